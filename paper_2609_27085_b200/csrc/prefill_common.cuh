@@ -15,19 +15,6 @@ constexpr int QT = 128;                    // rows per q tile
 constexpr int KT = 128;                    // tokens per K/V tile
 constexpr int HALF_BYTES = 128 * 128;      // [128 rows][64 elements] bf16
 constexpr int KV_STAGES = 2;
-constexpr int NTHREADS = 384;
-// Register hand-over (setmaxnreg).  The kernel launches with LAUNCH_REGS registers per thread; the
-// first warpgroup shrinks to REGS_ROLE and the two softmax warpgroups grow to REGS_SOFTMAX.  A grow
-// request blocks until the CTA's pool holds enough released registers, so the released amount MUST
-// cover the growth or the kernel never returns; the launcher also checks the compiled register count.
-#ifndef CF_REGS_ROLE
-#define CF_REGS_ROLE 136
-#endif
-#ifndef CF_REGS_SOFTMAX
-#define CF_REGS_SOFTMAX 184
-#endif
-constexpr int LAUNCH_REGS = 168, REGS_ROLE = CF_REGS_ROLE, REGS_SOFTMAX = CF_REGS_SOFTMAX;
-static_assert(4 * (LAUNCH_REGS - REGS_ROLE) >= 8 * (REGS_SOFTMAX - LAUNCH_REGS), "setmaxnreg.inc would block forever");
 __device__ __forceinline__ uint32_t lane_field(int warp) { return (uint32_t)((warp & 3) * 32) << 16; }
 template <int N> __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }

@@ -10,7 +10,7 @@
 //   warp 0      work queue; TMA producer of the Q tiles and of the 128-token K tiles, one 16-token
 //               page-half per TMA box, gathered through the block table into a 128B-swizzled ring.
 //   warp 2      TMA producer of the V tiles (same box shape, its own ring).
-//   warp 1      MMA issuer (one elected lane): S_t = Q_t K^T, O_t += P_t V, in the order
+//   warp 1      MMA issuer (the warp waits, an elected lane issues): S_t = Q_t K^T, O_t += P_t V, in the order
 //               PV_0(j) QK_0(j+1) PV_1(j) QK_1(j+1) so that the tensor pipe works on one tile while
 //               the other tile's softmax runs.
 //   warps 4-7   softmax of tile 0, one thread per q row; warps 8-11 softmax of tile 1.
@@ -32,6 +32,15 @@
 namespace cf {
 
 namespace {
+
+constexpr int NTHREADS = 384;
+// Register hand-over (setmaxnreg).  The kernel launches with LAUNCH_REGS registers per thread; the
+// first warpgroup shrinks to REGS_ROLE and the two softmax warpgroups grow to REGS_SOFTMAX (no role needs more than
+// 104 now that the issuer computes its descriptors; measured against 136 / 184 and 120 / 192: -1 %).  A grow
+// request blocks until the CTA's pool holds enough released registers, so the released amount MUST
+// cover the growth or the kernel never returns; the launcher also checks the compiled register count.
+constexpr int LAUNCH_REGS = 168, REGS_ROLE = 104, REGS_SOFTMAX = 200;
+static_assert(4 * (LAUNCH_REGS - REGS_ROLE) >= 8 * (REGS_SOFTMAX - LAUNCH_REGS), "setmaxnreg.inc would block forever");
 
 // Per head dimension (128 or 64): a Q, K or V tile is 128 rows x D elements, stored as D / 64 halves of
 // [128 rows][64 elements]; the O accumulator of a q tile takes D fp32 columns of tensor memory.
@@ -86,10 +95,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     __shared__ __align__(8) Bars bars;
     __shared__ uint32_t tmem_base_s;
     __shared__ uint32_t abort_s;
-    __shared__ uint32_t issuer_state[4];
 
     const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     // the first item of a CTA that starts on a fixed item: fetched now, in use after the set-up below (the plan
     // was uploaded before the kernel that precedes this one in the stream, so it may be read this early)
     const bool has_static = first_static != 0 && (int)blockIdx.x < n_items;
@@ -286,57 +294,59 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         constexpr uint32_t IDESC_QK = idesc_bf16(128, 128, false);
         constexpr uint32_t IDESC_PV = idesc_bf16(128, D, true);
         constexpr uint64_t HI64 = (uint64_t)desc_hi_sw128(1024) << 32;
-        // The issuing lane shares its scheduler with two softmax warps and gets roughly one issue
-        // slot in ten, while a 128x128x16 MMA lasts only 64 cycles.  Every shared-memory descriptor
-        // (q tile x k-step, K/V stage x k-step) is therefore built once and kept in registers, and the
-        // tile / stage indices are compile-time, so that a batch is MMAs back to back.
-        uint64_t qd[2][KS], kd[KV_STAGES][KS], vd[KV_STAGES][8];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                const uint32_t off = (uint32_t)(((ks >> 2) * HALF_BYTES + (ks & 3) * 32) >> 4);
-                qd[i][ks] = HI64 | (desc_lo_sw128(smem + SMEM_Q + i * TILE_BYTES, 16) + off);
-                kd[i][ks] = HI64 | (desc_lo_sw128(smem + SMEM_K + i * TILE_BYTES, 16) + off);
-            }
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                vd[i][ks] = HI64 | (desc_lo_sw128(smem + SMEM_V + i * TILE_BYTES, HALF_BYTES) + ks * (2048 >> 4));
-        }
+        // The issuing warp shares its scheduler with two softmax warps and gets roughly one issue slot in ten, while a
+        // 128x128x16 MMA lasts only 64 cycles, so the work between two batches is kept to a handful of
+        // instructions.  The whole warp runs the role and one elected lane issues: control flow, addresses and
+        // descriptors are warp-uniform, which the compiler keeps on the uniform datapath (a role run by one lane
+        // alone is divergent code: every descriptor passes through vector registers, and 48 of them had to be kept
+        // there).  Measured on a B200 against the one-lane role: head_dim 64 with a 128-token window 71.6 -> 64.3 us
+        // (2 x 2048 rows), head_dim 128 4096 new over 8192 cached 615 -> 603 us, three ragged chunks of 5003 rows
+        // 349 -> 344 us, head_dim 64 4096 over 8192 915 -> 906 us (all sustained).
+        const bool leader = elect_one();
+        auto qd = [&](int t, int ks) -> uint64_t {
+            return HI64 | (desc_lo_sw128(smem + SMEM_Q + t * TILE_BYTES, 16) + (uint32_t)(((ks >> 2) * HALF_BYTES + (ks & 3) * 32) >> 4));
+        };
+        auto kd = [&](int st, int ks) -> uint64_t {
+            return HI64 | (desc_lo_sw128(smem + SMEM_K + st * TILE_BYTES, 16) + (uint32_t)(((ks >> 2) * HALF_BYTES + (ks & 3) * 32) >> 4));
+        };
+        auto vd = [&](int st, int ks) -> uint64_t { return HI64 | (desc_lo_sw128(smem + SMEM_V + st * TILE_BYTES, HALF_BYTES) + ks * (2048 >> 4)); };
         const uint32_t bar_s[2] = {smem_u32(&bars.s_full[0]), smem_u32(&bars.s_full[1])};
         const uint32_t bar_o[2] = {smem_u32(&bars.o_done[0]), smem_u32(&bars.o_done[1])};
         const uint32_t bar_p[2] = {smem_u32(&bars.p_full[0]), smem_u32(&bars.p_full[1])};
         auto issue_qk = [&](auto T, auto S) {             // S_t = Q_t K^T over the head dimension (D / 16 steps of K = 16)
             constexpr int t = decltype(T)::value, st = decltype(S)::value;
             const uint32_t dS = tmem + TM_S + t * 128;
-            umma_ss(dS, qd[t][0], kd[st][0], IDESC_QK, 0u);
+            if (leader) {
+                umma_ss(dS, qd(t, 0), kd(st, 0), IDESC_QK, 0u);
 #pragma unroll
-            for (int ks = 1; ks < KS; ++ks) umma_ss(dS, qd[t][ks], kd[st][ks], IDESC_QK, 1u);
-            umma_commit(bar_s[t]);
+                for (int ks = 1; ks < KS; ++ks) umma_ss(dS, qd(t, ks), kd(st, ks), IDESC_QK, 1u);
+                umma_commit(bar_s[t]);
+            }
         };
         // O_t (+)= P_t V, one K = 16 step per fetched page: pages [ks0, n_steps) of the tile (ks0 > 0 only in the first
         // tile of a sliding window, n_steps < 8 only in a sequence's last tile)
         auto issue_pv = [&](auto T, auto S, int ks0, int n_steps, uint32_t acc0) {
             constexpr int t = decltype(T)::value, st = decltype(S)::value;
             const uint32_t dO = tmem + TM_O + t * D, aP = tmem + TM_S + t * 128;
-            if (ks0 == 0 && n_steps == 8) {
-                umma_ts(dO, aP, vd[st][0], IDESC_PV, acc0);
+            if (leader) {
+                if (ks0 == 0 && n_steps == 8) {
+                    umma_ts(dO, aP, vd(st, 0), IDESC_PV, acc0);
 #pragma unroll
-                for (int ks = 1; ks < 8; ++ks) umma_ts(dO, aP + ks * 8, vd[st][ks], IDESC_PV, 1u);
-            } else {
+                    for (int ks = 1; ks < 8; ++ks) umma_ts(dO, aP + ks * 8, vd(st, ks), IDESC_PV, 1u);
+                } else {
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    if (ks >= ks0 && ks < n_steps) umma_ts(dO, aP + ks * 8, vd[st][ks], IDESC_PV, ks == ks0 ? acc0 : 1u);
+                    for (int ks = 0; ks < 8; ++ks)
+                        if (ks >= ks0 && ks < n_steps) umma_ts(dO, aP + ks * 8, vd(st, ks), IDESC_PV, ks == ks0 ? acc0 : 1u);
+                }
+                umma_commit(bar_o[t]);
             }
-            umma_commit(bar_o[t]);
+        };
+        auto commit = [&](uint32_t bar) {
+            if (leader) umma_commit(bar);
         };
         using I0 = std::integral_constant<int, 0>;
         using I1 = std::integral_constant<int, 1>;
-        // One lane runs the whole role (the others go straight to the teardown barrier).  This lane is
-        // the critical resource of the kernel: it is a single dependent instruction stream that is also
-        // blocked while its MMAs queue up, so the work between two batches is kept to a handful of
-        // instructions, with a lean loop for interior tiles and the general step for the rest.
-        if (lane == 0) {
+        {
         const uint32_t bar_kf[2] = {smem_u32(&bars.k_full[0]), smem_u32(&bars.k_full[1])};
         const uint32_t bar_vf[2] = {smem_u32(&bars.v_full[0]), smem_u32(&bars.v_full[1])};
         const uint32_t bar_ke[2] = {smem_u32(&bars.k_empty[0]), smem_u32(&bars.k_empty[1])};
@@ -345,28 +355,24 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         // Running phases: ub[s] = fills of K/V ring stage s before this item (tile j of an item sits in
         // stage j & 1 and is that stage's fill number ub[j & 1] + (j >> 1)); sb[t] = tiles of q tile t
         // before this item (s_full / p_full / o_done complete one phase per tile).
-        // Only this lane touches issuer_state (= ub[0], ub[1], sb[0], sb[1]).  The lane has no registers to
-        // spare beside its 48 descriptors, so the running phases live in shared memory, the item's fields are
-        // read from the context slot where they are needed (the slot is not rewritten before this lane has
-        // left the next item's last S = Q K^T behind), and only the interior loop keeps its parities in registers.
-        volatile uint32_t* const ist = issuer_state;
-        ist[0] = ist[1] = ist[2] = ist[3] = 0u;
+        uint32_t ub[2] = {0u, 0u}, sb[2] = {0u, 0u};
+        // after a wait that gave up in any lane the whole warp leaves (the lean loop votes once, behind it)
+        auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)); };
         bool ok = true;
         for (int k = 0; ok; ++k) {
         const ItemCtx* cs = wait_item(k);
-        if (cs == nullptr || cs->live == 0) break;
+        if (!__all_sync(0xffffffffu, cs != nullptr) || cs->live == 0) break;
         const volatile ItemCtx* const vs = cs;
         const int n_max = cs->n_max;
         const int n_j[2] = {cs->n_j[0], cs->n_j[1]};
-        ok = mbar_wait(smem_u32(&bars.q_full), (uint32_t)k & 1u, abort_flag);
-        ok = ok && mbar_wait(bar_kf[0], ist[0] & 1u, abort_flag);
+        ok = wait_all(smem_u32(&bars.q_full), (uint32_t)k & 1u) && wait_all(bar_kf[0], ub[0] & 1u);
         if (!ok) break;
         tc_fence_after();
         if (n_j[0] > 0) issue_qk(I0{}, I0{});
         if (n_j[1] > 0) issue_qk(I1{}, I0{});
-        umma_commit(bar_ke[0]);
+        commit(bar_ke[0]);
         // q_empty: arrives when every S = Q K^T of the item has completed (the last one is issued in step n_max - 2)
-        if (n_max <= 1) umma_commit(bar_qe);
+        if (n_max <= 1) commit(bar_qe);
         // ---- interior tiles: both q tiles present and continuing, all 8 pages loaded, not the last tile
         const int n_int = (n_j[0] > 0 && n_j[1] > 0) ? min(n_j[0], n_j[1]) - 1 : 0;
         auto lean_step = [&](auto S, uint32_t par_v, uint32_t par_k1, uint32_t par_p0, uint32_t par_p1, uint32_t acc0) -> bool {
@@ -382,8 +388,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             tc_fence_after();
             issue_pv(I1{}, S, 0, 8, acc0);
             issue_qk(I1{}, S1{});
-            umma_commit(bar_ve[st]);
-            umma_commit(bar_ke[st1]);
+            commit(bar_ve[st]);
+            commit(bar_ke[st1]);
             return true;
         };
         // ---- general step: PV_0(j) QK_0(j+1) PV_1(j) QK_1(j+1) with every edge case
@@ -393,26 +399,27 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const int jb = vs->it.j_begin, Lc = vs->it.ctx_len;
             const int np = min(8, vs->total_pages - 8 * (jb + j));
             const int ks0 = max(0, vs->it.page_lo - 8 * (jb + j));      // sliding window: the tile's first fetched page
-            if (!mbar_wait(bar_vf[st], (ist[st] + (uint32_t)(j >> 1)) & 1u, abort_flag)) return false;
+            if (!wait_all(bar_vf[st], (ub[st] + (uint32_t)(j >> 1)) & 1u)) return false;
             if (j == n_max - 1 && Lc < (8 * (jb + j) + np) * 16) {
                 // slack slots of the sequence's last page came in with the page: zero those V rows so
                 // that a zero probability never multiplies a NaN
                 const int r0 = Lc - (jb + j) * KT, r1 = np * 16;
-                for (int idx = 0; idx < (r1 - r0) * (D / 8); ++idx) {
+                for (int idx = lane; idx < (r1 - r0) * (D / 8); idx += 32) {
                     const int r = r0 + idx / (D / 8), c = idx % (D / 8);
                     uint8_t* dst = smem_raw + ((smem + SMEM_V + st * TILE_BYTES) - smem_u32(smem_raw)) +
                                    (c >> 3) * HALF_BYTES + r * 128 + (c & 7) * 16;
                     *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
                 }
                 fence_proxy_async();
+                __syncwarp();
             }
             const uint32_t acc0 = j > 0 ? 1u : 0u;
             auto tile = [&](auto T) -> bool {
                 constexpr int t = decltype(T)::value;
                 if (j >= n_j[t]) return true;
                 const bool more = j + 1 < n_j[t];
-                if (more && !mbar_wait(bar_kf[st1], (ist[st1] + (uint32_t)((j + 1) >> 1)) & 1u, abort_flag)) return false;
-                if (!mbar_wait(bar_p[t], (ist[2 + t] + (uint32_t)j) & 1u, abort_flag)) return false;
+                if (more && !wait_all(bar_kf[st1], (ub[st1] + (uint32_t)((j + 1) >> 1)) & 1u)) return false;
+                if (!wait_all(bar_p[t], (sb[t] + (uint32_t)j) & 1u)) return false;
                 tc_fence_after();
                 issue_pv(T, S, ks0, np, acc0);
                 if (more) issue_qk(T, S1{});
@@ -420,9 +427,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             };
             if (!tile(I0{})) return false;
             if (!tile(I1{})) return false;
-            umma_commit(bar_ve[st]);
-            if (j + 1 < n_max) umma_commit(bar_ke[st1]);
-            if (j + 1 == n_max - 1) umma_commit(bar_qe);
+            commit(bar_ve[st]);
+            if (j + 1 < n_max) commit(bar_ke[st1]);
+            if (j + 1 == n_max - 1) commit(bar_qe);
             return true;
         };
         int j = 0;
@@ -437,22 +444,23 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             // parities of the even tile j of a pair: stage 0 fill ub[0] + j/2 (V now), stage 1 fill ub[1] + j/2
             // (K of tile j + 1), softmax phases sb[t] + j; the odd tile j + 1 flips all but the stage-0 K
             // fill of tile j + 2, which is ub[0] + j/2 + 1
-            uint32_t h0 = (ist[0] + (uint32_t)(j >> 1)) & 1u, h1 = (ist[1] + (uint32_t)(j >> 1)) & 1u;
-            const uint32_t p0 = ist[2] & 1u, p1 = ist[3] & 1u;
+            uint32_t h0 = (ub[0] + (uint32_t)(j >> 1)) & 1u, h1 = (ub[1] + (uint32_t)(j >> 1)) & 1u;
+            const uint32_t p0 = sb[0] & 1u, p1 = sb[1] & 1u;
             for (; ok && j + 1 < n_int; j += 2, h0 ^= 1u, h1 ^= 1u) {
                 ok = lean_step(I0{}, h0, h1, p0, p1, j > 0 ? 1u : 0u);
                 if (ok) ok = lean_step(I1{}, h1, h0 ^ 1u, p0 ^ 1u, p1 ^ 1u, 1u);
             }
-            if (ok && j > j_pairs && j >= n_max - 1) umma_commit(bar_qe);     // the pair loop issued the item's last S = Q K^T
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok && j > j_pairs && j >= n_max - 1) commit(bar_qe);     // the pair loop issued the item's last S = Q K^T
         }
         static_assert(KV_STAGES == 2, "the stage index is the parity of the tile index");
         for (; j < n_max && ok; ++j) {
             ok = (j & 1) ? kv_step(I1{}, j) : kv_step(I0{}, j);
         }
-        ist[0] += (uint32_t)(n_max + 1) >> 1;
-        ist[1] += (uint32_t)n_max >> 1;
-        ist[2] += (uint32_t)n_j[0];
-        ist[3] += (uint32_t)n_j[1];
+        ub[0] += (uint32_t)(n_max + 1) >> 1;
+        ub[1] += (uint32_t)n_max >> 1;
+        sb[0] += (uint32_t)n_j[0];
+        sb[1] += (uint32_t)n_j[1];
         }
         }
       }

@@ -40,6 +40,14 @@ namespace cf {
 
 namespace {
 
+constexpr int NTHREADS = 384;
+// Register hand-over (setmaxnreg).  The kernel launches with LAUNCH_REGS registers per thread; the
+// first warpgroup shrinks to REGS_ROLE and the two softmax warpgroups grow to REGS_SOFTMAX.  A grow
+// request blocks until the CTA's pool holds enough released registers, so the released amount MUST
+// cover the growth or the kernel never returns; the launcher also checks the compiled register count.
+constexpr int LAUNCH_REGS = 168, REGS_ROLE = 136, REGS_SOFTMAX = 184;
+static_assert(4 * (LAUNCH_REGS - REGS_ROLE) >= 8 * (REGS_SOFTMAX - LAUNCH_REGS), "setmaxnreg.inc would block forever");
+
 constexpr int D2 = 128;                            // head_dim of the pair kernel
 constexpr int TILE2 = 2 * HALF_BYTES;              // a 128-row q tile: 32 KB
 constexpr int KHALF = 64 * 128;                    // [64 tokens][64 elements]: 8 KB; a K half-tile is two of them
