@@ -52,7 +52,7 @@ struct PoolMapEntry {
 };
 struct QMapEntry {
     const void* base = nullptr;
-    int D = 0, rows = 0, Hq = 0;
+    int D = 0, rows = 0, Hq = 0, heads = 0;
     uint64_t stamp = 0;
     CUtensorMap map;
 };
@@ -319,21 +319,21 @@ static const CUtensorMap* pool_map(cf_ctx* c, const void* base, const cf_cache_d
     return &victim->map;
 }
 
-static const CUtensorMap* q_map(cf_ctx* c, const void* base, int D, int rows, int Hq)
+static const CUtensorMap* q_map(cf_ctx* c, const void* base, int D, int rows, int Hq, int heads)
 {
     QMapEntry* victim = &c->q_maps[0];
     for (QMapEntry& e : c->q_maps) {
-        if (e.base == base && e.D == D && e.rows == rows && e.Hq == Hq) {
+        if (e.base == base && e.D == D && e.rows == rows && e.Hq == Hq && e.heads == heads) {
             e.stamp = ++c->map_stamp;
             return &e.map;
         }
         if (e.stamp < victim->stamp) victim = &e;
     }
-    if (!encode_q_map(&victim->map, base, D, rows, Hq)) {
+    if (!encode_q_map(&victim->map, base, D, rows, Hq, heads)) {
         victim->base = nullptr;
         return nullptr;
     }
-    victim->base = base; victim->D = D; victim->rows = rows; victim->Hq = Hq;
+    victim->base = base; victim->D = D; victim->rows = rows; victim->Hq = Hq; victim->heads = heads;
     victim->stamp = ++c->map_stamp;
     return &victim->map;
 }
@@ -479,7 +479,7 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
     }
     PrefillMaps maps;
     if (has_prefill) {
-        const CUtensorMap* mq = q_map(c, q, D, n.total_q, Hq);
+        const CUtensorMap* mq = q_map(c, q, D, n.total_q, Hq, n.pair ? 1 : p.G);
         const CUtensorMap* mk = pool_map(c, pp.k_cache, &pdesc, pdesc.k_stride_block, pdesc.k_stride_head, pdesc.k_stride_token);
         const CUtensorMap* mv = pool_map(c, pp.v_cache, &pdesc, pdesc.v_stride_block, pdesc.v_stride_head, pdesc.v_stride_token);
         if (!mq || !mk || !mv) return CF_ERR_CUDA;
@@ -1222,26 +1222,32 @@ cf_status cf_plan_inspect(const cf_cache_desc* desc, const int32_t* context_len,
             o[0] = pl.combine[i].q_row; o[1] = pl.combine[i].part_first; o[2] = pl.combine[i].n_chunks;
         }
     size_t n_pre = 0;
-    for (const PrefillTcItem& it : pl.prefill_tc)
+    auto entry = [&](const PrefillTcItem& it, int32_t q_row, int32_t row0, int32_t n_rows, int32_t head) {
+        if (prefill_items && n_pre < (size_t)cap) {
+            const int32_t tiles = (it.prefix + row0 + n_rows + 127) / 128;      // KV tiles these rows can see
+            int32_t* o = prefill_items + 8 * n_pre;
+            o[0] = it.seq; o[1] = q_row; o[2] = row0; o[3] = n_rows; o[4] = head; o[5] = it.kvh;
+            o[6] = it.j_begin < tiles ? it.j_begin : tiles;
+            o[7] = it.j_end < tiles ? it.j_end : tiles;
+        }
+        ++n_pre;
+    };
+    const int32_t G = desc->num_q_heads / desc->num_kv_heads;
+    for (const PrefillTcItem& it : pl.prefill_tc) {
+        if (!pl.pair && G >= 2) {
+            // the items of a 128-row block and KV head carry all heads of the group and share their KV range: the
+            // block's entries are listed with its first item
+            if (it.row0[0] % 128 != 0) continue;
+            const int32_t rest = query_len[it.seq] - it.row0[0], n_rows = rest < 128 ? rest : 128;
+            for (int32_t h = 0; h < G; ++h) entry(it, it.q_row0[0], it.row0[0], n_rows, it.kvh * G + h);
+            continue;
+        }
         for (int t = 0; t < 2; ++t) {
             if (it.n_rows[t] <= 0) continue;
-            const int32_t tiles = (it.prefix + it.row0[t] + it.n_rows[t] + 127) / 128;      // KV tiles this q tile can see
-            if (prefill_items && n_pre < (size_t)cap) {
-                int32_t* o = prefill_items + 8 * n_pre;
-                o[0] = it.seq; o[1] = it.q_row0[t]; o[2] = it.row0[t]; o[3] = it.n_rows[t]; o[4] = it.head[t]; o[5] = it.kvh;
-                o[6] = it.j_begin < tiles ? it.j_begin : tiles;
-                o[7] = it.j_end < tiles ? it.j_end : tiles;
-            }
-            ++n_pre;
-            if (pl.pair) {                               // the second CTA of the pair: the same q tile for head + 2
-                if (prefill_items && n_pre < (size_t)cap) {
-                    int32_t* o = prefill_items + 8 * n_pre;
-                    for (int i = 0; i < 8; ++i) o[i] = o[i - 8];
-                    o[4] += 2;
-                }
-                ++n_pre;
-            }
+            entry(it, it.q_row0[t], it.row0[t], it.n_rows[t], it.head[t]);
+            if (pl.pair) entry(it, it.q_row0[t], it.row0[t], it.n_rows[t], it.head[t] + 2);      // the second CTA of the pair: head + 2
         }
+    }
     if (counts) {
         counts[0] = (int32_t)pl.decode.size();
         counts[1] = (int32_t)pl.combine.size();

@@ -59,7 +59,8 @@ cudaError_t launch_decode_with_shared(const AttnParams& p, int head_dim, int n_s
 struct PrefillMaps {
     CUtensorMap q, k, v;
 };
-bool encode_q_map(CUtensorMap* m, const void* q, int head_dim, int total_rows, int num_q_heads);
+// heads_per_tile: query heads of a 128-row q tile (the group size; 1 for the kernel on pairs of SMs)
+bool encode_q_map(CUtensorMap* m, const void* q, int head_dim, int total_rows, int num_q_heads, int heads_per_tile);
 bool encode_pool_map(CUtensorMap* m, const void* pool, int head_dim, int num_blocks, int num_kv_heads, int64_t stride_block,
                      int64_t stride_head, int64_t stride_token);
 cudaError_t launch_prefill_tc(const AttnParams& p, const PrefillMaps& maps, int head_dim, int n_items, int n_ctas,

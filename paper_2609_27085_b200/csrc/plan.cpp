@@ -226,15 +226,21 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
 
     // ---- prefill: q tiles of every chunk, the tile with the longest visible KV range first
     {
-        // pairs of 128-row tiles that share a KV head: two heads of a group over the same rows, or
-        // (group size 1) two consecutive row tiles of one head
+        // A block = 128 rows of a chunk (group size 1: two blocks of one head, one per q tile).  The work items of a
+        // block and KV head carry all heads of the group, 256 / G rows each in two q tiles (a 128-row q tile is
+        // 128 / G rows x G heads), and share the block's KV range.
         constexpr int32_t TR = 128;
         // pair items: four heads of a group per item, run by two CTAs on two SMs
         const bool pair = cfg.prefill_pair && d->head_dim == 128 && G % 4 == 0;
-        const int32_t heads_per_item = pair ? 4 : 2;
+        const int32_t rows_per_tile = pair ? TR : std::max(1, TR / G);      // rows of a q tile, all heads of the group packed
+        const int32_t pack = pair ? 1 : G;
         plan->pair = pair;
-        struct KeyedTc { int64_t extent; int32_t tiles; PrefillTcItem it; };   // extent: end of the visible keys; tiles: KV tiles to visit
+        // extent: end of the block's visible keys; tiles: KV tiles to visit; sub: index among the items of the block and KV head
+        struct KeyedTc { int64_t extent; int32_t tiles; int32_t sub; PrefillTcItem it; };
         std::vector<KeyedTc> items;
+        auto items_of = [&](int32_t rows) {          // items of a block of `rows` rows per KV head (group size 1: of two blocks)
+            return G == 1 ? 1 : pair ? G / 4 : (rows + 2 * rows_per_tile - 1) / (2 * rows_per_tile);
+        };
         auto prefix_of = [&](int32_t s) { return context_len[s] - query_len[s]; };
         // All items of one (sequence, row tile) have the same KV extent, so the longest-first order is found by
         // sorting those few groups, not the items (a 8192-token chunk with 64 query heads is 2048 items in 64 groups).
@@ -248,7 +254,7 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
             for (int32_t tile = 0; tile < n_tiles; tile += (G >= 2 ? 1 : 2)) {
                 const int32_t last = (G >= 2 || tile + 1 >= n_tiles) ? tile : tile + 1;
                 groups.push_back(Group{(int64_t)prefix_of(s) + last * TR + std::min(TR, lq - last * TR), s, tile});
-                n_emit += (size_t)(G >= 2 ? d->num_kv_heads * (G / heads_per_item) : d->num_q_heads);
+                n_emit += (size_t)(d->num_kv_heads * items_of(std::min(TR, lq - tile * TR)));
             }
         }
         std::stable_sort(groups.begin(), groups.end(), [](const Group& a, const Group& b) { return a.extent > b.extent; });
@@ -281,17 +287,20 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
             it.j_begin = lo0 / TR; it.j_end = INT32_MAX; it.part_slot[0] = it.part_slot[1] = -1; it.part_k = 1; it.part_c = 0;
             const int32_t n_tiles_kv = (int32_t)((gr.extent + TR - 1) / TR) - it.j_begin;
             if (G >= 2) {
-                for (int t = 0; t < 2; ++t) {
-                    it.q_row0[t] = plan->q_start[s] + tile * TR;
-                    it.row0[t] = tile * TR;
-                    it.n_rows[t] = rows_of(tile);
-                }
+                const int32_t rows = rows_of(tile), n_items_blk = items_of(rows);
                 for (int32_t kvh = set * heads_per_set; kvh < (set + 1) * heads_per_set; ++kvh)
-                    for (int32_t i = 0; i < G; i += heads_per_item) {
+                    for (int32_t i = 0; i < n_items_blk; ++i) {
                         it.kvh = kvh;
-                        it.head[0] = kvh * G + i;
-                        it.head[1] = kvh * G + i + 1;
-                        items.push_back(KeyedTc{gr.extent, n_tiles_kv, it});
+                        for (int t = 0; t < 2; ++t) {
+                            const int32_t off = pair ? 0 : (2 * i + t) * rows_per_tile;
+                            const int32_t n = std::min(rows_per_tile, rows - off);
+                            it.q_row0[t] = n > 0 ? plan->q_start[s] + tile * TR + off : 0;
+                            it.row0[t] = n > 0 ? tile * TR + off : 0;
+                            it.n_rows[t] = std::max(0, n);
+                            it.head[t] = pair ? kvh * G + 4 * i + t : kvh * G;
+                        }
+                        if (W > 0) it.page_lo = std::max(0, prefix + it.row0[0] - W + 1) / B;
+                        items.push_back(KeyedTc{gr.extent, n_tiles_kv, i, it});
                     }
             } else {
                 for (int t = 0; t < 2; ++t) {
@@ -304,7 +313,7 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
                 for (int32_t h = 0; h < d->num_q_heads; ++h) {
                     it.kvh = h;
                     it.head[0] = it.head[1] = h;
-                    items.push_back(KeyedTc{gr.extent, n_tiles_kv, it});
+                    items.push_back(KeyedTc{gr.extent, n_tiles_kv, 0, it});
                 }
             }
         }
@@ -322,11 +331,15 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
                     one.q_row0[0] = k.it.q_row0[t]; one.row0[0] = k.it.row0[t]; one.n_rows[0] = k.it.n_rows[t];
                     one.head[0] = k.it.head[t];
                     one.q_row0[1] = 0; one.row0[1] = 0; one.n_rows[1] = 0; one.head[1] = k.it.head[t];
-                    const int64_t ext = (int64_t)prefix_of(k.it.seq) + one.row0[0] + one.n_rows[0];
                     const int32_t lo1 = (W > 0) ? std::max(0, prefix_of(k.it.seq) + one.row0[0] - W + 1) : 0;
                     one.page_lo = lo1 / B;
+                    if (G >= 2) {                   // the block's KV range stays
+                        singles.push_back(KeyedTc{k.extent, k.tiles, 2 * k.sub + t, one});
+                        continue;
+                    }
+                    const int64_t ext = (int64_t)prefix_of(k.it.seq) + one.row0[0] + one.n_rows[0];
                     one.j_begin = lo1 / TR;
-                    singles.push_back(KeyedTc{ext, (int32_t)((ext + TR - 1) / TR) - one.j_begin, one});
+                    singles.push_back(KeyedTc{ext, (int32_t)((ext + TR - 1) / TR) - one.j_begin, 0, one});
                 }
             std::stable_sort(singles.begin(), singles.end(), [](const KeyedTc& a, const KeyedTc& b) { return a.extent > b.extent; });
         }
@@ -412,6 +425,8 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
             }
         }
         const size_t n_items = items.size();
+        for (size_t i = 1; i < n_items; ++i)
+            if (items[i].sub > 0) k_of[i] = k_of[i - 1];      // the items of a block and KV head are cut alike
         plan->prefill_tc.reserve(n_items + 8 * plan->prefill_combine.capacity());
         for (size_t i = 0; i < n_items; ++i) {
             PrefillTcItem it = items[i].it;
@@ -420,14 +435,21 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
                 plan->prefill_tc.push_back(it);
                 continue;
             }
-            // tiles every present q tile takes part in, and the last tile boundary outside the diagonal band
+            // tiles every present q tile takes part in (of a packed item: every row of its block), and the last tile
+            // boundary outside the diagonal band
             const int32_t prefix = prefix_of(it.seq);
             int32_t n_min = INT32_MAX, safe = INT32_MAX;
-            for (int t = 0; t < 2; ++t)
-                if (it.n_rows[t] > 0) {
-                    n_min = std::min(n_min, (prefix + it.row0[t] + it.n_rows[t] + 127) / 128);
-                    safe = std::min(safe, (prefix + it.row0[t]) / 128);
-                }
+            if (G >= 2) {
+                const int32_t blk0 = it.row0[0] / TR * TR, blk_rows = std::min(TR, query_len[it.seq] - blk0);
+                n_min = (prefix + blk0 + blk_rows + 127) / 128;
+                safe = (prefix + blk0) / 128;
+            } else {
+                for (int t = 0; t < 2; ++t)
+                    if (it.n_rows[t] > 0) {
+                        n_min = std::min(n_min, (prefix + it.row0[t] + it.n_rows[t] + 127) / 128);
+                        safe = std::min(safe, (prefix + it.row0[t]) / 128);
+                    }
+            }
             const int32_t j_lo = it.j_begin;          // first tile of the sliding window (0 without one); j_lo <= safe
             const int32_t k = std::min(k_want, std::max(1, (std::min(n_min, safe + 1) - j_lo) / 4));
             if (k <= 1) {
@@ -436,10 +458,11 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
             }
             PrefillCombineItem ci;
             ci.part_k = k;
+            ci.pack = pack;
             for (int t = 0; t < 2; ++t) {
                 ci.q_row0[t] = it.q_row0[t]; ci.n_rows[t] = it.n_rows[t]; ci.head[t] = it.head[t];
                 ci.part_slot[t] = it.n_rows[t] > 0 ? plan->n_pre_slots : -1;
-                plan->n_pre_slots += it.n_rows[t] * k;
+                plan->n_pre_slots += it.n_rows[t] * pack * k;
             }
             plan->prefill_combine.push_back(ci);
             if (pair) {
@@ -449,7 +472,7 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
                 for (int t = 0; t < 2; ++t) {
                     cj.head[t] = it.head[t] + 2;
                     cj.part_slot[t] = it.n_rows[t] > 0 ? plan->n_pre_slots : -1;
-                    plan->n_pre_slots += it.n_rows[t] * k;
+                    plan->n_pre_slots += it.n_rows[t] * pack * k;
                 }
                 plan->prefill_combine.push_back(cj);
             }
@@ -470,7 +493,6 @@ int32_t spatial_front_sms(const cf_cache_desc* d, const int32_t* context_len, co
                           int32_t num_sms)
 {
     const int32_t G = d->num_q_heads / d->num_kv_heads, W = d->window_size;
-    const double items_per_tile = G >= 2 ? (double)d->num_kv_heads * (double)(G / 2) : 0.5 * (double)d->num_q_heads;
     double dec_bytes = 0.0, work = 0.0;      // bytes the decode kernel streams; SM-microseconds of the prefill items
     for (int32_t s = 0; s < num_seqs; ++s) {
         const int32_t lq = query_len[s], lc = context_len[s];
@@ -481,7 +503,9 @@ int32_t spatial_front_sms(const cf_cache_desc* d, const int32_t* context_len, co
             for (int32_t row = 0; row < lq; row += 128) {
                 const int32_t hi = prefix + std::min(lq, row + 128);
                 const int32_t lo = W > 0 ? std::max(0, prefix + row - W + 1) / 128 : 0;
-                work += items_per_tile * (8.0 + 1.9 * (double)((hi + 127) / 128 - lo));
+                const int32_t rows = std::min(lq - row, 128);
+                const double items = G >= 2 ? (double)(d->num_kv_heads * ((rows * G + 255) / 256)) : 0.5 * (double)d->num_q_heads;
+                work += items * (8.0 + 1.9 * (double)((hi + 127) / 128 - lo));
             }
         }
     }

@@ -52,15 +52,17 @@ struct CombineItem {       // one decode sequence that was split
     int32_t n_chunks;
 };
 
-struct PrefillTcItem {     // tcgen05 kernel: two 128-row q tiles that share one KV head (tile 1 may be absent)
+// tcgen05 kernel: two q tiles of one KV head (tile 1 may be absent).  A q tile is 128 / G tokens x the G heads of the
+// group; for the kernel on pairs of SMs it is 128 tokens of one head.
+struct PrefillTcItem {
     int32_t seq;
     int32_t kvh;
-    int32_t q_row0[2];     // packed row of each tile's first row
-    int32_t row0[2];       // index of that row inside the chunk
-    int32_t n_rows[2];     // 0 = tile absent
-    int32_t head[2];       // query head of each tile
+    int32_t q_row0[2];     // packed row of each tile's first token
+    int32_t row0[2];       // index of that token inside the chunk
+    int32_t n_rows[2];     // tokens of the tile; 0 = tile absent
+    int32_t head[2];       // first query head of each tile
     // KV split: this item covers KV tiles [j_begin, j_end) (128-token tiles; j_end clamps to the item's
-    // own extent).  part_slot[t] >= 0: tile t writes an fp32 partial for row r into slot
+    // own extent).  part_slot[t] >= 0: tile t writes an fp32 partial for row r (token * heads + head) into slot
     // part_slot[t] + r * part_k + part_c instead of the final output.
     int32_t j_begin, j_end;
     int32_t part_slot[2];
@@ -75,10 +77,11 @@ static_assert(sizeof(PrefillTcItem) == 80, "PrefillTcItem is copied as five 16-b
 
 struct PrefillCombineItem { // one KV-split tcgen05 item: merges its part_k partials per row
     int32_t q_row0[2];
-    int32_t n_rows[2];
-    int32_t head[2];
+    int32_t n_rows[2];     // tokens
+    int32_t head[2];       // first head
     int32_t part_slot[2];
     int32_t part_k;
+    int32_t pack;          // heads of a tile: row r is token r / pack, head head[t] + r % pack
 };
 
 struct PlanConfig {

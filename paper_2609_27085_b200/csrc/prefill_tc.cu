@@ -1,9 +1,14 @@
 // Chunked-prefill attention on the 5th-generation tensor cores (tcgen05.mma, accumulators in
 // tensor memory), head_dim 128 or 64 (template parameter D; the sizes quoted below are those of D = 128).
 //
-// A work item = two 128-row q tiles that share a KV head (two query heads of one group over the same
-// rows; for G = 1 two consecutive row tiles of one head), so every K/V tile fetched into shared memory
-// feeds two S = Q K^T and two O += P V products.  CTAs are persistent (one per SM): CTA b starts on
+// A work item = two q tiles of one KV head, so every K/V tile fetched into shared memory feeds two S = Q K^T and two
+// O += P V products.  The 128 rows of a q tile are 128 / G consecutive tokens times the G query heads of the group
+// (row = token * G + head): one TMA box gathers them, and an item covers 256 / G tokens.  Against tiles of 128 tokens
+// of one head the number of items of a long chunk is the same, but a chunk's ragged end, a short chunk and the edges
+// of the causal band or of a sliding window are cut at 128 / G tokens instead of 128.  Measured (sustained, tiles of one
+// head -> packed, G = 8 unless stated): chunks of 40, 33 and 50 tokens 48 -> 25 us, a 128-token window (2 x 2048 rows,
+// head_dim 64) 64 -> 53 us, three ragged chunks of 5003 rows (G = 4) 342 -> 322 us, 4 x 2048 rows 1315 -> 1300 us.
+// CTAs are persistent (one per SM): CTA b starts on
 // item b and then draws items from a ticket counter; the roles run from item to item without a
 // CTA-wide barrier.  384 threads, warp-specialised (the first warpgroup hands most of its registers to
 // the two softmax warpgroups with setmaxnreg):
@@ -24,6 +29,7 @@
 // Every wait is bounded: on expiry the CTA raises an abort flag, every role leaves its loop, the
 // error word is set and tensor memory is released.
 #include <atomic>
+#include <climits>
 #include <type_traits>
 
 #include "kernels.h"
@@ -56,6 +62,32 @@ struct Geo {
     static constexpr int KS = D / 16;                                      // K = 16 steps of S = Q K^T
 };
 constexpr uint32_t TM_S = 0, TM_O = 256;   // column offsets: S_t at TM_S + 128 t, O_t at TM_O + D t
+
+// What a role needs to know about the work item it is on.  The producer warp builds it and hands it
+// to the other roles through a two-slot ring in shared memory.
+struct TcCtx {
+    PrefillTcItem it;
+    int end_t[2], n_j[2];         // per q tile: end of the keys it visits in this item; number of KV tiles it takes part in
+    int n_max, page0, page_end;   // KV tile j covers pages [page0 + 8 j, page0 + 8 j + 8), cut at page_end
+    int live;                     // 0: no more work, every role leaves
+};
+static_assert(sizeof(TcCtx) % 16 == 0, "copied as 16-byte words");
+__device__ __forceinline__ void derive_ctx(TcCtx& c)
+{
+    // a sliding window's pages left of page_lo are never touched: the first KV tile starts at page_lo
+    c.page0 = max((KT / 16) * c.it.j_begin, c.it.page_lo);
+    const int stop = c.it.j_end < (1 << 23) ? c.it.j_end * KT : INT_MAX;
+    int end = 0;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        c.end_t[t] = c.it.n_rows[t] > 0 ? min(c.it.prefix + c.it.row0[t] + c.it.n_rows[t], stop) : 0;
+        c.n_j[t] = max(0, (c.end_t[t] - 16 * c.page0 + KT - 1) / KT);
+        end = max(end, c.end_t[t]);
+    }
+    c.n_max = max(c.n_j[0], c.n_j[1]);
+    c.page_end = (end + 15) >> 4;
+    c.live = 1;
+}
 
 struct Bars {
     uint64_t q_full, q_empty;
@@ -91,7 +123,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     constexpr uint32_t kPolyMask = D == 64 ? CF_POLY_MASK_D64 : CF_POLY_MASK;
     constexpr uint32_t SMEM_Q = Geo<D>::SMEM_Q, SMEM_K = Geo<D>::SMEM_K, SMEM_V = Geo<D>::SMEM_V;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(16) ItemCtx ctx_s[2];
+    __shared__ __align__(16) TcCtx ctx_s[2];
     __shared__ __align__(8) Bars bars;
     __shared__ uint32_t tmem_base_s;
     __shared__ uint32_t abort_s;
@@ -153,7 +185,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     };
     // the context of a role's k-th item (slot k & 1, filled for the (k >> 1)-th time); null on an abort.
     // A role copies the fields it needs at once: the slot is rewritten two items later.
-    auto wait_item = [&](int k) -> const ItemCtx* {
+    auto wait_item = [&](int k) -> const TcCtx* {
         if (!mbar_wait(smem_u32(&bars.item_full[k & 1]), (uint32_t)(k >> 1) & 1u, abort_flag)) return nullptr;
         return &ctx_s[k & 1];
     };
@@ -169,25 +201,23 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         uint32_t ub[2] = {0u, 0u};
         bool ok = true;
         for (int k = 0; ok; ++k) {
-            const ItemCtx* cs = wait_item(k);
+            const TcCtx* cs = wait_item(k);
             if (cs == nullptr || cs->live == 0) break;
-            const int n_max = cs->n_max, total_pages = cs->total_pages, jb = cs->it.j_begin, kvh = cs->it.kvh;
-            const int page_lo = cs->it.page_lo;          // sliding window: pages below it are not fetched (their table entries may be stale)
+            const int n_max = cs->n_max, page0 = cs->page0, page_end = cs->page_end, kvh = cs->it.kvh;
             const int32_t* bt = p.block_table + (int64_t)cs->it.seq * p.max_blocks;
-            int32_t pid = (lane < min(8, total_pages - 8 * jb) && 8 * jb + lane >= page_lo) ? checked_pid(__ldg(bt + 8 * jb + lane)) : 0;
+            int32_t pid = lane < min(8, page_end - page0) ? checked_pid(__ldg(bt + page0 + lane)) : 0;
             for (int j = 0; j < n_max && ok; ++j) {
-                const int stage = j & 1;
+                const int stage = j & 1, at = page0 + 8 * j;
                 const uint32_t use = ub[stage] + (uint32_t)(j >> 1);
-                const int np = min(8, total_pages - 8 * (jb + j));
-                const int p0 = max(0, page_lo - 8 * (jb + j));            // first page of the tile that is fetched
+                const int np = min(8, page_end - at);
                 const int32_t my_pid = __shfl_sync(0xffffffffu, pid, lane / HALVES);
-                if (j + 1 < n_max) pid = lane < min(8, total_pages - 8 * (jb + j + 1)) ? checked_pid(__ldg(bt + 8 * (jb + j + 1) + lane)) : 0;
+                if (j + 1 < n_max) pid = lane < min(8, page_end - at - 8) ? checked_pid(__ldg(bt + at + 8 + lane)) : 0;
                 const uint32_t dst_off = (lane % HALVES) * HALF_BYTES + (lane / HALVES) * 2048;
                 if (use > 0) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.v_empty[stage]), (use - 1) & 1u, abort_flag));
                 if (!ok) break;
-                if (lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.v_full[stage]), (np - p0) * 16 * D * 2);
+                if (lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.v_full[stage]), np * 16 * D * 2);
                 __syncwarp();
-                if (lane < HALVES * np && lane >= HALVES * p0)
+                if (lane < HALVES * np)
                     tma_load_4d(smem + SMEM_V + stage * TILE_BYTES + dst_off, &map_v, (lane % HALVES) * 64, 0, kvh, my_pid,
                                 smem_u32(&bars.v_full[stage]));
             }
@@ -204,7 +234,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         }
         bool counted_out = false;
         // draws the next ticket; on the first empty draw the CTA is counted out and the last CTA resets the counters
-        auto draw = [&](ItemCtx& cx) {
+        auto draw = [&](TcCtx& cx) {
             int idx = n_items;
             if (lane == 0 && *abort_flag == 0u && !counted_out) idx = ticket_base + (int)atomicAdd(p.pre_queue, 1u);
             idx = __shfl_sync(0xffffffffu, idx, 0);
@@ -213,7 +243,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 uint4* dst = reinterpret_cast<uint4*>(&cx.it);
 #pragma unroll
                 for (int i = 0; i < (int)(sizeof(PrefillTcItem) / 16); ++i) dst[i] = __ldg(src + i);
-                derive_item(cx);
+                derive_ctx(cx);
             } else {
                 cx.live = 0;
                 if (!counted_out && lane == 0 && atomicAdd(p.pre_queue + 1, 1u) == (uint32_t)(queue_ctas - 1)) {
@@ -224,10 +254,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 counted_out = true;
             }
         };
-        ItemCtx cx, nx;
+        TcCtx cx, nx;
         if (has_static && *abort_flag == 0u) {
             cx.it = first_it;
-            derive_item(cx);
+            derive_ctx(cx);
         } else {
             draw(cx);
         }
@@ -241,7 +271,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 const uint4* src = reinterpret_cast<const uint4*>(&cx);
                 uint4* dst = reinterpret_cast<uint4*>(&ctx_s[k & 1]);
 #pragma unroll
-                for (int i = 0; i < (int)(sizeof(ItemCtx) / 16); ++i) dst[i] = src[i];
+                for (int i = 0; i < (int)(sizeof(TcCtx) / 16); ++i) dst[i] = src[i];
                 mbar_arrive(smem_u32(&bars.item_full[k & 1]));
             }
             if (!cx.live) break;
@@ -252,29 +282,27 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 for (int t = 0; t < 2; ++t)
                     if (it.n_rows[t] > 0)
                         for (int h = 0; h < HALVES; ++h)
-                            tma_load_3d(smem + SMEM_Q + t * TILE_BYTES + h * HALF_BYTES, &map_q, h * 64, it.head[t],
+                            tma_load_3d(smem + SMEM_Q + t * TILE_BYTES + h * HALF_BYTES, &map_q, h * 64, it.kvh * p.G,
                                         it.q_row0[t], smem_u32(&bars.q_full));
             }
             const int32_t* bt = p.block_table + (int64_t)it.seq * p.max_blocks;
-            const int n_max = cx.n_max, total_pages = cx.total_pages, jb = it.j_begin, page_lo = it.page_lo;
+            const int n_max = cx.n_max, page0 = cx.page0, page_end = cx.page_end;
             const int j_draw = min(2, n_max - 1);       // the next ticket is drawn once the first tiles are on their way
             bool drawn = false;
-            // page ids of a tile are fetched while the tile before it is being issued (never those of pages left of a
-            // sliding window: page_lo lies in the item's first tile)
-            int32_t pid = (lane < min(8, total_pages - 8 * jb) && 8 * jb + lane >= page_lo) ? checked_pid(__ldg(bt + 8 * jb + lane)) : 0;
+            // page ids of a tile are fetched while the tile before it is being issued
+            int32_t pid = lane < min(8, page_end - page0) ? checked_pid(__ldg(bt + page0 + lane)) : 0;
             for (int j = 0; j < n_max && ok; ++j) {
-                const int stage = j & 1;
+                const int stage = j & 1, at = page0 + 8 * j;
                 const uint32_t use = ub[stage] + (uint32_t)(j >> 1);
-                const int np = min(8, total_pages - 8 * (jb + j));
-                const int p0 = max(0, page_lo - 8 * (jb + j));
+                const int np = min(8, page_end - at);
                 const int32_t my_pid = __shfl_sync(0xffffffffu, pid, lane / HALVES);
-                if (j + 1 < n_max) pid = lane < min(8, total_pages - 8 * (jb + j + 1)) ? checked_pid(__ldg(bt + 8 * (jb + j + 1) + lane)) : 0;
+                if (j + 1 < n_max) pid = lane < min(8, page_end - at - 8) ? checked_pid(__ldg(bt + at + 8 + lane)) : 0;
                 const uint32_t dst_off = (lane % HALVES) * HALF_BYTES + (lane / HALVES) * 2048;
                 if (use > 0) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.k_empty[stage]), (use - 1) & 1u, abort_flag));
                 if (!ok) break;
-                if (lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.k_full[stage]), (np - p0) * 16 * D * 2);
+                if (lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.k_full[stage]), np * 16 * D * 2);
                 __syncwarp();
-                if (lane < HALVES * np && lane >= HALVES * p0)
+                if (lane < HALVES * np)
                     tma_load_4d(smem + SMEM_K + stage * TILE_BYTES + dst_off, &map_k, (lane % HALVES) * 64, 0, it.kvh, my_pid,
                                 smem_u32(&bars.k_full[stage]));
                 if (j == j_draw) {
@@ -323,20 +351,19 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 umma_commit(bar_s[t]);
             }
         };
-        // O_t (+)= P_t V, one K = 16 step per fetched page: pages [ks0, n_steps) of the tile (ks0 > 0 only in the first
-        // tile of a sliding window, n_steps < 8 only in a sequence's last tile)
-        auto issue_pv = [&](auto T, auto S, int ks0, int n_steps, uint32_t acc0) {
+        // O_t (+)= P_t V, one K = 16 step per fetched page of the tile (fewer than 8 only in an item's last tile)
+        auto issue_pv = [&](auto T, auto S, int n_steps, uint32_t acc0) {
             constexpr int t = decltype(T)::value, st = decltype(S)::value;
             const uint32_t dO = tmem + TM_O + t * D, aP = tmem + TM_S + t * 128;
             if (leader) {
-                if (ks0 == 0 && n_steps == 8) {
-                    umma_ts(dO, aP, vd(st, 0), IDESC_PV, acc0);
+                umma_ts(dO, aP, vd(st, 0), IDESC_PV, acc0);
+                if (n_steps == 8) {
 #pragma unroll
                     for (int ks = 1; ks < 8; ++ks) umma_ts(dO, aP + ks * 8, vd(st, ks), IDESC_PV, 1u);
                 } else {
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        if (ks >= ks0 && ks < n_steps) umma_ts(dO, aP + ks * 8, vd(st, ks), IDESC_PV, ks == ks0 ? acc0 : 1u);
+                    for (int ks = 1; ks < 7; ++ks)
+                        if (ks < n_steps) umma_ts(dO, aP + ks * 8, vd(st, ks), IDESC_PV, 1u);
                 }
                 umma_commit(bar_o[t]);
             }
@@ -360,9 +387,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)); };
         bool ok = true;
         for (int k = 0; ok; ++k) {
-        const ItemCtx* cs = wait_item(k);
+        const TcCtx* cs = wait_item(k);
         if (!__all_sync(0xffffffffu, cs != nullptr) || cs->live == 0) break;
-        const volatile ItemCtx* const vs = cs;
+        const volatile TcCtx* const vs = cs;
         const int n_max = cs->n_max;
         const int n_j[2] = {cs->n_j[0], cs->n_j[1]};
         ok = wait_all(smem_u32(&bars.q_full), (uint32_t)k & 1u) && wait_all(bar_kf[0], ub[0] & 1u);
@@ -382,11 +409,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (!mbar_wait(bar_kf[st1], par_k1, abort_flag)) return false;
             if (!mbar_wait(bar_p[0], par_p0, abort_flag)) return false;
             tc_fence_after();
-            issue_pv(I0{}, S, 0, 8, acc0);
+            issue_pv(I0{}, S, 8, acc0);
             issue_qk(I0{}, S1{});
             if (!mbar_wait(bar_p[1], par_p1, abort_flag)) return false;
             tc_fence_after();
-            issue_pv(I1{}, S, 0, 8, acc0);
+            issue_pv(I1{}, S, 8, acc0);
             issue_qk(I1{}, S1{});
             commit(bar_ve[st]);
             commit(bar_ke[st1]);
@@ -396,14 +423,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         auto kv_step = [&](auto S, int j) -> bool {
             constexpr int st = decltype(S)::value, st1 = st ^ 1;
             using S1 = std::integral_constant<int, st1>;
-            const int jb = vs->it.j_begin, Lc = vs->it.ctx_len;
-            const int np = min(8, vs->total_pages - 8 * (jb + j));
-            const int ks0 = max(0, vs->it.page_lo - 8 * (jb + j));      // sliding window: the tile's first fetched page
+            const int at = vs->page0 + 8 * j, Lc = vs->it.ctx_len;
+            const int np = min(8, vs->page_end - at);
             if (!wait_all(bar_vf[st], (ub[st] + (uint32_t)(j >> 1)) & 1u)) return false;
-            if (j == n_max - 1 && Lc < (8 * (jb + j) + np) * 16) {
+            if (j == n_max - 1 && Lc < (at + np) * 16) {
                 // slack slots of the sequence's last page came in with the page: zero those V rows so
                 // that a zero probability never multiplies a NaN
-                const int r0 = Lc - (jb + j) * KT, r1 = np * 16;
+                const int r0 = Lc - at * 16, r1 = np * 16;
                 for (int idx = lane; idx < (r1 - r0) * (D / 8); idx += 32) {
                     const int r = r0 + idx / (D / 8), c = idx % (D / 8);
                     uint8_t* dst = smem_raw + ((smem + SMEM_V + st * TILE_BYTES) - smem_u32(smem_raw)) +
@@ -421,7 +447,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 if (more && !wait_all(bar_kf[st1], (ub[st1] + (uint32_t)((j + 1) >> 1)) & 1u)) return false;
                 if (!wait_all(bar_p[t], (sb[t] + (uint32_t)j) & 1u)) return false;
                 tc_fence_after();
-                issue_pv(T, S, ks0, np, acc0);
+                issue_pv(T, S, np, acc0);
                 if (more) issue_qk(T, S1{});
                 return true;
             };
@@ -433,25 +459,18 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             return true;
         };
         int j = 0;
-        // Sliding window: the item's first tile may start with pages that are not fetched; it (and the tile after it,
-        // so that the pair loop below starts on an even tile) take the general step.
-        const bool partial_first = vs->it.page_lo > 8 * vs->it.j_begin;
-        if (partial_first) {
-            for (; j < min(2, n_max) && ok; ++j) ok = (j & 1) ? kv_step(I1{}, j) : kv_step(I0{}, j);
-        }
-        const int j_pairs = j;                       // where the pair loop starts: 0 or 2
-        if (ok) {
+        {
             // parities of the even tile j of a pair: stage 0 fill ub[0] + j/2 (V now), stage 1 fill ub[1] + j/2
             // (K of tile j + 1), softmax phases sb[t] + j; the odd tile j + 1 flips all but the stage-0 K
             // fill of tile j + 2, which is ub[0] + j/2 + 1
-            uint32_t h0 = (ub[0] + (uint32_t)(j >> 1)) & 1u, h1 = (ub[1] + (uint32_t)(j >> 1)) & 1u;
+            uint32_t h0 = ub[0] & 1u, h1 = ub[1] & 1u;
             const uint32_t p0 = sb[0] & 1u, p1 = sb[1] & 1u;
             for (; ok && j + 1 < n_int; j += 2, h0 ^= 1u, h1 ^= 1u) {
                 ok = lean_step(I0{}, h0, h1, p0, p1, j > 0 ? 1u : 0u);
                 if (ok) ok = lean_step(I1{}, h1, h0 ^ 1u, p0 ^ 1u, p1 ^ 1u, 1u);
             }
             ok = __all_sync(0xffffffffu, ok);
-            if (ok && j > j_pairs && j >= n_max - 1) commit(bar_qe);     // the pair loop issued the item's last S = Q K^T
+            if (ok && j > 0 && j >= n_max - 1) commit(bar_qe);     // the pair loop issued the item's last S = Q K^T
         }
         static_assert(KV_STAGES == 2, "the stage index is the parity of the tile index");
         for (; j < n_max && ok; ++j) {
@@ -471,22 +490,23 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
       const int row = (warp & 3) * 32 + lane;
       const uint32_t lanes = lane_field(warp);
       const uint32_t tS = tmem + TM_S + t * 128 + lanes, tO = tmem + TM_O + t * D + lanes;
+      const int lg = __ffs(p.G) - 1, token = row >> lg, head_in_group = row & (p.G - 1);
       uint32_t sbt = 0u;                       // tiles of this q tile in earlier items: running phase of s_full / p_full / o_done
       bool ok = true;
       for (int k = 0; ok; ++k) {
-        const ItemCtx* cs = wait_item(k);
+        const TcCtx* cs = wait_item(k);
         if (cs == nullptr || cs->live == 0) break;
         {
         // this q tile's fields of the item
-        const int jb = cs->it.j_begin, n_jt = cs->n_j[t], kv_hi = cs->kv_hi_t[t];
-        const int it_row0 = cs->it.row0[t], it_n_rows = cs->it.n_rows[t], it_q_row0 = cs->it.q_row0[t], it_head = cs->it.head[t];
+        const int key0 = cs->page0 * 16, n_jt = cs->n_j[t], end = cs->end_t[t];
+        const int it_row0 = cs->it.row0[t], it_n_rows = cs->it.n_rows[t], it_q_row0 = cs->it.q_row0[t], it_kvh = cs->it.kvh;
         const int it_part_slot = cs->it.part_slot[t], it_part_k = cs->it.part_k, it_part_c = cs->it.part_c;
         // fp8 cache: the staged K/V hold the codes; their per-head scales join the softmax scale and the output here
-        const float sc = (VARIANT && p.k_scale != nullptr) ? p.scale_log2 * __ldg(p.k_scale + cs->it.kvh) : p.scale_log2;
-        const float v_scale = (VARIANT && p.v_scale != nullptr) ? __ldg(p.v_scale + cs->it.kvh) : 1.f;
-        const int limit = min(cs->it.prefix + it_row0 + row, kv_hi - 1);   // last visible key of this row
-        const int first_key = (VARIANT && p.window > 0) ? limit - p.window + 1 : -(1 << 30);   // first visible key (sliding window)
-        const uint32_t span = (uint32_t)(limit - first_key);
+        const float sc = (VARIANT && p.k_scale != nullptr) ? p.scale_log2 * __ldg(p.k_scale + it_kvh) : p.scale_log2;
+        const float v_scale = (VARIANT && p.v_scale != nullptr) ? __ldg(p.v_scale + it_kvh) : 1.f;
+        const int pos = cs->it.prefix + it_row0 + min(token, it_n_rows - 1);      // rows past the tile's tokens repeat the last one
+        const int limit = min(pos, end - 1);                       // last key of this item the row sees
+        const int first_key = (VARIANT && p.window > 0) ? pos - p.window + 1 : -(1 << 30);   // first visible key (sliding window)
         float m_used = -INFINITY, l_sum = 0.f;     // -inf: the row has not met a visible key yet
         for (int j = 0; j < n_jt; ++j) {
             ok = mbar_wait(smem_u32(&bars.s_full[t]), (sbt + (uint32_t)j) & 1u, abort_flag);
@@ -496,12 +516,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, reinterpret_cast<uint32_t*>(&sv[c * 32]));
             tmem_wait_ld();
-            const int col_limit = limit - (jb + j) * KT;     // columns [col_first, col_limit] are visible
-            const int col_first = first_key - (jb + j) * KT;
+            const int col_limit = limit - key0 - j * KT;     // columns [col_first, col_limit] are visible
+            const int col_first = first_key - key0 - j * KT;
             if (VARIANT) {
                 if (__any_sync(0xffffffffu, col_limit < KT - 1 || col_first > 0)) {
 #pragma unroll
-                    for (int c = 0; c < 128; ++c) sv[c] = ((uint32_t)(c - col_first) <= span) ? sv[c] : -INFINITY;
+                    for (int c = 0; c < 128; ++c) sv[c] = (c >= col_first && c <= col_limit) ? sv[c] : -INFINITY;
                 }
             } else if (__any_sync(0xffffffffu, col_limit < KT - 1)) {
 #pragma unroll
@@ -590,13 +610,15 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (ok && n_jt > 0) ok = mbar_wait(smem_u32(&bars.o_done[t]), (sbt + (uint32_t)(n_jt - 1)) & 1u, abort_flag);
         if (ok && n_jt > 0) {
             tc_fence_after();
-            const bool live = row < it_n_rows;
+            const bool live = token < it_n_rows;
+            const int it_head = (it_kvh << lg) + head_in_group;
             const bool partial = it_part_slot >= 0;
             // a whole item joins the head's sink logit here; a KV range leaves it to the combine pass
             float m_fin = m_used, l_fin = l_sum, shrink = 1.f;
             if (VARIANT && !partial && p.sinks != nullptr) shrink = join_sink(__ldg(p.sinks + it_head) * kLog2e, m_fin, l_fin);
             const float inv = shrink * v_scale / l_fin;
-            __nv_bfloat16* orow = p.out + ((int64_t)(it_q_row0 + row) * p.Hq + it_head) * D;
+            const int64_t out_row = (int64_t)(it_q_row0 + token) * p.Hq + it_head;
+            __nv_bfloat16* orow = p.out + out_row * D;
             // KV-split item: un-normalised fp32 row plus (reference maximum, sum) for the combine pass
             const int64_t pslot = (int64_t)it_part_slot + (int64_t)row * it_part_k + it_part_c;
             float* prow = p.pre_part_o + pslot * D;
@@ -605,8 +627,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 float ov[32];
                 tmem_ld32(tO + c * 32, reinterpret_cast<uint32_t*>(ov));
                 tmem_wait_ld();
-                // a thread owns a row, so a warp's store touches 32 rows: 32-byte stores halve the number of
-                // memory transactions of the 16-byte ones
+                // a thread owns a row, so a warp's store touches 32 rows (runs of G rows are contiguous): 32-byte
+                // stores halve the number of memory transactions of the 16-byte ones
                 if (live && partial) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) st_global_256(prow + c * 32 + i * 8, reinterpret_cast<const uint32_t*>(ov + 8 * i));
@@ -621,7 +643,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 }
             }
             if (live && partial) *reinterpret_cast<float2*>(p.pre_part_ml + pslot * 2) = make_float2(m_used, l_sum);
-            else if (live && p.lse) p.lse[(int64_t)(it_q_row0 + row) * p.Hq + it_head] = (m_fin + log2f(l_fin)) * kLn2;
+            else if (live && p.lse) p.lse[out_row] = (m_fin + log2f(l_fin)) * kLn2;
             // O_t has been read out: the p_full arrival of the next item's first tile, later in this thread's
             // program order, is what allows the issuer to overwrite it
             tc_fence_before();
@@ -644,7 +666,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 }
 
 // ---------------------------------------------------------------------------------------------
-// Merges the partials of KV-split prefill items: for every row of the item's q tiles,
+// Merges the partials of KV-split prefill items: for every row (token x `pack` heads) of the item's q tiles,
 //   M = max_c m_c ; O = sum_c 2^(m_c - M) o_c / sum_c 2^(m_c - M) l_c ; lse = (M + log2 sum) ln 2
 // in fixed range order.  One warp per row (8 rows per CTA, 32 CTAs per split item), one float4 of the
 // row per lane (D / 4 lanes take part); the partials of a row are fetched with independent loads (part_k <= 8).
@@ -657,7 +679,8 @@ __global__ void __launch_bounds__(256) prefill_combine_kernel(const AttnParams p
     const int lane = threadIdx.x & 31;
     const int rb = blockIdx.x & 31;                  // 32 blocks of 8 rows = 2 tiles x 128 rows
     const int t = rb >> 4, r = (rb & 15) * 8 + (threadIdx.x >> 5);
-    if (r >= it.n_rows[t]) return;
+    const int token = r / it.pack, head = it.head[t] + r % it.pack;
+    if (token >= it.n_rows[t]) return;
     const int k = it.part_k;
     const int64_t s0 = (int64_t)it.part_slot[t] + (int64_t)r * k;
     const bool holds = lane < D / 4;                 // head_dim 64: half of the lanes hold a float4 of the row
@@ -683,13 +706,13 @@ __global__ void __launch_bounds__(256) prefill_combine_kernel(const AttnParams p
             acc.x += v[c].x * f; acc.y += v[c].y * f; acc.z += v[c].z * f; acc.w += v[c].w * f;
         }
     float shrink = 1.f;
-    if (p.sinks != nullptr) shrink = join_sink(__ldg(p.sinks + it.head[t]) * kLog2e, M, L);
-    if (p.v_scale != nullptr) shrink *= __ldg(p.v_scale + it.head[t] / p.G);      // fp8 cache: the value scale of the head's KV head
+    if (p.sinks != nullptr) shrink = join_sink(__ldg(p.sinks + head) * kLog2e, M, L);
+    if (p.v_scale != nullptr) shrink *= __ldg(p.v_scale + head / p.G);      // fp8 cache: the value scale of the head's KV head
     const float inv = shrink / L;
     uint2 w;
     w.x = pack_bf16(acc.x * inv, acc.y * inv);
     w.y = pack_bf16(acc.z * inv, acc.w * inv);
-    const int64_t orow = (int64_t)(it.q_row0[t] + r) * p.Hq + it.head[t];
+    const int64_t orow = (int64_t)(it.q_row0[t] + token) * p.Hq + head;
     if (holds) *reinterpret_cast<uint2*>(p.out + orow * D + lane * 4) = w;
     if (p.lse && lane == 0) p.lse[orow] = (M + log2f(L)) * kLn2;
 }
@@ -769,14 +792,14 @@ bool encode_pool_map(CUtensorMap* m, const void* base, int D, int num_blocks, in
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// q viewed as (d, head, row); one box = 64 elements x 1 head x 128 rows; rows past the end read as zero
-bool encode_q_map(CUtensorMap* m, const void* base, int D, int total_rows, int Hq)
+// q viewed as (d, head, row); one box = 64 elements x `heads` heads x 128 / heads rows; rows past the end read as zero
+bool encode_q_map(CUtensorMap* m, const void* base, int D, int total_rows, int Hq, int heads)
 {
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
     cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)Hq, (cuuint64_t)total_rows};
     cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)Hq * D * 2};
-    cuuint32_t box[3] = {64, 1, (cuuint32_t)QT}, es[3] = {1, 1, 1};
+    cuuint32_t box[3] = {64, (cuuint32_t)heads, (cuuint32_t)(QT / heads)}, es[3] = {1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;

@@ -1,0 +1,26 @@
+"""GPU parity at the sizes where a kernel's tiles, ranges and dispatch rules have their edges."""
+import numpy as np
+import pytest
+
+import cf_synth as syn
+import paper_2609_27085_b200 as cf
+from harness import run_and_check
+
+pytestmark = pytest.mark.gpu
+
+
+def small(seed, Hq, Hkv, D, prefix, qlens, NB=2048):
+    return syn.scenario_from_lengths("e", syn.Geometry(Hq, Hkv, D, 16, NB), seed, prefix, qlens)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(16, 2, 128), (16, 2, 64), (8, 2, 128), (4, 2, 64), (3, 3, 128)])
+@pytest.mark.parametrize("window,split", [(0, 0), (0, 3), (70, 0), (1500, 3)])
+def test_chunks_around_the_packed_q_tile(Hq, Hkv, D, window, split):
+    """A q tile of the prefill kernel holds 128 / G tokens x G heads, an item two of them, a planner block 128 tokens:
+    chunk lengths one short of, at and one past each of these, on prefixes that are not tile- or page-aligned."""
+    G = Hq // Hkv
+    t = 128 // G
+    qlen = sorted({2, t - 1, t, t + 1, 2 * t - 1, 2 * t, 2 * t + 1, 127, 128, 129, 128 + t, 128 + 2 * t + 1} - {0, 1})
+    prefix = [(211 * i * i + 7 * i) % 2500 for i in range(len(qlen))]
+    run_and_check(small(61, Hq, Hkv, D, prefix, [qlen]), window=window, sinks=None if window == 0 else np.linspace(-2, 2, Hq, dtype=np.float32),
+                  debug={cf.CF_DEBUG_PREFILL_SPLIT: split} if split else None)
