@@ -24,3 +24,11 @@ def test_chunks_around_the_packed_q_tile(Hq, Hkv, D, window, split):
     prefix = [(211 * i * i + 7 * i) % 2500 for i in range(len(qlen))]
     run_and_check(small(61, Hq, Hkv, D, prefix, [qlen]), window=window, sinks=None if window == 0 else np.linspace(-2, 2, Hq, dtype=np.float32),
                   debug={cf.CF_DEBUG_PREFILL_SPLIT: split} if split else None)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(16, 2, 64), (8, 2, 128), (2, 2, 128)])
+@pytest.mark.parametrize("window", [1, 31, 32, 33, 95, 129])
+def test_windows_around_the_skipped_column_chunks(Hq, Hkv, D, window):
+    """The softmax leaves out chunks of 32 columns that no row of a warp sees: windows one short of, at and one past a
+    chunk, on chunks of every length class, so that leading, middle and trailing chunks of a tile are dead."""
+    run_and_check(small(67, Hq, Hkv, D, [0, 5, 1000, 1023, 313, 64], [[150, 40, 129, 33, 300, 1]]), window=window)
