@@ -154,7 +154,7 @@ cf_status cf_mixed_attention_shared(cf_ctx* ctx, const cf_cache_desc* desc, cons
  * cf_mixed_attention_planned then only enqueue kernels - no allocation, no host synchronisation, no
  * host-side copy - with the same results as cf_kv_append / cf_mixed_attention.  That also makes the
  * two planned calls legal inside a CUDA stream capture (the pointers passed are baked into the graph;
- * the overlap variant and per-kernel timing do not apply to them when captured).  A plan must outlive
+ * per-kernel timing does not apply to them when captured).  A plan must outlive
  * every launch and every graph that uses it; cf_plan_destroy synchronises the device.  Planned calls
  * on one context share its error word and must be ordered like all other calls. */
 cf_status cf_plan_create(cf_ctx* ctx, const cf_cache_desc* desc, const int32_t* context_len, const int32_t* query_len,
@@ -198,11 +198,10 @@ cf_status cf_get_async_status(cf_ctx* ctx);
  *   cf_set_overlap(ctx, 0): serial sequence, decode -> (combine) -> prefill -> (prefill combine) on the
  *     caller's stream alone.
  *   cf_set_overlap(ctx, n), n > 0 (the initial state is n = 1): n persistent prefill CTAs, one per SM (n = 1:
- *     the library's default share of the SMs, cf_spatial_share), are enqueued first, on the caller's stream; a context-owned
- *     side stream, forked from the caller's, runs decode on the SMs left over as soon as those CTAs hold their
- *     SMs (it waits for their count with a stream memory operation), and behind it a second prefill
- *     grid that draws from the same work queue, so the SMs decode frees join the prefill.  The side stream is
- *     joined back into the caller's stream inside the call, so the caller still sees one stream.
+ *     the library's default share of the SMs, cf_spatial_share), are enqueued first; the decode grid, a programmatic
+ *     launch behind them on the same stream, starts as soon as those CTAs hold their SMs and runs on the SMs left
+ *     over; a second prefill grid behind it draws from the same work queue, so the SMs decode frees join the prefill.
+ *     Everything stays on the caller's stream, and whatever follows there sees all of it completed.
  * Environment at cf_create: CF_OVERLAP=0 (serial), CF_SPATIAL_SMS=n (the share that n = 1 stands for).
  * cf_set_timing and cf_mixed_step_host use the serial sequence. */
 cf_status cf_set_overlap(cf_ctx* ctx, int n);
@@ -231,9 +230,8 @@ cf_status cf_validate_block_table(cf_ctx* ctx, const cf_cache_desc* desc, const 
  *   CF_DEBUG_SEPARATE_COMBINE       1: merge split-K decode partials in the separate combine kernel
  *   CF_DEBUG_DECODE_WAVES           target number of decode CTA waves
  *   CF_DEBUG_DECODE_MIN_CHUNK_PAGES shortest decode chunk, in pages
- *   CF_DEBUG_SPATIAL_NO_WAIT        1: in the spatial sequence decode does not wait (through a stream memory
- *                                   operation) until the first prefill grid's CTAs hold their SMs, but relies on
- *                                   the order of the launches
+ *   CF_DEBUG_SPATIAL_NO_WAIT        accepted, no effect: the order in which the grids of the spatial sequence reach the
+ *                                   SMs is carried by the launches themselves
  *   CF_DEBUG_PREFILL_PAIRS          1: chunked prefill on pairs of SMs (tcgen05.mma.cta_group::2: two CTAs work on four
  *                                   heads of a group and share every K/V tile) where head_dim is 128 and the group
  *                                   size 4 or 8; correct and tested, but measured ~20 % slower than the default

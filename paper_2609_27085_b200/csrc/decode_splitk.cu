@@ -93,9 +93,7 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const int cta)
     const int item_id = cta / p.Hkv, kvh = cta % p.Hkv;
     const DecodeItem it = p.dec_items[item_id];
     const int G = p.G;
-    // lets the combine kernel (launched with programmatic stream serialisation) become resident while
-    // this grid drains; it still waits for this grid's completion before it reads a partial
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    decode_grid_start(p);
 
     // ---- Q^T fragments (B operand): thread holds Q[head = lane/4][d = 16*ks + 2*(lane%4) + {0,1} (+8)]
     uint32_t qf[KSTEPS][2];
@@ -357,10 +355,11 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, c = lane & 3;
+    if (decode_extra_cta(p)) return;
     const int item_id = blockIdx.x / p.Hkv, kvh = blockIdx.x % p.Hkv;
     const DecodeItem it = p.dec_items[item_id];
     const int G = p.G;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    decode_grid_start(p);
     const float score_scale = p.scale_log2 * __ldg(p.k_scale + kvh);
     const float out_scale = __ldg(p.v_scale + kvh);
 
@@ -605,7 +604,7 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const int
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int item_id = cta / p.Hkv, kvh = cta % p.Hkv;
     const SharedDecodeItem it = p.sh_items[item_id];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    decode_grid_start(p);
     const ShareMember* members = p.sh_members + it.member_first;
     const int G = p.G;
 
@@ -823,6 +822,7 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const int
 template <int D, int NWARPS, int NSTAGE>
 __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_kernel(const AttnParams p)
 {
+    if (decode_extra_cta(p)) return;
     decode_cta<D, NWARPS, NSTAGE>(p, (int)blockIdx.x);
 }
 
@@ -832,6 +832,7 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_kernel(const Att
 template <int D, int NWARPS, int NSTAGE, int NCG>
 __global__ void __launch_bounds__(NWARPS * 32, 2) decode_with_shared_kernel(const AttnParams p, const int n_shared_ctas)
 {
+    if (decode_extra_cta(p)) return;
     if ((int)blockIdx.x < n_shared_ctas) decode_shared_cta<D, NWARPS, NSTAGE, NCG>(p, (int)blockIdx.x);
     else decode_cta<D, NWARPS, NSTAGE>(p, (int)blockIdx.x - n_shared_ctas);
 }
@@ -872,6 +873,24 @@ static size_t decode_smem_bytes()
     return ring > merge ? ring : merge;
 }
 
+// Decode grids start before the grid ahead of them in the stream has completed (decode_grid_start): the launch, the
+// work item's fetch and the set-up are off the critical path.  `ctas` is one CTA per (item, KV head).
+template <class K, class... Rest>
+static cudaError_t launch_decode_grid(K kern, int ctas, size_t smem, cudaStream_t stream, const AttnParams& p, Rest... rest)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(ctas + (p.dec_chained ? 1 : 0)));
+    cfg.blockDim = dim3(kDecWarps * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, p, rest...);
+}
+
 template <int D>
 static cudaError_t launch_decode_t(const AttnParams& p, int n_items, cudaStream_t stream)
 {
@@ -886,8 +905,7 @@ static cudaError_t launch_decode_t(const AttnParams& p, int n_items, cudaStream_
         if (e != cudaSuccess) return e;
         configured[dev].store(true, std::memory_order_release);
     }
-    kern<<<n_items * p.Hkv, kDecWarps * 32, smem, stream>>>(p);
-    return cudaGetLastError();
+    return launch_decode_grid(kern, n_items * p.Hkv, smem, stream, p);
 }
 
 cudaError_t launch_decode_fp8(const AttnParams& p, int n_items, cudaStream_t stream)
@@ -905,8 +923,7 @@ cudaError_t launch_decode_fp8(const AttnParams& p, int n_items, cudaStream_t str
         if (e != cudaSuccess) return e;
         configured[dev].store(true, std::memory_order_release);
     }
-    kern<<<n_items * p.Hkv, kDecWarps * 32, smem, stream>>>(p);
-    return cudaGetLastError();
+    return launch_decode_grid(kern, n_items * p.Hkv, smem, stream, p);
 }
 
 cudaError_t launch_decode(const AttnParams& p, int head_dim, int n_items, cudaStream_t stream)
@@ -931,8 +948,7 @@ static cudaError_t launch_decode_shared_t(const AttnParams& p, int n_shared_item
         if (e != cudaSuccess) return e;
         configured[dev].store(true, std::memory_order_release);
     }
-    kern<<<(n_shared_items + n_items) * p.Hkv, kDecWarps * 32, smem, stream>>>(p, n_shared_items * p.Hkv);
-    return cudaGetLastError();
+    return launch_decode_grid(kern, (n_shared_items + n_items) * p.Hkv, smem, stream, p, n_shared_items * p.Hkv);
 }
 
 cudaError_t launch_decode_with_shared(const AttnParams& p, int head_dim, int n_shared_items, int n_items, cudaStream_t stream)

@@ -35,6 +35,7 @@ struct AttnParams {
     const PrefillTcItem* pre_tc_items;
     float* part_o;                    // [slot, Hq, D] fp32 un-normalised partial outputs
     float* part_ml;                   // [slot, Hq, 2] running max (log2 domain) and sum
+    int32_t dec_chained;              // the decode grid runs beside the prefill grid before it in the stream (spatial sequence)
     uint32_t* dec_counters;           // [first slot of a split sequence, Hkv] chunks finished; null: the combine kernel merges
     float* pre_part_o;                // [row slot, D] fp32 partial rows of KV-split prefill items
     float* pre_part_ml;               // [row slot, 2]
@@ -42,6 +43,24 @@ struct AttnParams {
     uint32_t* pre_queue;              // [2] ticket counter of the persistent prefill CTAs, and how many of them have left
     uint32_t* err;                    // device error word (bits below); may be null
 };
+
+// Start of a decode grid.  Every decode kernel is launched with programmatic stream serialisation.  On its own it waits
+// for the grid before it in the stream (the append) before its first read of anything but its work item.  Behind the
+// front prefill grid of the spatial sequence (p.dec_chained) it must not wait for that grid, and need not: every CTA of
+// the front grid has waited for the append before it allowed this grid to start.  There the grid has one CTA more than
+// work, which waits for the front grid, so that completion of this grid implies completion of that one.
+__device__ __forceinline__ void decode_grid_start(const AttnParams& p)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!p.dec_chained) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ bool decode_extra_cta(const AttnParams& p)      // true in that extra CTA, once it has waited
+{
+    if (!p.dec_chained || blockIdx.x != gridDim.x - 1) return false;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return true;
+}
 
 // Bits of the device error word
 constexpr uint32_t kErrTimeout = 1u;      // a bounded wait expired

@@ -52,8 +52,8 @@ cudaError_t launch_decode_with_shared(const AttnParams& p, int head_dim, int n_s
 // PrefillTcItems from the ticket counter p.pre_queue, which `queue_ctas` CTAs share in total (several
 // launches may draw from one counter; the last CTA to leave resets it).  Ticket t stands for item
 // ticket_base + t; with first_static set, CTA b starts on item b without a draw (then ticket_base = n_ctas of
-// that grid, also for a second grid that shares the counter).  `resident`, when not null, is a device word that
-// every CTA increments as it starts.
+// that grid, also for a second grid that shares the counter).  `tail`: the grid runs beside
+// the grid before it in the stream (the decode grid of the spatial sequence) and waits for its completion at the end.
 // The kernel reads q and the two pools through TMA tensor maps; a map depends only on the base address and the
 // geometry, so the caller may build it once and keep it (encode_* return false when the driver refuses).
 struct PrefillMaps {
@@ -64,14 +64,14 @@ bool encode_q_map(CUtensorMap* m, const void* q, int head_dim, int total_rows, i
 bool encode_pool_map(CUtensorMap* m, const void* pool, int head_dim, int num_blocks, int num_kv_heads, int64_t stride_block,
                      int64_t stride_head, int64_t stride_token);
 cudaError_t launch_prefill_tc(const AttnParams& p, const PrefillMaps& maps, int head_dim, int n_items, int n_ctas,
-                              int queue_ctas, int first_static, int ticket_base, uint32_t* resident, cudaStream_t stream);
+                              int queue_ctas, int first_static, int ticket_base, int tail, cudaStream_t stream);
 
 // The same work on pairs of SMs (tcgen05.mma.cta_group::2; head_dim 128, group size a multiple of 4): an item is four
 // q tiles (four heads of a group over the same rows), CTA r of a pair taking heads head[t] + 2 r and partial slots
 // part_slot[t] + r * pad; n_pairs persistent pairs (2 n_pairs CTAs), queue_pairs pairs drawing from the counter.
 bool prefill_pair_supported(const cf_cache_desc* desc);
 cudaError_t launch_prefill_tc2(const AttnParams& p, const PrefillMaps& maps, int n_items, int n_pairs, int queue_pairs,
-                               int first_static, int ticket_base, uint32_t* resident, cudaStream_t stream);
+                               int first_static, int ticket_base, int tail, cudaStream_t stream);
 
 // merges the fp32 partials of KV-split prefill items into `out` (one CTA per split item)
 cudaError_t launch_prefill_combine(const AttnParams& p, int head_dim, int n_items, cudaStream_t stream);

@@ -119,7 +119,7 @@ template <int D, int MODE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                   const __grid_constant__ CUtensorMap map_v, const AttnParams p, const int n_items, const int queue_ctas,
-                  const int first_static, const int ticket_base, uint32_t* const resident)
+                  const int first_static, const int ticket_base, const int tail)
 {
     constexpr bool VARIANT = MODE > 0, WINDOW = MODE == 2;
     constexpr int HALVES = Geo<D>::HALVES, TILE_BYTES = Geo<D>::TILE_BYTES, KS = Geo<D>::KS;
@@ -143,16 +143,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 #pragma unroll
         for (int i = 0; i < (int)(sizeof(PrefillTcItem) / 16); ++i) dst[i] = __ldg(src + i);
     }
-    // lets the next grid of the stream become resident while this grid drains (it waits for this grid's
-    // completion before it reads anything this grid wrote)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     volatile uint32_t* abort_flag = &abort_s;
 
     if (threadIdx.x == 0) {
         abort_s = (p.err != nullptr && (*reinterpret_cast<volatile uint32_t*>(p.err) & kErrTimeout) != 0u) ? 2u : 0u;   // an earlier CTA gave up
-        // spatial launch sequence: the stream that carries the decode kernel waits (a
-        // stream memory operation, not a kernel) until every CTA of this grid holds its SM
-        if (resident != nullptr) atomicAdd(resident, 1u);
         mbar_init(smem_u32(&bars.q_full), 1);
         mbar_init(smem_u32(&bars.q_empty), 1);
         for (int s = 0; s < KV_STAGES; ++s) {
@@ -174,10 +168,14 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
-    // Launched with programmatic stream serialisation: everything above overlaps the tail of the kernel
-    // before this one in the stream; from here on that kernel has completed and its writes are visible
-    // (the K/V rows of cf_kv_append when the batch has no decode part).
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // Launched with programmatic stream serialisation: everything above overlaps the tail of the kernel before this
+    // one in the stream.  From here on that kernel has completed and its writes are visible (the K/V rows of
+    // cf_kv_append) - except for the tail grid of the spatial sequence, which runs beside the decode grid before it:
+    // that one started after the front grid had passed this wait, and the tail grid makes up for it at its end.
+    if (!tail) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // Allows the next grid of the stream to start: the decode grid of the spatial sequence once every CTA of this
+    // grid holds its SM, a grid that waits for this one's completion (combine pass, next append) for its set-up.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // A block id outside the pool is not used as a TMA coordinate: page 0 is fetched in its place and the error
     // word is set (the rows of that sequence are then meaningless, but nothing is read outside the pool).
@@ -687,6 +685,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         __syncthreads();
     }
     if (warp == 0) tmem_dealloc<512>(tmem);
+    // the tail grid counts as complete only when the decode grid before it is (which in turn waits for the front grid)
+    if (tail) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -833,7 +833,7 @@ namespace {
 
 template <int D, int MODE>
 cudaError_t launch_prefill_tc_t(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const AttnParams& p,
-                                int n_items, int n_ctas, int queue_ctas, int first_static, int ticket_base, uint32_t* resident,
+                                int n_items, int n_ctas, int queue_ctas, int first_static, int ticket_base, int tail,
                                 cudaStream_t stream)
 {
     const size_t smem = Geo<D>::SMEM_TOTAL + 1024;
@@ -867,17 +867,17 @@ cudaError_t launch_prefill_tc_t(const CUtensorMap& mq, const CUtensorMap& mk, co
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, MODE>, mq, mk, mv, p, n_items, queue_ctas, first_static, ticket_base, resident);
+    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, MODE>, mq, mk, mv, p, n_items, queue_ctas, first_static, ticket_base, tail);
 }
 
 }  // namespace
 
 cudaError_t launch_prefill_tc(const AttnParams& p, const PrefillMaps& maps, int head_dim, int n_items, int n_ctas,
-                              int queue_ctas, int first_static, int ticket_base, uint32_t* resident, cudaStream_t stream)
+                              int queue_ctas, int first_static, int ticket_base, int tail, cudaStream_t stream)
 {
     if (n_items <= 0 || n_ctas <= 0) return cudaSuccess;
     auto launch = [&](auto DIM, auto MODE) {
-        return launch_prefill_tc_t<decltype(DIM)::value, decltype(MODE)::value>(maps.q, maps.k, maps.v, p, n_items, n_ctas, queue_ctas, first_static, ticket_base, resident, stream);
+        return launch_prefill_tc_t<decltype(DIM)::value, decltype(MODE)::value>(maps.q, maps.k, maps.v, p, n_items, n_ctas, queue_ctas, first_static, ticket_base, tail, stream);
     };
     using std::integral_constant;
     const int mode = p.window > 0 ? 2 : (p.sinks != nullptr || p.k_scale != nullptr) ? 1 : 0;

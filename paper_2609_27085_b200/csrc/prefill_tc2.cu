@@ -74,7 +74,7 @@ struct Bars2 {
 __global__ void __launch_bounds__(NTHREADS, 1)
 prefill_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const AttnParams p, const int n_items, const int queue_pairs,
-                   const int first_static, const int ticket_base, uint32_t* const resident)
+                   const int first_static, const int ticket_base, const int tail)
 {
     constexpr int D = D2, KS = D / 16;
     constexpr uint32_t kPolyMask = CF_POLY_MASK;
@@ -98,13 +98,11 @@ prefill_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
         for (int i = 0; i < (int)(sizeof(PrefillTcItem) / 16); ++i) dst[i] = __ldg(src + i);
     }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     volatile uint32_t* abort_flag = &abort_s;
     const uint32_t peer_abort = mapa_cluster(smem_u32(&abort_s), rank ^ 1u);
 
     if (threadIdx.x == 0) {
         abort_s = (p.err != nullptr && (*reinterpret_cast<volatile uint32_t*>(p.err) & kErrTimeout) != 0u) ? 2u : 0u;
-        if (resident != nullptr) atomicAdd(resident, 1u);
         mbar_init(smem_u32(&bars.q_full), 1);
         mbar_init(smem_u32(&bars.q_ready), 2);            // one arrival per CTA
         mbar_init(smem_u32(&bars.q_empty), 1);
@@ -130,7 +128,9 @@ prefill_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     cluster_sync_all();                                   // both CTAs: barriers initialised, tensor memory allocated
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // as in the one-CTA kernel: the tail grid of the spatial sequence waits at its end instead
+    if (!tail) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // a wait that gave up raises the other CTA's abort flag as well, so that both leave together
     auto wait_local = [&](uint32_t bar, uint32_t parity) -> bool {
@@ -631,6 +631,7 @@ prefill_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     }
     cluster_sync_all();                                   // neither CTA leaves while the other may still touch its memory
     if (warp == 0) tmem_dealloc2<512>(tmem);
+    if (tail) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 bool prefill_pair_supported(const cf_cache_desc* d)
@@ -640,7 +641,7 @@ bool prefill_pair_supported(const cf_cache_desc* d)
 }
 
 cudaError_t launch_prefill_tc2(const AttnParams& p, const PrefillMaps& maps, int n_items, int n_pairs, int queue_pairs,
-                               int first_static, int ticket_base, uint32_t* resident, cudaStream_t stream)
+                               int first_static, int ticket_base, int tail, cudaStream_t stream)
 {
     if (n_items <= 0 || n_pairs <= 0) return cudaSuccess;
     const size_t smem = P_SMEM_TOTAL + 1024;
@@ -675,7 +676,7 @@ cudaError_t launch_prefill_tc2(const AttnParams& p, const PrefillMaps& maps, int
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, prefill_tc2_kernel, maps.q, maps.k, maps.v, p, n_items, queue_pairs, first_static, ticket_base, resident);
+    return cudaLaunchKernelEx(&cfg, prefill_tc2_kernel, maps.q, maps.k, maps.v, p, n_items, queue_pairs, first_static, ticket_base, tail);
 }
 
 }  // namespace cf
