@@ -32,3 +32,17 @@ def test_windows_around_the_skipped_column_chunks(Hq, Hkv, D, window):
     """The softmax leaves out chunks of 32 columns that no row of a warp sees: windows one short of, at and one past a
     chunk, on chunks of every length class, so that leading, middle and trailing chunks of a tile are dead."""
     run_and_check(small(67, Hq, Hkv, D, [0, 5, 1000, 1023, 313, 64], [[150, 40, 129, 33, 300, 1]]), window=window)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,fp8", [(2, 2, 64, False), (8, 2, 128, False), (24, 24, 64, False), (32, 8, 128, True), (24, 24, 128, True)])
+@pytest.mark.parametrize("n_seqs", [1, 2, 31, 32, 33, 65, 1030])
+def test_append_at_the_edges_of_the_row_search(Hq, Hkv, D, fp8, n_seqs):
+    """The append's search splits the sequences 32 ways per step and moves a row in rounds of 32 x 8 loads: sequence counts
+    around powers of 32, empty sequences at the front, between and at the end, rows of less and more than one round
+    (24 heads).  Bit-exact whole-pool compare (inside run_and_check) and attention on top."""
+    rng = np.random.default_rng(n_seqs)
+    qlen = rng.choice([0, 0, 1, 1, 2, 5], size=n_seqs)
+    qlen[rng.integers(n_seqs)] = 3
+    prefix = rng.integers(0, 40, size=n_seqs)
+    scales = (rng.uniform(0.01, 0.03, Hkv).astype(np.float32), rng.uniform(0.01, 0.03, Hkv).astype(np.float32)) if fp8 else None
+    run_and_check(small(71, Hq, Hkv, D, prefix, [qlen], NB=4096), fp8=scales)
