@@ -14,6 +14,7 @@ length arrays are host ``int32`` numpy arrays (anything array-like is converted)
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional, Tuple
 
@@ -21,6 +22,7 @@ import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libcrossflow_attn.so")
+MARSHAL_PATH = os.path.join(_HERE, "_marshal.so")
 
 CF_OK = 0
 CF_ERR_INVALID_ARG = 1
@@ -73,15 +75,19 @@ class CfError(RuntimeError):
 
 
 _lib = None
+_fast = None       # compiled marshalling of the entry points that are called per layer or per step (csrc/marshal.cpp)
+_FAST = ("cf_kv_append", "cf_mixed_attention", "cf_mixed_attention_shared", "cf_kv_append_planned", "cf_mixed_attention_planned",
+         "cf_mixed_step_host", "cf_host_steps_flush", "cf_decode_attention_static")
 
 
 def load_library() -> ctypes.CDLL:
     """Loads the C-ABI library; raises if it has not been built (no fallback of any kind)."""
-    global _lib
+    global _lib, _fast
     if _lib is not None:
         return _lib
-    if not os.path.exists(LIB_PATH):
-        raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2609_27085_b200.build`")
+    for path in (LIB_PATH, MARSHAL_PATH):
+        if not os.path.exists(path):
+            raise ImportError(f"{path} is missing: build it with `python -m paper_2609_27085_b200.build`")
     lib = ctypes.CDLL(LIB_PATH)
     vp, i32, i32p, fp = ctypes.c_void_p, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_float)
     dp = ctypes.POINTER(CacheDesc)
@@ -117,8 +123,20 @@ def load_library() -> ctypes.CDLL:
     for name in EXPORTS:
         if name != "cf_status_string":
             getattr(lib, name).restype = ctypes.c_int
+    spec = importlib.util.spec_from_file_location(f"{__name__}._marshal", MARSHAL_PATH)
+    fast = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(fast)
+    fast.bind(_host_i32, *(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _FAST))
+    _fast = fast
     _lib = lib
     return lib
+
+
+def _native():
+    """The compiled marshalling functions (loads the library on first use)."""
+    if _fast is None:
+        load_library()
+    return _fast
 
 
 def cf_status_string(status: int) -> str:
@@ -179,10 +197,8 @@ def cf_destroy(ctx) -> None:
 
 def cf_kv_append(ctx, desc: CacheDesc, k_cache, v_cache, k_new, v_new, block_table, max_blocks_per_seq: int,
                  context_len, query_len, stream=None, check: bool = True) -> int:
-    lc, lq = _host_i32(context_len), _host_i32(query_len)
-    st = load_library().cf_kv_append(ctx, ctypes.byref(desc), _dev(k_cache), _dev(v_cache), _dev(k_new), _dev(v_new),
-                                     _dev(block_table), int(max_blocks_per_seq), lc.ctypes.data, lq.ctypes.data,
-                                     int(lc.shape[0]), _stream(stream))
+    st = (_fast or _native()).kv_append(ctx, desc, k_cache, v_cache, k_new, v_new, block_table, max_blocks_per_seq, context_len,
+                                        query_len, stream)
     if check:
         _check(st, "cf_kv_append")
     return st
@@ -190,10 +206,8 @@ def cf_kv_append(ctx, desc: CacheDesc, k_cache, v_cache, k_new, v_new, block_tab
 
 def cf_mixed_attention(ctx, desc: CacheDesc, q, k_cache, v_cache, block_table, max_blocks_per_seq: int,
                        context_len, query_len, out, lse=None, stream=None, check: bool = True) -> int:
-    lc, lq = _host_i32(context_len), _host_i32(query_len)
-    st = load_library().cf_mixed_attention(ctx, ctypes.byref(desc), _dev(q), _dev(k_cache), _dev(v_cache),
-                                           _dev(block_table), int(max_blocks_per_seq), lc.ctypes.data, lq.ctypes.data,
-                                           int(lc.shape[0]), _dev(out), _dev(lse), _stream(stream))
+    st = (_fast or _native()).mixed_attention(ctx, desc, q, k_cache, v_cache, block_table, max_blocks_per_seq, context_len,
+                                              query_len, out, lse, stream)
     if check:
         _check(st, "cf_mixed_attention")
     return st
@@ -204,12 +218,8 @@ def cf_mixed_attention_shared(ctx, desc: CacheDesc, q, k_cache, v_cache, block_t
                               check: bool = True) -> int:
     """cf_mixed_attention with shared prefixes described: share_group[s] >= 0 names the group whose members have
     the same pages for their first shared_len[s] tokens (host int32 arrays)."""
-    lc, lq = _host_i32(context_len), _host_i32(query_len)
-    sg, sl = _host_i32(share_group), _host_i32(shared_len)
-    st = load_library().cf_mixed_attention_shared(ctx, ctypes.byref(desc), _dev(q), _dev(k_cache), _dev(v_cache),
-                                                  _dev(block_table), int(max_blocks_per_seq), lc.ctypes.data, lq.ctypes.data,
-                                                  sg.ctypes.data, sl.ctypes.data, int(lc.shape[0]), _dev(out), _dev(lse),
-                                                  _stream(stream))
+    st = (_fast or _native()).mixed_attention_shared(ctx, desc, q, k_cache, v_cache, block_table, max_blocks_per_seq, context_len,
+                                                     query_len, share_group, shared_len, out, lse, stream)
     if check:
         _check(st, "cf_mixed_attention_shared")
     return st
@@ -225,11 +235,8 @@ def cf_get_last_plan_counts(ctx) -> np.ndarray:
 def cf_mixed_step_host(ctx, desc: CacheDesc, q_host, k_new_host, v_new_host, k_cache, v_cache, block_table,
                        max_blocks_per_seq: int, context_len, query_len, out_host, stream=None, check: bool = True) -> int:
     """q_host / k_new_host / v_new_host / out_host: host tensors (pinned recommended) or addresses."""
-    lc, lq = _host_i32(context_len), _host_i32(query_len)
-    st = load_library().cf_mixed_step_host(ctx, ctypes.byref(desc), _dev(q_host), _dev(k_new_host), _dev(v_new_host),
-                                           _dev(k_cache), _dev(v_cache), _dev(block_table), int(max_blocks_per_seq),
-                                           lc.ctypes.data, lq.ctypes.data, int(lc.shape[0]), _dev(out_host),
-                                           _stream(stream))
+    st = (_fast or _native()).mixed_step_host(ctx, desc, q_host, k_new_host, v_new_host, k_cache, v_cache, block_table,
+                                              max_blocks_per_seq, context_len, query_len, out_host, stream)
     if check:
         _check(st, "cf_mixed_step_host")
     return st
@@ -237,7 +244,7 @@ def cf_mixed_step_host(ctx, desc: CacheDesc, q_host, k_new_host, v_new_host, k_c
 
 def cf_host_steps_flush(ctx, stream=None) -> None:
     """Makes `stream` wait for the read-backs of every cf_mixed_step_host call issued so far."""
-    _check(load_library().cf_host_steps_flush(ctx, _stream(stream)), "cf_host_steps_flush")
+    _check((_fast or _native()).host_steps_flush(ctx, stream), "cf_host_steps_flush")
 
 
 def cf_get_async_status(ctx) -> int:
@@ -314,10 +321,8 @@ def cf_decode_attention_static(desc: CacheDesc, q, k_cache, v_cache, block_table
     split-K scratch is a fixed 16 MiB array inside the library.  One query token per sequence;
     runs on the current device; calls sharing the array must not overlap on the GPU.  Batches beyond
     the fixed limits return CF_ERR_WORKSPACE."""
-    lc = _host_i32(context_len)
-    st = load_library().cf_decode_attention_static(ctypes.byref(desc), _dev(q), _dev(k_cache), _dev(v_cache),
-                                                   _dev(block_table), int(max_blocks_per_seq), lc.ctypes.data,
-                                                   int(lc.shape[0]), _dev(out), _dev(lse), _stream(stream))
+    st = (_fast or _native()).decode_attention_static(desc, q, k_cache, v_cache, block_table, max_blocks_per_seq, context_len, out,
+                                                      lse, stream)
     if check:
         _check(st, "cf_decode_attention_static")
     return st
@@ -337,13 +342,12 @@ def cf_plan_destroy(plan) -> None:
 
 
 def cf_kv_append_planned(plan, k_cache, v_cache, k_new, v_new, block_table, stream=None) -> None:
-    _check(load_library().cf_kv_append_planned(plan, _dev(k_cache), _dev(v_cache), _dev(k_new), _dev(v_new),
-                                               _dev(block_table), _stream(stream)), "cf_kv_append_planned")
+    _check((_fast or _native()).kv_append_planned(plan, k_cache, v_cache, k_new, v_new, block_table, stream), "cf_kv_append_planned")
 
 
 def cf_mixed_attention_planned(plan, q, k_cache, v_cache, block_table, out, lse=None, stream=None) -> None:
-    _check(load_library().cf_mixed_attention_planned(plan, _dev(q), _dev(k_cache), _dev(v_cache), _dev(block_table),
-                                                     _dev(out), _dev(lse), _stream(stream)), "cf_mixed_attention_planned")
+    _check((_fast or _native()).mixed_attention_planned(plan, q, k_cache, v_cache, block_table, out, lse, stream),
+           "cf_mixed_attention_planned")
 
 
 def cf_spatial_share(desc: CacheDesc, context_len, query_len, num_sms: int = 148) -> int:

@@ -1,4 +1,5 @@
-"""Builds libcrossflow_attn.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Builds libcrossflow_attn.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _marshal.so (the CPython
+extension that marshals the arguments of the hot entry points) with g++.
 
     python -m paper_2609_27085_b200.build [--force] [--verbose]
 
@@ -11,10 +12,12 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcrossflow_attn.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")      # CPython extension: argument marshalling of the hot entry points
 SOURCES = ["api.cu", "plan.cpp", "kv_append.cu", "decode_splitk.cu", "prefill_tc.cu", "prefill_tc2.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
@@ -26,9 +29,9 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(MARSHAL)):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [
         os.path.join(HERE, "..", "include", "crossflow_attn.h"), os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
@@ -48,6 +51,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
             cmd.insert(1, "-Xptxas")
             cmd.insert(2, "-v")
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    tmp_marshal = MARSHAL + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-Wall", "-I", sysconfig.get_paths()["include"],
+           os.path.join(CSRC, "marshal.cpp"), "-o", tmp_marshal]
+    procs.append(("marshal.cpp", subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = False
     for src, p in procs:
         out, _ = p.communicate()
@@ -60,6 +67,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.check_call([_nvcc(), "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp, *objs,
                            "-cudart", "static"])
     os.replace(tmp, LIB)
+    os.replace(tmp_marshal, MARSHAL)
     return LIB
 
 
