@@ -78,6 +78,7 @@ struct cf_ctx {
     float* workspace = nullptr;
     size_t workspace_bytes = 0;
     bool workspace_fixed = false;
+    uint32_t* queue_dev = nullptr;    // ticket and exit counter of the persistent prefill CTAs of unplanned calls: zero between calls (the last CTA resets them)
     uint32_t* err_dev = nullptr;      // [0] device-side findings (bit 0: a wait expired, bit 1: block id outside the pool); [1] scratch counter of cf_validate_block_table
     bool fused_combine = true; // split-K merge inside the decode kernel (CF_DEBUG_SEPARATE_COMBINE: the separate combine kernel)
     bool use_pairs = false;    // CF_DEBUG_PREFILL_PAIRS: chunked prefill on pairs of SMs where the geometry allows it (measured slower
@@ -119,9 +120,9 @@ struct cf_plan {
     uint8_t* dev = nullptr;
     float* part = nullptr;         // this plan's own split-K partials
     int n_part_slots = 0, n_pre_slots = 0;
-    size_t off_stage = 0;
     int n_stage_seqs = 0, n_stage_pages = 0, max_stage_pages = 0;
-    size_t off_qstart = 0, off_ctx = 0, off_qlen = 0, off_dec = 0, off_comb = 0, off_sh = 0, off_shm = 0, off_pre_tc = 0, off_pre_comb = 0, off_queue = 0, total = 0;
+    cf::PlanRef ref;               // the lists in `dev`; behind them the lengths and the queue counters
+    size_t off_len = 0, off_queue = 0, total = 0;
     int n_dec = 0, n_comb = 0, n_pre_tc = 0, n_pre_comb = 0, total_q = 0;
     bool pair = false;
     int front_sms = 0;          // spatial sequence: SMs of the first prefill grid (spatial_front_sms or cf_set_overlap)
@@ -191,69 +192,60 @@ static cf_status ensure_workspace(cf_ctx* c, size_t need)
     return CF_OK;
 }
 
-// Layout of one uploaded plan: [q_start S+1][context_len S][query_len S][decode][combine][prefill]
-struct PlanLayout {
-    size_t off_qstart, off_ctx, off_qlen, off_dec, off_comb, off_sh, off_shm, off_pre_tc, off_pre_comb, off_stage, off_queue, total;
-};
-
-static PlanLayout layout_of(int32_t S, const Plan& pl, size_t n_stage_seqs = 0)
+// The lists of one call's plan, one behind the other (every offset a multiple of 16)
+static size_t layout_of(const Plan& pl, size_t n_stage_seqs, PlanRef* r)
 {
-    PlanLayout L;
     size_t at = 0;
-    L.off_qstart = at; at = align_up(at + sizeof(int32_t) * ((size_t)S + 1), 16);
-    L.off_ctx = at;    at = align_up(at + sizeof(int32_t) * (size_t)S, 16);
-    L.off_qlen = at;   at = align_up(at + sizeof(int32_t) * (size_t)S, 16);
-    L.off_dec = at;    at = align_up(at + sizeof(DecodeItem) * pl.decode.size(), 16);
-    L.off_comb = at;   at = align_up(at + sizeof(CombineItem) * pl.combine.size(), 16);
-    L.off_sh = at;     at = align_up(at + sizeof(SharedDecodeItem) * pl.shared_decode.size(), 16);
-    L.off_shm = at;    at = align_up(at + sizeof(ShareMember) * pl.share_members.size(), 16);
-    L.off_pre_tc = at; at = align_up(at + sizeof(PrefillTcItem) * pl.prefill_tc.size(), 16);
-    L.off_pre_comb = at; at = align_up(at + sizeof(PrefillCombineItem) * pl.prefill_combine.size(), 16);
-    L.off_stage = at;  at = align_up(at + sizeof(StageSeq) * n_stage_seqs, 16);
-    L.off_queue = at;  at += 16;   // ticket counter + exit counter of the persistent prefill CTAs; uploaded as zeros
-    L.total = at;
-    return L;
+    auto list = [&](int32_t* off, size_t bytes) {
+        *off = (int32_t)at;
+        at = align_up(at + bytes, 16);
+    };
+    r->base = nullptr;
+    list(&r->dec, sizeof(DecodeItem) * pl.decode.size());
+    list(&r->comb, sizeof(CombineItem) * pl.combine.size());
+    list(&r->sh, sizeof(SharedDecodeItem) * pl.shared_decode.size());
+    list(&r->shm, sizeof(ShareMember) * pl.share_members.size());
+    list(&r->pre_tc, sizeof(PrefillTcItem) * pl.prefill_tc.size());
+    list(&r->pre_comb, sizeof(PrefillCombineItem) * pl.prefill_combine.size());
+    list(&r->stage, sizeof(StageSeq) * n_stage_seqs);
+    return at;
+}
+static void write_plan(uint8_t* dst, const Plan& pl, const std::vector<StageSeq>& stage, const PlanRef& r)
+{
+    auto list = [&](int32_t off, const void* src, size_t bytes) {
+        if (bytes) std::memcpy(dst + off, src, bytes);
+    };
+    list(r.dec, pl.decode.data(), sizeof(DecodeItem) * pl.decode.size());
+    list(r.comb, pl.combine.data(), sizeof(CombineItem) * pl.combine.size());
+    list(r.sh, pl.shared_decode.data(), sizeof(SharedDecodeItem) * pl.shared_decode.size());
+    list(r.shm, pl.share_members.data(), sizeof(ShareMember) * pl.share_members.size());
+    list(r.pre_tc, pl.prefill_tc.data(), sizeof(PrefillTcItem) * pl.prefill_tc.size());
+    list(r.pre_comb, pl.prefill_combine.data(), sizeof(PrefillCombineItem) * pl.prefill_combine.size());
+    list(r.stage, stage.data(), sizeof(StageSeq) * stage.size());
 }
 
-// Copies the plan into the next pinned slot and enqueues its upload.  Returns the device base.
-static cf_status upload_plan(cf_ctx* c, int32_t S, const int32_t* context_len, const int32_t* query_len,
-                             const Plan& pl, cudaStream_t stream, PlanLayout* L, uint8_t** dev_base, PlanSlot** slot_out,
-                             const std::vector<StageSeq>* stage = nullptr)
+// Takes the next pinned slot (waits for its last use) ...
+static cf_status next_slot(cf_ctx* c, size_t bytes, PlanSlot** out)
 {
-    *L = layout_of(S, pl, stage ? stage->size() : 0);
-    cf_status st = ensure_plan_capacity(c, L->total);
+    cf_status st = ensure_plan_capacity(c, bytes);
     if (st != CF_OK) return st;
     PlanSlot& s = c->slots[c->next_slot];
     c->next_slot = (c->next_slot + 1) % kRing;
     if (s.used && cudaEventSynchronize(s.done) != cudaSuccess) return CF_ERR_CUDA;   // slot still in flight
-    std::memcpy(s.host + L->off_qstart, pl.q_start.data(), sizeof(int32_t) * ((size_t)S + 1));
-    if (S > 0) {
-        std::memcpy(s.host + L->off_ctx, context_len, sizeof(int32_t) * (size_t)S);
-        std::memcpy(s.host + L->off_qlen, query_len, sizeof(int32_t) * (size_t)S);
-    }
-    if (!pl.decode.empty()) std::memcpy(s.host + L->off_dec, pl.decode.data(), sizeof(DecodeItem) * pl.decode.size());
-    if (!pl.combine.empty()) std::memcpy(s.host + L->off_comb, pl.combine.data(), sizeof(CombineItem) * pl.combine.size());
-    if (!pl.shared_decode.empty())
-        std::memcpy(s.host + L->off_sh, pl.shared_decode.data(), sizeof(SharedDecodeItem) * pl.shared_decode.size());
-    if (!pl.share_members.empty())
-        std::memcpy(s.host + L->off_shm, pl.share_members.data(), sizeof(ShareMember) * pl.share_members.size());
-    if (!pl.prefill_tc.empty())
-        std::memcpy(s.host + L->off_pre_tc, pl.prefill_tc.data(), sizeof(PrefillTcItem) * pl.prefill_tc.size());
-    if (!pl.prefill_combine.empty())
-        std::memcpy(s.host + L->off_pre_comb, pl.prefill_combine.data(), sizeof(PrefillCombineItem) * pl.prefill_combine.size());
-    if (stage && !stage->empty()) std::memcpy(s.host + L->off_stage, stage->data(), sizeof(StageSeq) * stage->size());
-    std::memset(s.host + L->off_queue, 0, 16);
-    // The copy does not go on the caller's stream: there it would start only when that stream's earlier
-    // kernels are done (a few microseconds of copy-engine latency between kernels, every call) and, queued in
-    // the copy engine meanwhile, hold back copies enqueued after it.  It runs on a context-owned stream (a
-    // host-staged step: on its input copy stream) and the caller's stream waits for it through an event; the
-    // slot's device buffer is free by then (the host waited for the slot's last use above).
+    *out = &s;
+    return CF_OK;
+}
+// ... and enqueues its upload.  The copy does not go on the caller's stream: there it would start only when that
+// stream's earlier kernels are done (a few microseconds of copy-engine latency between kernels, every call) and, queued in
+// the copy engine meanwhile, hold back copies enqueued after it.  It runs on a context-owned stream (a host-staged step:
+// on its input copy stream) and the caller's stream waits for it through an event; the slot's device buffer is free by
+// then (the host waited for the slot's last use).
+static cf_status upload_slot(cf_ctx* c, PlanSlot* s, size_t bytes, cudaStream_t stream)
+{
     cudaStream_t copy_stream = c->plan_copy_stream ? c->plan_copy_stream : c->upload_stream;
-    if (cudaMemcpyAsync(s.dev, s.host, L->total, cudaMemcpyHostToDevice, copy_stream) != cudaSuccess) return CF_ERR_CUDA;
-    if (cudaEventRecord(s.uploaded, copy_stream) != cudaSuccess || cudaStreamWaitEvent(stream, s.uploaded, 0) != cudaSuccess)
+    if (cudaMemcpyAsync(s->dev, s->host, bytes, cudaMemcpyHostToDevice, copy_stream) != cudaSuccess) return CF_ERR_CUDA;
+    if (cudaEventRecord(s->uploaded, copy_stream) != cudaSuccess || cudaStreamWaitEvent(stream, s->uploaded, 0) != cudaSuccess)
         return CF_ERR_CUDA;
-    *dev_base = s.dev;
-    *slot_out = &s;
     return CF_OK;
 }
 
@@ -373,9 +365,11 @@ static void stage_list(const cf_cache_desc* d, const int32_t* context_len, const
     }
 }
 
-// Enqueues decode -> combine -> prefill for a plan that already sits in device memory at `base`.
-static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const PlanCounts& n, const PlanLayout& L,
-                                  uint8_t* base, float* ws, const WsLayout& W, const void* q, const void* k_cache,
+// Enqueues decode -> combine -> prefill for a plan that already sits in device memory
+// (plan.base), or in host memory (hp), from where the launches carry it.  `queue`: the two counter words of the
+// persistent prefill CTAs.
+static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const PlanCounts& n, const PlanRef& plan, const HostPlan& hp,
+                                  uint32_t* queue, float* ws, const WsLayout& W, const void* q, const void* k_cache,
                                   const void* v_cache, const int32_t* block_table, int32_t max_blocks_per_seq, void* out,
                                   float* lse, cudaStream_t stream, bool allow_timing)
 {
@@ -398,14 +392,7 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
     const bool fp8 = desc->kv_dtype == CF_KV_FP8_E4M3;
     p.k_scale = fp8 ? desc->k_scale : nullptr;
     p.v_scale = fp8 ? desc->v_scale : nullptr;
-    p.q_start = (const int32_t*)(base + L.off_qstart);
-    p.context_len = (const int32_t*)(base + L.off_ctx);
-    p.query_len = (const int32_t*)(base + L.off_qlen);
-    p.dec_items = (const DecodeItem*)(base + L.off_dec);
-    p.comb_items = (const CombineItem*)(base + L.off_comb);
-    p.sh_items = (const SharedDecodeItem*)(base + L.off_sh);
-    p.sh_members = (const ShareMember*)(base + L.off_shm);
-    p.pre_tc_items = (const PrefillTcItem*)(base + L.off_pre_tc);
+    p.plan = plan;
     p.part_o = (float*)((uint8_t*)ws + W.dec_o);
     p.part_ml = (float*)((uint8_t*)ws + W.dec_ml);
     const bool fused_combine = c->fused_combine && (size_t)n.n_part_slots * desc->num_kv_heads * sizeof(uint32_t) <= kCounterBytes;
@@ -413,8 +400,7 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
     p.dec_counters = fused_combine ? (uint32_t*)ws : nullptr;
     p.pre_part_o = (float*)((uint8_t*)ws + W.pre_o);
     p.pre_part_ml = (float*)((uint8_t*)ws + W.pre_ml);
-    p.pre_comb_items = (const PrefillCombineItem*)(base + L.off_pre_comb);
-    p.pre_queue = (uint32_t*)(base + L.off_queue);
+    p.pre_queue = queue;
     p.err = c->err_dev;
 
     cudaError_t e = cudaSuccess;
@@ -461,12 +447,12 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
     // it waits for the grid before it in the stream to complete before its first read)
     auto stage_pages = [&](cudaStream_t st) -> cudaError_t {
         if (!(fp8 && has_prefill)) return cudaSuccess;
-        return launch_kv_dequant_gather(p, (const StageSeq*)(base + L.off_stage), n.n_stage_seqs, n.max_stage_pages,
+        return launch_kv_dequant_gather(p, hp, n.n_stage_seqs, n.max_stage_pages,
                                         (__nv_bfloat16*)((uint8_t*)ws + W.stage_k), (__nv_bfloat16*)((uint8_t*)ws + W.stage_v),
                                         (int32_t*)((uint8_t*)ws + W.stage_bt), st);
     };
     auto decode_launch = [&](cudaStream_t st) -> cudaError_t {
-        return fp8 ? launch_decode_fp8(p, n.n_dec, st) : launch_decode_with_shared(p, D, n.n_shared, n.n_dec, st);
+        return fp8 ? launch_decode_fp8(p, hp, n.n_dec, st) : launch_decode_with_shared(p, hp, D, n.n_shared, n.n_dec, st);
     };
     int second_grid = 0;
     // Slots that take a prefill item: SMs, or pairs of SMs for pair items.  Grid sizes, the shared work queue and
@@ -476,7 +462,7 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
     const int pre_ctas = n.n_pre_tc < sms ? n.n_pre_tc : sms;      // persistent CTAs (pairs) of the serial sequence
     auto launch_prefill = [&](int n_slots, int queue_slots, int first_static, int ticket_base, int tail) {
         return n.pair ? launch_prefill_tc2(pp, maps, n.n_pre_tc, n_slots, queue_slots, first_static, ticket_base, tail, stream)
-                      : launch_prefill_tc(pp, maps, D, n.n_pre_tc, n_slots, queue_slots, first_static, ticket_base, tail, stream);
+                      : launch_prefill_tc(pp, hp, maps, D, n.n_pre_tc, n_slots, queue_slots, first_static, ticket_base, tail, stream);
     };
     if (c->overlap && !c->in_host_step && !tc && has_prefill && (n.n_dec > 0)) {
         // Spatial partition, three grids of one stream that run at the same time by programmatic launches.  `front`
@@ -505,7 +491,7 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
         if (e == cudaSuccess) e = decode_launch(stream);
         if (e == cudaSuccess) e = launch_prefill(tail, front + tail, 0, front, 1);
         if (e == cudaSuccess) e = launch_combine(p, D, fused_combine ? 0 : n.n_comb, stream);
-        if (e == cudaSuccess) e = launch_prefill_combine(pp, D, n.n_pre_comb, stream);
+        if (e == cudaSuccess) e = launch_prefill_combine(pp, hp, D, n.n_pre_comb, stream);
     } else {
         if (tc) cudaEventRecord(tc->ev[0], stream);
         if (e == cudaSuccess) e = decode_launch(stream);
@@ -514,10 +500,12 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
         if (tc) cudaEventRecord(tc->ev[2], stream);
         if (e == cudaSuccess) e = stage_pages(stream);
         if (e == cudaSuccess) e = launch_prefill(pre_ctas, pre_ctas, 1, pre_ctas, 0);
-        if (e == cudaSuccess) e = launch_prefill_combine(pp, D, n.n_pre_comb, stream);
+        if (e == cudaSuccess) e = launch_prefill_combine(pp, hp, D, n.n_pre_comb, stream);
         if (tc) cudaEventRecord(tc->ev[3], stream);
     }
     c->launches = (int)(n.n_dec > 0) + (int)(n.n_comb > 0 && !fused_combine) + (int)(n.n_pre_tc > 0) + (int)(n.n_pre_comb > 0) + second_grid;
+    // a launch that failed half-way leaves tickets that no CTA will draw: the counters go back to zero behind the rest
+    if (e != cudaSuccess && has_prefill) cudaMemsetAsync(queue, 0, 2 * sizeof(uint32_t), stream);
     return e == cudaSuccess ? CF_OK : CF_ERR_CUDA;
 }
 
@@ -587,6 +575,8 @@ cf_status cf_create(cf_ctx** out, int device, size_t workspace_bytes)
     }
     ok = ok && cudaMalloc((void**)&c->err_dev, 2 * sizeof(uint32_t)) == cudaSuccess;
     ok = ok && cudaMemset(c->err_dev, 0, 2 * sizeof(uint32_t)) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
+    ok = ok && cudaMalloc((void**)&c->queue_dev, 2 * sizeof(uint32_t)) == cudaSuccess;
+    ok = ok && cudaMemset(c->queue_dev, 0, 2 * sizeof(uint32_t)) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
         cf_destroy(c);
         return CF_ERR_CUDA;
@@ -612,6 +602,7 @@ cf_status cf_destroy(cf_ctx* c)
             if (tc.ev[i]) cudaEventDestroy(tc.ev[i]);
     if (c->workspace) cudaFree(c->workspace);
     if (c->err_dev) cudaFree(c->err_dev);
+    if (c->queue_dev) cudaFree(c->queue_dev);
     if (c->upload_stream) cudaStreamDestroy(c->upload_stream);
     for (int i = 0; i < kHostStages; ++i) {
         HostStage& hs = c->stage[i];
@@ -626,6 +617,25 @@ cf_status cf_destroy(cf_ctx* c)
     if (c->d2h_stream) cudaStreamDestroy(c->d2h_stream);
     delete c;
     return CF_OK;
+}
+
+static AppendParams append_params(cf_ctx* c, const cf_cache_desc* desc, void* k_cache, void* v_cache, const void* k_new, const void* v_new,
+                                  const int32_t* block_table, int32_t max_blocks, int32_t num_seqs, int32_t total_rows)
+{
+    AppendParams p = {};
+    p.k_cache = (__nv_bfloat16*)k_cache;
+    p.v_cache = (__nv_bfloat16*)v_cache;
+    p.k_new = (const __nv_bfloat16*)k_new;
+    p.v_new = (const __nv_bfloat16*)v_new;
+    p.block_table = block_table;
+    p.max_blocks = max_blocks;
+    p.ks_block = desc->k_stride_block; p.ks_head = desc->k_stride_head; p.ks_token = desc->k_stride_token;
+    p.vs_block = desc->v_stride_block; p.vs_head = desc->v_stride_head; p.vs_token = desc->v_stride_token;
+    p.Hkv = desc->num_kv_heads; p.D = desc->head_dim; p.num_seqs = num_seqs; p.total_rows = total_rows;
+    p.num_blocks = desc->num_blocks; p.err = c->err_dev;
+    p.k_scale = desc->kv_dtype == CF_KV_FP8_E4M3 ? desc->k_scale : nullptr;
+    p.v_scale = desc->kv_dtype == CF_KV_FP8_E4M3 ? desc->v_scale : nullptr;
+    return p;
 }
 
 cf_status cf_kv_append(cf_ctx* c, const cf_cache_desc* desc, void* k_cache, void* v_cache,
@@ -646,29 +656,25 @@ cf_status cf_kv_append(cf_ctx* c, const cf_cache_desc* desc, void* k_cache, void
     DeviceGuard guard(c->device);
     if (!guard.ok) return CF_ERR_CUDA;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    PlanLayout L;
-    uint8_t* base = nullptr;
+    for (int32_t i = 0; i < num_seqs; ++i) pl.prefix.push_back(context_len[i] - query_len[i]);
     PlanSlot* slot = nullptr;
-    st = upload_plan(c, num_seqs, context_len, query_len, pl, stream, &L, &base, &slot);
-    if (st != CF_OK) return st;
-    AppendParams p;
-    p.k_cache = (__nv_bfloat16*)k_cache;
-    p.v_cache = (__nv_bfloat16*)v_cache;
-    p.k_new = (const __nv_bfloat16*)k_new;
-    p.v_new = (const __nv_bfloat16*)v_new;
-    p.block_table = block_table;
-    p.max_blocks = max_blocks_per_seq;
-    p.ks_block = desc->k_stride_block; p.ks_head = desc->k_stride_head; p.ks_token = desc->k_stride_token;
-    p.vs_block = desc->v_stride_block; p.vs_head = desc->v_stride_head; p.vs_token = desc->v_stride_token;
-    p.Hkv = desc->num_kv_heads; p.D = desc->head_dim; p.num_seqs = num_seqs; p.total_rows = pl.total_q;
-    p.num_blocks = desc->num_blocks; p.err = c->err_dev;
-    p.k_scale = desc->kv_dtype == CF_KV_FP8_E4M3 ? desc->k_scale : nullptr;
-    p.v_scale = desc->kv_dtype == CF_KV_FP8_E4M3 ? desc->v_scale : nullptr;
-    p.q_start = (const int32_t*)(base + L.off_qstart);
-    p.context_len = (const int32_t*)(base + L.off_ctx);
-    p.query_len = (const int32_t*)(base + L.off_qlen);
+    AppendParams p = append_params(c, desc, k_cache, v_cache, k_new, v_new, block_table, max_blocks_per_seq, num_seqs, pl.total_q);
+    if (num_seqs <= kAppendInlineSeqs) {
+        p.host_q_start = pl.q_start.data();
+        p.host_prefix = pl.prefix.data();
+    } else {
+        const size_t qs_bytes = sizeof(int32_t) * ((size_t)num_seqs + 1), pf_bytes = sizeof(int32_t) * (size_t)num_seqs;
+        st = next_slot(c, qs_bytes + pf_bytes, &slot);
+        if (st != CF_OK) return st;
+        std::memcpy(slot->host, pl.q_start.data(), qs_bytes);
+        std::memcpy(slot->host + qs_bytes, pl.prefix.data(), pf_bytes);
+        st = upload_slot(c, slot, qs_bytes + pf_bytes, stream);
+        if (st != CF_OK) return st;
+        p.q_start = (const int32_t*)slot->dev;
+        p.prefix = (const int32_t*)(slot->dev + qs_bytes);
+    }
     const cudaError_t e = launch_kv_append(p, stream);
-    const cf_status fs = finish_slot(slot, stream);
+    const cf_status fs = slot ? finish_slot(slot, stream) : CF_OK;
     c->host_ns_append += now_ns() - t_in;
     ++c->host_calls_append;
     if (e != cudaSuccess) return CF_ERR_CUDA;
@@ -722,11 +728,26 @@ cf_status cf_mixed_attention_shared(cf_ctx* c, const cf_cache_desc* desc, const 
     st = ensure_workspace(c, W.total);
     if (st != CF_OK) return st;
 
-    PlanLayout L;
-    uint8_t* base = nullptr;
+    // A small plan travels with the launches: up to kSmallPlanBytes with every kernel of the sequence, up to kMidPlanBytes
+    // with the decode kernel when it is the only one that needs it.  Larger ones go through a pinned slot and a copy.
+    PlanRef ref;
+    HostPlan hp;
     PlanSlot* slot = nullptr;
-    st = upload_plan(c, num_seqs, context_len, query_len, pl, stream, &L, &base, &slot, &stage);
-    if (st != CF_OK) return st;
+    const size_t bytes = layout_of(pl, stage.size(), &ref);
+    const bool fused = c->fused_combine && (size_t)pl.n_part_slots * desc->num_kv_heads * sizeof(uint32_t) <= kCounterBytes;
+    alignas(16) uint8_t inline_plan[kMidPlanBytes];
+    if (bytes <= (size_t)(pl.prefill_tc.empty() ? kMidPlanBytes : kSmallPlanBytes) && (fused || pl.combine.empty()) && !pl.pair) {
+        write_plan(inline_plan, pl, stage, ref);
+        hp.bytes = inline_plan;
+        hp.size = bytes;
+    } else {
+        st = next_slot(c, bytes, &slot);
+        if (st != CF_OK) return st;
+        write_plan(slot->host, pl, stage, ref);
+        st = upload_slot(c, slot, bytes, stream);
+        if (st != CF_OK) return st;
+        ref.base = slot->dev;
+    }
 
     PlanCounts n;
     n.n_dec = (int)pl.decode.size(); n.n_comb = (int)pl.combine.size(); n.n_shared = (int)pl.shared_decode.size();
@@ -738,9 +759,9 @@ cf_status cf_mixed_attention_shared(cf_ctx* c, const cf_cache_desc* desc, const 
     c->last_counts[4] = n.n_pre_comb; c->last_counts[5] = n.n_shared; c->last_counts[6] = (int32_t)pl.share_members.size();
     c->last_counts[7] = pl.pair ? 1 : 0;
     n.front_sms = front_sms;
-    const cf_status ls = launch_attention(c, desc, n, L, base, c->workspace, W,
+    const cf_status ls = launch_attention(c, desc, n, ref, hp, c->queue_dev, c->workspace, W,
                                           q, k_cache, v_cache, block_table, max_blocks_per_seq, out, lse, stream, true);
-    const cf_status fs = finish_slot(slot, stream);
+    const cf_status fs = slot ? finish_slot(slot, stream) : CF_OK;
     c->host_ns_attention += now_ns() - t_in;
     ++c->host_calls_attention;
     return ls != CF_OK ? ls : fs;
@@ -772,12 +793,11 @@ cf_status cf_plan_create(cf_ctx* c, const cf_cache_desc* desc, const int32_t* co
     std::vector<StageSeq> stage;
     int n_stage_pages = 0, max_stage_pages = 0;
     if (!pl.prefill_tc.empty()) stage_list(desc, context_len, query_len, num_seqs, &stage, &n_stage_pages, &max_stage_pages);
-    const PlanLayout L = layout_of(num_seqs, pl, stage.size());
-    P->off_stage = L.off_stage;
+    P->off_len = align_up(layout_of(pl, stage.size(), &P->ref), 16);
+    const size_t qs_bytes = sizeof(int32_t) * ((size_t)num_seqs + 1), pf_bytes = sizeof(int32_t) * (size_t)num_seqs;
+    P->off_queue = align_up(P->off_len + qs_bytes + pf_bytes, 16);
+    P->total = P->off_queue + 16;
     P->n_stage_seqs = (int)stage.size(); P->n_stage_pages = n_stage_pages; P->max_stage_pages = max_stage_pages;
-    P->off_qstart = L.off_qstart; P->off_ctx = L.off_ctx; P->off_qlen = L.off_qlen; P->off_dec = L.off_dec;
-    P->off_comb = L.off_comb; P->off_sh = L.off_sh; P->off_shm = L.off_shm; P->off_pre_tc = L.off_pre_tc; P->off_pre_comb = L.off_pre_comb; P->off_queue = L.off_queue;
-    P->total = L.total;
     P->n_dec = (int)pl.decode.size(); P->n_comb = (int)pl.combine.size();
     P->n_pre_tc = (int)pl.prefill_tc.size(); P->n_pre_comb = (int)pl.prefill_combine.size(); P->total_q = pl.total_q;
     P->front_sms = front_sms;
@@ -785,26 +805,20 @@ cf_status cf_plan_create(cf_ctx* c, const cf_cache_desc* desc, const int32_t* co
     P->pair = pl.pair;
     const size_t part_bytes = ws_layout(pl.n_part_slots, pl.n_pre_slots, desc->num_q_heads, desc->head_dim, n_stage_pages,
                                         desc->num_kv_heads, (int64_t)num_seqs * max_blocks_per_seq).total;
-    bool ok = cudaMallocHost((void**)&P->host, L.total) == cudaSuccess && cudaMalloc((void**)&P->dev, L.total) == cudaSuccess;
+    bool ok = cudaMallocHost((void**)&P->host, P->total) == cudaSuccess && cudaMalloc((void**)&P->dev, P->total) == cudaSuccess;
     // the ticket counters are zeroed on the caller's stream, like the plan copy: every launch that uses the plan
     // is ordered behind this call on that stream (or by the caller)
     if (ok && part_bytes)
         ok = cudaMalloc((void**)&P->part, part_bytes) == cudaSuccess &&
              cudaMemsetAsync(P->part, 0, kCounterBytes, (cudaStream_t)cuda_stream) == cudaSuccess;
     if (ok) {
-        std::memcpy(P->host + L.off_qstart, pl.q_start.data(), sizeof(int32_t) * ((size_t)num_seqs + 1));
-        if (num_seqs > 0) {
-            std::memcpy(P->host + L.off_ctx, context_len, sizeof(int32_t) * (size_t)num_seqs);
-            std::memcpy(P->host + L.off_qlen, query_len, sizeof(int32_t) * (size_t)num_seqs);
-        }
-        if (P->n_dec) std::memcpy(P->host + L.off_dec, pl.decode.data(), sizeof(DecodeItem) * pl.decode.size());
-        if (P->n_comb) std::memcpy(P->host + L.off_comb, pl.combine.data(), sizeof(CombineItem) * pl.combine.size());
-        if (P->n_pre_tc) std::memcpy(P->host + L.off_pre_tc, pl.prefill_tc.data(), sizeof(PrefillTcItem) * pl.prefill_tc.size());
-        if (P->n_pre_comb)
-            std::memcpy(P->host + L.off_pre_comb, pl.prefill_combine.data(), sizeof(PrefillCombineItem) * pl.prefill_combine.size());
-        if (!stage.empty()) std::memcpy(P->host + L.off_stage, stage.data(), sizeof(StageSeq) * stage.size());
-        std::memset(P->host + L.off_queue, 0, 16);
-        ok = cudaMemcpyAsync(P->dev, P->host, L.total, cudaMemcpyHostToDevice, (cudaStream_t)cuda_stream) == cudaSuccess;
+        for (int32_t i = 0; i < num_seqs; ++i) pl.prefix.push_back(context_len[i] - query_len[i]);
+        write_plan(P->host, pl, stage, P->ref);
+        std::memcpy(P->host + P->off_len, pl.q_start.data(), qs_bytes);
+        if (pf_bytes) std::memcpy(P->host + P->off_len + qs_bytes, pl.prefix.data(), pf_bytes);
+        std::memset(P->host + P->off_queue, 0, 16);
+        P->ref.base = P->dev;
+        ok = cudaMemcpyAsync(P->dev, P->host, P->total, cudaMemcpyHostToDevice, (cudaStream_t)cuda_stream) == cudaSuccess;
     }
     c->live_plans.fetch_add(1);
     if (!ok) {
@@ -836,23 +850,15 @@ cf_status cf_kv_append_planned(cf_plan* P, void* k_cache, void* v_cache, const v
     if (!k_cache || !v_cache || !k_new || !v_new || !block_table) return CF_ERR_INVALID_ARG;
     DeviceGuard guard(P->ctx->device);
     if (!guard.ok) return CF_ERR_CUDA;
-    const cf_cache_desc* desc = &P->desc;
-    AppendParams p;
-    p.k_cache = (__nv_bfloat16*)k_cache;
-    p.v_cache = (__nv_bfloat16*)v_cache;
-    p.k_new = (const __nv_bfloat16*)k_new;
-    p.v_new = (const __nv_bfloat16*)v_new;
-    p.block_table = block_table;
-    p.max_blocks = P->max_blocks;
-    p.ks_block = desc->k_stride_block; p.ks_head = desc->k_stride_head; p.ks_token = desc->k_stride_token;
-    p.vs_block = desc->v_stride_block; p.vs_head = desc->v_stride_head; p.vs_token = desc->v_stride_token;
-    p.Hkv = desc->num_kv_heads; p.D = desc->head_dim; p.num_seqs = P->num_seqs; p.total_rows = P->total_q;
-    p.num_blocks = desc->num_blocks; p.err = P->ctx->err_dev;
-    p.k_scale = desc->kv_dtype == CF_KV_FP8_E4M3 ? desc->k_scale : nullptr;
-    p.v_scale = desc->kv_dtype == CF_KV_FP8_E4M3 ? desc->v_scale : nullptr;
-    p.q_start = (const int32_t*)(P->dev + P->off_qstart);
-    p.context_len = (const int32_t*)(P->dev + P->off_ctx);
-    p.query_len = (const int32_t*)(P->dev + P->off_qlen);
+    AppendParams p = append_params(P->ctx, &P->desc, k_cache, v_cache, k_new, v_new, block_table, P->max_blocks, P->num_seqs, P->total_q);
+    const size_t qs_bytes = sizeof(int32_t) * ((size_t)P->num_seqs + 1);
+    if (P->num_seqs <= kAppendInlineSeqs) {
+        p.host_q_start = (const int32_t*)(P->host + P->off_len);
+        p.host_prefix = (const int32_t*)(P->host + P->off_len + qs_bytes);
+    } else {
+        p.q_start = (const int32_t*)(P->dev + P->off_len);
+        p.prefix = (const int32_t*)(P->dev + P->off_len + qs_bytes);
+    }
     return launch_kv_append(p, (cudaStream_t)cuda_stream) == cudaSuccess ? CF_OK : CF_ERR_CUDA;
 }
 
@@ -865,10 +871,6 @@ cf_status cf_mixed_attention_planned(cf_plan* P, const void* q, const void* k_ca
     if (!q || !k_cache || !v_cache || !block_table || !out) return CF_ERR_INVALID_ARG;
     DeviceGuard guard(P->ctx->device);
     if (!guard.ok) return CF_ERR_CUDA;
-    PlanLayout L;
-    L.off_qstart = P->off_qstart; L.off_ctx = P->off_ctx; L.off_qlen = P->off_qlen; L.off_dec = P->off_dec;
-    L.off_comb = P->off_comb; L.off_sh = P->off_sh; L.off_shm = P->off_shm; L.off_pre_tc = P->off_pre_tc; L.off_stage = P->off_stage; L.off_pre_comb = P->off_pre_comb; L.off_queue = P->off_queue;
-    L.total = P->total;
     PlanCounts n;
     n.n_dec = P->n_dec; n.n_comb = P->n_comb; n.n_pre_tc = P->n_pre_tc; n.n_pre_comb = P->n_pre_comb;
     n.total_q = P->total_q;
@@ -878,7 +880,7 @@ cf_status cf_mixed_attention_planned(cf_plan* P, const void* q, const void* k_ca
     n.n_stage_seqs = P->n_stage_seqs; n.n_stage_pages = P->n_stage_pages; n.max_stage_pages = P->max_stage_pages; n.num_seqs = P->num_seqs;
     const WsLayout W = ws_layout(P->n_part_slots, P->n_pre_slots, P->desc.num_q_heads, P->desc.head_dim, P->n_stage_pages,
                                  P->desc.num_kv_heads, (int64_t)P->num_seqs * P->max_blocks);
-    return launch_attention(P->ctx, &P->desc, n, L, P->dev, P->part, W, q, k_cache,
+    return launch_attention(P->ctx, &P->desc, n, P->ref, HostPlan(), (uint32_t*)(P->dev + P->off_queue), P->part, W, q, k_cache,
                             v_cache, block_table, P->max_blocks, out, lse, (cudaStream_t)cuda_stream, false);
 }
 
@@ -1005,14 +1007,16 @@ cf_status cf_validate_block_table(cf_ctx* c, const cf_cache_desc* desc, const in
     DeviceGuard guard(c->device);
     if (!guard.ok) return CF_ERR_CUDA;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    PlanLayout L;
-    uint8_t* base = nullptr;
     PlanSlot* slot = nullptr;
-    st = upload_plan(c, num_seqs, context_len, query_len, pl, stream, &L, &base, &slot);
+    const size_t bytes = sizeof(int32_t) * (size_t)num_seqs;
+    st = next_slot(c, bytes, &slot);
+    if (st != CF_OK) return st;
+    std::memcpy(slot->host, context_len, bytes);
+    st = upload_slot(c, slot, bytes, stream);
     if (st != CF_OK) return st;
     uint32_t* counter = c->err_dev + 1;      // context-owned scratch word
     bool ok = cudaMemsetAsync(counter, 0, sizeof(uint32_t), stream) == cudaSuccess;
-    ok = ok && launch_validate_table(block_table, max_blocks_per_seq, (const int32_t*)(base + L.off_ctx), num_seqs,
+    ok = ok && launch_validate_table(block_table, max_blocks_per_seq, (const int32_t*)slot->dev, num_seqs,
                                      desc->num_blocks, counter, stream) == cudaSuccess;
     finish_slot(slot, stream);
     uint32_t host = 0;

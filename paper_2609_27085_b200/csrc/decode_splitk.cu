@@ -19,7 +19,9 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "device_common.cuh"
 #include "kernels.h"
@@ -79,7 +81,7 @@ __device__ __forceinline__ void merge_partials(const AttnParams& p, int q_row, i
 }
 
 template <int D, int NWARPS, int NSTAGE>
-__device__ __forceinline__ void decode_cta(const AttnParams& p, const int cta)
+__device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* plan, const int cta)
 {
     constexpr int CPR = D / 8;                  // 16-byte chunks per token row
     constexpr int PAGE_BYTES = 16 * D * 2;      // one (page, head) of K or of V
@@ -91,7 +93,7 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const int cta)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int item_id = cta / p.Hkv, kvh = cta % p.Hkv;
-    const DecodeItem it = p.dec_items[item_id];
+    const DecodeItem it = plan_list<DecodeItem>(plan, p.plan.dec)[item_id];
     const int G = p.G;
     decode_grid_start(p);
 
@@ -342,9 +344,10 @@ __device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t v)
     return pack_f16(f.x, f.y);
 }
 
-template <int NWARPS, int NSTAGE>
-__global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const AttnParams p)
+template <int NWARPS, int NSTAGE, int INL>
+__global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const AttnParams p, const __grid_constant__ PlanBytes<INL> inl)
 {
+    const uint8_t* const plan = INL > 0 ? inl.bytes : p.plan.base;
     constexpr int D = 128;
     constexpr int PAGE_BYTES = 16 * D;          // one (page, head) of K or of V: 16 tokens x 128 one-byte codes
     constexpr int STAGE_BYTES = 2 * PAGE_BYTES;
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const
     const int g = lane >> 2, c = lane & 3;
     if (decode_extra_cta(p)) return;
     const int item_id = blockIdx.x / p.Hkv, kvh = blockIdx.x % p.Hkv;
-    const DecodeItem it = p.dec_items[item_id];
+    const DecodeItem it = plan_list<DecodeItem>(plan, p.plan.dec)[item_id];
     const int G = p.G;
     decode_grid_start(p);
     const float score_scale = p.scale_log2 * __ldg(p.k_scale + kvh);
@@ -590,7 +593,7 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const
 // partial in the member's slot for this chunk; the member's own chunks and the merge follow in the next kernel.
 // Pages are fetched with the default L2 policy: other member sets of the group read them again.
 template <int D, int NWARPS, int NSTAGE, int NCG>
-__device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const int cta)
+__device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const uint8_t* plan, const int cta)
 {
     constexpr int CPR = D / 8;
     constexpr int PAGE_BYTES = 16 * D * 2;
@@ -603,9 +606,9 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const int
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int item_id = cta / p.Hkv, kvh = cta % p.Hkv;
-    const SharedDecodeItem it = p.sh_items[item_id];
+    const SharedDecodeItem it = plan_list<SharedDecodeItem>(plan, p.plan.sh)[item_id];
     decode_grid_start(p);
-    const ShareMember* members = p.sh_members + it.member_first;
+    const ShareMember* members = plan_list<ShareMember>(plan, p.plan.shm) + it.member_first;
     const int G = p.G;
 
     // ---- Q^T fragments of every column group (B operands)
@@ -615,7 +618,7 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const int
         const int col = cg * 8 + (lane >> 2);
         const int m = col / G, head = col % G;
         const bool live = m < it.n_members;
-        const int q_row = live ? __ldg(&members[m].q_row) : 0;
+        const int q_row = live ? members[m].q_row : 0;
         const uint32_t* qrow = reinterpret_cast<const uint32_t*>(p.q + ((int64_t)q_row * p.Hq + (int64_t)kvh * G + head) * D);
 #pragma unroll
         for (int ks = 0; ks < KSTEPS; ++ks) {
@@ -785,7 +788,7 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const int
             o1 += mo[(w * NCOL + col) * DP + d + 1] * f;
         }
         const int m = col / G, hq = kvh * G + col % G;
-        const int64_t pr = (int64_t)(__ldg(&members[m].part_first) + it.chunk) * p.Hq + hq;
+        const int64_t pr = (int64_t)(members[m].part_first + it.chunk) * p.Hq + hq;
         *reinterpret_cast<float2*>(p.part_o + pr * D + d) = make_float2(o0, o1);
         if (d == 0) *reinterpret_cast<float2*>(p.part_ml + pr * 2) = make_float2(M, L);
     }
@@ -798,8 +801,8 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const int
         __threadfence();
         __syncthreads();
         if ((int)threadIdx.x < it.n_members) {
-            uint32_t* counter = p.dec_counters + (int64_t)__ldg(&members[threadIdx.x].part_first) * p.Hkv + kvh;
-            if (atomicAdd(counter, 1u) == (uint32_t)(__ldg(&members[threadIdx.x].n_chunks) - 1)) atomicOr(&last_mask_s, 1u << threadIdx.x);
+            uint32_t* counter = p.dec_counters + (int64_t)members[threadIdx.x].part_first * p.Hkv + kvh;
+            if (atomicAdd(counter, 1u) == (uint32_t)(members[threadIdx.x].n_chunks - 1)) atomicOr(&last_mask_s, 1u << threadIdx.x);
         }
         __syncthreads();
         const uint32_t last_mask = last_mask_s;
@@ -807,8 +810,8 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const int
             __threadfence();
             for (int m = 0; m < it.n_members; ++m) {
                 if (!((last_mask >> m) & 1u)) continue;
-                const int q_row = __ldg(&members[m].q_row), part_first = __ldg(&members[m].part_first);
-                const int n_chunks = __ldg(&members[m].n_chunks);
+                const int q_row = members[m].q_row, part_first = members[m].part_first;
+                const int n_chunks = members[m].n_chunks;
                 for (int idx = threadIdx.x; idx < G * (D / 4); idx += NWARPS * 32) {
                     const int head = idx / (D / 4), d = (idx % (D / 4)) * 4;
                     merge_partials<D>(p, q_row, part_first, n_chunks, kvh * G + head, d, d == 0);
@@ -819,22 +822,23 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const int
     }
 }
 
-template <int D, int NWARPS, int NSTAGE>
-__global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_kernel(const AttnParams p)
+template <int D, int NWARPS, int NSTAGE, int INL>
+__global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_kernel(const AttnParams p, const __grid_constant__ PlanBytes<INL> inl)
 {
     if (decode_extra_cta(p)) return;
-    decode_cta<D, NWARPS, NSTAGE>(p, (int)blockIdx.x);
+    decode_cta<D, NWARPS, NSTAGE>(p, INL > 0 ? inl.bytes : p.plan.base, (int)blockIdx.x);
 }
 
 // One grid for a batch with shared prefixes: the first n_shared_ctas CTAs serve the shared chunks (longer items
 // first), the rest the sequences' own chunks.  Both kinds need half an SM's shared memory, so the larger register
 // footprint of the shared role costs no occupancy; batches without sharing launch decode_splitk_kernel.
-template <int D, int NWARPS, int NSTAGE, int NCG>
-__global__ void __launch_bounds__(NWARPS * 32, 2) decode_with_shared_kernel(const AttnParams p, const int n_shared_ctas)
+template <int D, int NWARPS, int NSTAGE, int NCG, int INL>
+__global__ void __launch_bounds__(NWARPS * 32, 2) decode_with_shared_kernel(const AttnParams p, const __grid_constant__ PlanBytes<INL> inl, const int n_shared_ctas)
 {
     if (decode_extra_cta(p)) return;
-    if ((int)blockIdx.x < n_shared_ctas) decode_shared_cta<D, NWARPS, NSTAGE, NCG>(p, (int)blockIdx.x);
-    else decode_cta<D, NWARPS, NSTAGE>(p, (int)blockIdx.x - n_shared_ctas);
+    const uint8_t* const plan = INL > 0 ? inl.bytes : p.plan.base;
+    if ((int)blockIdx.x < n_shared_ctas) decode_shared_cta<D, NWARPS, NSTAGE, NCG>(p, plan, (int)blockIdx.x);
+    else decode_cta<D, NWARPS, NSTAGE>(p, plan, (int)blockIdx.x - n_shared_ctas);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -845,7 +849,7 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_with_shared_kernel(cons
 template <int D>
 __global__ void __launch_bounds__(D / 4) combine_kernel(const AttnParams p)
 {
-    const CombineItem it = p.comb_items[blockIdx.x];
+    const CombineItem it = plan_list<CombineItem>(p.plan.base, p.plan.comb)[blockIdx.x];
     const int hq = blockIdx.y;
     asm volatile("griddepcontrol.wait;" ::: "memory");     // the decode grid has completed and its partials are visible
     merge_partials<D>(p, it.q_row, it.part_first, it.n_chunks, hq, threadIdx.x * 4, threadIdx.x == 0);
@@ -875,9 +879,18 @@ static size_t decode_smem_bytes()
 
 // Decode grids start before the grid ahead of them in the stream has completed (decode_grid_start): the launch, the
 // work item's fetch and the set-up are off the critical path.  `ctas` is one CTA per (item, KV head).
-template <class K, class... Rest>
-static cudaError_t launch_decode_grid(K kern, int ctas, size_t smem, cudaStream_t stream, const AttnParams& p, Rest... rest)
+template <auto KERN, int INL, class... Rest>
+static cudaError_t launch_decode_grid(int ctas, size_t smem, cudaStream_t stream, const AttnParams& p, const PlanBytes<INL>& inl, Rest... rest)
 {
+    // set once per kernel and device; two host threads racing here both set the same value
+    static std::atomic<bool> configured[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !configured[dev].load(std::memory_order_acquire)) {
+        cudaError_t e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        configured[dev].store(true, std::memory_order_release);
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(ctas + (p.dec_chained ? 1 : 0)));
     cfg.blockDim = dim3(kDecWarps * 32);
@@ -888,75 +901,67 @@ static cudaError_t launch_decode_grid(K kern, int ctas, size_t smem, cudaStream_
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, p, rest...);
+    return cudaLaunchKernelEx(&cfg, KERN, p, inl, rest...);
+}
+
+// launch(size, block) with the parameter block that the plan fits in: none (it is in device memory), small or mid
+template <class F>
+static cudaError_t with_plan_bytes(const HostPlan& hp, F launch)
+{
+    if (!hp.bytes) return launch(std::integral_constant<int, 0>{}, PlanBytes<0>{});
+    auto carry = [&](auto size) {
+        PlanBytes<decltype(size)::value> b;
+        std::memcpy(b.bytes, hp.bytes, hp.size);
+        return launch(size, b);
+    };
+    if (hp.size <= (size_t)kSmallPlanBytes) return carry(std::integral_constant<int, kSmallPlanBytes>{});
+    return hp.size <= (size_t)kMidPlanBytes ? carry(std::integral_constant<int, kMidPlanBytes>{}) : cudaErrorInvalidValue;
 }
 
 template <int D>
-static cudaError_t launch_decode_t(const AttnParams& p, int n_items, cudaStream_t stream)
+static cudaError_t launch_decode_t(const AttnParams& p, const HostPlan& hp, int n_items, cudaStream_t stream)
 {
-    auto kern = decode_splitk_kernel<D, kDecWarps, dec_stages<D>()>;
-    const size_t smem = decode_smem_bytes<D>();
-    // set once per device; two host threads racing here both set the same value
-    static std::atomic<bool> configured[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured[dev].store(true, std::memory_order_release);
-    }
-    return launch_decode_grid(kern, n_items * p.Hkv, smem, stream, p);
+    return with_plan_bytes(hp, [&](auto size, const auto& inl) {
+        return launch_decode_grid<decode_splitk_kernel<D, kDecWarps, dec_stages<D>(), decltype(size)::value>>(
+            n_items * p.Hkv, decode_smem_bytes<D>(), stream, p, inl);
+    });
 }
 
-cudaError_t launch_decode_fp8(const AttnParams& p, int n_items, cudaStream_t stream)
+cudaError_t launch_decode_fp8(const AttnParams& p, const HostPlan& hp, int n_items, cudaStream_t stream)
 {
     if (n_items <= 0) return cudaSuccess;
-    auto kern = decode_splitk_fp8_kernel<kDecWarps, kDecStagesFp8>;
     const size_t ring = (size_t)kDecWarps * kDecStagesFp8 * 2 * 16 * 128;
     const size_t merge = (size_t)kDecWarps * 8 * (128 + 4) * 4 + (size_t)kDecWarps * 8 * 4 * 2;
-    const size_t smem = ring > merge ? ring : merge;
-    static std::atomic<bool> configured[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured[dev].store(true, std::memory_order_release);
-    }
-    return launch_decode_grid(kern, n_items * p.Hkv, smem, stream, p);
+    return with_plan_bytes(hp, [&](auto size, const auto& inl) {
+        return launch_decode_grid<decode_splitk_fp8_kernel<kDecWarps, kDecStagesFp8, decltype(size)::value>>(
+            n_items * p.Hkv, std::max(ring, merge), stream, p, inl);
+    });
 }
 
-cudaError_t launch_decode(const AttnParams& p, int head_dim, int n_items, cudaStream_t stream)
+cudaError_t launch_decode(const AttnParams& p, const HostPlan& hp, int head_dim, int n_items, cudaStream_t stream)
 {
     if (n_items <= 0) return cudaSuccess;
-    return head_dim == 128 ? launch_decode_t<128>(p, n_items, stream) : launch_decode_t<64>(p, n_items, stream);
+    return head_dim == 128 ? launch_decode_t<128>(p, hp, n_items, stream) : launch_decode_t<64>(p, hp, n_items, stream);
 }
 
 template <int D>
-static cudaError_t launch_decode_shared_t(const AttnParams& p, int n_shared_items, int n_items, cudaStream_t stream)
+static cudaError_t launch_decode_shared_t(const AttnParams& p, const HostPlan& hp, int n_shared_items, int n_items, cudaStream_t stream)
 {
     constexpr int NCG = kSharedColumns / 8;
-    auto kern = decode_with_shared_kernel<D, kDecWarps, kDecStages, NCG>;
     const size_t ring = (size_t)kDecWarps * kDecStages * 2 * 16 * D * 2;
     const size_t merge = (size_t)kDecWarps * kSharedColumns * (D + 4) * 4 + (size_t)kDecWarps * kSharedColumns * 4 * 2;
-    const size_t smem = ring > merge ? ring : merge;
-    static std::atomic<bool> configured[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured[dev].store(true, std::memory_order_release);
-    }
-    return launch_decode_grid(kern, (n_shared_items + n_items) * p.Hkv, smem, stream, p, n_shared_items * p.Hkv);
+    return with_plan_bytes(hp, [&](auto size, const auto& inl) {
+        return launch_decode_grid<decode_with_shared_kernel<D, kDecWarps, kDecStages, NCG, decltype(size)::value>>(
+            (n_shared_items + n_items) * p.Hkv, std::max(ring, merge), stream, p, inl, n_shared_items * p.Hkv);
+    });
 }
 
-cudaError_t launch_decode_with_shared(const AttnParams& p, int head_dim, int n_shared_items, int n_items, cudaStream_t stream)
+cudaError_t launch_decode_with_shared(const AttnParams& p, const HostPlan& hp, int head_dim, int n_shared_items, int n_items, cudaStream_t stream)
 {
     if (n_shared_items + n_items <= 0) return cudaSuccess;
-    if (n_shared_items <= 0) return launch_decode(p, head_dim, n_items, stream);
-    return head_dim == 128 ? launch_decode_shared_t<128>(p, n_shared_items, n_items, stream)
-                           : launch_decode_shared_t<64>(p, n_shared_items, n_items, stream);
+    if (n_shared_items <= 0) return launch_decode(p, hp, head_dim, n_items, stream);
+    return head_dim == 128 ? launch_decode_shared_t<128>(p, hp, n_shared_items, n_items, stream)
+                           : launch_decode_shared_t<64>(p, hp, n_shared_items, n_items, stream);
 }
 
 cudaError_t launch_combine(const AttnParams& p, int head_dim, int n_items, cudaStream_t stream)
@@ -1142,14 +1147,14 @@ extern "C" cf_status cf_decode_attention_static(const cf_cache_desc* desc, const
     p.scale_log2 = (desc->softmax_scale > 0.f ? desc->softmax_scale : 1.0f / sqrtf((float)D)) * 1.4426950408889634f;
     p.window = desc->window_size;
     p.sinks = desc->sink_logits;
-    p.dec_items = reinterpret_cast<const DecodeItem*>(su.base);
-    p.comb_items = reinterpret_cast<const CombineItem*>(su.base + comb_off);
+    p.plan.base = su.base;
+    p.plan.comb = (int32_t)comb_off;
     // Partials need no clearing: every slot the combine kernel reads is fully written by its decode CTA
     // in the same call.  This entry point keeps the separate combine kernel (no ticket counters), so nothing
     // in the array has to start at zero; the merge routine and its chunk order are those of the fused merge.
     p.part_o = reinterpret_cast<float*>(su.base + kStaticPlanBytes);
     p.part_ml = reinterpret_cast<float*>(su.base + kStaticPlanBytes + part_o_bytes);
-    if (launch_decode(p, D, pl.n_items, stream) != cudaSuccess) return CF_ERR_CUDA;
+    if (launch_decode(p, HostPlan(), D, pl.n_items, stream) != cudaSuccess) return CF_ERR_CUDA;
     if (launch_combine(p, D, pl.n_comb, stream) != cudaSuccess) return CF_ERR_CUDA;
     return CF_OK;
 }

@@ -99,6 +99,7 @@ struct PlanConfig {
 
 struct Plan {
     std::vector<int32_t> q_start;     // [S+1] exclusive prefix sum of query_len
+    std::vector<int32_t> prefix;      // [S] context_len - query_len (filled by the callers that append)
     std::vector<DecodeItem> decode;   // longest chunk first
     std::vector<CombineItem> combine;
     std::vector<SharedDecodeItem> shared_decode;   // shared-prefix chunks (empty unless the caller described sharing)

@@ -30,6 +30,7 @@
 // error word is set and tensor memory is released.
 #include <atomic>
 #include <climits>
+#include <cstring>
 #include <type_traits>
 
 #include "kernels.h"
@@ -118,7 +119,8 @@ struct Bars {
 template <int D, int MODE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                  const __grid_constant__ CUtensorMap map_v, const AttnParams p, const int n_items, const int queue_ctas,
+                  const __grid_constant__ CUtensorMap map_v, const AttnParams p,
+                  const __grid_constant__ PlanBytes<kSmallPlanBytes> inl, const int n_items, const int queue_ctas,
                   const int first_static, const int ticket_base, const int tail)
 {
     constexpr bool VARIANT = MODE > 0, WINDOW = MODE == 2;
@@ -136,12 +138,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     // the first item of a CTA that starts on a fixed item: fetched now, in use after the set-up below (the plan
     // was uploaded before the kernel that precedes this one in the stream, so it may be read this early)
     const bool has_static = first_static != 0 && (int)blockIdx.x < n_items;
+    const PrefillTcItem* const items = plan_list<PrefillTcItem>(p.plan.base != nullptr ? p.plan.base : inl.bytes, p.plan.pre_tc);
     PrefillTcItem first_it;
     if (warp == 0 && has_static) {
-        const uint4* src = reinterpret_cast<const uint4*>(p.pre_tc_items + blockIdx.x);
+        const uint4* src = reinterpret_cast<const uint4*>(items + blockIdx.x);
         uint4* dst = reinterpret_cast<uint4*>(&first_it);
 #pragma unroll
-        for (int i = 0; i < (int)(sizeof(PrefillTcItem) / 16); ++i) dst[i] = __ldg(src + i);
+        for (int i = 0; i < (int)(sizeof(PrefillTcItem) / 16); ++i) dst[i] = src[i];
     }
     volatile uint32_t* abort_flag = &abort_s;
 
@@ -240,10 +243,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (lane == 0 && *abort_flag == 0u && !counted_out) idx = ticket_base + (int)atomicAdd(p.pre_queue, 1u);
             idx = __shfl_sync(0xffffffffu, idx, 0);
             if (idx < n_items) {
-                const uint4* src = reinterpret_cast<const uint4*>(p.pre_tc_items + idx);
+                const uint4* src = reinterpret_cast<const uint4*>(items + idx);
                 uint4* dst = reinterpret_cast<uint4*>(&cx.it);
 #pragma unroll
-                for (int i = 0; i < (int)(sizeof(PrefillTcItem) / 16); ++i) dst[i] = __ldg(src + i);
+                for (int i = 0; i < (int)(sizeof(PrefillTcItem) / 16); ++i) dst[i] = src[i];
                 derive_ctx(cx);
             } else {
                 cx.live = 0;
@@ -696,9 +699,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 // row per lane (D / 4 lanes take part); the partials of a row are fetched with independent loads (part_k <= 8).
 constexpr int kMaxSplit = 8;
 template <int D>
-__global__ void __launch_bounds__(256) prefill_combine_kernel(const AttnParams p)
+__global__ void __launch_bounds__(256) prefill_combine_kernel(const AttnParams p, const __grid_constant__ PlanBytes<kSmallPlanBytes> inl)
 {
-    const PrefillCombineItem it = p.pre_comb_items[blockIdx.x >> 5];
+    const PrefillCombineItem it = plan_list<PrefillCombineItem>(p.plan.base != nullptr ? p.plan.base : inl.bytes, p.plan.pre_comb)[blockIdx.x >> 5];
     asm volatile("griddepcontrol.wait;" ::: "memory");     // the prefill grid has completed and its partials are visible
     const int lane = threadIdx.x & 31;
     const int rb = blockIdx.x & 31;                  // 32 blocks of 8 rows = 2 tiles x 128 rows
@@ -741,9 +744,11 @@ __global__ void __launch_bounds__(256) prefill_combine_kernel(const AttnParams p
     if (p.lse && lane == 0) p.lse[orow] = (M + log2f(L)) * kLn2;
 }
 
-cudaError_t launch_prefill_combine(const AttnParams& p, int head_dim, int n_items, cudaStream_t stream)
+cudaError_t launch_prefill_combine(const AttnParams& p, const HostPlan& hp, int head_dim, int n_items, cudaStream_t stream)
 {
     if (n_items <= 0) return cudaSuccess;
+    PlanBytes<kSmallPlanBytes> inl;
+    if (hp.bytes) std::memcpy(inl.bytes, hp.bytes, hp.size);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_items * 32);
     cfg.blockDim = dim3(256);
@@ -753,7 +758,7 @@ cudaError_t launch_prefill_combine(const AttnParams& p, int head_dim, int n_item
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return head_dim == 128 ? cudaLaunchKernelEx(&cfg, prefill_combine_kernel<128>, p) : cudaLaunchKernelEx(&cfg, prefill_combine_kernel<64>, p);
+    return head_dim == 128 ? cudaLaunchKernelEx(&cfg, prefill_combine_kernel<128>, p, inl) : cudaLaunchKernelEx(&cfg, prefill_combine_kernel<64>, p, inl);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -832,11 +837,13 @@ bool encode_q_map(CUtensorMap* m, const void* base, int D, int total_rows, int H
 namespace {
 
 template <int D, int MODE>
-cudaError_t launch_prefill_tc_t(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const AttnParams& p,
+cudaError_t launch_prefill_tc_t(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const AttnParams& p, const HostPlan& hp,
                                 int n_items, int n_ctas, int queue_ctas, int first_static, int ticket_base, int tail,
                                 cudaStream_t stream)
 {
     const size_t smem = Geo<D>::SMEM_TOTAL + 1024;
+    PlanBytes<kSmallPlanBytes> inl;
+    if (hp.bytes) std::memcpy(inl.bytes, hp.bytes, hp.size);
     // The register hand-over inside the kernel (setmaxnreg) is sized for LAUNCH_REGS registers per thread at
     // launch; with any other count a grow request could block forever, so such a build is never launched.
     // (both are set once; host threads racing here compute and store the same values)
@@ -867,17 +874,17 @@ cudaError_t launch_prefill_tc_t(const CUtensorMap& mq, const CUtensorMap& mk, co
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, MODE>, mq, mk, mv, p, n_items, queue_ctas, first_static, ticket_base, tail);
+    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, MODE>, mq, mk, mv, p, inl, n_items, queue_ctas, first_static, ticket_base, tail);
 }
 
 }  // namespace
 
-cudaError_t launch_prefill_tc(const AttnParams& p, const PrefillMaps& maps, int head_dim, int n_items, int n_ctas,
+cudaError_t launch_prefill_tc(const AttnParams& p, const HostPlan& hp, const PrefillMaps& maps, int head_dim, int n_items, int n_ctas,
                               int queue_ctas, int first_static, int ticket_base, int tail, cudaStream_t stream)
 {
     if (n_items <= 0 || n_ctas <= 0) return cudaSuccess;
     auto launch = [&](auto DIM, auto MODE) {
-        return launch_prefill_tc_t<decltype(DIM)::value, decltype(MODE)::value>(maps.q, maps.k, maps.v, p, n_items, n_ctas, queue_ctas, first_static, ticket_base, tail, stream);
+        return launch_prefill_tc_t<decltype(DIM)::value, decltype(MODE)::value>(maps.q, maps.k, maps.v, p, hp, n_items, n_ctas, queue_ctas, first_static, ticket_base, tail, stream);
     };
     using std::integral_constant;
     const int mode = p.window > 0 ? 2 : (p.sinks != nullptr || p.k_scale != nullptr) ? 1 : 0;

@@ -93,7 +93,7 @@ prefill_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const bool has_static = first_static != 0 && pair < n_items;
     PrefillTcItem first_it;
     if (warp == 0 && leader && has_static) {
-        const uint4* src = reinterpret_cast<const uint4*>(p.pre_tc_items + pair);
+        const uint4* src = reinterpret_cast<const uint4*>(plan_list<PrefillTcItem>(p.plan.base, p.plan.pre_tc) + pair);
         uint4* dst = reinterpret_cast<uint4*>(&first_it);
 #pragma unroll
         for (int i = 0; i < (int)(sizeof(PrefillTcItem) / 16); ++i) dst[i] = __ldg(src + i);
@@ -236,7 +236,7 @@ prefill_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             if (lane == 0 && *abort_flag == 0u && !counted_out) idx = ticket_base + (int)atomicAdd(p.pre_queue, 1u);
             idx = __shfl_sync(0xffffffffu, idx, 0);
             if (idx < n_items) {
-                const uint4* src = reinterpret_cast<const uint4*>(p.pre_tc_items + idx);
+                const uint4* src = reinterpret_cast<const uint4*>(plan_list<PrefillTcItem>(p.plan.base, p.plan.pre_tc) + idx);
                 uint4* dst = reinterpret_cast<uint4*>(&cx.it);
 #pragma unroll
                 for (int i = 0; i < (int)(sizeof(PrefillTcItem) / 16); ++i) dst[i] = __ldg(src + i);
