@@ -171,7 +171,8 @@ cf_status cf_mixed_attention_planned(cf_plan* plan, const void* q, const void* k
  * out_host.  The caches and the block table stay DEVICE pointers (they are the node's resident
  * state).  The input copy and the read-back run on two context-owned copy streams, ordered against
  * the kernels by events and triple-buffered, so that consecutive calls overlap step i+1's input copy
- * and step i-1's read-back with step i's kernels.  Asynchronous.  out_host of every call issued so far
+ * and step i-1's read-back with step i's kernels.  A step with many prefill rows is computed in parts, prefill first, and
+ * each part is read back while the next one runs.  Asynchronous.  out_host of every call issued so far
  * is valid once cf_host_steps_flush(ctx, stream) has been called and `stream` synchronised; the host
  * input buffers of a call must stay unchanged until then as well. */
 cf_status cf_mixed_step_host(cf_ctx* ctx, const cf_cache_desc* desc,
@@ -203,7 +204,7 @@ cf_status cf_get_async_status(cf_ctx* ctx);
  *     over; a second prefill grid behind it draws from the same work queue, so the SMs decode frees join the prefill.
  *     Everything stays on the caller's stream, and whatever follows there sees all of it completed.
  * Environment at cf_create: CF_OVERLAP=0 (serial), CF_SPATIAL_SMS=n (the share that n = 1 stands for).
- * cf_set_timing and cf_mixed_step_host use the serial sequence. */
+ * cf_set_timing uses the serial sequence, cf_mixed_step_host a sequence of its own choice. */
 cf_status cf_set_overlap(cf_ctx* ctx, int n);
 
 /* The library's default share (host only, no GPU needed): how many of num_sms SMs (0 = 148) the first prefill grid

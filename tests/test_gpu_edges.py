@@ -1,10 +1,12 @@
 """GPU parity at the sizes where a kernel's tiles, ranges and dispatch rules have their edges."""
 import numpy as np
 import pytest
+import torch
 
 import cf_synth as syn
+import oracle
 import paper_2609_27085_b200 as cf
-from harness import run_and_check
+from harness import GpuScenario, compare, run_and_check
 
 pytestmark = pytest.mark.gpu
 
@@ -46,3 +48,34 @@ def test_append_at_the_edges_of_the_row_search(Hq, Hkv, D, fp8, n_seqs):
     prefix = rng.integers(0, 40, size=n_seqs)
     scales = (rng.uniform(0.01, 0.03, Hkv).astype(np.float32), rng.uniform(0.01, 0.03, Hkv).astype(np.float32)) if fp8 else None
     run_and_check(small(71, Hq, Hkv, D, prefix, [qlen], NB=4096), fp8=scales)
+
+
+@pytest.mark.parametrize("prefix,qlen", [
+    ([900, 100, 2000, 50, 40], [650, 1, 1, 1, 1]),                    # one chunk, decode behind it
+    ([3000, 100, 7, 0, 700, 512], [1, 1, 700, 0, 130, 2]),            # decode first; an empty sequence inside the prefill run
+    ([0, 31, 16], [1500, 257, 900]),                                  # prefill alone, cut into parts
+    ([5, 77, 300, 1000], [300, 1, 400, 1]),                           # four runs of alternating kind
+    ([5, 77, 300, 1000, 9], [300, 1, 400, 1, 200]),                   # five runs: computed in one piece
+])
+@pytest.mark.parametrize("window", [0, 200])
+def test_host_steps_in_parts(prefix, qlen, window):
+    """A host-staged step with at least 4 MB of prefill rows is computed and read back in parts."""
+    sc = small(73, 32, 8, 128, prefix, [qlen], NB=1024)
+    b = sc.batches[0]
+    g = GpuScenario(sc, window=window)
+    pin = lambda x: torch.from_numpy(x.view(np.int16)).pin_memory()
+    bt, qh, kh, vh = torch.from_numpy(b.block_table).cuda(), pin(b.q), pin(b.k_new), pin(b.v_new)
+    k_ref, v_ref = sc.k_pool.copy(), sc.v_pool.copy()
+    oracle.kv_append(k_ref, v_ref, b.k_new, b.v_new, b.block_table, b.context_len, b.query_len)
+    rows = syn.tile_edge_rows(b)
+    ref_o, _ = oracle.mixed_attention(b.q, k_ref, v_ref, b.block_table, b.context_len, b.query_len, rows=rows, window=window)
+    for _ in range(4):                                                # more steps than staging sets
+        oh = torch.full_like(qh, -1).pin_memory()
+        cf.cf_mixed_step_host(g.ctx, g.desc, qh, kh, vh, g.k, g.v, bt, b.max_blocks, b.context_len, b.query_len, oh)
+        cf.cf_host_steps_flush(g.ctx)
+    torch.cuda.synchronize()
+    assert cf.cf_get_async_status(g.ctx) == cf.CF_OK
+    compare(oh.numpy().view(np.uint16), None, ref_o, None, rows=rows)
+    kg, vg = g.pools_host()
+    assert np.array_equal(kg, k_ref) and np.array_equal(vg, v_ref)
+    g.close()
