@@ -781,8 +781,7 @@ cf_status cf_plan_create(cf_ctx* c, const cf_cache_desc* desc, const int32_t* co
     if (st != CF_OK) return st;
     Plan pl;
     PlanConfig cfg = c->cfg;
-    const int front_sms = !(c->overlap && !c->in_host_step) ? 0 : c->spatial_sms > 0 ? c->spatial_sms
-                              : spatial_front_sms(desc, context_len, query_len, num_seqs, c->num_sms);
+    const int front_sms = !c->overlap ? 0 : c->spatial_sms > 0 ? c->spatial_sms : spatial_front_sms(desc, context_len, query_len, num_seqs, c->num_sms);
     cfg.prefill_sms_mixed = front_sms;
     cfg.prefill_pair = c->use_pairs && prefill_pair_supported(desc);
     st = build_plan(desc, context_len, query_len, num_seqs, max_blocks_per_seq, cfg, &pl);

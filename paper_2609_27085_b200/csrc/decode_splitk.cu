@@ -1082,7 +1082,7 @@ extern "C" cf_status cf_decode_attention_static(const cf_cache_desc* desc, const
     auto first_page_of = [&](int32_t lc) -> int64_t { return (W > 0 && lc > W) ? (lc - W) / B : 0; };
     const int64_t target = decode_target_pages(
         num_seqs, [&](int32_t s) -> int64_t { return (int64_t)context_len[s] - first_page_of(context_len[s]) * B; }, B,
-        desc->num_kv_heads, D, cfg, false);
+        desc->num_kv_heads, D, false, cfg);
 
     StaticPlan pl;
     for (int32_t s = 0; s < num_seqs; ++s) {

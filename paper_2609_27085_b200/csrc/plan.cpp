@@ -91,7 +91,6 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         if (query_len[s] == 1) ++plan->n_decode_seqs;
         else if (query_len[s] > 1) ++plan->n_prefill_seqs;
     const int32_t quantum = std::max(1, cfg.decode_page_quantum);
-    const bool shares_sms = cfg.prefill_sms_mixed > 0 && plan->n_prefill_seqs > 0;   // spatial sequence: decode runs on part of the machine, beside prefill
     // With a sliding window a decode token at position Lc - 1 sees keys [Lc - W, Lc): the chunks cover the pages
     // from the one that holds the window's left edge onwards, and nothing left of it is ever touched.
     const int32_t W = d->window_size;
@@ -142,7 +141,7 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
     const int64_t target = decode_target_pages(
         num_seqs,
         [&](int32_t s) -> int64_t { return query_len[s] == 1 ? (int64_t)context_len[s] - own_first_page(s) * B : -1; },
-        B, d->num_kv_heads, d->head_dim, cfg, shares_sms, extra_pages);
+        B, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, cfg, extra_pages);
 
     // chunks of the shared part of every group, the same for all of its members
     std::vector<int32_t> n_shared_chunks;      // per sequence

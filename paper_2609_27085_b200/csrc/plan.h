@@ -4,6 +4,7 @@
 // its local prefill queue (Section 5); the planner only partitions work, it does no arithmetic
 // on tensor data.
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <vector>
 
@@ -86,9 +87,8 @@ struct PrefillCombineItem { // one KV-split tcgen05 item: merges its part_k part
 
 struct PlanConfig {
     int32_t num_sms = 148;
-    int32_t decode_ctas_per_sm = 2;   // resident decode CTAs per SM the kernel is built for
-    int32_t decode_waves = 4;         // target number of CTA waves (load balance vs. partial traffic)
-    int32_t decode_min_chunk_pages = 32;
+    int32_t decode_waves = 4;         // most CTA waves that the decode chunks are sized for
+    int32_t decode_min_chunk_pages = 8;
     int32_t decode_page_quantum = 4;  // chunk lengths are multiples of this many pages (warps per CTA)
     int32_t prefill_sms_mixed = 0;    // > 0: SMs the prefill items are balanced over when the batch also holds decode
                                       // work (spatial launch sequence: the first prefill grid's share); 0: num_sms
@@ -122,56 +122,85 @@ cf_status validate_lengths(const cf_cache_desc* d, const int32_t* context_len, c
 // Decode chunking, shared by build_plan and by the allocation-free entry point (plain loops over the
 // caller's arrays: nothing here allocates).  `lc_of(s)` returns the context length of sequence s if it is
 // a decode sequence and a negative number otherwise.
-//   decode_target_pages: the chunk length (in pages) that fills the machine `decode_waves` times, or, for a
-//     batch too small for that, the length from [min, 4 x min] with the smallest waves x CTA time.
+//   decode_target_pages: the chunk length (in pages) with the smallest predicted time among those that fill the resident
+//     CTA slots exactly one, two, ... `decode_waves` times, longer ones, and no split at all.
 //   decode_split: near-equal chunks of at most `target` pages, each a multiple of the page quantum.
+// The prediction, in microseconds, was fitted to 800 (batch, chunk length) pairs: 90 batches of 2 to 256 sequences on all
+// geometries, measured on a B200.  Streaming at full bandwidth (B) and one CTA's way through the longest chunk (g per page)
+// add up in the 1.7-norm, 2.5 for a split (partials, ticket, merge; fp8 cache: 3.2), 1.2 for every further eight chunks of a
+// sequence (the merge takes eight at a time), 2.2 (fp8: 3.5) for every further wave.  Against chunks of at least 32 pages
+// in four waves, decode kernel alone: 40 sequences of 400 tokens, 64 over 8 heads 18.2 -> 14.2 us; 100 of 600 tokens 54 -> 47 us,
+// with head_dim 64 31 -> 23 us; 16 of 600 tokens (head_dim 64) 9.3 -> 7.8 us; 64 of 1500 tokens on an fp8 cache 54 -> 47 us;
+// 64 of 4000 tokens, which four waves fitted, 167 -> 168 us; the 90 shapes 1.06 in the mean.
 template <class LcOf>
-inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int32_t Hkv, int32_t D, const PlanConfig& cfg,
-                                   bool shares_sms, int64_t extra_pages = 0)
+inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int32_t Hkv, int32_t D, bool fp8, const PlanConfig& cfg,
+                                   int64_t extra_pages = 0)
 {
-    const int64_t wave = (int64_t)(cfg.num_sms > 1 ? cfg.num_sms : 1) * (cfg.decode_ctas_per_sm > 1 ? cfg.decode_ctas_per_sm : 1);
-    const int64_t slots = wave * (cfg.decode_waves > 1 ? cfg.decode_waves : 1);
-    const int64_t quantum = cfg.decode_page_quantum > 1 ? cfg.decode_page_quantum : 1;
-    const int64_t min_pages = cfg.decode_min_chunk_pages > 1 ? cfg.decode_min_chunk_pages : 1;
-    int64_t total_pages = 0;
+    constexpr int32_t kMax = 2048;                      // larger batches: whole sequences are chunks enough
+    float pages[kMax];
+    int32_t n = 0;
+    int64_t total = extra_pages, longest = 1;           // extra: pages streamed by shared-prefix items
     for (int32_t s = 0; s < num_seqs; ++s) {
         const int64_t lc = lc_of(s);
-        if (lc >= 0) total_pages += (lc + B - 1) / B;
+        if (lc < 0) continue;
+        const int64_t pg = (lc + B - 1) / B;
+        total += pg;
+        longest = pg > longest ? pg : longest;
+        if (n < kMax) pages[n] = (float)pg;
+        ++n;
     }
-    total_pages += extra_pages;                         // pages streamed by shared-prefix items
-    int64_t target = (total_pages * Hkv + slots - 1) / slots;
-    if (target < min_pages && total_pages > 0 && !shares_sms && extra_pages == 0) {
-        // A small batch: chunks of the minimum length would not fill `decode_waves` waves, and how many waves
-        // of (num_sms x ctas_per_sm) CTAs they do fall into decides the time (a last wave that is a quarter
-        // full costs a whole CTA time).  Try chunk lengths from the minimum to four times it and keep the
-        // one with the smallest waves x (CTA start-up + chunk streaming time).  (Not when decode shares the SMs
-        // with a prefill grid: there the short chunks measured better.)
-        const double page_us = (2.0 * B * D * 2.0) / (7.56e6 / (double)wave);   // one (page, head) of K and V at a CTA's share of HBM
-        const double cta_us = 2.5;
-        double best = 1e30;
-        int64_t best_c = min_pages;
-        for (int64_t c = (min_pages + quantum - 1) / quantum * quantum; c <= 4 * min_pages; c += quantum) {
-            int64_t ctas = 0, longest = 0;
-            for (int32_t s = 0; s < num_seqs; ++s) {
-                const int64_t lc = lc_of(s);
-                if (lc < 0) continue;
-                const int64_t pages = (lc + B - 1) / B;
-                int64_t n = (pages + c - 1) / c;
-                if (n < 1) n = 1;
-                const int64_t per = ((pages + n - 1) / n + quantum - 1) / quantum * quantum;
-                n = per > 0 ? (pages + per - 1) / per : 1;
-                ctas += n;
-                const int64_t len = per < pages ? per : pages;
-                if (len > longest) longest = len;
+    const int64_t quantum = cfg.decode_page_quantum > 1 ? cfg.decode_page_quantum : 1;
+    const int64_t lo = ((cfg.decode_min_chunk_pages > 1 ? cfg.decode_min_chunk_pages : 1) + quantum - 1) / quantum * quantum;
+    const int64_t sms = cfg.num_sms > 1 ? cfg.num_sms : 1;      // of a mixed batch too: the sequences of launches agree bit for bit
+    const int64_t slots = sms * (D == 64 || fp8 ? 3 : 2);      // resident CTAs: 64 KB of shared memory each, or 96 KB
+    const int32_t waves = cfg.decode_waves > 1 ? cfg.decode_waves : 1;
+    auto round_up = [&](int64_t c) { return (c + quantum - 1) / quantum * quantum; };
+    if (n > kMax || extra_pages > 0) {
+        const int64_t c = round_up((total * Hkv + slots * waves - 1) / (slots * waves));
+        return extra_pages > 0 ? (c > 32 ? c : c > lo ? 32 : lo) : (c > lo ? c : lo);
+    }
+    auto chunks = [&](int64_t c) -> int64_t {           // over all sequences (near-equal chunks are rounded up later: at most this)
+        const float inv = 1.0f / (float)c, up = (float)(c - 1);
+        int32_t sum = 0;
+        for (int32_t i = 0; i < n; ++i) sum += (int32_t)((pages[i] + up) * inv + 1e-4f);
+        return sum > n ? sum : n;
+    };
+    const double page_bytes = 2.0 * B * D * (fp8 ? 1.0 : 2.0), g = fp8 ? 0.15 : D == 64 ? 0.077 : 0.113;
+    const double rate = (fp8 ? 6.3e6 : 7.6e6) * (double)sms / 148.0;
+    const double bytes_us = std::pow((double)total * Hkv * page_bytes / rate, 1.7);
+    double best = 1e30;
+    int64_t best_c = lo;
+    // chunks longer than this only unbalance the end of the grid
+    const int64_t hi = lo > 192 ? lo : 192;
+    auto consider = [&](int64_t c) {
+        c = round_up(c < lo ? lo : c);
+        if (c > hi && c < longest) c = hi / quantum * quantum;
+        const int64_t ctas = chunks(c) * Hkv, len = c < longest ? c : longest, of_longest = (longest + c - 1) / c;
+        // further waves: a whole one for any remainder when the chunks are alike, the remainder's part of one when most
+        // are shorter than the longest (they leave their slots early)
+        const double w = (double)ctas / (double)slots, alike = (double)total * Hkv / ((double)ctas * (double)len);
+        const double more = w > 1.0 ? (w - 1.0) + (std::ceil(w) - w) * alike * alike * alike : 0.0;
+        const double t = std::pow(bytes_us + std::pow(g * (double)len, 1.7), 1.0 / 1.7) +
+                         (of_longest > 1 ? (fp8 ? 3.2 : 2.5) + 1.2 * (double)((of_longest - 1) / 8) : 0.0) + (fp8 ? 3.5 : 2.2) * more;
+        if (t < best - 1e-3) { best = t; best_c = c; }
+    };
+    for (int32_t k = 1; k <= waves; ++k) {
+        // the shortest chunk with at most k waves of CTAs (none when even whole sequences are more)
+        int64_t a = lo / quantum, z = round_up(longest > lo ? longest : lo) / quantum;
+        if (chunks(z * quantum) * Hkv <= k * slots) {
+            while (a < z) {
+                const int64_t m = (a + z) / 2;
+                if (chunks(m * quantum) * Hkv <= k * slots) z = m; else a = m + 1;
             }
-            ctas *= Hkv;
-            const double t = (double)((ctas + wave - 1) / wave) * (cta_us + page_us * (double)longest);
-            if (t < best * 0.999) { best = t; best_c = c; }
+            consider(a * quantum);
+            if (k == 1)
+                for (int64_t f : {5, 6, 8, 12}) consider(a * quantum * f / 4);
         }
-        target = best_c;
     }
-    if (target < min_pages) target = min_pages;
-    return (target + quantum - 1) / quantum * quantum;
+    if (longest > 64)
+        for (int64_t c : {32, 64, 96, 128, 160}) consider(c);
+    if (longest <= hi) consider(longest);
+    return best_c;
 }
 inline void decode_split(int64_t pages, int64_t target, int32_t quantum, int64_t* n_chunks, int64_t* pages_per_chunk)
 {

@@ -79,3 +79,17 @@ def test_host_steps_in_parts(prefix, qlen, window):
     kg, vg = g.pools_host()
     assert np.array_equal(kg, k_ref) and np.array_equal(vg, v_ref)
     g.close()
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,fp8", [(16, 2, 64, False), (8, 2, 128, False), (2, 2, 128, False), (16, 2, 128, True)])
+@pytest.mark.parametrize("lens", [
+    [1], [16], [128], [129],                                          # one page, one shortest chunk, one page more
+    [31 * 16, 32 * 16 + 1, 33 * 16],
+    [2500, 1, 77, 4000, 640],                                         # chunks of 8 to 32 pages
+    [193 * 16] * 3 + [192 * 16],                                      # around the longest chunk
+    [300] * 150,                                                      # whole sequences fill the slots
+])
+def test_decode_chunk_lengths(Hq, Hkv, D, fp8, lens):
+    """The decode chunk rule picks chunks of 8 to 192 pages or whole sequences: batches on both sides of its lines."""
+    scales = (np.full(Hkv, 0.02, np.float32), np.full(Hkv, 0.015, np.float32)) if fp8 else None
+    run_and_check(small(79, Hq, Hkv, D, [l - 1 for l in lens], [[1] * len(lens)], NB=4096), fp8=scales)
