@@ -763,7 +763,7 @@ cf_status cf_mixed_attention_shared(cf_ctx* c, const cf_cache_desc* desc, const 
     c->last_counts[0] = n.n_dec; c->last_counts[1] = n.n_comb; c->last_counts[2] = n.n_pre_tc; c->last_counts[3] = n.n_part_slots;
     c->last_counts[4] = n.n_pre_comb; c->last_counts[5] = n.n_shared; c->last_counts[6] = (int32_t)pl.share_members.size();
     c->last_counts[7] = pl.pair ? 1 : 0;
-    n.front_sms = front_sms;
+    n.front_sms = c->spatial_sms > 0 ? front_sms : pl.front_sms;
     const cf_status ls = launch_attention(c, desc, n, ref, hp, c->queue_dev, c->workspace, W,
                                           q, k_cache, v_cache, block_table, max_blocks_per_seq, out, lse, stream, true);
     const cf_status fs = slot ? finish_slot(slot, stream) : CF_OK;
@@ -804,7 +804,7 @@ cf_status cf_plan_create(cf_ctx* c, const cf_cache_desc* desc, const int32_t* co
     P->n_stage_seqs = (int)stage.size(); P->n_stage_pages = n_stage_pages; P->max_stage_pages = max_stage_pages;
     P->n_dec = (int)pl.decode.size(); P->n_comb = (int)pl.combine.size();
     P->n_pre_tc = (int)pl.prefill_tc.size(); P->n_pre_comb = (int)pl.prefill_combine.size(); P->total_q = pl.total_q;
-    P->front_sms = front_sms;
+    P->front_sms = c->spatial_sms > 0 ? front_sms : pl.front_sms;
     P->n_part_slots = pl.n_part_slots; P->n_pre_slots = pl.n_pre_slots;
     P->pair = pl.pair;
     const size_t part_bytes = ws_layout(pl.n_part_slots, pl.n_pre_slots, desc->num_q_heads, desc->head_dim, n_stage_pages,

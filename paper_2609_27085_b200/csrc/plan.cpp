@@ -348,6 +348,19 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         // least 4 tiles.
         const size_t M = (size_t)std::max(1, ((cfg.prefill_sms_mixed > 0 && !plan->decode.empty()) ? cfg.prefill_sms_mixed : cfg.num_sms) /
                                                  (pair ? 2 : 1));      // slots that take an item: SMs, or pairs of SMs
+        // Beside decode that lasts longer than the uncut items an incomplete last wave costs nothing - the call ends with
+        // decode - while ranges would cost their partials and the combine pass (chat mix, 128 items on 88 SMs, one pass:
+        // 40 of them cut in two 277 us, none 263 us).
+        bool decode_outlasts = false;
+        if (cfg.prefill_sms_mixed > 0 && cfg.prefill_sms_mixed < cfg.num_sms && !plan->decode.empty() && !items.empty()) {
+            double bytes = 0.0, tiles = 0.0;
+            for (int32_t s = 0; s < num_seqs; ++s)
+                if (query_len[s] == 1)
+                    bytes += 2.0 * (W > 0 ? std::min(context_len[s], W) : context_len[s]) * d->num_kv_heads * d->head_dim * (d->kv_dtype == CF_KV_FP8_E4M3 ? 1 : 2);
+            for (const KeyedTc& k : items) tiles += k.tiles;
+            const double rounds = std::ceil((double)items.size() / (double)M), rate = std::min(7.1e6, 8.5e4 * (cfg.num_sms - cfg.prefill_sms_mixed));
+            decode_outlasts = 8.0 + bytes / rate >= rounds * (8.0 + 1.9 * tiles / (double)items.size());
+        }
         // decides the KV ranges per item for one candidate item list; returns the predicted time (us)
         auto decide = [&](const std::vector<KeyedTc>& its, const double tile_us, std::vector<int32_t>& k_of) -> double {
         const size_t n_items = its.size();
@@ -392,7 +405,7 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
                 const double t = list_schedule(jobs, M) + split_extra(n_ranges);
                 if (t < best * 0.95) { best = t; k_of = cand; predicted = t; }
             }
-        } else if (n_items % M != 0) {
+        } else if (n_items % M != 0 && !decode_outlasts) {
             // Several waves of similar items: after the full waves the remaining r items would hold r SMs
             // for a whole item time; cutting each into k ranges lets them fill the machine.
             const size_t r = n_items % M, first_tail = n_items - r;
@@ -424,6 +437,17 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
             }
         }
         const size_t n_items = items.size();
+        // The first prefill grid: as many SMs as the batch's share, or fewer that need no more rounds when the items are alike
+        // (chat mix: two rounds of 64 instead of 88 and 40: 263 -> 256 us, decode has the SMs).
+        if (cfg.prefill_sms_mixed > 0 && !plan->decode.empty()) {
+            plan->front_sms = cfg.prefill_sms_mixed;
+            const size_t slots = M, rounds = n_items > 0 ? (n_items + slots - 1) / slots : 1;
+            const bool whole = std::all_of(k_of.begin(), k_of.end(), [](int32_t k) { return k == 1; });
+            int32_t least = INT32_MAX, most = 0;
+            for (const KeyedTc& k : items) { least = std::min(least, k.tiles); most = std::max(most, k.tiles); }
+            if (whole && rounds >= 2 && rounds <= 4 && (double)most <= 1.25 * (double)least)
+                plan->front_sms = (int32_t)((n_items + rounds - 1) / rounds) * (pair ? 2 : 1);
+        }
         for (size_t i = 1; i < n_items; ++i)
             if (items[i].sub > 0) k_of[i] = k_of[i - 1];      // the items of a block and KV head are cut alike
         plan->prefill_tc.reserve(n_items + 8 * plan->prefill_combine.capacity());
@@ -510,7 +534,7 @@ int32_t spatial_front_sms(const cf_cache_desc* d, const int32_t* context_len, co
     }
     if (dec_bytes == 0.0 || work == 0.0) return 0;
     const double sms = (double)std::max(1, num_sms);
-    const double t_dec = 17.0 + dec_bytes / 7.1e6, k_sat = G > 4 ? 100.0 : 65.0;
+    const double t_dec = 8.0 + dec_bytes / 7.1e6, k_sat = G > 4 ? 100.0 : 65.0;
     const double t_call = work / sms + t_dec * k_sat / sms;              // both parts packed without idle SMs
     const double k_dec = 1.15 * k_sat * t_dec / t_call;
     const double front = std::min(std::max(sms - k_dec, 0.6 * sms), 0.875 * sms);

@@ -112,6 +112,8 @@ struct Plan {
     int32_t n_decode_seqs = 0;
     int32_t n_prefill_seqs = 0;
     bool pair = false;                // prefill_tc items are pair items (four q tiles, two CTAs)
+    int32_t front_sms = 0;            // mixed batch of the spatial sequence: SMs that the first prefill grid takes (at most
+                                      // cfg.prefill_sms_mixed; fewer when they need no more rounds for items of like length)
 };
 
 // Validates geometry (supported head_dim / block_size / group / strides).
