@@ -492,13 +492,13 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
         p.dec_chained = 1;
         if (e == cudaSuccess) e = decode_launch(stream);
         if (e == cudaSuccess) e = launch_prefill(tail, front + tail, 0, front, 1);
-        if (e == cudaSuccess) e = launch_combine(p, D, fused_combine ? 0 : n.n_comb, stream);
+        if (e == cudaSuccess) e = launch_combine(p, hp, D, fused_combine ? 0 : n.n_comb, stream);
         if (e == cudaSuccess) e = launch_prefill_combine(pp, hp, D, n.n_pre_comb, stream);
     } else {
         if (tc) cudaEventRecord(tc->ev[0], stream);
         if (e == cudaSuccess) e = decode_launch(stream);
         if (tc) cudaEventRecord(tc->ev[1], stream);
-        if (e == cudaSuccess) e = launch_combine(p, D, fused_combine ? 0 : n.n_comb, stream);
+        if (e == cudaSuccess) e = launch_combine(p, hp, D, fused_combine ? 0 : n.n_comb, stream);
         if (tc) cudaEventRecord(tc->ev[2], stream);
         if (e == cudaSuccess) e = stage_pages(stream);
         if (e == cudaSuccess) e = launch_prefill(pre_ctas, pre_ctas, 1, pre_ctas, 0);

@@ -34,7 +34,7 @@ cudaError_t launch_kv_append(const AppendParams& p, cudaStream_t stream);
 cudaError_t launch_validate_table(const int32_t* block_table, int32_t max_blocks, const int32_t* context_len_dev,
                                   int32_t num_seqs, int32_t num_blocks, uint32_t* bad_count, cudaStream_t stream);
 cudaError_t launch_decode(const AttnParams& p, const HostPlan& hp, int head_dim, int n_items, cudaStream_t stream);
-cudaError_t launch_combine(const AttnParams& p, int head_dim, int n_items, cudaStream_t stream);
+cudaError_t launch_combine(const AttnParams& p, const HostPlan& hp, int head_dim, int n_items, cudaStream_t stream);
 // split-K decode over an fp8 (e4m3) cache, head_dim 128: same items, partials and merge as launch_decode
 cudaError_t launch_decode_fp8(const AttnParams& p, const HostPlan& hp, int n_items, cudaStream_t stream);
 // fp8 cache: expands the pages that prefill chunks need into bf16 staging pools [n_stage_pages, Hkv, 16, 128] (the codes
