@@ -36,6 +36,13 @@ def test_windows_around_the_skipped_column_chunks(Hq, Hkv, D, window):
     run_and_check(small(67, Hq, Hkv, D, [0, 5, 1000, 1023, 313, 64], [[150, 40, 129, 33, 300, 1]]), window=window)
 
 
+@pytest.mark.parametrize("Hq,Hkv,D", [(16, 2, 64), (8, 2, 128), (2, 2, 128)])
+def test_causal_edges_around_the_masked_column_chunks(Hq, Hkv, D):
+    """The causal mask is applied to the 32-column chunks that it crosses: prefixes one short of, at and one past a
+    chunk's and a tile's edge."""
+    run_and_check(small(68, Hq, Hkv, D, [0, 30, 31, 32, 33, 95, 127, 128], [[1, 33, 40, 2, 64, 130, 3, 31]]))
+
+
 @pytest.mark.parametrize("Hq,Hkv,D,fp8", [(2, 2, 64, False), (8, 2, 128, False), (24, 24, 64, False), (32, 8, 128, True), (24, 24, 128, True)])
 @pytest.mark.parametrize("n_seqs", [1, 2, 31, 32, 33, 65, 1030])
 def test_append_at_the_edges_of_the_row_search(Hq, Hkv, D, fp8, n_seqs):
