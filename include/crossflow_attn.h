@@ -269,7 +269,7 @@ cf_status cf_get_host_time_sums(cf_ctx* ctx, double* us_append, double* us_atten
                                 int32_t* num_steps);
 /* Item counts of the plan the last cf_mixed_attention(_shared) built, for tests and reports: counts[8] =
  * {decode items, split decode sequences, prefill CTAs, decode partial slots, KV-split prefill items,
- *  shared-prefix items, members of shared-prefix sets, 1 if the prefill items are pair items (two CTAs each)}. */
+ *  shared-prefix units (a shared KV chunk x 16 query-head columns), members of shared-prefix sets, 1 if the prefill items are pair items (two CTAs each)}. */
 cf_status cf_get_last_plan_counts(cf_ctx* ctx, int32_t* counts);
 /* Number of kernels the last cf_mixed_attention launched. */
 cf_status cf_get_last_launch_count(cf_ctx* ctx, int32_t* num_launches);

@@ -212,6 +212,13 @@ static size_t layout_of(const Plan& pl, size_t n_stage_seqs, PlanRef* r)
     list(&r->stage, sizeof(StageSeq) * n_stage_seqs);
     return at;
 }
+static int32_t shared_units(const Plan& pl, const cf_cache_desc* d)
+{
+    const int32_t per_unit = std::max(1, 16 / (d->num_q_heads / d->num_kv_heads));       // members whose heads fill 16 columns
+    int32_t n = 0;
+    for (const SharedDecodeItem& it : pl.shared_decode) n += (it.n_members + per_unit - 1) / per_unit;
+    return n;
+}
 static void write_plan(uint8_t* dst, const Plan& pl, const std::vector<StageSeq>& stage, const PlanRef& r)
 {
     auto list = [&](int32_t off, const void* src, size_t bytes) {
@@ -397,7 +404,7 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
     p.plan = plan;
     p.part_o = (float*)((uint8_t*)ws + W.dec_o);
     p.part_ml = (float*)((uint8_t*)ws + W.dec_ml);
-    const bool fused_combine = c->fused_combine && (size_t)n.n_part_slots * desc->num_kv_heads * sizeof(uint32_t) <= kCounterBytes;
+    const bool fused_combine = c->fused_combine && n.n_shared == 0 && (size_t)n.n_part_slots * desc->num_kv_heads * sizeof(uint32_t) <= kCounterBytes;
     p.dec_chained = 0;
     p.dec_counters = fused_combine ? (uint32_t*)ws : nullptr;
     p.pre_part_o = (float*)((uint8_t*)ws + W.pre_o);
@@ -761,7 +768,7 @@ cf_status cf_mixed_attention_shared(cf_ctx* c, const cf_cache_desc* desc, const 
     n.pair = pl.pair;
     n.n_stage_seqs = (int)stage.size(); n.n_stage_pages = n_stage_pages; n.max_stage_pages = max_stage_pages; n.num_seqs = num_seqs;
     c->last_counts[0] = n.n_dec; c->last_counts[1] = n.n_comb; c->last_counts[2] = n.n_pre_tc; c->last_counts[3] = n.n_part_slots;
-    c->last_counts[4] = n.n_pre_comb; c->last_counts[5] = n.n_shared; c->last_counts[6] = (int32_t)pl.share_members.size();
+    c->last_counts[4] = n.n_pre_comb; c->last_counts[5] = shared_units(pl, desc); c->last_counts[6] = (int32_t)pl.share_members.size();
     c->last_counts[7] = pl.pair ? 1 : 0;
     n.front_sms = c->spatial_sms > 0 ? front_sms : pl.front_sms;
     const cf_status ls = launch_attention(c, desc, n, ref, hp, c->queue_dev, c->workspace, W,

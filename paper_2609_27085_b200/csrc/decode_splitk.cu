@@ -34,39 +34,46 @@ namespace cf {
 //   M = max_c m_c ; O = sum_c 2^(m_c - M) o_c / sum_c 2^(m_c - M) l_c ; lse = (M + log2 sum) ln 2
 // evaluated as a running merge over groups of eight chunks.  Partials are fetched eight chunks at a time
 // with independent L2 loads (a dependent load per chunk would cost a memory round trip each; L2 loads,
-// because in the fused path other CTAs of the same grid wrote them).
-template <int D>
+// because in the fused path other CTAs of the same grid wrote them).  GROUPS groups are fetched at once where registers
+// are free for it; the arithmetic is the same.
+template <int D, int GROUPS = 1>
 __device__ __forceinline__ void merge_partials(const AttnParams& p, int q_row, int part_first, int n_chunks, int hq, int d,
                                                bool write_lse)
 {
     constexpr int GROUP = 8;
     float M = -INFINITY, L = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int c0 = 0; c0 < n_chunks; c0 += GROUP) {
-        float2 ml[GROUP];
-        float4 v[GROUP];
+    for (int c0 = 0; c0 < n_chunks; c0 += GROUPS * GROUP) {
+        float2 ml[GROUPS * GROUP];
+        float4 v[GROUPS * GROUP];
 #pragma unroll
-        for (int i = 0; i < GROUP; ++i)
+        for (int i = 0; i < GROUPS * GROUP; ++i)
             if (c0 + i < n_chunks) {
                 const int64_t pr = (int64_t)(part_first + c0 + i) * p.Hq + hq;
                 ml[i] = __ldcg(reinterpret_cast<const float2*>(p.part_ml + pr * 2));
                 v[i] = __ldcg(reinterpret_cast<const float4*>(p.part_o + pr * D + d));
             }
-        float Mg = M;
 #pragma unroll
-        for (int i = 0; i < GROUP; ++i)
-            if (c0 + i < n_chunks) Mg = fmaxf(Mg, ml[i].x);
-        const float fold = fast_exp2(M - Mg);               // 0 on the first group (M = -inf)
-        L *= fold;
-        acc.x *= fold; acc.y *= fold; acc.z *= fold; acc.w *= fold;
-        M = Mg;
+        for (int g = 0; g < GROUPS; ++g) {
+            if (c0 + g * GROUP >= n_chunks) break;
+            float Mg = M;
 #pragma unroll
-        for (int i = 0; i < GROUP; ++i)
-            if (c0 + i < n_chunks) {
-                const float f = fast_exp2(ml[i].x - M);
-                L += ml[i].y * f;
-                acc.x += v[i].x * f; acc.y += v[i].y * f; acc.z += v[i].z * f; acc.w += v[i].w * f;
-            }
+            for (int i = g * GROUP; i < (g + 1) * GROUP; ++i)
+                if (c0 + i < n_chunks) Mg = fmaxf(Mg, ml[i].x);
+            const float fold = fast_exp2(M - Mg);               // 0 on the first group (M = -inf)
+            // products and sums spelled out: the compiler's choice of what to fuse must not depend on GROUPS
+            L = __fmul_rn(L, fold);
+            acc.x = __fmul_rn(acc.x, fold); acc.y = __fmul_rn(acc.y, fold); acc.z = __fmul_rn(acc.z, fold); acc.w = __fmul_rn(acc.w, fold);
+            M = Mg;
+#pragma unroll
+            for (int i = g * GROUP; i < (g + 1) * GROUP; ++i)
+                if (c0 + i < n_chunks) {
+                    const float f = fast_exp2(ml[i].x - M);
+                    L = __fmaf_rn(ml[i].y, f, L);
+                    acc.x = __fmaf_rn(v[i].x, f, acc.x); acc.y = __fmaf_rn(v[i].y, f, acc.y);
+                    acc.z = __fmaf_rn(v[i].z, f, acc.z); acc.w = __fmaf_rn(v[i].w, f, acc.w);
+                }
+        }
     }
     float shrink = 1.f;
     if (p.sinks != nullptr) shrink = join_sink(__ldg(p.sinks + hq) * kLog2e, M, L);
@@ -80,22 +87,25 @@ __device__ __forceinline__ void merge_partials(const AttnParams& p, int q_row, i
     if (p.lse && write_lse) p.lse[(int64_t)q_row * p.Hq + hq] = (M + log2f(L)) * kLn2;
 }
 
-// Exponentials of one page's scores of one column group (8 heads) and running sums.  The reference maximum of a head is
+// Exponentials of one page's scores (N = 4 per thread; two pages: 8) of one column group (8 heads) and running sums.  The reference maximum of a head is
 // only raised when some score exceeds it by more than 2^kRaise: then the exact maximum over the page is taken (three shuffles
 // per head) and the accumulators are rescaled; a page without such a score costs a vote.  (Probabilities up to 2^kRaise keep
 // their relative precision, in bf16, fp16 and in the fp32 sums.)  Raising at every page instead is six shuffles, two
 // exponentials and 32 multiplications per page more, which show where the kernel is not bound by HBM: shared-prefix
 // decode 39.2 -> 38.1 us per pass, 256 sequences on an fp8 cache beside four chunks 294 -> 288 us, chat mix 264 -> 258 us.
 constexpr float kRaise = 8.f;
-template <int KSTEPS>
-__device__ __forceinline__ void page_softmax(float (&s)[4], float (&m_run)[2], float (&l_run)[2], float (&o)[KSTEPS][4])
+template <int N, int KSTEPS>
+__device__ __forceinline__ void page_softmax(float (&s)[N], float (&m_run)[2], float (&l_run)[2], float (&o)[KSTEPS][4])
 {
-    const bool raise = fmaxf(s[0], s[2]) > m_run[0] + kRaise || fmaxf(s[1], s[3]) > m_run[1] + kRaise;
+    float top[2] = {s[0], s[1]};            // element e belongs to head e & 1; four elements per page
+#pragma unroll
+    for (int e = 2; e < N; ++e) top[e & 1] = fmaxf(top[e & 1], s[e]);
+    const bool raise = top[0] > m_run[0] + kRaise || top[1] > m_run[1] + kRaise;
     if (__any_sync(0xffffffffu, raise)) {
         float alpha[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            float mx = fmaxf(s[j], s[2 + j]);
+            float mx = top[j];
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
@@ -111,11 +121,13 @@ __device__ __forceinline__ void page_softmax(float (&s)[4], float (&m_run)[2], f
         }
     }
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        s[j] = fast_exp2(s[j] - m_run[j]);
-        s[2 + j] = fast_exp2(s[2 + j] - m_run[j]);
-        l_run[j] += s[j] + s[2 + j];
-    }
+    for (int e = 0; e < N; e += 4)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            s[e + j] = fast_exp2(s[e + j] - m_run[j]);
+            s[e + 2 + j] = fast_exp2(s[e + 2 + j] - m_run[j]);
+            l_run[j] += s[e + j] + s[e + 2 + j];
+        }
 }
 
 template <int D, int NWARPS, int NSTAGE>
@@ -594,35 +606,44 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const
 // ---------------------------------------------------------------------------------------------
 // Shared-prefix decode: one CTA serves one (share group, shared KV chunk, KV head) for a SET of member sequences.
 // The chunk lies inside the prefix that all members have in common (same physical pages), so its K/V is streamed
-// once and the members' query heads ride along as MMA columns: NCG column groups of 8, column c of the set =
-// head c % G of member c / G.  Loop structure, ring and fragment layouts are those of decode_splitk_kernel; there
+// once and the members' query heads ride along as MMA columns: column c of the set = head c % G of member c / G.  A warp
+// carries NCG column groups of 8; WC warps split the columns of a page between them and the NWARPS / WC such teams
+// split the pages.  A team shares a page ring (every member fetches its part of a page, one barrier per page), so a
+// page comes in once for up to 64 columns.  Fragment layouts are those of decode_splitk_kernel; there
 // is no masking at all (whole pages, every token visible to every member).  Every (member, head) gets an fp32
-// partial in the member's slot for this chunk; the member's own chunks and the merge follow in the next kernel.
+// partial in the member's slot for this chunk; the merge follows in the combine kernel (a set's members all become
+// complete at the same time, and one CTA merging them one after the other took longer than the launch).
 // Pages are fetched with the default L2 policy: other member sets of the group read them again.
-template <int D, int NWARPS, int NSTAGE, int NCG>
-__device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const uint8_t* plan, const int cta)
+// What bounds it is the chain of a page inside a warp and what a CTA pays around its pages, not HBM.  One pass on a B200, 8192
+// tokens shared, 32 / 8 heads of 128, 4 / 16 / 64 sequences: 32.3 / 38.4 / 102.8 us with 16 columns per CTA and
+// the merge inside the kernel, 17.3 / 29.1 / 75.7 us with this layout.  Of that: two pages per step instead of one
+// 0.51 -> 0.45 us per page; partials written by float4 with the row of a column looked up once 5500 -> 1500 cycles.
+template <int D, int NWARPS, int NSTAGE, int NCG, int WC>
+__device__ __forceinline__ void decode_shared_team(const AttnParams& p, const SharedDecodeItem& it, const ShareMember* members, const int kvh)
 {
     constexpr int CPR = D / 8;
     constexpr int PAGE_BYTES = 16 * D * 2;
     constexpr int STAGE_BYTES = 2 * PAGE_BYTES;
-    constexpr int WARP_BYTES = NSTAGE * STAGE_BYTES;
+    constexpr int WP = NWARPS / WC, DEPTH = NSTAGE * WC;
     constexpr int KSTEPS = D / 16;
     constexpr int DP = D + 4;
     constexpr int NCOL = NCG * 8;
+    constexpr int NP = DEPTH >= 6 ? 2 : 1;            // pages per step: two hide each other's chains of dependent MMAs
     extern __shared__ __align__(1024) uint8_t smem[];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int item_id = cta / p.Hkv, kvh = cta % p.Hkv;
-    const SharedDecodeItem it = plan_list<SharedDecodeItem>(plan, p.plan.sh)[item_id];
-    decode_grid_start(p);
-    const ShareMember* members = plan_list<ShareMember>(plan, p.plan.shm) + it.member_first;
-    const int G = p.G;
+    const int wc = warp % WC, wp = warp / WC;
+    const int G = p.G, n_cols = it.n_members * G;
+    // row of the partials that a column goes to
+    __shared__ int32_t col_row[kSharedColumns];
+    if ((int)threadIdx.x < n_cols)
+        col_row[threadIdx.x] = (members[threadIdx.x / G].part_first + it.chunk) * p.Hq + kvh * G + (int)threadIdx.x % G;
 
     // ---- Q^T fragments of every column group (B operands)
     uint32_t qf[NCG][KSTEPS][2];
 #pragma unroll
     for (int cg = 0; cg < NCG; ++cg) {
-        const int col = cg * 8 + (lane >> 2);
+        const int col = wc * NCOL + cg * 8 + (lane >> 2);
         const int m = col / G, head = col % G;
         const bool live = m < it.n_members;
         const int q_row = live ? members[m].q_row : 0;
@@ -636,9 +657,13 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const uin
 
     const int first_page = it.kv_begin >> 4;
     const int n_pages = (it.kv_end - it.kv_begin) >> 4;
-    const int my_n = n_pages > warp ? (n_pages - warp + NWARPS - 1) / NWARPS : 0;
-    const int32_t* bt = p.block_table + (int64_t)it.seq * p.max_blocks + first_page + warp;
-    const uint32_t wbase = smem_u32(smem) + warp * WARP_BYTES;
+    const int my_n = n_pages > wp ? (n_pages - wp + WP - 1) / WP : 0;
+    const int32_t* bt = p.block_table + (int64_t)it.seq * p.max_blocks + first_page + wp;
+    const uint32_t wbase = smem_u32(smem) + wp * (DEPTH * STAGE_BYTES);
+    auto team_sync = [&]() {
+        if constexpr (WC == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + wp), "n"(WC * 32) : "memory");
+    };
     const __nv_bfloat16* kbase = p.k_cache + (int64_t)kvh * p.ks_head;
     const __nv_bfloat16* vbase = p.v_cache + (int64_t)kvh * p.vs_head;
 
@@ -648,20 +673,20 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const uin
         return 0;
     };
     int cache_base = 0;
-    int32_t pid_cache = (lane < my_n) ? checked(__ldg(bt + lane * NWARPS)) : 0;
+    int32_t pid_cache = (lane < my_n) ? checked(__ldg(bt + lane * WP)) : 0;
 
     auto issue = [&](int i) {
         if (i - cache_base == 32) {
             cache_base = i;
-            pid_cache = (i + lane < my_n) ? checked(__ldg(bt + (i + lane) * NWARPS)) : 0;
+            pid_cache = (i + lane < my_n) ? checked(__ldg(bt + (i + lane) * WP)) : 0;
         }
         const int32_t pid = __shfl_sync(0xffffffffu, pid_cache, i - cache_base);
-        const uint32_t sbase = wbase + (i % NSTAGE) * STAGE_BYTES;
+        const uint32_t sbase = wbase + (i % DEPTH) * STAGE_BYTES;
         const __nv_bfloat16* kp = kbase + (int64_t)pid * p.ks_block;
         const __nv_bfloat16* vp = vbase + (int64_t)pid * p.vs_block;
 #pragma unroll
-        for (int r = 0; r < (16 * CPR) / 32; ++r) {
-            const int id = r * 32 + lane;
+        for (int r = 0; r < (16 * CPR) / (32 * WC); ++r) {
+            const int id = (r * WC + wc) * 32 + lane;
             const int t = id / CPR, c = id % CPR;
             cp_async16(sbase + tile_off<16>(t, c), kp + t * p.ks_token + c * 8, 16);
             cp_async16(sbase + PAGE_BYTES + tile_off<16>(t, c), vp + t * p.vs_token + c * 8, 16);
@@ -679,54 +704,70 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const uin
     }
 
 #pragma unroll
-    for (int s = 0; s < NSTAGE - 1; ++s) {
+    for (int s = 0; s < DEPTH - NP; ++s) {
         if (s < my_n) issue(s);
         cp_async_commit();
     }
 
-    for (int i = 0; i < my_n; ++i) {
-        cp_async_wait<NSTAGE - 2>();
-        __syncwarp();
-        if (i + NSTAGE - 1 < my_n) issue(i + NSTAGE - 1);
-        cp_async_commit();
-
-        const uint32_t sK = wbase + (i % NSTAGE) * STAGE_BYTES;
-        const uint32_t sV = sK + PAGE_BYTES;
-
-        // S^T = K Q^T: one K fragment feeds every column group
-        float sacc[NCG][4];
+    auto step = [&](auto PAGES, const int i) {
+        constexpr int np = decltype(PAGES)::value;
+        uint32_t sK[np];
 #pragma unroll
-        for (int cg = 0; cg < NCG; ++cg) sacc[cg][0] = sacc[cg][1] = sacc[cg][2] = sacc[cg][3] = 0.f;
+        for (int u = 0; u < np; ++u) sK[u] = wbase + ((i + u) % DEPTH) * STAGE_BYTES;
+        // S^T = K Q^T: one K fragment feeds every column group
+        float sacc[NCG][np][4];
+#pragma unroll
+        for (int cg = 0; cg < NCG; ++cg)
+#pragma unroll
+            for (int u = 0; u < np; ++u) sacc[cg][u][0] = sacc[cg][u][1] = sacc[cg][u][2] = sacc[cg][u][3] = 0.f;
         {
             const int t = (lane & 7) + ((lane >> 3) & 1) * 8;
 #pragma unroll
-            for (int ks = 0; ks < KSTEPS; ++ks) {
-                uint32_t a[4];
-                ldmatrix_x4(a, sK + tile_off<16>(t, 2 * ks + (lane >> 4)));
+            for (int ks = 0; ks < KSTEPS; ++ks)
 #pragma unroll
-                for (int cg = 0; cg < NCG; ++cg) mma_bf16_16816(sacc[cg], a, qf[cg][ks][0], qf[cg][ks][1]);
-            }
+                for (int u = 0; u < np; ++u) {
+                    uint32_t a[4];
+                    ldmatrix_x4(a, sK[u] + tile_off<16>(t, 2 * ks + (lane >> 4)));
+#pragma unroll
+                    for (int cg = 0; cg < NCG; ++cg) mma_bf16_16816(sacc[cg][u], a, qf[cg][ks][0], qf[cg][ks][1]);
+                }
         }
-        uint32_t pb[NCG][2];
+        uint32_t pb[NCG][np][2];
 #pragma unroll
         for (int cg = 0; cg < NCG; ++cg) {
-            float s[4];
+            float s[4 * np];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) s[e] = sacc[cg][e] * p.scale_log2;
+            for (int e = 0; e < 4 * np; ++e) s[e] = sacc[cg][e >> 2][e & 3] * p.scale_log2;
             page_softmax(s, m_run[cg], l_run[cg], o[cg]);
-            pb[cg][0] = movmatrix_trans(pack_bf16(s[0], s[1]));
-            pb[cg][1] = movmatrix_trans(pack_bf16(s[2], s[3]));
+#pragma unroll
+            for (int u = 0; u < np; ++u) {
+                pb[cg][u][0] = movmatrix_trans(pack_bf16(s[4 * u], s[4 * u + 1]));
+                pb[cg][u][1] = movmatrix_trans(pack_bf16(s[4 * u + 2], s[4 * u + 3]));
+            }
         }
         {
             const int t = (lane & 7) + (lane >> 4) * 8;
 #pragma unroll
-            for (int mt = 0; mt < KSTEPS; ++mt) {
-                uint32_t a[4];
-                ldmatrix_x4_trans(a, sV + tile_off<16>(t, 2 * mt + ((lane >> 3) & 1)));
+            for (int mt = 0; mt < KSTEPS; ++mt)
 #pragma unroll
-                for (int cg = 0; cg < NCG; ++cg) mma_bf16_16816(o[cg][mt], a, pb[cg][0], pb[cg][1]);
-            }
+                for (int u = 0; u < np; ++u) {
+                    uint32_t a[4];
+                    ldmatrix_x4_trans(a, sK[u] + PAGE_BYTES + tile_off<16>(t, 2 * mt + ((lane >> 3) & 1)));
+#pragma unroll
+                    for (int cg = 0; cg < NCG; ++cg) mma_bf16_16816(o[cg][mt], a, pb[cg][u][0], pb[cg][u][1]);
+                }
         }
+    };
+    for (int i = 0; i < my_n; i += NP) {
+        cp_async_wait<DEPTH - 2 * NP>();
+        team_sync();                                   // the pages are in, and the slots of the step before are free
+#pragma unroll
+        for (int u = 0; u < NP; ++u) {
+            if (i + DEPTH - NP + u < my_n) issue(i + DEPTH - NP + u);
+            cp_async_commit();
+        }
+        if (NP == 1 || i + 1 < my_n) step(std::integral_constant<int, NP>{}, i);
+        else step(std::integral_constant<int, 1>{}, i);
     }
     cp_async_wait<0>();
 
@@ -762,53 +803,41 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const uin
     }
     __syncthreads();
 
-    const int n_cols = it.n_members * G;
-    for (int idx = threadIdx.x; idx < n_cols * (D / 2); idx += NWARPS * 32) {
-        const int col = idx / (D / 2), d = (idx % (D / 2)) * 2;
+    // the warps w0, w0 + WC, ... carried column w0 * NCOL + c
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < n_cols * (D / 4); idx += NWARPS * 32) {
+        const int col = idx / (D / 4), d = (idx % (D / 4)) * 4;
+        const int w0 = col / NCOL, c = col % NCOL;
         float M = -INFINITY;
 #pragma unroll
-        for (int w = 0; w < NWARPS; ++w) M = fmaxf(M, mm[w * NCOL + col]);
-        float L = 0.f, o0 = 0.f, o1 = 0.f;
+        for (int w = 0; w < WP; ++w) M = fmaxf(M, mm[(w * WC + w0) * NCOL + c]);
+        float L = 0.f;
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int w = 0; w < NWARPS; ++w) {
-            const float f = fast_exp2(mm[w * NCOL + col] - M);   // idle warps: 2^(-inf) = 0
-            L += ml[w * NCOL + col] * f;
-            o0 += mo[(w * NCOL + col) * DP + d] * f;
-            o1 += mo[(w * NCOL + col) * DP + d + 1] * f;
+        for (int w = 0; w < WP; ++w) {
+            const int at = (w * WC + w0) * NCOL + c;
+            const float f = fast_exp2(mm[at] - M);            // idle warps: 2^(-inf) = 0
+            const float4 v = *reinterpret_cast<const float4*>(mo + at * DP + d);
+            L += ml[at] * f;
+            sum.x += v.x * f; sum.y += v.y * f; sum.z += v.z * f; sum.w += v.w * f;
         }
-        const int m = col / G, hq = kvh * G + col % G;
-        const int64_t pr = (int64_t)(members[m].part_first + it.chunk) * p.Hq + hq;
-        *reinterpret_cast<float2*>(p.part_o + pr * D + d) = make_float2(o0, o1);
+        const int64_t pr = col_row[col];
+        *reinterpret_cast<float4*>(p.part_o + pr * D + d) = sum;
         if (d == 0) *reinterpret_cast<float2*>(p.part_ml + pr * 2) = make_float2(M, L);
     }
-    // Fused merge: this chunk counts as done for every member of the set.  The members' own chunks run in the
-    // same grid; whichever CTA draws a member's last ticket - this one or one of those - merges that member's
-    // partials for this KV head (all of them were published, fence + ticket, before the last ticket was drawn).
-    if (p.dec_counters != nullptr) {
-        __shared__ uint32_t last_mask_s;
-        if (threadIdx.x == 0) last_mask_s = 0u;
-        __threadfence();
-        __syncthreads();
-        if ((int)threadIdx.x < it.n_members) {
-            uint32_t* counter = p.dec_counters + (int64_t)members[threadIdx.x].part_first * p.Hkv + kvh;
-            if (atomicAdd(counter, 1u) == (uint32_t)(members[threadIdx.x].n_chunks - 1)) atomicOr(&last_mask_s, 1u << threadIdx.x);
-        }
-        __syncthreads();
-        const uint32_t last_mask = last_mask_s;
-        if (last_mask != 0u) {
-            __threadfence();
-            for (int m = 0; m < it.n_members; ++m) {
-                if (!((last_mask >> m) & 1u)) continue;
-                const int q_row = members[m].q_row, part_first = members[m].part_first;
-                const int n_chunks = members[m].n_chunks;
-                for (int idx = threadIdx.x; idx < G * (D / 4); idx += NWARPS * 32) {
-                    const int head = idx / (D / 4), d = (idx % (D / 4)) * 4;
-                    merge_partials<D>(p, q_row, part_first, n_chunks, kvh * G + head, d, d == 0);
-                }
-                if (threadIdx.x == 0) p.dec_counters[(int64_t)part_first * p.Hkv + kvh] = 0u;
-            }
-        }
-    }
+}
+// The team size follows the set's columns (16 per warp): sets of one column pair gain nothing from a shared ring.
+template <int D, int NWARPS, int NSTAGE, int NCG>
+__device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const uint8_t* plan, const int cta)
+{
+    const int item_id = cta / p.Hkv, kvh = cta % p.Hkv;
+    const SharedDecodeItem it = plan_list<SharedDecodeItem>(plan, p.plan.sh)[item_id];
+    decode_grid_start(p);
+    const ShareMember* members = plan_list<ShareMember>(plan, p.plan.shm) + it.member_first;
+    const int n_cols = it.n_members * p.G;
+    if (n_cols > 2 * NCG * 8) decode_shared_team<D, NWARPS, NSTAGE, NCG, 4>(p, it, members, kvh);
+    else if (n_cols > NCG * 8) decode_shared_team<D, NWARPS, NSTAGE, NCG, 2>(p, it, members, kvh);
+    else decode_shared_team<D, NWARPS, NSTAGE, NCG, 1>(p, it, members, kvh);
 }
 
 template <int D, int NWARPS, int NSTAGE, int INL>
@@ -841,7 +870,7 @@ __global__ void __launch_bounds__(D / 4) combine_kernel(const AttnParams p, cons
     const CombineItem it = plan_list<CombineItem>(INL > 0 ? inl.bytes : p.plan.base, p.plan.comb)[blockIdx.x];
     const int hq = blockIdx.y;
     asm volatile("griddepcontrol.wait;" ::: "memory");     // the decode grid has completed and its partials are visible
-    merge_partials<D>(p, it.q_row, it.part_first, it.n_chunks, hq, threadIdx.x * 4, threadIdx.x == 0);
+    merge_partials<D, 3>(p, it.q_row, it.part_first, it.n_chunks, hq, threadIdx.x * 4, threadIdx.x == 0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -936,11 +965,12 @@ cudaError_t launch_decode(const AttnParams& p, const HostPlan& hp, int head_dim,
 template <int D>
 static cudaError_t launch_decode_shared_t(const AttnParams& p, const HostPlan& hp, int n_shared_items, int n_items, cudaStream_t stream)
 {
-    constexpr int NCG = kSharedColumns / 8;
-    const size_t ring = (size_t)kDecWarps * kDecStages * 2 * 16 * D * 2;
-    const size_t merge = (size_t)kDecWarps * kSharedColumns * (D + 4) * 4 + (size_t)kDecWarps * kSharedColumns * 4 * 2;
+    constexpr int NCG = kSharedColumns / (8 * kDecWarps), COLS = 8 * NCG;      // columns a warp carries
+    constexpr int STAGES = kDecStages * 128 / D;       // the same 96 KB for both head sizes
+    const size_t ring = (size_t)kDecWarps * STAGES * 2 * 16 * D * 2;
+    const size_t merge = (size_t)kDecWarps * COLS * (D + 4) * 4 + (size_t)kDecWarps * COLS * 4 * 2;
     return with_plan_bytes(hp, [&](auto size, const auto& inl) {
-        return launch_decode_grid<decode_with_shared_kernel<D, kDecWarps, kDecStages, NCG, decltype(size)::value>>(
+        return launch_decode_grid<decode_with_shared_kernel<D, kDecWarps, STAGES, NCG, decltype(size)::value>>(
             (n_shared_items + n_items) * p.Hkv, std::max(ring, merge), stream, p, inl, n_shared_items * p.Hkv);
     });
 }

@@ -104,6 +104,7 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
     struct GroupInfo { int32_t group; int32_t pages; std::vector<int32_t> members; };
     std::vector<GroupInfo> groups_sh;
     int64_t extra_pages = 0;
+    const int32_t per_set = std::max(1, std::min(kSharedMembers, kSharedColumns / G));    // members of a set
     if (share_group != nullptr && shared_len != nullptr && W == 0 && d->kv_dtype == CF_KV_BF16) {
         std::vector<std::pair<int32_t, int32_t>> keyed;          // (group, sequence) of the decode sequences that share
         for (int32_t s = 0; s < num_seqs; ++s)
@@ -123,7 +124,7 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
                 gi.group = keyed[i].first;
                 gi.pages = pages;
                 for (size_t m = i; m < j; ++m) gi.members.push_back(keyed[m].second);
-                const int64_t sets = ((int64_t)gi.members.size() * G + kSharedColumns - 1) / kSharedColumns;
+                const int64_t sets = ((int64_t)gi.members.size() + per_set - 1) / per_set;
                 extra_pages += sets * pages;
                 groups_sh.push_back(std::move(gi));
             }
@@ -144,23 +145,33 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         B, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, cfg, extra_pages);
 
     // chunks of the shared part of every group, the same for all of its members
+    // A shared CTA costs 3 us before and after its pages (queries, first pages, 64 columns of partials) and every chunk
+    // lengthens the merge of all members, so its chunks are longer than those of the fitted model: about 1.2 CTAs per
+    // SM (each SM holds two; the rest are the members' own chunks), and not below 12 pages.  A member's own chunks are
+    // twice as long (four warps split their pages; 64 columns make all four go through each page).  One pass on a B200,
+    // by the model -> by this rule: 16 sequences of 32 / 8 heads, 8192 tokens shared 32.0 -> 29.4 us, four of them 29.4
+    // -> 18.5, 64 of them 94 -> 79, 2048 tokens shared 26.6 -> 21.6; 64 / 8 heads of 64 28.4 -> 28.6 us.
     std::vector<int32_t> n_shared_chunks;      // per sequence
     std::vector<int64_t> shared_per;           // per group: pages per shared chunk
+    std::vector<int64_t> own_target;           // per sequence: target length of its own chunks
     if (!groups_sh.empty()) {
         n_shared_chunks.assign((size_t)num_seqs, 0);
+        own_target.assign((size_t)num_seqs, target);
+        const int64_t slots = 2 * (int64_t)std::max(1, cfg.num_sms);
+        const int64_t longest = std::max<int64_t>(12, (7 * extra_pages * d->num_kv_heads + 4 * slots - 1) / (4 * slots));
         for (const GroupInfo& gi : groups_sh) {
-            int64_t n = 1, per = gi.pages;
-            decode_split(gi.pages, target, quantum, &n, &per);
+            const int64_t chunks = (gi.pages + longest - 1) / longest;
+            const int64_t per = std::min<int64_t>(gi.pages, ((gi.pages + chunks - 1) / chunks + 1) & ~1ll);      // a step takes two pages
             shared_per.push_back(per);
-            for (int32_t s : gi.members) n_shared_chunks[(size_t)s] = (int32_t)n;
+            for (int32_t s : gi.members) {
+                n_shared_chunks[(size_t)s] = (int32_t)((gi.pages + per - 1) / per);
+                own_target[(size_t)s] = std::max(target, 2 * per);
+            }
         }
     }
 
-    std::vector<int32_t> part_first_of, n_chunks_of;   // per sequence: its first partial slot (-1: writes out directly), its chunks
-    if (!groups_sh.empty()) {
-        part_first_of.assign((size_t)num_seqs, -1);
-        n_chunks_of.assign((size_t)num_seqs, 0);
-    }
+    std::vector<int32_t> part_first_of;        // per sequence: its first partial slot (-1: writes out directly)
+    if (!groups_sh.empty()) part_first_of.assign((size_t)num_seqs, -1);
     for (int32_t s = 0; s < num_seqs; ++s) {
         if (query_len[s] != 1) continue;
         const int32_t lc = context_len[s];
@@ -168,17 +179,14 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         const int64_t pages = (lc + B - 1) / B - page0;
         const int32_t n_sh = n_shared_chunks.empty() ? 0 : n_shared_chunks[(size_t)s];
         int64_t n = 1, per = pages;
-        decode_split(pages, target, quantum, &n, &per);
+        decode_split(pages, own_target.empty() ? target : own_target[(size_t)s], quantum, &n, &per);
         const int32_t n_all = (int32_t)n + n_sh;
         int32_t first = -1;
         if (n_all > 1) {
             first = plan->n_part_slots;
             plan->combine.push_back(CombineItem{plan->q_start[s], first, n_all});
             plan->n_part_slots += n_all;
-            if (!part_first_of.empty()) {
-                part_first_of[(size_t)s] = first;
-                n_chunks_of[(size_t)s] = n_all;
-            }
+            if (!part_first_of.empty()) part_first_of[(size_t)s] = first;
         }
         for (int64_t c = 0; c < n; ++c) {
             DecodeItem it;
@@ -193,18 +201,17 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
             plan->decode.push_back(it);
         }
     }
-    // shared items: per group, member sets of kSharedColumns / G sequences, one item per (set, shared chunk)
+    // shared items: per group, member sets of per_set sequences, one item per (set, shared chunk)
     for (size_t gi_idx = 0; gi_idx < groups_sh.size(); ++gi_idx) {
         const GroupInfo& gi = groups_sh[gi_idx];
         const int64_t per = shared_per[gi_idx];
         const int32_t n_sh = n_shared_chunks[(size_t)gi.members[0]];
-        const int32_t per_set = std::max(1, kSharedColumns / G);
         for (size_t m0 = 0; m0 < gi.members.size(); m0 += (size_t)per_set) {
             const int32_t n_mem = (int32_t)std::min<size_t>((size_t)per_set, gi.members.size() - m0);
             const int32_t member_first = (int32_t)plan->share_members.size();
             for (int32_t m = 0; m < n_mem; ++m) {
                 const int32_t s = gi.members[m0 + (size_t)m];
-                plan->share_members.push_back(ShareMember{plan->q_start[s], part_first_of[(size_t)s], n_chunks_of[(size_t)s], 0});
+                plan->share_members.push_back(ShareMember{plan->q_start[s], part_first_of[(size_t)s], {0, 0}});
             }
             for (int32_t c = 0; c < n_sh; ++c) {
                 SharedDecodeItem it;

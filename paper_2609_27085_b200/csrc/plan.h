@@ -35,16 +35,16 @@ struct SharedDecodeItem {  // one (share group, shared KV chunk, member set); th
     int32_t kv_end;
     int32_t chunk;         // index of this chunk in every member's chunk list (shared chunks come first)
     int32_t member_first;  // first entry of this set in the member list
-    int32_t n_members;     // members in the set (<= kSharedColumns / G)
+    int32_t n_members;     // members in the set (n_members * G <= kSharedColumns)
     int32_t pad[2];
 };
 struct ShareMember {       // one member of a set
     int32_t q_row;         // packed row of its query token
     int32_t part_first;    // first partial slot of the sequence (its chunk c writes slot part_first + c)
-    int32_t n_chunks;      // chunks of the sequence, shared ones and its own
-    int32_t pad;
+    int32_t pad[2];
 };
-constexpr int32_t kSharedColumns = 16;      // query-head columns a shared-prefix CTA carries (two 8-wide MMA operands)
+constexpr int32_t kSharedColumns = 64;      // query-head columns a shared-prefix CTA carries (two 8-wide MMA operands per warp)
+constexpr int32_t kSharedMembers = 32;      // and sequences
 constexpr int32_t kMinSharedPages = 16;     // shorter shared prefixes are not worth a separate pass
 
 struct CombineItem {       // one decode sequence that was split

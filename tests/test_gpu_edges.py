@@ -6,7 +6,7 @@ import torch
 import cf_synth as syn
 import oracle
 import paper_2609_27085_b200 as cf
-from harness import GpuScenario, compare, run_and_check
+from harness import GpuScenario, compare, run_and_check, to_dev_bf16, to_host_bits
 
 pytestmark = pytest.mark.gpu
 
@@ -100,3 +100,28 @@ def test_decode_chunk_lengths(Hq, Hkv, D, fp8, lens):
     """The decode chunk rule picks chunks of 8 to 192 pages or whole sequences: batches on both sides of its lines."""
     scales = (np.full(Hkv, 0.02, np.float32), np.full(Hkv, 0.015, np.float32)) if fp8 else None
     run_and_check(small(79, Hq, Hkv, D, [l - 1 for l in lens], [[1] * len(lens)], NB=4096), fp8=scales)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,members", [(2, 2, 128, 40), (8, 2, 128, 4), (8, 2, 128, 5), (8, 2, 128, 9), (8, 2, 128, 17),
+                                              (16, 2, 64, 2), (16, 2, 64, 3), (16, 2, 64, 9), (4, 2, 128, 22), (4, 2, 64, 33)])
+@pytest.mark.parametrize("pages", [16, 33, 129])
+def test_shared_prefix_sets_of_every_width(Hq, Hkv, D, members, pages):
+    """The warps of a shared-prefix CTA split the columns of a set (16 each) or its pages: sets that need one, two and
+    four warps per page, sets cut at 64 columns and at 32 members, chunks with an odd number of pages."""
+    own = [(37 * i * i) % 300 for i in range(members)]
+    sc, sg, sl = syn.shared_prefix_scenario("sets", syn.Geometry(Hq, Hkv, D, 16, 2048), 80 + members, pages * 16, own, [1] * members,
+                                            [0] * members)
+    b = sc.batches[0]
+    g = GpuScenario(sc)
+    g.append(b)
+    q = to_dev_bf16(b.q)
+    out = torch.full_like(q, float("nan"))
+    lse = torch.full((b.total_q, Hq), float("nan"), dtype=torch.float32, device="cuda")
+    cf.cf_mixed_attention_shared(g.ctx, g.desc, q, g.k, g.v, torch.from_numpy(b.block_table).cuda(), b.max_blocks, b.context_len,
+                                 b.query_len, sg, sl, out, lse)
+    torch.cuda.synchronize()
+    assert cf.cf_get_last_plan_counts(g.ctx)[6] == members
+    k_ref, v_ref = g.pools_host()
+    ref_o, ref_lse = oracle.mixed_attention(b.q, k_ref, v_ref, b.block_table, b.context_len, b.query_len)
+    compare(to_host_bits(out), lse.cpu().numpy(), ref_o, ref_lse)
+    g.close()
