@@ -17,7 +17,7 @@
 //   warp 2      TMA producer of the V tiles (same box shape, its own ring).
 //   warp 1      MMA issuer (the warp waits, an elected lane issues): S_t = Q_t K^T, O_t += P_t V, in the order
 //               PV_0(j) QK_0(j+1) PV_1(j) QK_1(j+1) so that the tensor pipe works on one tile while
-//               the other tile's softmax runs.
+//               the other tile's softmax runs; PV in two parts, the first as soon as three quarters of P are there.
 //   warps 4-7   softmax of tile 0, one thread per q row; warps 8-11 softmax of tile 1.
 // Tensor memory (512 columns): S_0 | S_1 | O_0 | O_1, 128 fp32 columns each; P_t (bf16) overwrites
 // the first 64 columns of S_t and is consumed by the PV product straight from tensor memory.
@@ -117,7 +117,7 @@ struct Bars {
     uint64_t q_full, q_empty;
     uint64_t k_full[KV_STAGES], k_empty[KV_STAGES];
     uint64_t v_full[KV_STAGES], v_empty[KV_STAGES];
-    uint64_t s_full[2], p_full[2], o_done[2];
+    uint64_t s_full[2], p_part[2], p_full[2], o_done[2];      // p_part: the first PART chunks of P, p_full: all of it
     uint64_t item_full[2];    // the producer has put an item context into slot s
 };
 
@@ -147,6 +147,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                   const int first_static, const int ticket_base, const int tail)
 {
     constexpr bool VARIANT = MODE > 0, WINDOW = MODE == 2;
+    constexpr int PART = 3;            // of a tile's four 32-column chunks, those that P V may start on before the last is done
     constexpr int HALVES = Geo<D>::HALVES, TILE_BYTES = Geo<D>::TILE_BYTES, KS = Geo<D>::KS;
     constexpr uint32_t kPolyMask = D == 64 ? CF_POLY_MASK_D64 : CF_POLY_MASK;
     constexpr uint32_t SMEM_Q = Geo<D>::SMEM_Q, SMEM_K = Geo<D>::SMEM_K, SMEM_V = Geo<D>::SMEM_V;
@@ -183,7 +184,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         }
         for (int t = 0; t < 2; ++t) {
             mbar_init(smem_u32(&bars.s_full[t]), 1);
-            mbar_init(smem_u32(&bars.p_full[t]), 4);      // one arrival per softmax warp
+            mbar_init(smem_u32(&bars.p_part[t]), 4);      // one arrival per softmax warp
+            mbar_init(smem_u32(&bars.p_full[t]), 4);
             mbar_init(smem_u32(&bars.o_done[t]), 1);
             mbar_init(smem_u32(&bars.item_full[t]), 1);
         }
@@ -395,6 +397,30 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 umma_commit(bar_o[t]);
             }
         };
+        // The same for a whole tile in two parts: the columns that the softmax hands over first (p_part), then the rest
+        // (p_full).  The first product runs while the last chunk's exponentials are computed, which takes it out of the
+        // chain S -> softmax -> P V -> next S that bounds a tile.  Sustained, whole -> in parts (three chunks, then one; two and
+        // two: -1 % less): head_dim 128, 4096 rows over 8192 cached 596 -> 575 us, three ragged chunks of 5003 rows 298
+        // -> 293 us, 4 x 2048 rows 944 -> 928 us, 2 x 512 rows 106 -> 104 us; head_dim 64 -0.5 %.
+        auto issue_pv_part = [&](auto T, auto S, uint32_t acc0) {
+            constexpr int t = decltype(T)::value, st = decltype(S)::value;
+            const uint32_t dO = tmem + TM_O + t * D, aP = tmem + TM_S + t * 128;
+            if (leader) {
+                umma_ts(dO, aP, vd(st, 0), IDESC_PV, acc0);
+#pragma unroll
+                for (int ks = 1; ks < 2 * PART; ++ks) umma_ts(dO, aP + ks * 8, vd(st, ks), IDESC_PV, 1u);
+            }
+        };
+        auto issue_pv_rest = [&](auto T, auto S) {
+            constexpr int t = decltype(T)::value, st = decltype(S)::value;
+            const uint32_t dO = tmem + TM_O + t * D, aP = tmem + TM_S + t * 128;
+            if (leader) {
+#pragma unroll
+                for (int ks = 2 * PART; ks < 8; ++ks) umma_ts(dO, aP + ks * 8, vd(st, ks), IDESC_PV, 1u);
+                umma_commit(bar_o[t]);
+            }
+        };
+        const uint32_t bar_pp[2] = {smem_u32(&bars.p_part[0]), smem_u32(&bars.p_part[1])};
         auto commit = [&](uint32_t bar) {
             if (leader) umma_commit(bar);
         };
@@ -434,13 +460,19 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             using S1 = std::integral_constant<int, st1>;
             if (!mbar_wait(bar_vf[st], par_v, abort_flag)) return false;
             if (!mbar_wait(bar_kf[st1], par_k1, abort_flag)) return false;
+            if (!mbar_wait(bar_pp[0], par_p0, abort_flag)) return false;
+            tc_fence_after();
+            issue_pv_part(I0{}, S, acc0);
             if (!mbar_wait(bar_p[0], par_p0, abort_flag)) return false;
             tc_fence_after();
-            issue_pv(I0{}, S, 8, acc0);
+            issue_pv_rest(I0{}, S);
             issue_qk(I0{}, S1{});
+            if (!mbar_wait(bar_pp[1], par_p1, abort_flag)) return false;
+            tc_fence_after();
+            issue_pv_part(I1{}, S, acc0);
             if (!mbar_wait(bar_p[1], par_p1, abort_flag)) return false;
             tc_fence_after();
-            issue_pv(I1{}, S, 8, acc0);
+            issue_pv_rest(I1{}, S);
             issue_qk(I1{}, S1{});
             commit(bar_ve[st]);
             commit(bar_ke[st1]);
@@ -598,12 +630,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             // sum (a probability above 2^8 makes it exceed 2^15 long before anything can overflow); only
             // then is the exact maximum taken, O_t rescaled in tensor memory and the pass repeated.
             float2 acc2[4];
-            auto exp_pass = [&](auto EDGE, const float neg_m) {
+            auto exp_pass = [&](auto EDGE, auto C0, auto C1, const float neg_m) {
                 const float2 sc2 = make_float2(sc, sc), nm2 = make_float2(neg_m, neg_m);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc2[i] = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
+                for (int c = decltype(C0)::value; c < decltype(C1)::value; ++c) {
                     uint32_t pk[16];
                     if (decltype(EDGE)::value && ((dead >> c) & 1u)) {
 #pragma unroll
@@ -624,6 +656,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             };
             using Edge = std::bool_constant<WINDOW>;
             using Interior = std::false_type;
+            using First = std::integral_constant<int, 0>;
+            using Cut = std::integral_constant<int, PART>;
+            using Last = std::integral_constant<int, 4>;
             auto neg_reference = [&]() -> float { return (WINDOW && m_used == -INFINITY) ? 0.f : -m_used; };
             // Written as a loop so that the exponential pass exists once in the code: a second copy for the repetition (and the
             // registers kept for it) slowed the tile loop down although it hardly ever runs.  Measured, copy -> loop: head_dim
@@ -633,8 +668,14 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             float tile_sum = 0.f;
 #pragma unroll (WINDOW ? 2 : 1)
             for (int pass = 0; pass < 2; ++pass) {
-                tile_sum = WINDOW && (edge || pass == 1) ? exp_pass(Edge{}, neg_reference()) : exp_pass(Interior{}, neg_reference());
-                if (pass == 1 || !__any_sync(0xffffffffu, !(tile_sum <= 32768.f))) break;
+                tile_sum = WINDOW && (edge || pass == 1) ? exp_pass(Edge{}, First{}, Cut{}, neg_reference()) : exp_pass(Interior{}, First{}, Cut{}, neg_reference());
+                // the last chunk's exponentials follow when the others have been handed over: its scores decide now
+                float mx = sv[PART * 32];
+#pragma unroll
+                for (int i = PART * 32 + 1; i + 1 < 128; i += 2) mx = max3(mx, sv[i], sv[i + 1]);
+                mx = fmaxf(mx, sv[127]);
+                const bool high = !(tile_sum <= 32768.f) || !((WINDOW && ((dead >> PART) & 1u)) || fmaf(mx, sc, neg_reference()) <= 15.f);
+                if (pass == 1 || !__any_sync(0xffffffffu, high)) break;
                 const float rise = row_max() * sc - m_used;
                 const float d = fmaxf(rise, 0.f);            // rows that did not rise keep their reference (a row without
                                                              // a visible key so far: -inf - -inf is NaN, which fmaxf drops)
@@ -659,6 +700,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             if (!ok) break;
             l_sum += tile_sum;
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bars.p_part[t]));
+            l_sum += WINDOW && edge ? exp_pass(Edge{}, Cut{}, Last{}, neg_reference()) : exp_pass(Interior{}, Cut{}, Last{}, neg_reference());
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();

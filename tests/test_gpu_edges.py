@@ -7,6 +7,7 @@ import cf_synth as syn
 import oracle
 import paper_2609_27085_b200 as cf
 from harness import GpuScenario, compare, run_and_check, to_dev_bf16, to_host_bits
+from test_gpu_parity import _spike_run
 
 pytestmark = pytest.mark.gpu
 
@@ -125,3 +126,13 @@ def test_shared_prefix_sets_of_every_width(Hq, Hkv, D, members, pages):
     ref_o, ref_lse = oracle.mixed_attention(b.q, k_ref, v_ref, b.block_table, b.context_len, b.query_len)
     compare(to_host_bits(out), lse.cpu().numpy(), ref_o, ref_lse)
     g.close()
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(8, 2, 128), (16, 2, 64)])
+@pytest.mark.parametrize("spike", [96.0, 192.0])
+def test_spikes_around_the_chunk_that_is_handed_over_last(Hq, Hkv, D, spike):
+    """The product P V starts on the first 96 columns of a tile before the exponentials of the last 32 exist, so whether
+    the reference has to be raised is decided from those columns' scores: a towering key on both sides of that line."""
+    Lq, P = 200, 1000
+    cand = [128 * t + c for t in (1, 2, 5, P // 128) for c in (94, 95, 96, 97, 110, 111, 126, 127)]
+    _spike_run(small(71, Hq, Hkv, D, [P], [[Lq]]), cand, [0, 1, 31, 32, 127, 128, Lq - 1], spike)
