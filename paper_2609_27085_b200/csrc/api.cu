@@ -90,6 +90,7 @@ struct cf_ctx {
     bool overlap = true;
     cudaStream_t upload_stream = nullptr;      // plan uploads of cf_kv_append / cf_mixed_attention
     cudaStream_t plan_copy_stream = nullptr;   // set while cf_mixed_step_host runs
+    uint64_t unflushed_steps = 0;   // host-staged steps since the last flush
     bool in_host_step = false; // inside a cf_mixed_step_host call that keeps the serial sequence (a step bound by the host copies)
     int spatial_sms = 0;       // SMs given to the first prefill grid in that mode (0 = three fifths)
     int spatial_sms_default = 0;   // CF_SPATIAL_SMS at cf_create: what cf_set_overlap(ctx, 1) goes back to
@@ -915,7 +916,7 @@ struct HostPart {
 
 // Parts of the step, or none when it is better computed and read back as one: few bytes, or too many runs.
 static std::vector<HostPart> host_parts(const cf_cache_desc* d, const int32_t* context_len, const int32_t* query_len, int32_t S,
-                                        const std::vector<int32_t>& q_start, int num_sms)
+                                        const std::vector<int32_t>& q_start, int num_sms, bool pipelined)
 {
     constexpr double kMinPrefillBytes = 4 << 20;      // below: the read-back is shorter than what the parts cost
     constexpr double kLinkBytesPerUs = 52e3, kPartUs = 12.0;
@@ -957,6 +958,10 @@ static std::vector<HostPart> host_parts(const cf_cache_desc* d, const int32_t* c
     const double link_us = pre_rows * row_bytes / kLinkBytesPerUs;
     const double in_us = ((double)q_start.back() * (row_bytes + 4.0 * d->num_kv_heads * d->head_dim)) / kLinkBytesPerUs;
     if (in_us > pre_us + dec_us + link_us) return parts;
+    // A step that follows another without a flush in between has its read-back under the kernels of the next one anyway.
+    // Where the kernels outweigh both directions of the link such steps are bound by them and go in one piece, decode beside
+    // prefill (agentic, back to back: 994 -> 899 us per step); where the link weighs as much, parts still help (chat mix: 296 against 349 us).
+    if (pipelined && pre_us + dec_us > 1.25 * std::max(in_us, link_us)) return parts;
     // how many pieces to cut the prefill rows into: the end of the last read-back, all pieces taken as equal
     int32_t cuts = 1;
     double best = 1e30;
@@ -1070,7 +1075,7 @@ cf_status cf_mixed_step_host(cf_ctx* c, const cf_cache_desc* desc,
         c->plan_copy_stream = nullptr;
         return CF_ERR_CUDA;
     }
-    const std::vector<HostPart> parts = host_parts(desc, context_len, query_len, num_seqs, pl.q_start, c->num_sms);
+    const std::vector<HostPart> parts = host_parts(desc, context_len, query_len, num_seqs, pl.q_start, c->num_sms, c->unflushed_steps++ > 0);
     if (!parts.empty()) {
         const size_t row_bytes = (size_t)desc->num_q_heads * desc->head_dim * 2;
         bool ok = true;
@@ -1118,6 +1123,7 @@ cf_status cf_host_steps_flush(cf_ctx* c, void* cuda_stream)
     for (int i = 0; i < kHostStages; ++i)
         if (c->stage[i].used && cudaStreamWaitEvent((cudaStream_t)cuda_stream, c->stage[i].d2h_done, 0) != cudaSuccess)
             return CF_ERR_CUDA;
+    c->unflushed_steps = 0;
     return CF_OK;
 }
 

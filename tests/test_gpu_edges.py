@@ -89,6 +89,30 @@ def test_host_steps_in_parts(prefix, qlen, window):
     g.close()
 
 
+def test_host_steps_without_a_flush_in_between():
+    """A step whose kernels outweigh its copies goes in parts when it comes first after a flush and in one piece when it
+    follows another: both against the oracle, three in flight."""
+    sc = small(74, 32, 8, 128, [40000, 3000], [[600, 1]], NB=3072)
+    b = sc.batches[0]
+    g = GpuScenario(sc)
+    pin = lambda x: torch.from_numpy(x.view(np.int16)).pin_memory()
+    bt, qh, kh, vh = torch.from_numpy(b.block_table).cuda(), pin(b.q), pin(b.k_new), pin(b.v_new)
+    k_ref, v_ref = sc.k_pool.copy(), sc.v_pool.copy()
+    oracle.kv_append(k_ref, v_ref, b.k_new, b.v_new, b.block_table, b.context_len, b.query_len)
+    rows = np.array([0, 31, 32, 127, 128, 599, 600])
+    ref_o, _ = oracle.mixed_attention(b.q, k_ref, v_ref, b.block_table, b.context_len, b.query_len, rows=rows)
+    outs = [torch.full_like(qh, -1).pin_memory() for _ in range(3)]
+    for oh in outs:
+        cf.cf_mixed_step_host(g.ctx, g.desc, qh, kh, vh, g.k, g.v, bt, b.max_blocks, b.context_len, b.query_len, oh)
+    cf.cf_host_steps_flush(g.ctx)
+    torch.cuda.synchronize()
+    assert cf.cf_get_async_status(g.ctx) == cf.CF_OK
+    for oh in outs:
+        compare(oh.numpy().view(np.uint16), None, ref_o, None, rows=rows)
+    assert torch.equal(outs[1], outs[2])
+    g.close()
+
+
 @pytest.mark.parametrize("Hq,Hkv,D,fp8", [(16, 2, 64, False), (8, 2, 128, False), (2, 2, 128, False), (16, 2, 128, True)])
 @pytest.mark.parametrize("lens", [
     [1], [16], [128], [129],                                          # one page, one shortest chunk, one page more
