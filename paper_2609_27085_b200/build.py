@@ -42,32 +42,38 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     objdir = os.path.join(HERE, "build")
     os.makedirs(objdir, exist_ok=True)
-    procs, objs = [], []
-    for src in SOURCES:
-        obj = os.path.join(objdir, os.path.splitext(src)[0] + ".o")
-        objs.append(obj)
-        cmd = [_nvcc(), *NVCC_FLAGS, *os.environ.get("CF_NVCC_EXTRA", "").split(), "-c", os.path.join(CSRC, src), "-o", obj]
-        if verbose:
-            cmd.insert(1, "-Xptxas")
-            cmd.insert(2, "-v")
-        procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-    tmp_marshal = MARSHAL + f".tmp{os.getpid()}"
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-Wall", "-I", sysconfig.get_paths()["include"],
-           os.path.join(CSRC, "marshal.cpp"), "-o", tmp_marshal]
-    procs.append(("marshal.cpp", subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-    failed = False
-    for src, p in procs:
-        out, _ = p.communicate()
-        if p.returncode != 0 or verbose:
-            sys.stderr.write(f"--- {src}\n{out}\n")
-        failed = failed or p.returncode != 0
-    if failed:
-        raise RuntimeError("nvcc failed")
-    tmp = LIB + f".tmp{os.getpid()}"
-    subprocess.check_call([_nvcc(), "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp, *objs,
-                           "-cudart", "static"])
-    os.replace(tmp, LIB)
-    os.replace(tmp_marshal, MARSHAL)
+    # both results are built under temporary names, put in place together and never left behind
+    tmp_marshal, tmp = MARSHAL + f".tmp{os.getpid()}", LIB + f".tmp{os.getpid()}"
+    try:
+        procs, objs = [], []
+        for src in SOURCES:
+            obj = os.path.join(objdir, os.path.splitext(src)[0] + ".o")
+            objs.append(obj)
+            cmd = [_nvcc(), *NVCC_FLAGS, *os.environ.get("CF_NVCC_EXTRA", "").split(), "-c", os.path.join(CSRC, src), "-o", obj]
+            if verbose:
+                cmd.insert(1, "-Xptxas")
+                cmd.insert(2, "-v")
+            procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+        cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-Wall", "-I", sysconfig.get_paths()["include"],
+               os.path.join(CSRC, "marshal.cpp"), "-o", tmp_marshal]
+        procs.append(("marshal.cpp", subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+        failed = []
+        for src, p in procs:
+            out, _ = p.communicate()
+            if p.returncode != 0 or verbose:
+                sys.stderr.write(f"--- {src}\n{out}\n")
+            if p.returncode != 0:
+                failed.append(src)
+        if failed:
+            raise RuntimeError(f"compilation failed: {', '.join(failed)}")
+        subprocess.check_call([_nvcc(), "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp, *objs,
+                               "-cudart", "static"])
+        os.replace(tmp, LIB)
+        os.replace(tmp_marshal, MARSHAL)
+    finally:
+        for path in (tmp, tmp_marshal):
+            if os.path.exists(path):
+                os.remove(path)
     return LIB
 
 
