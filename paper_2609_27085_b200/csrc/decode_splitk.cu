@@ -87,20 +87,20 @@ __device__ __forceinline__ void merge_partials(const AttnParams& p, int q_row, i
     if (p.lse && write_lse) p.lse[(int64_t)q_row * p.Hq + hq] = (M + log2f(L)) * kLn2;
 }
 
-// Exponentials of one page's scores (N = 4 per thread; two pages: 8) of one column group (8 heads) and running sums.  The reference maximum of a head is
-// only raised when some score exceeds it by more than 2^kRaise: then the exact maximum over the page is taken (three shuffles
-// per head) and the accumulators are rescaled; a page without such a score costs a vote.  (Probabilities up to 2^kRaise keep
-// their relative precision, in bf16, fp16 and in the fp32 sums.)  Raising at every page instead is six shuffles, two
-// exponentials and 32 multiplications per page more, which show where the kernel is not bound by HBM: shared-prefix
-// decode 39.2 -> 38.1 us per pass, 256 sequences on an fp8 cache beside four chunks 294 -> 288 us, chat mix 264 -> 258 us.
-constexpr float kRaise = 8.f;
+// Exponentials of one page's scores (N = 4 per thread; two pages: 8) of one column group (8 heads) and running sums.  The reference
+// of a head is the running maximum itself: the largest probability is exactly 1 and carries no rounding to 16 bits.  A
+// reference that may lag behind (raised only when a score exceeds it by 2^8) is 0-4 % cheaper (64 sequences of 1K-8K 182.0
+// against 182.3 us, five short ones 10.1 against 10.5 us, 256 on an fp8 cache beside four chunks 287 against 293 us) and
+// 8 % further from fp64 (relative error of 64 sequences' rows 0.00233 against 0.00217).  A page that raises no head of the warp
+// costs a vote; only the others take the maximum over the page (three shuffles per head) and rescale the accumulators - with
+// factors of exactly 1 for the heads that did not rise, so the vote changes no bit.
 template <int N, int KSTEPS>
 __device__ __forceinline__ void page_softmax(float (&s)[N], float (&m_run)[2], float (&l_run)[2], float (&o)[KSTEPS][4])
 {
     float top[2] = {s[0], s[1]};            // element e belongs to head e & 1; four elements per page
 #pragma unroll
     for (int e = 2; e < N; ++e) top[e & 1] = fmaxf(top[e & 1], s[e]);
-    const bool raise = top[0] > m_run[0] + kRaise || top[1] > m_run[1] + kRaise;
+    const bool raise = top[0] > m_run[0] || top[1] > m_run[1];
     if (__any_sync(0xffffffffu, raise)) {
         float alpha[2];
 #pragma unroll

@@ -160,3 +160,42 @@ def test_spikes_around_the_chunk_that_is_handed_over_last(Hq, Hkv, D, spike):
     Lq, P = 200, 1000
     cand = [128 * t + c for t in (1, 2, 5, P // 128) for c in (94, 95, 96, 97, 110, 111, 126, 127)]
     _spike_run(small(71, Hq, Hkv, D, [P], [[Lq]]), cand, [0, 1, 31, 32, 127, 128, Lq - 1], spike)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,members", [(8, 2, 128, 0), (16, 2, 128, 0), (16, 2, 64, 0), (8, 2, 128, 4), (8, 2, 128, 9), (8, 2, 128, 16),
+                                              (16, 2, 64, 8)])
+def test_the_dominant_probability_is_not_rounded(Hq, Hkv, D, members):
+    """One key, well behind the pages that a warp starts with, outweighs each of the others by 2^1 to 2^7.9 and alone has a
+    value: relative to the running maximum its probability is 1, so the result differs from the oracle's by its own rounding to bf16
+    (half a unit in the last place) and by what fp32 sums of 300 terms add (below 2^-13); a rounded probability adds up to 2^-8.  members > 0: the key is part of a shared prefix."""
+    n = max(1, members)
+    geom = syn.Geometry(Hq, Hkv, D, 16, 1024)
+    if members:
+        sc, sg, sl = syn.shared_prefix_scenario("dominant", geom, 91, 256, [5] * n, [1] * n, [0] * n)
+    else:
+        sc = small(91, Hq, Hkv, D, [127], [[1]], NB=1024)
+    b = sc.batches[0]
+    at = 150 if members else 70
+    rng = np.random.default_rng(91)
+    k, v = np.zeros_like(sc.k_pool), np.zeros_like(sc.v_pool)
+    page, slot = int(b.block_table[0, at // 16]), at % 16
+    k[page, :, slot, 0] = syn.f32_to_bf16_bits(np.float32(1.0))
+    v[page, :, slot, :] = syn.f32_to_bf16_bits(rng.uniform(1.0, 2.0, (Hkv, D)).astype(np.float32))
+    q = np.zeros_like(b.q)
+    lead = np.linspace(1.0, 7.9, n * Hq).reshape(n, Hq)                    # log2 of the key's weight
+    q[:, :, 0] = syn.f32_to_bf16_bits((lead * np.log(2.0) * np.sqrt(D)).astype(np.float32))
+    g = GpuScenario(sc)
+    g.k, g.v, qd = to_dev_bf16(k), to_dev_bf16(v), to_dev_bf16(q)
+    out = torch.full_like(qd, float("nan"))
+    args = (g.ctx, g.desc, qd, g.k, g.v, torch.from_numpy(b.block_table).cuda(), b.max_blocks, b.context_len, b.query_len)
+    if members:
+        cf.cf_mixed_attention_shared(*args, sg, sl, out)
+        assert cf.cf_get_last_plan_counts(g.ctx)[6] == members
+    else:
+        cf.cf_mixed_attention(*args, out)
+    torch.cuda.synchronize()
+    ref, _ = oracle.mixed_attention(q, k, v, b.block_table, b.context_len, b.query_len)
+    half_ulp = 2.0 ** (np.floor(np.log2(ref)) - 8)
+    excess = (np.abs(syn.bf16_bits_to_f64(to_host_bits(out)) - ref) - half_ulp) / ref
+    assert excess.max() <= 2.0 ** -13, excess.max()
+    g.close()
