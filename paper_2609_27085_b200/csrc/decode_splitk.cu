@@ -1024,8 +1024,9 @@ namespace {
 
 constexpr size_t kStaticScratchBytes = (size_t)16 << 20;          // whole array
 constexpr size_t kStaticPlanBytes = (size_t)128 << 10;            // items + combine items
+static_assert(kStaticScratchBytes - kStaticPlanBytes == (size_t)cf::kStaticPartBytes, "what the planner keeps within");
 constexpr int kStaticMaxSeqs = 1024;
-constexpr int kStaticMaxItems = 3584;                             // 3584 x 32 B + 1024 x 12 B fits the plan region
+using cf::kStaticMaxItems;                                         // 3584 x 32 B + 1024 x 12 B fits the plan region
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
@@ -1104,7 +1105,7 @@ extern "C" cf_status cf_decode_attention_static(const cf_cache_desc* desc, const
     auto first_page_of = [&](int32_t lc) -> int64_t { return (W > 0 && lc > W) ? (lc - W) / B : 0; };
     const int64_t target = decode_target_pages(
         num_seqs, [&](int32_t s) -> int64_t { return (int64_t)context_len[s] - first_page_of(context_len[s]) * B; }, B,
-        desc->num_kv_heads, D, false, cfg);
+        Hq, desc->num_kv_heads, D, false, cfg);
 
     StaticPlan pl;
     for (int32_t s = 0; s < num_seqs; ++s) {

@@ -142,7 +142,7 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
     const int64_t target = decode_target_pages(
         num_seqs,
         [&](int32_t s) -> int64_t { return query_len[s] == 1 ? (int64_t)context_len[s] - own_first_page(s) * B : -1; },
-        B, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, cfg, extra_pages);
+        B, d->num_q_heads, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, cfg, extra_pages);
 
     // chunks of the shared part of every group, the same for all of its members
     // A shared CTA costs 3 us before and after its pages (queries, first pages, 64 columns of partials) and every chunk

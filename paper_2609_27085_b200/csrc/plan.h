@@ -4,6 +4,7 @@
 // its local prefill queue (Section 5); the planner only partitions work, it does no arithmetic
 // on tensor data.
 #pragma once
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <vector>
@@ -125,7 +126,8 @@ cf_status validate_lengths(const cf_cache_desc* d, const int32_t* context_len, c
 // caller's arrays: nothing here allocates).  `lc_of(s)` returns the context length of sequence s if it is
 // a decode sequence and a negative number otherwise.
 //   decode_target_pages: the chunk length (in pages) with the smallest predicted time among those that fill the resident
-//     CTA slots exactly one, two, ... `decode_waves` times, longer ones, and no split at all.
+//     CTA slots exactly one, two, ... `decode_waves` times, a ladder of longer ones, and no split at all, of those whose partials
+//     fit the limits of the allocation-free entry point, which plans with this routine (no split needs none).
 //   decode_split: near-equal chunks of at most `target` pages, each a multiple of the page quantum.
 // The prediction, in microseconds, was fitted to 800 (batch, chunk length) pairs: 90 batches of 2 to 256 sequences on all
 // geometries, measured on a B200.  Streaming at full bandwidth (B) and one CTA's way through the longest chunk (g per page)
@@ -134,9 +136,11 @@ cf_status validate_lengths(const cf_cache_desc* d, const int32_t* context_len, c
 // in four waves, decode kernel alone: 40 sequences of 400 tokens, 64 over 8 heads 18.2 -> 14.2 us; 100 of 600 tokens 54 -> 47 us,
 // with head_dim 64 31 -> 23 us; 16 of 600 tokens (head_dim 64) 9.3 -> 7.8 us; 64 of 1500 tokens on an fp8 cache 54 -> 47 us;
 // 64 of 4000 tokens, which four waves fitted, 167 -> 168 us; the 90 shapes 1.06 in the mean.
+constexpr int64_t kStaticPartBytes = (16ll << 20) - (128ll << 10);      // partials of the allocation-free entry point
+constexpr int32_t kStaticMaxItems = 3584;                              // and its chunks
 template <class LcOf>
-inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int32_t Hkv, int32_t D, bool fp8, const PlanConfig& cfg,
-                                   int64_t extra_pages = 0)
+inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int32_t Hq, int32_t Hkv, int32_t D, bool fp8,
+                                   const PlanConfig& cfg, int64_t extra_pages = 0)
 {
     constexpr int32_t kMax = 2048;                      // larger batches: whole sequences are chunks enough
     float pages[kMax];
@@ -157,27 +161,44 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
     const int64_t slots = sms * (D == 64 || fp8 ? 3 : 2);      // resident CTAs: 64 KB of shared memory each, or 96 KB
     const int32_t waves = cfg.decode_waves > 1 ? cfg.decode_waves : 1;
     auto round_up = [&](int64_t c) { return (c + quantum - 1) / quantum * quantum; };
+    const int64_t slot_bytes = (int64_t)Hq * (D + 2) * 4;
     if (n > kMax || extra_pages > 0) {
         const int64_t c = round_up((total * Hkv + slots * waves - 1) / (slots * waves));
         return extra_pages > 0 ? (c > 32 ? c : c > lo ? 32 : lo) : (c > lo ? c : lo);
     }
-    auto chunks = [&](int64_t c) -> int64_t {           // over all sequences (near-equal chunks are rounded up later: at most this)
-        const float inv = 1.0f / (float)c, up = (float)(c - 1);
-        int32_t sum = 0;
-        for (int32_t i = 0; i < n; ++i) sum += (int32_t)((pages[i] + up) * inv + 1e-4f);
+    // all chunks, and those of sequences with more than one: upper bounds (near-equal chunks are rounded up later, and the
+    // slack covers the reciprocal's rounding)
+    auto chunks = [&](int64_t c, int64_t* split = nullptr) -> int64_t {
+        const float inv = 1.000001f / (float)c, up = (float)(c - 1);
+        int64_t sum = 0, parts = 0;
+        for (int32_t i = 0; i < n; ++i) {
+            const int32_t k = (int32_t)((pages[i] + up) * inv + 1e-4f);
+            sum += k;
+            parts += k > 1 ? k : 0;
+        }
+        if (split) *split = parts;
         return sum > n ? sum : n;
     };
     const double page_bytes = 2.0 * B * D * (fp8 ? 1.0 : 2.0), g = fp8 ? 0.15 : D == 64 ? 0.077 : 0.113;
     const double rate = (fp8 ? 6.3e6 : 7.6e6) * (double)sms / 148.0;
     const double bytes_us = std::pow((double)total * Hkv * page_bytes / rate, 1.7);
     double best = 1e30;
-    int64_t best_c = lo;
-    // chunks longer than this only unbalance the end of the grid
-    const int64_t hi = lo > 192 ? lo : 192;
+    int64_t best_c = round_up(longest > lo ? longest : lo);      // no split
+    // Chunks longer than 192 pages unbalance the end of the grid, except where there is so much to stream that even
+    // `decode_waves` waves of two CTAs per SM hold longer ones: there a chunk's start, its partials and its share of the merge
+    // weigh more.  Decode kernel alone, at most 192 pages -> with this limit: 256 ragged sequences around 5000 tokens 759 ->
+    // 741 us (64 over 8 heads 771 -> 743, head_dim 64 389 -> 381), 600 around 3000 1553 -> 1533 us, one of 1 M tokens 654 -> 634
+    // us (head_dim 64 357 -> 329, fp8 cache 411 -> 367).
+    const int64_t full = round_up((total * Hkv + 2 * sms * waves - 1) / (2 * sms * waves));
+    const int64_t hi = std::max(std::max(lo, full), (int64_t)192);
     auto consider = [&](int64_t c) {
         c = round_up(c < lo ? lo : c);
         if (c > hi && c < longest) c = hi / quantum * quantum;
-        const int64_t ctas = chunks(c) * Hkv, len = c < longest ? c : longest, of_longest = (longest + c - 1) / c;
+        int64_t split = 0;
+        const int64_t all = chunks(c, &split);
+        if (all > kStaticMaxItems && all > n) return;
+        if (split * slot_bytes + 256 > kStaticPartBytes) return;
+        const int64_t ctas = all * Hkv, len = c < longest ? c : longest, of_longest = (longest + c - 1) / c;
         // further waves: a whole one for any remainder when the chunks are alike, the remainder's part of one when most
         // are shorter than the longest (they leave their slots early)
         const double w = (double)ctas / (double)slots, alike = (double)total * Hkv / ((double)ctas * (double)len);
@@ -201,6 +222,11 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
     }
     if (longest > 64)
         for (int64_t c : {32, 64, 96, 128, 160}) consider(c);
+    if (full > 192) {
+        for (int64_t c : {192, 256, 384, 512, 768, 1024})
+            if (c < full) consider(c);
+        consider(full);
+    }
     if (longest <= hi) consider(longest);
     return best_c;
 }

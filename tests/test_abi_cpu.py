@@ -284,3 +284,16 @@ def test_shared_prefix_argument_check_needs_no_device():
     st = lib.cf_mixed_attention_shared(fake_ctx, ctypes.byref(d), None, None, None, None, 4, arr.ctypes.data, arr.ctypes.data,
                                        arr.ctypes.data, None, 2, None, None, None)
     assert st == cf.CF_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(32, 8, 128), (64, 8, 128), (64, 8, 64), (8, 1, 128), (256, 32, 128)])
+def test_decode_plans_fit_the_allocation_free_entry_point(Hq, Hkv, D):
+    """cf_decode_attention_static plans with the same routine and holds 3584 chunks and 16 MiB - 128 KiB of partials: no
+    batch of up to 1024 sequences is cut finer than that, few or many, equal or ragged, short or of a million tokens."""
+    d = cf.make_desc(Hq, Hkv, D, 16, 1 << 22)
+    rng = np.random.default_rng(0)
+    for S in (1, 16, 64, 192, 256, 512, 1024):
+        for L in (600, 3100, 4096, 8192, 16384, 131072, 1 << 20):
+            for lens in (np.full(S, L), (L * rng.lognormal(0, 1, S)).clip(1, 1 << 22)):
+                *_, parts, counts = cf.cf_plan_inspect(d, lens.astype(np.int32), np.ones(S, np.int32), 1 << 20, want_counts=True, cap=1)
+                assert counts[0] <= 3584 and parts * Hq * (D + 2) * 4 + 256 <= (16 << 20) - (128 << 10), (S, L)

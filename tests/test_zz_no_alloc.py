@@ -103,3 +103,30 @@ def test_static_scratch_entry_refuses_a_capturing_stream():
     torch.cuda.synchronize()
     del graph
     g.close()
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,S,L", [(64, 8, 128, 256, 4096), (64, 8, 64, 512, 6000), (256, 32, 128, 64, 8192)])
+def test_static_scratch_entry_serves_many_long_sequences(Hq, Hkv, D, S, L):
+    """Batches whose partials in chunks of at most 192 pages would outgrow the fixed array (all sequences draw their pages
+    from one small pool): served, with the bits of the context entry point, and right in a sample of rows."""
+    rng = np.random.default_rng(35)
+    lens = rng.integers(L - 500, L + 1, size=S).astype(np.int32)
+    NB, width = 256, (L + 15) // 16
+    k_bits, v_bits = (syn.normal_bf16(rng, (NB, Hkv, 16, D)) for _ in range(2))
+    q_bits = syn.normal_bf16(rng, (S, Hq, D))
+    table = rng.integers(0, NB, size=(S, width)).astype(np.int32)
+    k, v, q, bt = to_dev_bf16(k_bits), to_dev_bf16(v_bits), to_dev_bf16(q_bits), torch.from_numpy(table).cuda()
+    desc = cf.make_desc(Hq, Hkv, D, 16, NB)
+    ctx = cf.cf_create(0)
+    outs = []
+    for call in (lambda o, l: cf.cf_mixed_attention(ctx, desc, q, k, v, bt, width, lens, np.ones(S, np.int32), o, l),
+                 lambda o, l: cf.cf_decode_attention_static(desc, q, k, v, bt, width, lens, o, l)):
+        o, l = torch.full_like(q, float("nan")), torch.full((S, Hq), float("nan"), dtype=torch.float32, device="cuda")
+        call(o, l)
+        torch.cuda.synchronize()
+        outs.append((to_host_bits(o), l.cpu().numpy()))
+    cf.cf_destroy(ctx)
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+    rows = np.array([0, 1, S // 2, S - 1])
+    ref_o, ref_lse = oracle.mixed_attention(q_bits, k_bits, v_bits, table, lens, np.ones(S, np.int32), rows=rows)
+    compare(outs[1][0], outs[1][1], ref_o, ref_lse, rows=rows)
