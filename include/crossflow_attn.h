@@ -95,7 +95,8 @@ enum { CF_KV_BF16 = 0, CF_KV_FP8_E4M3 = 1 };
 
 /* Create a context on `device`.  workspace_bytes = 0: the split-K workspace starts at a default
  * size and grows when a batch needs more (growth allocates and synchronises the device);
- * workspace_bytes > 0: fixed size, a batch that needs more gets CF_ERR_WORKSPACE. */
+ * workspace_bytes > 0: fixed size; a batch whose partials do not fit is cut into fewer pieces, and one that does not fit
+ * in long pieces either gets CF_ERR_WORKSPACE. */
 cf_status cf_create(cf_ctx** out, int device, size_t workspace_bytes);
 /* Synchronises the device and frees everything the context owns.  A context that still has live plans
  * (cf_plan_create without cf_plan_destroy) is not destroyed: CF_ERR_BUSY, nothing freed. */

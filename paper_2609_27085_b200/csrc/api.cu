@@ -736,8 +736,19 @@ cf_status cf_mixed_attention_shared(cf_ctx* c, const cf_cache_desc* desc, const 
     std::vector<StageSeq> stage;
     int n_stage_pages = 0, max_stage_pages = 0;
     if (!pl.prefill_tc.empty()) stage_list(desc, context_len, query_len, num_seqs, &stage, &n_stage_pages, &max_stage_pages);
-    const WsLayout W = ws_layout(pl.n_part_slots, pl.n_pre_slots, Hq, D, n_stage_pages, desc->num_kv_heads,
-                                 (int64_t)num_seqs * max_blocks_per_seq);
+    auto layout = [&](int n_part_slots, int n_pre_slots) {
+        return ws_layout(n_part_slots, n_pre_slots, Hq, D, n_stage_pages, desc->num_kv_heads, (int64_t)num_seqs * max_blocks_per_seq);
+    };
+    WsLayout W = layout(pl.n_part_slots, pl.n_pre_slots);
+    if (c->workspace_fixed && W.total > c->workspace_bytes) {
+        // the batch is planned again for the partials that fit the caller's workspace (1 KB: the lists' alignment); one that
+        // does not even fit without any is refused
+        const int64_t left = (int64_t)c->workspace_bytes - (int64_t)layout(0, 0).total - 1024;
+        cfg.part_bytes = left > 0 ? left : 0;
+        st = build_plan(desc, context_len, query_len, num_seqs, max_blocks_per_seq, cfg, &pl, share_group, shared_len);
+        if (st != CF_OK) return st;
+        W = layout(pl.n_part_slots, pl.n_pre_slots);
+    }
     st = ensure_workspace(c, W.total);
     if (st != CF_OK) return st;
 

@@ -139,10 +139,13 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
     auto own_first_page = [&](int32_t s) -> int64_t {
         return shared_pages.empty() ? first_page_of(context_len[s]) : (int64_t)shared_pages[(size_t)s];
     };
-    const int64_t target = decode_target_pages(
-        num_seqs,
-        [&](int32_t s) -> int64_t { return query_len[s] == 1 ? (int64_t)context_len[s] - own_first_page(s) * B : -1; },
-        B, d->num_q_heads, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, cfg, extra_pages);
+    auto decode_target = [&]() {
+        return decode_target_pages(
+            num_seqs,
+            [&](int32_t s) -> int64_t { return query_len[s] == 1 ? (int64_t)context_len[s] - own_first_page(s) * B : -1; },
+            B, d->num_q_heads, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, cfg, extra_pages);
+    };
+    int64_t target = decode_target();
 
     // chunks of the shared part of every group, the same for all of its members
     // A shared CTA costs 3 us before and after its pages (queries, first pages, 64 columns of partials) and every chunk
@@ -167,6 +170,36 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
                 n_shared_chunks[(size_t)s] = (int32_t)((gi.pages + per - 1) / per);
                 own_target[(size_t)s] = std::max(target, 2 * per);
             }
+        }
+    }
+
+    // A budget for the partials that shared chunks outgrow: the shared part and every sequence's own in one chunk each, then
+    // no shared items at all (their result is that of the ordinary way).
+    const int64_t slot_bytes = (int64_t)d->num_q_heads * (d->head_dim + 2) * 4;
+    auto over_budget = [&]() {
+        int64_t slots = 0;
+        for (int32_t s = 0; s < num_seqs; ++s) {
+            if (query_len[s] != 1) continue;
+            int64_t n = 1, per = 1;
+            decode_split((context_len[s] + B - 1) / B - own_first_page(s), own_target[(size_t)s], quantum, &n, &per);
+            n += n_shared_chunks[(size_t)s];
+            slots += n > 1 ? n : 0;
+        }
+        return slots * slot_bytes > cfg.part_bytes;
+    };
+    if (!groups_sh.empty() && cfg.part_bytes != INT64_MAX && over_budget()) {
+        own_target.assign((size_t)num_seqs, INT32_MAX);
+        for (size_t g = 0; g < groups_sh.size(); ++g) {
+            shared_per[g] = groups_sh[g].pages;
+            for (int32_t s : groups_sh[g].members) n_shared_chunks[(size_t)s] = 1;
+        }
+        if (over_budget()) {
+            groups_sh.clear();
+            shared_pages.clear();
+            n_shared_chunks.clear();
+            own_target.clear();
+            extra_pages = 0;
+            target = decode_target();
         }
     }
 
@@ -457,6 +490,20 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         }
         for (size_t i = 1; i < n_items; ++i)
             if (items[i].sub > 0) k_of[i] = k_of[i - 1];      // the items of a block and KV head are cut alike
+        if (cfg.part_bytes != INT64_MAX) {                      // fewer ranges where the partial rows would outgrow the budget
+            const int64_t left = cfg.part_bytes - (int64_t)plan->n_part_slots * slot_bytes;
+            auto row_bytes = [&](int32_t most) {
+                int64_t rows = 0;
+                for (size_t i = 0; i < n_items; ++i) {
+                    const int32_t k = std::min(most, k_of[i]);
+                    if (k > 1) rows += (int64_t)k * (items[i].it.n_rows[0] + items[i].it.n_rows[1]) * pack * (pair ? 2 : 1);
+                }
+                return rows * (d->head_dim + 2) * 4;
+            };
+            int32_t most = 8;
+            while (most > 1 && row_bytes(most) > left) --most;
+            for (int32_t& k : k_of) k = std::min(k, most);
+        }
         plan->prefill_tc.reserve(n_items + 8 * plan->prefill_combine.capacity());
         for (size_t i = 0; i < n_items; ++i) {
             PrefillTcItem it = items[i].it;

@@ -94,6 +94,7 @@ struct PlanConfig {
     int32_t prefill_sms_mixed = 0;    // > 0: SMs the prefill items are balanced over when the batch also holds decode
                                       // work (spatial launch sequence: the first prefill grid's share); 0: num_sms
     int32_t prefill_force_split = 0;  // >= 2: split every tcgen05 item that many ways (tests); 0: cost model decides
+    int64_t part_bytes = INT64_MAX;   // bytes that the fp32 partials of split sequences and items may take (fixed workspace)
     bool prefill_pair = false;        // plan for the two-CTA kernel where the geometry allows it (head_dim 128, group
                                       // size a multiple of 4): an item carries four heads, the machine has num_sms / 2 slots
 };
@@ -127,7 +128,8 @@ cf_status validate_lengths(const cf_cache_desc* d, const int32_t* context_len, c
 // a decode sequence and a negative number otherwise.
 //   decode_target_pages: the chunk length (in pages) with the smallest predicted time among those that fill the resident
 //     CTA slots exactly one, two, ... `decode_waves` times, a ladder of longer ones, and no split at all, of those whose partials
-//     fit the limits of the allocation-free entry point, which plans with this routine (no split needs none).
+//     fit the budget: cfg.part_bytes, and the limits of the allocation-free entry point, which plans with this routine (no
+//     split needs none).
 //   decode_split: near-equal chunks of at most `target` pages, each a multiple of the page quantum.
 // The prediction, in microseconds, was fitted to 800 (batch, chunk length) pairs: 90 batches of 2 to 256 sequences on all
 // geometries, measured on a B200.  Streaming at full bandwidth (B) and one CTA's way through the longest chunk (g per page)
@@ -161,10 +163,20 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
     const int64_t slots = sms * (D == 64 || fp8 ? 3 : 2);      // resident CTAs: 64 KB of shared memory each, or 96 KB
     const int32_t waves = cfg.decode_waves > 1 ? cfg.decode_waves : 1;
     auto round_up = [&](int64_t c) { return (c + quantum - 1) / quantum * quantum; };
-    const int64_t slot_bytes = (int64_t)Hq * (D + 2) * 4;
+    const int64_t full = round_up((total * Hkv + 2 * sms * waves - 1) / (2 * sms * waves));      // fills `waves` waves of two CTAs per SM
+    const int64_t slot_bytes = (int64_t)Hq * (D + 2) * 4, budget = std::min(cfg.part_bytes, kStaticPartBytes);
     if (n > kMax || extra_pages > 0) {
-        const int64_t c = round_up((total * Hkv + slots * waves - 1) / (slots * waves));
-        return extra_pages > 0 ? (c > 32 ? c : c > lo ? 32 : lo) : (c > lo ? c : lo);
+        int64_t c = round_up((total * Hkv + slots * waves - 1) / (slots * waves));
+        c = extra_pages > 0 ? (c > 32 ? c : c > lo ? 32 : lo) : (c > lo ? c : lo);
+        if (cfg.part_bytes != INT64_MAX) {
+            int64_t parts = 0;
+            for (int32_t s = 0; s < num_seqs; ++s) {
+                const int64_t pg = (lc_of(s) + B - 1) / B;
+                if (pg > c) parts += (pg + c - 1) / c;
+            }
+            if (parts * slot_bytes > cfg.part_bytes) c = std::max(c, std::max<int64_t>(full, 32));
+        }
+        return c;
     }
     // all chunks, and those of sequences with more than one: upper bounds (near-equal chunks are rounded up later, and the
     // slack covers the reciprocal's rounding)
@@ -183,13 +195,12 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
     const double rate = (fp8 ? 6.3e6 : 7.6e6) * (double)sms / 148.0;
     const double bytes_us = std::pow((double)total * Hkv * page_bytes / rate, 1.7);
     double best = 1e30;
-    int64_t best_c = round_up(longest > lo ? longest : lo);      // no split
+    int64_t best_c = std::max(std::max(lo, full), round_up(128));      // for a budget that none of the candidates fits
     // Chunks longer than 192 pages unbalance the end of the grid, except where there is so much to stream that even
-    // `decode_waves` waves of two CTAs per SM hold longer ones: there a chunk's start, its partials and its share of the merge
+    // `decode_waves` waves of two CTAs per SM hold longer ones (`full`): there a chunk's start, its partials and its share of the merge
     // weigh more.  Decode kernel alone, at most 192 pages -> with this limit: 256 ragged sequences around 5000 tokens 759 ->
     // 741 us (64 over 8 heads 771 -> 743, head_dim 64 389 -> 381), 600 around 3000 1553 -> 1533 us, one of 1 M tokens 654 -> 634
     // us (head_dim 64 357 -> 329, fp8 cache 411 -> 367).
-    const int64_t full = round_up((total * Hkv + 2 * sms * waves - 1) / (2 * sms * waves));
     const int64_t hi = std::max(std::max(lo, full), (int64_t)192);
     auto consider = [&](int64_t c) {
         c = round_up(c < lo ? lo : c);
@@ -197,7 +208,7 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
         int64_t split = 0;
         const int64_t all = chunks(c, &split);
         if (all > kStaticMaxItems && all > n) return;
-        if (split * slot_bytes + 256 > kStaticPartBytes) return;
+        if (split * slot_bytes + 256 > budget) return;
         const int64_t ctas = all * Hkv, len = c < longest ? c : longest, of_longest = (longest + c - 1) / c;
         // further waves: a whole one for any remainder when the chunks are alike, the remainder's part of one when most
         // are shorter than the longest (they leave their slots early)

@@ -199,3 +199,46 @@ def test_the_dominant_probability_is_not_rounded(Hq, Hkv, D, members):
     excess = (np.abs(syn.bf16_bits_to_f64(to_host_bits(out)) - ref) - half_ulp) / ref
     assert excess.max() <= 2.0 ** -13, excess.max()
     g.close()
+
+
+@pytest.mark.parametrize("prefix,qlen", [
+    ([3000, 4500, 6000], [45, 45, 45]),                               # few short chunks: KV ranges, planned anew without
+    ([2500, 5000, 300, 1800, 40, 2900, 700], [1, 300, 1, 1, 1, 1, 1]),
+    ([700] * 31, [1] * 31),                                           # a wave of short chunks, planned anew with long ones
+    ([2600, 9, 1500, 2600, 1100, 2600], [1, 2, 1, 1, 600, 1]),
+])
+@pytest.mark.parametrize("window,fp8", [(0, False), (1000, False), (0, True)])
+def test_a_small_fixed_workspace_is_planned_for(prefix, qlen, window, fp8):
+    """A fixed workspace that the default plan's partials do not fit (1 MB, a quarter of it the ticket counters; an fp8 cache:
+    the chunks' staging on top) is planned for with fewer chunks and KV ranges: whatever fits with 128-page decode chunks and
+    uncut prefill items is served."""
+    sc = small(95, 32, 8, 128, prefix, [qlen], NB=2048)
+    pages = sum((p + q + 15) // 16 for p, q in zip(prefix, qlen) if q > 1)
+    ctx = cf.cf_create(0, workspace_bytes=4096 + (2 * pages * 8 * 16 * 128 * 2 + 4 * len(prefix) * 1024 if fp8 else 0))
+    scales = (np.full(8, 0.02, np.float32), np.full(8, 0.015, np.float32)) if fp8 else None
+    run_and_check(sc, ctx=ctx, window=window, fp8=scales)
+    cf.cf_destroy(ctx)
+
+
+@pytest.mark.parametrize("members,served_shared", [(8, True), (20, True), (40, False)])
+def test_a_small_fixed_workspace_and_shared_prefixes(members, served_shared):
+    """The partials of eleven shared chunks per member outgrow 1 MB: the shared part goes in one chunk, or, where two slots per
+    member are too many as well, the sequences are served one by one."""
+    sc, sg, sl = syn.shared_prefix_scenario("ws", syn.Geometry(32, 8, 128, 16, 2048), 96, 2048, [7 * i for i in range(members)], [1] * members,
+                                            [0] * members)
+    b = sc.batches[0]
+    ctx = cf.cf_create(0, workspace_bytes=4096)
+    g = GpuScenario(sc, ctx=ctx)
+    g.append(b)
+    q = to_dev_bf16(b.q)
+    out = torch.full_like(q, float("nan"))
+    lse = torch.full((b.total_q, 32), float("nan"), dtype=torch.float32, device="cuda")
+    cf.cf_mixed_attention_shared(ctx, g.desc, q, g.k, g.v, torch.from_numpy(b.block_table).cuda(), b.max_blocks, b.context_len,
+                                 b.query_len, sg, sl, out, lse)
+    torch.cuda.synchronize()
+    assert (cf.cf_get_last_plan_counts(ctx)[6] > 0) == served_shared
+    k_ref, v_ref = g.pools_host()
+    ref_o, ref_lse = oracle.mixed_attention(b.q, k_ref, v_ref, b.block_table, b.context_len, b.query_len)
+    compare(to_host_bits(out), lse.cpu().numpy(), ref_o, ref_lse)
+    g.close()
+    cf.cf_destroy(ctx)
