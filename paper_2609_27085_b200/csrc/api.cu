@@ -89,9 +89,7 @@ struct cf_ctx {
     // concurrent execution of the prefill kernel beside decode + combine
     bool overlap = true;
     cudaStream_t upload_stream = nullptr;      // plan uploads of cf_kv_append / cf_mixed_attention
-    cudaStream_t plan_copy_stream = nullptr;   // set while cf_mixed_step_host runs
     uint64_t unflushed_steps = 0;   // host-staged steps since the last flush
-    bool in_host_step = false; // inside a cf_mixed_step_host call that keeps the serial sequence (a step bound by the host copies)
     int spatial_sms = 0;       // SMs given to the first prefill grid in that mode (0 = three fifths)
     int spatial_sms_default = 0;   // CF_SPATIAL_SMS at cf_create: what cf_set_overlap(ctx, 1) goes back to
     // host-staged step
@@ -250,9 +248,8 @@ static cf_status next_slot(cf_ctx* c, size_t bytes, PlanSlot** out)
 // the copy engine meanwhile, hold back copies enqueued after it.  It runs on a context-owned stream (a host-staged step:
 // on its input copy stream) and the caller's stream waits for it through an event; the slot's device buffer is free by
 // then (the host waited for the slot's last use).
-static cf_status upload_slot(cf_ctx* c, PlanSlot* s, size_t bytes, cudaStream_t stream)
+static cf_status upload_slot(PlanSlot* s, size_t bytes, cudaStream_t copy_stream, cudaStream_t stream)
 {
-    cudaStream_t copy_stream = c->plan_copy_stream ? c->plan_copy_stream : c->upload_stream;
     if (cudaMemcpyAsync(s->dev, s->host, bytes, cudaMemcpyHostToDevice, copy_stream) != cudaSuccess) return CF_ERR_CUDA;
     if (cudaEventRecord(s->uploaded, copy_stream) != cudaSuccess || cudaStreamWaitEvent(stream, s->uploaded, 0) != cudaSuccess)
         return CF_ERR_CUDA;
@@ -377,11 +374,11 @@ static void stage_list(const cf_cache_desc* d, const int32_t* context_len, const
 
 // Enqueues decode -> combine -> prefill for a plan that already sits in device memory
 // (plan.base), or in host memory (hp), from where the launches carry it.  `queue`: the two counter words of the
-// persistent prefill CTAs.
+// persistent prefill CTAs.  `serial`: not the spatial sequence, whatever cf_set_overlap says.
 static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const PlanCounts& n, const PlanRef& plan, const HostPlan& hp,
                                   uint32_t* queue, float* ws, const WsLayout& W, const void* q, const void* k_cache,
                                   const void* v_cache, const int32_t* block_table, int32_t max_blocks_per_seq, void* out,
-                                  float* lse, cudaStream_t stream, bool allow_timing)
+                                  float* lse, cudaStream_t stream, bool serial, bool allow_timing)
 {
     const int Hq = desc->num_q_heads, D = desc->head_dim;
     AttnParams p;
@@ -474,7 +471,7 @@ static cf_status launch_attention(cf_ctx* c, const cf_cache_desc* desc, const Pl
         return n.pair ? launch_prefill_tc2(pp, maps, n.n_pre_tc, n_slots, queue_slots, first_static, ticket_base, tail, stream)
                       : launch_prefill_tc(pp, hp, maps, D, n.n_pre_tc, n_slots, queue_slots, first_static, ticket_base, tail, stream);
     };
-    if (c->overlap && !c->in_host_step && !tc && has_prefill && (n.n_dec > 0)) {
+    if (c->overlap && !serial && !tc && has_prefill && (n.n_dec > 0)) {
         // Spatial partition, three grids of one stream that run at the same time by programmatic launches.  `front`
         // persistent prefill CTAs (one per SM: a CTA takes an SM's whole shared memory) go first.  The decode grid is
         // allowed to start once every one of them holds its SM (they say so with griddepcontrol.launch_dependents) and
@@ -632,6 +629,10 @@ cf_status cf_destroy(cf_ctx* c)
     return CF_OK;
 }
 
+}  // extern "C"
+
+namespace cf {
+
 static AppendParams append_params(cf_ctx* c, const cf_cache_desc* desc, void* k_cache, void* v_cache, const void* k_new, const void* v_new,
                                   const int32_t* block_table, int32_t max_blocks, int32_t num_seqs, int32_t total_rows)
 {
@@ -651,6 +652,125 @@ static AppendParams append_params(cf_ctx* c, const cf_cache_desc* desc, void* k_
     return p;
 }
 
+// Enqueues the append of a validated batch (`pl`: q_start and total_q filled); a plan slot is uploaded on copy_stream.
+static cf_status enqueue_append(cf_ctx* c, const cf_cache_desc* desc, Plan& pl, void* k_cache, void* v_cache, const void* k_new,
+                                const void* v_new, const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_len,
+                                const int32_t* query_len, int32_t num_seqs, cudaStream_t copy_stream, cudaStream_t stream)
+{
+    pl.prefix.clear();
+    for (int32_t i = 0; i < num_seqs; ++i) pl.prefix.push_back(context_len[i] - query_len[i]);
+    PlanSlot* slot = nullptr;
+    AppendParams p = append_params(c, desc, k_cache, v_cache, k_new, v_new, block_table, max_blocks_per_seq, num_seqs, pl.total_q);
+    if (num_seqs <= kAppendInlineSeqs) {
+        p.host_q_start = pl.q_start.data();
+        p.host_prefix = pl.prefix.data();
+    } else {
+        const size_t qs_bytes = sizeof(int32_t) * ((size_t)num_seqs + 1), pf_bytes = sizeof(int32_t) * (size_t)num_seqs;
+        cf_status st = next_slot(c, qs_bytes + pf_bytes, &slot);
+        if (st != CF_OK) return st;
+        std::memcpy(slot->host, pl.q_start.data(), qs_bytes);
+        std::memcpy(slot->host + qs_bytes, pl.prefix.data(), pf_bytes);
+        st = upload_slot(slot, qs_bytes + pf_bytes, copy_stream, stream);
+        if (st != CF_OK) return st;
+        p.q_start = (const int32_t*)slot->dev;
+        p.prefix = (const int32_t*)(slot->dev + qs_bytes);
+    }
+    const cudaError_t e = launch_kv_append(p, stream);
+    const cf_status fs = slot ? finish_slot(slot, stream) : CF_OK;
+    return e != cudaSuccess ? CF_ERR_CUDA : fs;
+}
+
+// One attention call, planned: everything that is decided from the lengths and can be refused, before anything is enqueued.
+struct Unit {
+    Plan pl;
+    std::vector<StageSeq> stage;             // fp8 cache: pages to expand for the prefill chunks
+    int n_stage_pages = 0, max_stage_pages = 0;
+    int32_t num_seqs = 0, max_blocks = 0;
+    WsLayout W;
+    int front_sms = 0;
+    bool serial = false;
+};
+static cf_status plan_unit(cf_ctx* c, const cf_cache_desc* desc, const int32_t* context_len, const int32_t* query_len, int32_t num_seqs,
+                           int32_t max_blocks_per_seq, const int32_t* share_group, const int32_t* shared_len, bool serial, Unit* u)
+{
+    const int64_t t_in = now_ns();
+    PlanConfig cfg = c->cfg;
+    const int front_sms = !c->overlap || serial ? 0 : c->spatial_sms > 0 ? c->spatial_sms
+                              : spatial_front_sms(desc, context_len, query_len, num_seqs, c->num_sms);
+    cfg.prefill_sms_mixed = c->timing ? 0 : front_sms;
+    cfg.prefill_pair = c->use_pairs && prefill_pair_supported(desc);
+    Plan& pl = u->pl;
+    cf_status st = build_plan(desc, context_len, query_len, num_seqs, max_blocks_per_seq, cfg, &pl, share_group, shared_len);
+    if (st != CF_OK) return st;
+    u->num_seqs = num_seqs;
+    u->max_blocks = max_blocks_per_seq;
+    u->serial = serial;
+    if (!pl.prefill_tc.empty()) stage_list(desc, context_len, query_len, num_seqs, &u->stage, &u->n_stage_pages, &u->max_stage_pages);
+    auto layout = [&](int n_part_slots, int n_pre_slots) {
+        return ws_layout(n_part_slots, n_pre_slots, desc->num_q_heads, desc->head_dim, u->n_stage_pages, desc->num_kv_heads,
+                         (int64_t)num_seqs * max_blocks_per_seq);
+    };
+    u->W = layout(pl.n_part_slots, pl.n_pre_slots);
+    if (c->workspace_fixed && u->W.total > c->workspace_bytes) {
+        // the batch is planned again for the partials that fit the caller's workspace (1 KB: the lists' alignment); one that
+        // does not even fit without any is refused
+        const int64_t left = (int64_t)c->workspace_bytes - (int64_t)layout(0, 0).total - 1024;
+        cfg.part_bytes = left > 0 ? left : 0;
+        st = build_plan(desc, context_len, query_len, num_seqs, max_blocks_per_seq, cfg, &pl, share_group, shared_len);
+        if (st != CF_OK) return st;
+        u->W = layout(pl.n_part_slots, pl.n_pre_slots);
+        if (u->W.total > c->workspace_bytes) return CF_ERR_WORKSPACE;
+    }
+    u->front_sms = c->spatial_sms > 0 ? front_sms : pl.front_sms;
+    c->host_ns_planner += now_ns() - t_in;
+    return CF_OK;
+}
+
+// Enqueues a planned call.  ensure_workspace(c, u.W.total) has been called.
+static cf_status enqueue_unit(cf_ctx* c, const cf_cache_desc* desc, const Unit& u, const void* q, const void* k_cache, const void* v_cache,
+                              const int32_t* block_table, void* out, float* lse, cudaStream_t copy_stream, cudaStream_t stream)
+{
+    const Plan& pl = u.pl;
+    // A small plan travels with the launches: up to kSmallPlanBytes with every kernel of the sequence, up to kMidPlanBytes
+    // with the decode kernel when it is the only one that needs it.  Larger ones go through a pinned slot and a copy.
+    PlanRef ref;
+    HostPlan hp;
+    PlanSlot* slot = nullptr;
+    const size_t bytes = layout_of(pl, u.stage.size(), &ref);
+    const bool fused = c->fused_combine && (size_t)pl.n_part_slots * desc->num_kv_heads * sizeof(uint32_t) <= kCounterBytes;
+    alignas(16) uint8_t inline_plan[kMidPlanBytes];
+    if (bytes <= (size_t)(pl.prefill_tc.empty() ? kMidPlanBytes : kSmallPlanBytes) && (fused || pl.combine.empty()) && !pl.pair) {
+        write_plan(inline_plan, pl, u.stage, ref);
+        hp.bytes = inline_plan;
+        hp.size = bytes;
+    } else {
+        cf_status st = next_slot(c, bytes, &slot);
+        if (st != CF_OK) return st;
+        write_plan(slot->host, pl, u.stage, ref);
+        st = upload_slot(slot, bytes, copy_stream, stream);
+        if (st != CF_OK) return st;
+        ref.base = slot->dev;
+    }
+    PlanCounts n;
+    n.n_dec = (int)pl.decode.size(); n.n_comb = (int)pl.combine.size(); n.n_shared = (int)pl.shared_decode.size();
+    n.n_pre_tc = (int)pl.prefill_tc.size(); n.n_pre_comb = (int)pl.prefill_combine.size(); n.total_q = pl.total_q;
+    n.n_part_slots = pl.n_part_slots;
+    n.pair = pl.pair;
+    n.n_stage_seqs = (int)u.stage.size(); n.n_stage_pages = u.n_stage_pages; n.max_stage_pages = u.max_stage_pages; n.num_seqs = u.num_seqs;
+    c->last_counts[0] = n.n_dec; c->last_counts[1] = n.n_comb; c->last_counts[2] = n.n_pre_tc; c->last_counts[3] = n.n_part_slots;
+    c->last_counts[4] = n.n_pre_comb; c->last_counts[5] = shared_units(pl, desc); c->last_counts[6] = (int32_t)pl.share_members.size();
+    c->last_counts[7] = pl.pair ? 1 : 0;
+    n.front_sms = u.front_sms;
+    const cf_status ls = launch_attention(c, desc, n, ref, hp, c->queue_dev, c->workspace, u.W, q, k_cache, v_cache, block_table,
+                                          u.max_blocks, out, lse, stream, u.serial, true);
+    const cf_status fs = slot ? finish_slot(slot, stream) : CF_OK;
+    return ls != CF_OK ? ls : fs;
+}
+
+}  // namespace cf
+
+extern "C" {
+
 cf_status cf_kv_append(cf_ctx* c, const cf_cache_desc* desc, void* k_cache, void* v_cache,
                        const void* k_new, const void* v_new,
                        const int32_t* block_table, int32_t max_blocks_per_seq,
@@ -668,30 +788,11 @@ cf_status cf_kv_append(cf_ctx* c, const cf_cache_desc* desc, void* k_cache, void
     if (!k_cache || !v_cache || !k_new || !v_new || !block_table) return CF_ERR_INVALID_ARG;
     DeviceGuard guard(c->device);
     if (!guard.ok) return CF_ERR_CUDA;
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
-    for (int32_t i = 0; i < num_seqs; ++i) pl.prefix.push_back(context_len[i] - query_len[i]);
-    PlanSlot* slot = nullptr;
-    AppendParams p = append_params(c, desc, k_cache, v_cache, k_new, v_new, block_table, max_blocks_per_seq, num_seqs, pl.total_q);
-    if (num_seqs <= kAppendInlineSeqs) {
-        p.host_q_start = pl.q_start.data();
-        p.host_prefix = pl.prefix.data();
-    } else {
-        const size_t qs_bytes = sizeof(int32_t) * ((size_t)num_seqs + 1), pf_bytes = sizeof(int32_t) * (size_t)num_seqs;
-        st = next_slot(c, qs_bytes + pf_bytes, &slot);
-        if (st != CF_OK) return st;
-        std::memcpy(slot->host, pl.q_start.data(), qs_bytes);
-        std::memcpy(slot->host + qs_bytes, pl.prefix.data(), pf_bytes);
-        st = upload_slot(c, slot, qs_bytes + pf_bytes, stream);
-        if (st != CF_OK) return st;
-        p.q_start = (const int32_t*)slot->dev;
-        p.prefix = (const int32_t*)(slot->dev + qs_bytes);
-    }
-    const cudaError_t e = launch_kv_append(p, stream);
-    const cf_status fs = slot ? finish_slot(slot, stream) : CF_OK;
+    st = enqueue_append(c, desc, pl, k_cache, v_cache, k_new, v_new, block_table, max_blocks_per_seq, context_len, query_len, num_seqs,
+                        c->upload_stream, (cudaStream_t)cuda_stream);
     c->host_ns_append += now_ns() - t_in;
     ++c->host_calls_append;
-    if (e != cudaSuccess) return CF_ERR_CUDA;
-    return fs;
+    return st;
 }
 
 cf_status cf_mixed_attention(cf_ctx* c, const cf_cache_desc* desc, const void* q,
@@ -716,79 +817,22 @@ cf_status cf_mixed_attention_shared(cf_ctx* c, const cf_cache_desc* desc, const 
     const int64_t t_in = now_ns();
     cf_status st = validate_desc(desc);
     if (st != CF_OK) return st;
-    Plan pl;
-    PlanConfig cfg = c->cfg;
-    const int front_sms = !(c->overlap && !c->in_host_step) ? 0 : c->spatial_sms > 0 ? c->spatial_sms
-                              : spatial_front_sms(desc, context_len, query_len, num_seqs, c->num_sms);
-    cfg.prefill_sms_mixed = c->timing ? 0 : front_sms;
-    cfg.prefill_pair = c->use_pairs && prefill_pair_supported(desc);
-    st = build_plan(desc, context_len, query_len, num_seqs, max_blocks_per_seq, cfg, &pl, share_group, shared_len);
+    Unit u;
+    st = validate_lengths(desc, context_len, query_len, num_seqs, max_blocks_per_seq, &u.pl);
     if (st != CF_OK) return st;
-    c->host_ns_planner += now_ns() - t_in;
     c->launches = 0;
-    if (pl.total_q == 0) return CF_OK;
+    if (u.pl.total_q == 0) return CF_OK;
     if (!q || !k_cache || !v_cache || !block_table || !out) return CF_ERR_INVALID_ARG;
+    st = plan_unit(c, desc, context_len, query_len, num_seqs, max_blocks_per_seq, share_group, shared_len, false, &u);
+    if (st != CF_OK) return st;
     DeviceGuard guard(c->device);
     if (!guard.ok) return CF_ERR_CUDA;
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
-
-    const int Hq = desc->num_q_heads, D = desc->head_dim;
-    std::vector<StageSeq> stage;
-    int n_stage_pages = 0, max_stage_pages = 0;
-    if (!pl.prefill_tc.empty()) stage_list(desc, context_len, query_len, num_seqs, &stage, &n_stage_pages, &max_stage_pages);
-    auto layout = [&](int n_part_slots, int n_pre_slots) {
-        return ws_layout(n_part_slots, n_pre_slots, Hq, D, n_stage_pages, desc->num_kv_heads, (int64_t)num_seqs * max_blocks_per_seq);
-    };
-    WsLayout W = layout(pl.n_part_slots, pl.n_pre_slots);
-    if (c->workspace_fixed && W.total > c->workspace_bytes) {
-        // the batch is planned again for the partials that fit the caller's workspace (1 KB: the lists' alignment); one that
-        // does not even fit without any is refused
-        const int64_t left = (int64_t)c->workspace_bytes - (int64_t)layout(0, 0).total - 1024;
-        cfg.part_bytes = left > 0 ? left : 0;
-        st = build_plan(desc, context_len, query_len, num_seqs, max_blocks_per_seq, cfg, &pl, share_group, shared_len);
-        if (st != CF_OK) return st;
-        W = layout(pl.n_part_slots, pl.n_pre_slots);
-    }
-    st = ensure_workspace(c, W.total);
+    st = ensure_workspace(c, u.W.total);
     if (st != CF_OK) return st;
-
-    // A small plan travels with the launches: up to kSmallPlanBytes with every kernel of the sequence, up to kMidPlanBytes
-    // with the decode kernel when it is the only one that needs it.  Larger ones go through a pinned slot and a copy.
-    PlanRef ref;
-    HostPlan hp;
-    PlanSlot* slot = nullptr;
-    const size_t bytes = layout_of(pl, stage.size(), &ref);
-    const bool fused = c->fused_combine && (size_t)pl.n_part_slots * desc->num_kv_heads * sizeof(uint32_t) <= kCounterBytes;
-    alignas(16) uint8_t inline_plan[kMidPlanBytes];
-    if (bytes <= (size_t)(pl.prefill_tc.empty() ? kMidPlanBytes : kSmallPlanBytes) && (fused || pl.combine.empty()) && !pl.pair) {
-        write_plan(inline_plan, pl, stage, ref);
-        hp.bytes = inline_plan;
-        hp.size = bytes;
-    } else {
-        st = next_slot(c, bytes, &slot);
-        if (st != CF_OK) return st;
-        write_plan(slot->host, pl, stage, ref);
-        st = upload_slot(c, slot, bytes, stream);
-        if (st != CF_OK) return st;
-        ref.base = slot->dev;
-    }
-
-    PlanCounts n;
-    n.n_dec = (int)pl.decode.size(); n.n_comb = (int)pl.combine.size(); n.n_shared = (int)pl.shared_decode.size();
-    n.n_pre_tc = (int)pl.prefill_tc.size(); n.n_pre_comb = (int)pl.prefill_combine.size(); n.total_q = pl.total_q;
-    n.n_part_slots = pl.n_part_slots;
-    n.pair = pl.pair;
-    n.n_stage_seqs = (int)stage.size(); n.n_stage_pages = n_stage_pages; n.max_stage_pages = max_stage_pages; n.num_seqs = num_seqs;
-    c->last_counts[0] = n.n_dec; c->last_counts[1] = n.n_comb; c->last_counts[2] = n.n_pre_tc; c->last_counts[3] = n.n_part_slots;
-    c->last_counts[4] = n.n_pre_comb; c->last_counts[5] = shared_units(pl, desc); c->last_counts[6] = (int32_t)pl.share_members.size();
-    c->last_counts[7] = pl.pair ? 1 : 0;
-    n.front_sms = c->spatial_sms > 0 ? front_sms : pl.front_sms;
-    const cf_status ls = launch_attention(c, desc, n, ref, hp, c->queue_dev, c->workspace, W,
-                                          q, k_cache, v_cache, block_table, max_blocks_per_seq, out, lse, stream, true);
-    const cf_status fs = slot ? finish_slot(slot, stream) : CF_OK;
+    st = enqueue_unit(c, desc, u, q, k_cache, v_cache, block_table, out, lse, c->upload_stream, (cudaStream_t)cuda_stream);
     c->host_ns_attention += now_ns() - t_in;
     ++c->host_calls_attention;
-    return ls != CF_OK ? ls : fs;
+    return st;
 }
 
 cf_status cf_plan_create(cf_ctx* c, const cf_cache_desc* desc, const int32_t* context_len, const int32_t* query_len,
@@ -904,7 +948,7 @@ cf_status cf_mixed_attention_planned(cf_plan* P, const void* q, const void* k_ca
     const WsLayout W = ws_layout(P->n_part_slots, P->n_pre_slots, P->desc.num_q_heads, P->desc.head_dim, P->n_stage_pages,
                                  P->desc.num_kv_heads, (int64_t)P->num_seqs * P->max_blocks);
     return launch_attention(P->ctx, &P->desc, n, P->ref, HostPlan(), (uint32_t*)(P->dev + P->off_queue), P->part, W, q, k_cache,
-                            v_cache, block_table, P->max_blocks, out, lse, (cudaStream_t)cuda_stream, false);
+                            v_cache, block_table, P->max_blocks, out, lse, (cudaStream_t)cuda_stream, false, false);
 }
 
 }  // extern "C"
@@ -1036,16 +1080,40 @@ cf_status cf_mixed_step_host(cf_ctx* c, const cf_cache_desc* desc,
     st = validate_lengths(desc, context_len, query_len, num_seqs, max_blocks_per_seq, &pl);
     if (st != CF_OK) return st;
     if (pl.total_q == 0) return CF_OK;
-    if (!q_host || !k_new_host || !v_new_host || !out_host) return CF_ERR_INVALID_ARG;
+    if (!q_host || !k_new_host || !v_new_host || !out_host || !k_cache || !v_cache || !block_table) return CF_ERR_INVALID_ARG;
     DeviceGuard guard(c->device);
     if (!guard.ok) return CF_ERR_CUDA;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
+
+    // The step is planned, all of its parts, before anything is enqueued: a part that does not fit a fixed workspace refuses the
+    // step while the caches and out_host are as they were.
+    const int64_t t_in = now_ns();
+    std::vector<HostPart> parts = host_parts(desc, context_len, query_len, num_seqs, pl.q_start, c->num_sms, c->unflushed_steps > 0);
+    const bool whole = parts.empty();
+    std::vector<Unit> units(whole ? 1 : parts.size());
+    size_t ws_bytes = 0;
+    for (size_t i = 0; i < units.size(); ++i) {
+        // In one piece: a step whose decode part weighs as much as its prefill part is bound by the copies over the host link,
+        // not by the kernels, and keeps the serial sequence; a prefill-heavy step (the spatial share above its floor) runs
+        // the sequence cf_mixed_attention would run.
+        if (whole)
+            st = plan_unit(c, desc, context_len, query_len, num_seqs, max_blocks_per_seq, nullptr, nullptr,
+                           spatial_front_sms(desc, context_len, query_len, num_seqs, c->num_sms) <= (c->num_sms * 3) / 5, &units[i]);
+        else
+            st = plan_unit(c, desc, parts[i].context_len.data(), parts[i].query_len.data(), parts[i].num_seqs, max_blocks_per_seq, nullptr,
+                           nullptr, true, &units[i]);
+        if (st != CF_OK) return st;
+        ws_bytes = std::max(ws_bytes, units[i].W.total);
+    }
+    st = ensure_workspace(c, ws_bytes);
+    if (st != CF_OK) return st;
+    c->launches = 0;
+
     const size_t T = (size_t)pl.total_q;
     const size_t q_bytes = align_up(T * desc->num_q_heads * desc->head_dim * 2, 256);
     const size_t kv_bytes = align_up(T * desc->num_kv_heads * desc->head_dim * 2, 256);
     const size_t need = 2 * q_bytes + 2 * kv_bytes;
     HostStage& hs = c->stage[c->next_stage];
-    c->next_stage = (c->next_stage + 1) % kHostStages;
     if (need > hs.bytes) {
         if (cudaDeviceSynchronize() != cudaSuccess) return CF_ERR_CUDA;
         if (hs.dev) cudaFree(hs.dev);
@@ -1055,75 +1123,62 @@ cf_status cf_mixed_step_host(cf_ctx* c, const cf_cache_desc* desc,
         hs.bytes = need;
         hs.used = false;
     }
+    c->next_stage = (c->next_stage + 1) % kHostStages;
     uint8_t* dq = hs.dev;
     uint8_t* dk = dq + q_bytes;
     uint8_t* dv = dk + kv_bytes;
     uint8_t* dout = dv + kv_bytes;
-    const size_t qb = T * desc->num_q_heads * desc->head_dim * 2, kb = T * desc->num_kv_heads * desc->head_dim * 2;
-    // inputs: copy stream, after the kernels and the read-back that last used this staging set
-    // (q on one copy stream, k_new and v_new on a second: the small copies run at two thirds of the link rate
-    // on their own and fill in beside the large one)
-    if (hs.used) {
-        if (cudaStreamWaitEvent(c->h2d_stream, hs.compute_done, 0) != cudaSuccess) return CF_ERR_CUDA;
-        if (cudaStreamWaitEvent(c->h2d_stream, hs.d2h_done, 0) != cudaSuccess) return CF_ERR_CUDA;
-        if (cudaStreamWaitEvent(c->h2d_kv_stream, hs.compute_done, 0) != cudaSuccess) return CF_ERR_CUDA;
-    }
-    if (cudaMemcpyAsync(dk, k_new_host, kb, cudaMemcpyHostToDevice, c->h2d_kv_stream) != cudaSuccess) return CF_ERR_CUDA;
-    if (cudaMemcpyAsync(dv, v_new_host, kb, cudaMemcpyHostToDevice, c->h2d_kv_stream) != cudaSuccess) return CF_ERR_CUDA;
-    if (cudaEventRecord(hs.h2d_kv_done, c->h2d_kv_stream) != cudaSuccess) return CF_ERR_CUDA;
-    if (cudaMemcpyAsync(dq, q_host, qb, cudaMemcpyHostToDevice, c->h2d_stream) != cudaSuccess) return CF_ERR_CUDA;
-    if (cudaEventRecord(hs.h2d_done, c->h2d_stream) != cudaSuccess) return CF_ERR_CUDA;
-    // kernels: the caller's stream
-    if (cudaStreamWaitEvent(stream, hs.h2d_kv_done, 0) != cudaSuccess) return CF_ERR_CUDA;
-    c->plan_copy_stream = c->h2d_stream;
-    st = cf_kv_append(c, desc, k_cache, v_cache, dk, dv, block_table, max_blocks_per_seq, context_len, query_len,
-                      num_seqs, cuda_stream);
-    if (st != CF_OK) {
-        c->plan_copy_stream = nullptr;
-        return st;
-    }
-    if (cudaStreamWaitEvent(stream, hs.h2d_done, 0) != cudaSuccess) {
-        c->plan_copy_stream = nullptr;
-        return CF_ERR_CUDA;
-    }
-    const std::vector<HostPart> parts = host_parts(desc, context_len, query_len, num_seqs, pl.q_start, c->num_sms, c->unflushed_steps++ > 0);
-    if (!parts.empty()) {
-        const size_t row_bytes = (size_t)desc->num_q_heads * desc->head_dim * 2;
-        bool ok = true;
-        for (size_t i = 0; i < parts.size() && ok && st == CF_OK; ++i) {
-            const HostPart& r = parts[i];
-            const size_t off = (size_t)r.row * row_bytes, bytes = (size_t)r.rows * row_bytes;
-            c->in_host_step = true;
-            st = cf_mixed_attention(c, desc, dq + off, k_cache, v_cache, block_table + (int64_t)r.seq * max_blocks_per_seq, max_blocks_per_seq,
-                                    r.context_len.data(), r.query_len.data(), r.num_seqs, dout + off, nullptr, cuda_stream);
-            c->in_host_step = false;
-            if (st != CF_OK) break;
-            ok = cudaEventRecord(hs.part_done[i], stream) == cudaSuccess && cudaStreamWaitEvent(c->d2h_stream, hs.part_done[i], 0) == cudaSuccess &&
-                 cudaMemcpyAsync((uint8_t*)out_host + off, dout + off, bytes, cudaMemcpyDeviceToHost, c->d2h_stream) == cudaSuccess;
-        }
-        c->plan_copy_stream = nullptr;
-        if (st != CF_OK) return st;
-        if (!ok || cudaEventRecord(hs.compute_done, stream) != cudaSuccess || cudaEventRecord(hs.d2h_done, c->d2h_stream) != cudaSuccess)
+    const size_t row_bytes = (size_t)desc->num_q_heads * desc->head_dim * 2;
+    const size_t qb = T * row_bytes, kb = T * desc->num_kv_heads * desc->head_dim * 2;
+    auto run = [&]() -> cf_status {
+        auto ok = [](cudaError_t e) { return e == cudaSuccess; };
+        // inputs: copy stream, after the kernels and the read-back that last used this staging set
+        // (q on one copy stream, k_new and v_new on a second: the small copies run at two thirds of the link rate
+        // on their own and fill in beside the large one)
+        if (hs.used && !(ok(cudaStreamWaitEvent(c->h2d_stream, hs.compute_done, 0)) && ok(cudaStreamWaitEvent(c->h2d_stream, hs.d2h_done, 0)) &&
+                         ok(cudaStreamWaitEvent(c->h2d_kv_stream, hs.compute_done, 0))))
             return CF_ERR_CUDA;
-        hs.used = true;
+        if (!ok(cudaMemcpyAsync(dk, k_new_host, kb, cudaMemcpyHostToDevice, c->h2d_kv_stream)) ||
+            !ok(cudaMemcpyAsync(dv, v_new_host, kb, cudaMemcpyHostToDevice, c->h2d_kv_stream)) ||
+            !ok(cudaEventRecord(hs.h2d_kv_done, c->h2d_kv_stream)) ||
+            !ok(cudaMemcpyAsync(dq, q_host, qb, cudaMemcpyHostToDevice, c->h2d_stream)) || !ok(cudaEventRecord(hs.h2d_done, c->h2d_stream)))
+            return CF_ERR_CUDA;
+        // kernels: the caller's stream; plans are uploaded on the input copy stream
+        if (!ok(cudaStreamWaitEvent(stream, hs.h2d_kv_done, 0))) return CF_ERR_CUDA;
+        cf_status e = enqueue_append(c, desc, pl, k_cache, v_cache, dk, dv, block_table, max_blocks_per_seq, context_len, query_len, num_seqs,
+                                     c->h2d_stream, stream);
+        if (e != CF_OK) return e;
+        if (!ok(cudaStreamWaitEvent(stream, hs.h2d_done, 0))) return CF_ERR_CUDA;
+        for (size_t i = 0; i < units.size(); ++i) {
+            const size_t off = whole ? 0 : (size_t)parts[i].row * row_bytes, bytes = whole ? qb : (size_t)parts[i].rows * row_bytes;
+            const int32_t* table = whole ? block_table : block_table + (int64_t)parts[i].seq * max_blocks_per_seq;
+            e = enqueue_unit(c, desc, units[i], dq + off, k_cache, v_cache, table, dout + off, nullptr, c->h2d_stream, stream);
+            if (e != CF_OK) return e;
+            // result: second copy stream
+            if (!ok(cudaEventRecord(hs.part_done[i], stream)) || !ok(cudaStreamWaitEvent(c->d2h_stream, hs.part_done[i], 0)) ||
+                !ok(cudaMemcpyAsync((uint8_t*)out_host + off, dout + off, bytes, cudaMemcpyDeviceToHost, c->d2h_stream)))
+                return CF_ERR_CUDA;
+        }
         return CF_OK;
+    };
+    st = run();
+    // Also where a call failed half-way: what has been enqueued is ordered before the staging set's next use and before the flush.
+    if (st != CF_OK) {
+        cudaEventRecord(hs.h2d_done, c->h2d_stream);
+        cudaEventRecord(hs.h2d_kv_done, c->h2d_kv_stream);
+        cudaStreamWaitEvent(stream, hs.h2d_done, 0);
+        cudaStreamWaitEvent(stream, hs.h2d_kv_done, 0);
     }
-    // In one piece: a step whose decode part weighs as much as its prefill part is bound by the copies over the host link,
-    // not by the kernels, and keeps the serial sequence; a prefill-heavy step (the spatial share above its floor) runs
-    // the sequence cf_mixed_attention would run.
-    c->in_host_step = spatial_front_sms(desc, context_len, query_len, num_seqs, c->num_sms) <= (c->num_sms * 3) / 5;
-    st = cf_mixed_attention(c, desc, dq, k_cache, v_cache, block_table, max_blocks_per_seq, context_len, query_len,
-                            num_seqs, dout, nullptr, cuda_stream);
-    c->in_host_step = false;
-    c->plan_copy_stream = nullptr;
-    if (st != CF_OK) return st;
-    if (cudaEventRecord(hs.compute_done, stream) != cudaSuccess) return CF_ERR_CUDA;
-    // result: second copy stream
-    if (cudaStreamWaitEvent(c->d2h_stream, hs.compute_done, 0) != cudaSuccess) return CF_ERR_CUDA;
-    if (cudaMemcpyAsync(out_host, dout, qb, cudaMemcpyDeviceToHost, c->d2h_stream) != cudaSuccess) return CF_ERR_CUDA;
-    if (cudaEventRecord(hs.d2h_done, c->d2h_stream) != cudaSuccess) return CF_ERR_CUDA;
+    const bool done = cudaEventRecord(hs.compute_done, stream) == cudaSuccess &&
+                      (st == CF_OK || cudaStreamWaitEvent(c->d2h_stream, hs.compute_done, 0) == cudaSuccess) &&
+                      cudaEventRecord(hs.d2h_done, c->d2h_stream) == cudaSuccess;
     hs.used = true;
-    return CF_OK;
+    c->host_ns_attention += now_ns() - t_in;
+    c->host_calls_append += 1;
+    c->host_calls_attention += (int32_t)units.size();
+    if (st == CF_OK && !done) st = CF_ERR_CUDA;
+    if (st == CF_OK) ++c->unflushed_steps;
+    return st;
 }
 
 cf_status cf_host_steps_flush(cf_ctx* c, void* cuda_stream)
@@ -1172,7 +1227,7 @@ cf_status cf_validate_block_table(cf_ctx* c, const cf_cache_desc* desc, const in
     st = next_slot(c, bytes, &slot);
     if (st != CF_OK) return st;
     std::memcpy(slot->host, context_len, bytes);
-    st = upload_slot(c, slot, bytes, stream);
+    st = upload_slot(slot, bytes, c->upload_stream, stream);
     if (st != CF_OK) return st;
     uint32_t* counter = c->err_dev + 1;      // context-owned scratch word
     bool ok = cudaMemsetAsync(counter, 0, sizeof(uint32_t), stream) == cudaSuccess;

@@ -242,3 +242,41 @@ def test_a_small_fixed_workspace_and_shared_prefixes(members, served_shared):
     compare(to_host_bits(out), lse.cpu().numpy(), ref_o, ref_lse)
     g.close()
     cf.cf_destroy(ctx)
+
+
+def test_a_host_step_that_does_not_fit_is_refused_before_anything_is_enqueued():
+    """fp8 cache: the staging of one chunk's context outgrows the fixed workspace.  The step is refused with the caches, out_host
+    and the staging sets as they were, and the steps around it are served."""
+    sc = small(97, 32, 8, 128, [0, 6000, 50], [[600, 40, 1]], NB=1024)
+    b = sc.batches[0]
+    scales = (np.full(8, 0.02, np.float32), np.full(8, 0.015, np.float32))
+    ctx = cf.cf_create(0, workspace_bytes=8 << 20)                    # 38 staged pages (2.5 MB) fit, 378 (25 MB) do not
+    g = GpuScenario(sc, ctx=ctx, fp8=scales)
+    pin = lambda x: torch.from_numpy(x.view(np.int16)).pin_memory()
+    qh, kh, vh, bt = pin(b.q), pin(b.k_new), pin(b.v_new), torch.from_numpy(b.block_table).cuda()
+    fits = (np.array([600, 0, 51], np.int32), np.array([600, 0, 1], np.int32))
+    idx = np.r_[0:600, 640]
+    qs, ks, vs = (torch.from_numpy(x.view(np.int16)[idx].copy()).pin_memory() for x in (b.q, b.k_new, b.v_new))
+    outs = []
+    for step in range(7):                                             # the set of a refused step comes round again
+        if step % 2:
+            k0, v0 = g.pools_host()
+            oh = torch.full_like(qh, 77).pin_memory()
+            st = cf.cf_mixed_step_host(ctx, g.desc, qh, kh, vh, g.k, g.v, bt, b.max_blocks, b.context_len, b.query_len, oh, check=False)
+            assert st == cf.CF_ERR_WORKSPACE
+            cf.cf_host_steps_flush(ctx)
+            torch.cuda.synchronize()
+            k1, v1 = g.pools_host()
+            assert bool((oh == 77).all()) and np.array_equal(k0, k1) and np.array_equal(v0, v1)
+        else:
+            outs.append(torch.full_like(qs, 77).pin_memory())
+            cf.cf_mixed_step_host(ctx, g.desc, qs, ks, vs, g.k, g.v, bt, b.max_blocks, *fits, outs[-1])
+    cf.cf_host_steps_flush(ctx)
+    torch.cuda.synchronize()
+    assert cf.cf_get_async_status(ctx) == cf.CF_OK
+    kr, vr = g.pools_host()
+    ref, _ = oracle.mixed_attention(b.q[idx], kr, vr, b.block_table, *fits, k_scale=g.k_scale, v_scale=g.v_scale)
+    for o in outs:
+        compare(o.numpy().view(np.uint16), None, ref, None)
+    g.close()
+    cf.cf_destroy(ctx)
