@@ -174,7 +174,8 @@ cf_status cf_mixed_attention_planned(cf_plan* plan, const void* q, const void* k
  * the kernels by events and triple-buffered, so that consecutive calls overlap step i+1's input copy
  * and step i-1's read-back with step i's kernels.  A step with many prefill rows is computed in parts, prefill first, and
  * each part is read back while the next one runs - except one that follows another without a flush in between and whose
- * kernels outweigh its copies: that one runs as cf_mixed_attention would.  Asynchronous.  out_host of every call issued so far
+ * kernels outweigh its copies: there the parts' work items run in one call, decode beside prefill, with the same bits.
+ * Asynchronous.  out_host of every call issued so far
  * is valid once cf_host_steps_flush(ctx, stream) has been called and `stream` synchronised; the host
  * input buffers of a call must stay unchanged until then as well. */
 cf_status cf_mixed_step_host(cf_ctx* ctx, const cf_cache_desc* desc,

@@ -970,8 +970,9 @@ struct HostPart {
 };
 
 // Parts of the step, or none when it is better computed and read back as one: few bytes, or too many runs.
+// *kernel_bound: the kernels outweigh both directions of the link.
 static std::vector<HostPart> host_parts(const cf_cache_desc* d, const int32_t* context_len, const int32_t* query_len, int32_t S,
-                                        const std::vector<int32_t>& q_start, int num_sms, bool pipelined)
+                                        const std::vector<int32_t>& q_start, int num_sms, bool* kernel_bound)
 {
     constexpr double kMinPrefillBytes = 4 << 20;      // below: the read-back is shorter than what the parts cost
     constexpr double kLinkBytesPerUs = 52e3, kPartUs = 12.0;
@@ -1013,10 +1014,7 @@ static std::vector<HostPart> host_parts(const cf_cache_desc* d, const int32_t* c
     const double link_us = pre_rows * row_bytes / kLinkBytesPerUs;
     const double in_us = ((double)q_start.back() * (row_bytes + 4.0 * d->num_kv_heads * d->head_dim)) / kLinkBytesPerUs;
     if (in_us > pre_us + dec_us + link_us) return parts;
-    // A step that follows another without a flush in between has its read-back under the kernels of the next one anyway.
-    // Where the kernels outweigh both directions of the link such steps are bound by them and go in one piece, decode beside
-    // prefill (agentic, back to back: 994 -> 899 us per step); where the link weighs as much, parts still help (chat mix: 296 against 349 us).
-    if (pipelined && pre_us + dec_us > 1.25 * std::max(in_us, link_us)) return parts;
+    *kernel_bound = pre_us + dec_us > 1.25 * std::max(in_us, link_us);
     // how many pieces to cut the prefill rows into: the end of the last read-back, all pieces taken as equal
     int32_t cuts = 1;
     double best = 1e30;
@@ -1062,6 +1060,29 @@ static std::vector<HostPart> host_parts(const cf_cache_desc* d, const int32_t* c
     return parts;
 }
 
+// The planned parts of a step as one call (join_plans); false where it does not fit a fixed workspace.
+static bool join_units(cf_ctx* c, const cf_cache_desc* desc, const std::vector<HostPart>& parts, const std::vector<Unit>& units,
+                       const int32_t* context_len, const int32_t* query_len, int32_t num_seqs, int32_t max_blocks_per_seq, Unit* u)
+{
+    std::vector<const Plan*> plans;
+    std::vector<int32_t> seqs;
+    std::vector<int64_t> rows;
+    for (size_t i = 0; i < parts.size(); ++i) {
+        plans.push_back(&units[i].pl);
+        seqs.push_back(parts[i].seq);
+        rows.push_back(parts[i].row);
+    }
+    join_plans(desc, plans, seqs, rows, &u->pl);
+    stage_list(desc, context_len, query_len, num_seqs, &u->stage, &u->n_stage_pages, &u->max_stage_pages);
+    u->W = ws_layout(u->pl.n_part_slots, u->pl.n_pre_slots, desc->num_q_heads, desc->head_dim, u->n_stage_pages, desc->num_kv_heads,
+                     (int64_t)num_seqs * max_blocks_per_seq);
+    u->num_seqs = num_seqs;
+    u->max_blocks = max_blocks_per_seq;
+    u->front_sms = spatial_front_sms(desc, context_len, query_len, num_seqs, c->num_sms);
+    u->serial = u->front_sms <= (c->num_sms * 3) / 5;      // as for a step that is not cut
+    return !c->workspace_fixed || u->W.total <= c->workspace_bytes;
+}
+
 }  // namespace cf
 
 extern "C" {
@@ -1085,28 +1106,46 @@ cf_status cf_mixed_step_host(cf_ctx* c, const cf_cache_desc* desc,
     if (!guard.ok) return CF_ERR_CUDA;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
 
-    // The step is planned, all of its parts, before anything is enqueued: a part that does not fit a fixed workspace refuses the
-    // step while the caches and out_host are as they were.
+    // Plans the step, all of its parts.  With a fixed workspace this comes before anything is enqueued: a part that does not fit
+    // refuses the step while the caches and out_host are as they were.  A growing workspace refuses nothing, and the planning
+    // runs beside the input copies (a step that is waited for: chat mix 581 -> 566 us, 512 rows on an fp8 cache 723 -> 697 us).
     const int64_t t_in = now_ns();
-    std::vector<HostPart> parts = host_parts(desc, context_len, query_len, num_seqs, pl.q_start, c->num_sms, c->unflushed_steps > 0);
-    const bool whole = parts.empty();
-    std::vector<Unit> units(whole ? 1 : parts.size());
-    size_t ws_bytes = 0;
-    for (size_t i = 0; i < units.size(); ++i) {
-        // In one piece: a step whose decode part weighs as much as its prefill part is bound by the copies over the host link,
-        // not by the kernels, and keeps the serial sequence; a prefill-heavy step (the spatial share above its floor) runs
-        // the sequence cf_mixed_attention would run.
-        if (whole)
-            st = plan_unit(c, desc, context_len, query_len, num_seqs, max_blocks_per_seq, nullptr, nullptr,
-                           spatial_front_sms(desc, context_len, query_len, num_seqs, c->num_sms) <= (c->num_sms * 3) / 5, &units[i]);
-        else
-            st = plan_unit(c, desc, parts[i].context_len.data(), parts[i].query_len.data(), parts[i].num_seqs, max_blocks_per_seq, nullptr,
-                           nullptr, true, &units[i]);
-        if (st != CF_OK) return st;
-        ws_bytes = std::max(ws_bytes, units[i].W.total);
-    }
-    st = ensure_workspace(c, ws_bytes);
-    if (st != CF_OK) return st;
+    std::vector<HostPart> parts;
+    std::vector<Unit> units;
+    bool whole = false;
+    auto plan = [&]() -> cf_status {
+        bool kernel_bound = false;
+        parts = host_parts(desc, context_len, query_len, num_seqs, pl.q_start, c->num_sms, &kernel_bound);
+        whole = parts.empty();
+        units.resize(whole ? 1 : parts.size());
+        size_t ws_bytes = 0;
+        for (size_t i = 0; i < units.size(); ++i) {
+            // In one piece: a step whose decode part weighs as much as its prefill part is bound by the copies over the host link,
+            // not by the kernels, and keeps the serial sequence; a prefill-heavy step (the spatial share above its floor) runs
+            // the sequence cf_mixed_attention would run.
+            const cf_status e = whole ? plan_unit(c, desc, context_len, query_len, num_seqs, max_blocks_per_seq, nullptr, nullptr,
+                                                  spatial_front_sms(desc, context_len, query_len, num_seqs, c->num_sms) <= (c->num_sms * 3) / 5, &units[i])
+                                      : plan_unit(c, desc, parts[i].context_len.data(), parts[i].query_len.data(), parts[i].num_seqs,
+                                                  max_blocks_per_seq, nullptr, nullptr, true, &units[i]);
+            if (e != CF_OK) return e;
+            ws_bytes = std::max(ws_bytes, units[i].W.total);
+        }
+        // A step that follows another without a flush in between has its read-back under the kernels of the next one anyway.
+        // Where the kernels outweigh both directions of the link such steps are bound by them, and the parts' items run as one
+        // call, decode beside prefill (agentic, back to back: 994 -> 905 us per step); where the link weighs as much, parts
+        // still help.  The items are the parts' own, so a step's result does not depend on the steps before it.
+        if (!whole && kernel_bound && c->unflushed_steps > 0) {
+            Unit u;
+            if (join_units(c, desc, parts, units, context_len, query_len, num_seqs, max_blocks_per_seq, &u)) {
+                units.clear();
+                units.push_back(std::move(u));
+                ws_bytes = units[0].W.total;
+                whole = true;
+            }
+        }
+        return ensure_workspace(c, ws_bytes);
+    };
+    if (c->workspace_fixed && (st = plan()) != CF_OK) return st;
     c->launches = 0;
 
     const size_t T = (size_t)pl.total_q;
@@ -1143,9 +1182,11 @@ cf_status cf_mixed_step_host(cf_ctx* c, const cf_cache_desc* desc,
             !ok(cudaEventRecord(hs.h2d_kv_done, c->h2d_kv_stream)) ||
             !ok(cudaMemcpyAsync(dq, q_host, qb, cudaMemcpyHostToDevice, c->h2d_stream)) || !ok(cudaEventRecord(hs.h2d_done, c->h2d_stream)))
             return CF_ERR_CUDA;
+        cf_status e = c->workspace_fixed ? CF_OK : plan();
+        if (e != CF_OK) return e;
         // kernels: the caller's stream; plans are uploaded on the input copy stream
         if (!ok(cudaStreamWaitEvent(stream, hs.h2d_kv_done, 0))) return CF_ERR_CUDA;
-        cf_status e = enqueue_append(c, desc, pl, k_cache, v_cache, dk, dv, block_table, max_blocks_per_seq, context_len, query_len, num_seqs,
+        e = enqueue_append(c, desc, pl, k_cache, v_cache, dk, dv, block_table, max_blocks_per_seq, context_len, query_len, num_seqs,
                                      c->h2d_stream, stream);
         if (e != CF_OK) return e;
         if (!ok(cudaStreamWaitEvent(stream, hs.h2d_done, 0))) return CF_ERR_CUDA;

@@ -77,6 +77,13 @@ cf_status validate_lengths(const cf_cache_desc* d, const int32_t* context_len, c
     return CF_OK;
 }
 
+// Prefill items are queued KV head by KV head (build_plan says why)
+static bool head_by_head(const cf_cache_desc* d, int64_t longest)
+{
+    constexpr int64_t kKvSetBytes = CF_KV_SET_BYTES;
+    return d->num_q_heads / d->num_kv_heads >= 2 && longest * 2 * d->num_kv_heads * d->head_dim * 2 > kKvSetBytes;
+}
+
 cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const int32_t* query_len,
                      int32_t num_seqs, int32_t max_blocks_per_seq, const PlanConfig& cfg, Plan* plan,
                      const int32_t* share_group, const int32_t* shared_len)
@@ -303,13 +310,9 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         // other (longest item first inside each), so that the items in flight share two or three heads instead of all:
         // the same work, a third of the trips to DRAM (measured on 2048 new over 24,576 cached tokens: +1.8 %).
         // Below that size the order makes no difference to DRAM and the globally longest-first order is kept.
-        constexpr int64_t kKvSetBytes = CF_KV_SET_BYTES;
-        int32_t kv_sets = 1;
-        if (G >= 2) {
-            int64_t longest = 0;
-            for (const Group& gr : groups) longest = std::max(longest, gr.extent);
-            if (longest * 2 * d->num_kv_heads * d->head_dim * 2 > kKvSetBytes) kv_sets = d->num_kv_heads;
-        }
+        int64_t longest_kv = 0;
+        for (const Group& gr : groups) longest_kv = std::max(longest_kv, gr.extent);
+        const int32_t kv_sets = head_by_head(d, longest_kv) ? d->num_kv_heads : 1;
         const int32_t heads_per_set = d->num_kv_heads / kv_sets;
         for (int32_t set = 0; set < kv_sets; ++set)
         for (const Group& gr : groups) {
@@ -564,6 +567,58 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         }
     }
     return CF_OK;
+}
+
+void join_plans(const cf_cache_desc* d, const std::vector<const Plan*>& parts, const std::vector<int32_t>& seqs,
+                const std::vector<int64_t>& rows, Plan* plan)
+{
+    int64_t longest = 0;
+    for (size_t i = 0; i < parts.size(); ++i) {
+        const Plan& a = *parts[i];
+        const int32_t seq = seqs[i], row = (int32_t)rows[i], slot = plan->n_part_slots, pre_slot = plan->n_pre_slots;
+        for (DecodeItem it : a.decode) {
+            it.seq += seq;
+            it.q_row += row;
+            if (it.part_slot >= 0) it.part_slot += slot;
+            plan->decode.push_back(it);
+        }
+        for (CombineItem it : a.combine) plan->combine.push_back(CombineItem{it.q_row + row, it.part_first + slot, it.n_chunks});
+        auto shift = [&](auto& it) {
+            for (int t = 0; t < 2; ++t) {
+                if (it.n_rows[t] > 0) it.q_row0[t] += row;
+                if (it.part_slot[t] >= 0) it.part_slot[t] += pre_slot;
+            }
+        };
+        for (PrefillTcItem it : a.prefill_tc) {
+            it.seq += seq;
+            shift(it);
+            longest = std::max<int64_t>(longest, it.ctx_len);
+            plan->prefill_tc.push_back(it);
+        }
+        for (PrefillCombineItem it : a.prefill_combine) {
+            shift(it);
+            plan->prefill_combine.push_back(it);
+        }
+        plan->n_part_slots += a.n_part_slots;
+        plan->n_pre_slots += a.n_pre_slots;
+        plan->total_q += a.total_q;
+        plan->n_decode_seqs += a.n_decode_seqs;
+        plan->n_prefill_seqs += a.n_prefill_seqs;
+        plan->pair = plan->pair || a.pair;
+    }
+    std::stable_sort(plan->decode.begin(), plan->decode.end(), [](const DecodeItem& a, const DecodeItem& b) {
+        return (a.kv_end - a.kv_begin) > (b.kv_end - b.kv_begin);
+    });
+    const bool by_head = head_by_head(d, longest);
+    auto tiles = [](const PrefillTcItem& it) {
+        int32_t end = 0;
+        for (int t = 0; t < 2; ++t)
+            if (it.n_rows[t] > 0) end = std::max(end, it.prefix + it.row0[t] + it.n_rows[t]);
+        return std::min((end + 127) / 128, it.j_end) - it.j_begin;
+    };
+    std::stable_sort(plan->prefill_tc.begin(), plan->prefill_tc.end(), [&](const PrefillTcItem& a, const PrefillTcItem& b) {
+        return by_head && a.kvh != b.kvh ? a.kvh < b.kvh : tiles(a) > tiles(b);
+    });
 }
 
 int32_t spatial_front_sms(const cf_cache_desc* d, const int32_t* context_len, const int32_t* query_len, int32_t num_seqs,

@@ -260,6 +260,12 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
                      int32_t num_seqs, int32_t max_blocks_per_seq, const PlanConfig& cfg, Plan* plan,
                      const int32_t* share_group = nullptr, const int32_t* shared_len = nullptr);
 
+// The plans of consecutive parts of one batch (part i: sequences from seqs[i] on, packed rows from rows[i] on) as one plan of
+// the batch: the same items, chunks and KV ranges, so every row has the bits that its part gives it, queued as build_plan
+// queues them.
+void join_plans(const cf_cache_desc* d, const std::vector<const Plan*>& parts, const std::vector<int32_t>& seqs,
+                const std::vector<int64_t>& rows, Plan* plan);
+
 // Predicted device time of one cf_mixed_attention call, in microseconds, from a model fitted to this
 // library's measured kernel times on B200 (decode: fixed cost + bytes at the sustained split-K rate;
 // prefill: work items scheduled longest-first onto the SMs, each costing a fixed part plus a time per

@@ -280,3 +280,37 @@ def test_a_host_step_that_does_not_fit_is_refused_before_anything_is_enqueued():
         compare(o.numpy().view(np.uint16), None, ref, None)
     g.close()
     cf.cf_destroy(ctx)
+
+
+@pytest.mark.parametrize("prefix,qlen,fp8", [
+    ([40000, 3000], [600, 1], False),
+    ([70, 9000, 40000, 3000, 500, 20000], [1, 1, 600, 300, 1, 1], False),
+    ([40000, 36000, 100, 100], [300, 400, 0, 1], False),
+    ([30000, 9000, 700], [600, 1, 1], True),
+])
+def test_a_host_step_does_not_depend_on_the_steps_before_it(prefix, qlen, fp8):
+    """The first step after a flush goes in parts; those behind it, bound by their kernels, in one piece: the same bits, which are
+    right."""
+    sc = small(98, 32, 8, 128, prefix, [qlen], NB=5120)
+    b = sc.batches[0]
+    scales = (np.full(8, 0.02, np.float32), np.full(8, 0.015, np.float32)) if fp8 else None
+    g = GpuScenario(sc, fp8=scales)
+    pin = lambda x: torch.from_numpy(x.view(np.int16)).pin_memory()
+    qh, kh, vh, bt = pin(b.q), pin(b.k_new), pin(b.v_new), torch.from_numpy(b.block_table).cuda()
+    outs, kernels = [], []
+    for _ in range(5):
+        outs.append(torch.full_like(qh, -1).pin_memory())
+        cf.cf_mixed_step_host(g.ctx, g.desc, qh, kh, vh, g.k, g.v, bt, b.max_blocks, b.context_len, b.query_len, outs[-1])
+        kernels.append(cf.cf_get_last_plan_counts(g.ctx)[2])
+    cf.cf_host_steps_flush(g.ctx)
+    torch.cuda.synchronize()
+    assert cf.cf_get_async_status(g.ctx) == cf.CF_OK
+    assert kernels[0] == 0 < kernels[1]                               # the last call of a step in parts is its decode part
+    assert all(torch.equal(outs[0], o) for o in outs[1:])
+    k_ref, v_ref = g.pools_host()
+    rows = syn.tile_edge_rows(b)
+    rows = np.unique(np.r_[rows[::9], rows[-3:], b.total_q - 1])
+    variant = dict(k_scale=g.k_scale, v_scale=g.v_scale) if fp8 else {}
+    ref, _ = oracle.mixed_attention(b.q, k_ref, v_ref, b.block_table, b.context_len, b.query_len, rows=rows, **variant)
+    compare(outs[0].numpy().view(np.uint16), None, ref, None, rows=rows)
+    g.close()
