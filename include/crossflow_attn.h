@@ -310,7 +310,7 @@ cf_status cf_decode_attention_static(const cf_cache_desc* desc, const void* q,
  * (microseconds) of the decode, combine and prefill kernels that cf_mixed_attention would launch for
  * these lengths on a B200 with num_sms SMs (0 = 148), from a model fitted to this library's measured
  * times: a scheduler can size the next prefill chunk so that the iteration stays inside its ITL budget.
- * Accuracy on the five workload configurations: within about 15 %.  Any output pointer may be NULL. */
+ * Accuracy on the five workload configurations: within about 20 %.  Any output pointer may be NULL. */
 cf_status cf_estimate_us(const cf_cache_desc* desc, const int32_t* context_len, const int32_t* query_len,
                          int32_t num_seqs, int32_t max_blocks_per_seq, int32_t num_sms,
                          float* us_decode, float* us_combine, float* us_prefill);

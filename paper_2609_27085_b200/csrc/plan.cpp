@@ -653,19 +653,23 @@ int32_t spatial_front_sms(const cf_cache_desc* d, const int32_t* context_len, co
 Estimate estimate_us(const cf_cache_desc* d, const int32_t* context_len, const int32_t* query_len, const Plan& plan,
                      int32_t num_sms)
 {
-    // Constants fitted to CUDA-event times of the kernels on a B200: split-K decode (with the merge of the
-    // partials fused in) sustains ~7.56 TB/s on top of ~22 us of launch, ramp and tail; the separate combine
-    // launch, when it is used, ~8 us, reported as 0 here because the default path has none; one tcgen05
-    // prefill item costs ~8 us plus ~1.9 us per 128-token KV tile.
-    constexpr double kDecodeFixedUs = 22.0, kDecodeBytesPerUs = 7.56e6, kCombineUs = 0.0;
-    constexpr double kTcItemFixedUs = 8.0, kTcTileUs = 1.9, kLaunchUs = 4.0;
+    // Constants fitted to CUDA-event times of the kernels on a B200.  Split-K decode (with the merge of the partials fused in):
+    // 10 us of launch, ramp and tail on top of its bytes at 6.8 TB/s, of an fp8 cache's codes at 6.3 TB/s; measured / predicted: five
+    // sequences of 600 tokens 13 / 12 us, 40 of 800 (32 over 8 heads) 31 / 29, 64 of 2000 84 / 87, 64 of 1K-8K 191 / 187,
+    // 256 on an fp8 cache 178 / 180.  The separate combine launch, when it is used, is reported as 0: the default path has none.
+    // One tcgen05 prefill item costs ~8 us plus ~1.9 us per 128-token KV tile (head_dim 64: 1.4), at the clock that a long
+    // prefill settles at; a short one at full clock takes up to 20 % less.
+    constexpr double kDecodeFixedUs = 10.0, kCombineUs = 0.0;
+    constexpr double kTcItemFixedUs = 8.0, kLaunchUs = 4.0;
+    const bool fp8 = d->kv_dtype == CF_KV_FP8_E4M3;
+    const double kDecodeBytesPerUs = fp8 ? 6.3e6 : 6.8e6, kTcTileUs = d->head_dim == 64 ? 1.4 : 1.9;
     Estimate e;
     const int32_t S = (int32_t)plan.q_start.size() - 1;
     double dec_bytes = 0.0;
     for (int32_t s = 0; s < S; ++s)
         if (query_len[s] == 1)
             dec_bytes += (double)(d->window_size > 0 ? std::min(context_len[s], d->window_size) : context_len[s]) * 2.0 *
-                             d->num_kv_heads * d->head_dim * 2.0 + 4.0 * d->num_q_heads * d->head_dim;
+                             d->num_kv_heads * d->head_dim * (fp8 ? 1.0 : 2.0) + 4.0 * d->num_q_heads * d->head_dim;
     if (!plan.decode.empty()) e.us_decode = (float)(kDecodeFixedUs + dec_bytes / kDecodeBytesPerUs);
     if (!plan.combine.empty()) e.us_combine = (float)kCombineUs;
     if (!plan.prefill_tc.empty()) {

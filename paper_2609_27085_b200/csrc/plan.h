@@ -278,8 +278,8 @@ struct Estimate {
 // balances the prefill items over this many SMs.  Decode gets what it needs to be done when the prefill is, and no
 // more: it saturates HBM from k_sat SMs (about 65 with up to four heads per KV head, about 100 with eight, where the
 // MMAs per byte double), so over a call of length T it needs k_sat * t_decode / T of them, taken with a margin of 1.15;
-// the share of the prefill grid is clamped to [3/5, 7/8] of the SMs.  t_decode and the prefill work come from the
-// constants of estimate_us.  Fitted against sweeps of the share on the bench configurations (within a few per
+// the share of the prefill grid is clamped to [3/5, 7/8] of the SMs.  t_decode and the prefill work come from constants of
+// its own (decode beside prefill, not on its own).  Fitted against sweeps of the share on the bench configurations (within a few per
 // cent of the best share on each).
 int32_t spatial_front_sms(const cf_cache_desc* d, const int32_t* context_len, const int32_t* query_len, int32_t num_seqs,
                           int32_t num_sms);

@@ -297,3 +297,17 @@ def test_decode_plans_fit_the_allocation_free_entry_point(Hq, Hkv, D):
             for lens in (np.full(S, L), (L * rng.lognormal(0, 1, S)).clip(1, 1 << 22)):
                 *_, parts, counts = cf.cf_plan_inspect(d, lens.astype(np.int32), np.ones(S, np.int32), 1 << 20, want_counts=True, cap=1)
                 assert counts[0] <= 3584 and parts * Hq * (D + 2) * 4 + 256 <= (16 << 20) - (128 << 10), (S, L)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,fp8,n,L,measured", [
+    (64, 8, 128, False, 5, 600, 13.2), (32, 8, 128, False, 16, 400, 11.3), (32, 8, 128, False, 40, 800, 30.7),
+    (32, 8, 128, False, 64, 2000, 84.1), (32, 8, 128, False, 16, 20000, 199.9), (8, 2, 128, False, 64, 2000, 28.9),
+    (64, 8, 64, False, 64, 2000, 54.5), (64, 8, 64, False, 5, 600, 12.6), (64, 8, 128, True, 64, 2000, 55.7), (64, 8, 128, True, 16, 20000, 114.0),
+])
+def test_decode_estimates_follow_the_present_kernels(Hq, Hkv, D, fp8, n, L, measured):
+    """cf_estimate_us against CUDA-event times (us) of the decode kernels on a B200: within 25 %, small batches and fp8 caches
+    included."""
+    d = cf.make_desc(Hq, Hkv, D, 16, 65536, kv_dtype=cf.CF_KV_FP8_E4M3 if fp8 else cf.CF_KV_BF16, k_scale=16 if fp8 else None,
+                     v_scale=16 if fp8 else None)
+    us, _, _ = cf.cf_estimate_us(d, [L] * n, [1] * n, 4096)
+    assert abs(us / measured - 1.0) < 0.25, us
