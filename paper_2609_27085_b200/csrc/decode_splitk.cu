@@ -895,10 +895,30 @@ static size_t decode_smem_bytes()
     return ring > merge ? ring : merge;
 }
 
-// Decode grids start before the grid ahead of them in the stream has completed (decode_grid_start): the launch, the
-// work item's fetch and the set-up are off the critical path.  `ctas` is one CTA per (item, KV head).
+// Launches with programmatic stream serialisation: the grid starts before the grid ahead of it in the stream has completed
+// (decode_grid_start; the combine kernel executes griddepcontrol.wait before it touches a partial), so that the launch, the
+// work item's fetch and the set-up are off the critical path.  The plan that the launch carries is read from the caller's
+// buffer; by-value parameters would be copies of 12 KB each on the stack of a call that promises a small one.
+template <class... Args>
+static cudaError_t launch_serialised(const void* kernel, dim3 grid, int threads, size_t smem, cudaStream_t stream, const Args*... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* values[] = {const_cast<void*>(static_cast<const void*>(args))...};
+    return cudaLaunchKernelExC(&cfg, kernel, values);
+}
+
+// Decode grids: `ctas` is one CTA per (item, KV head).
 template <auto KERN, int INL, class... Rest>
-static cudaError_t launch_decode_grid(int ctas, size_t smem, cudaStream_t stream, const AttnParams& p, const PlanBytes<INL>& inl, Rest... rest)
+static cudaError_t launch_decode_grid(int ctas, size_t smem, cudaStream_t stream, const AttnParams& p, const PlanBytes<INL>* inl, const Rest*... rest)
 {
     // set once per kernel and device; two host threads racing here both set the same value
     static std::atomic<bool> configured[64];
@@ -909,29 +929,16 @@ static cudaError_t launch_decode_grid(int ctas, size_t smem, cudaStream_t stream
         if (e != cudaSuccess) return e;
         configured[dev].store(true, std::memory_order_release);
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(ctas + (p.dec_chained ? 1 : 0)));
-    cfg.blockDim = dim3(kDecWarps * 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, KERN, p, inl, rest...);
+    return launch_serialised((const void*)KERN, dim3((unsigned)(ctas + (p.dec_chained ? 1 : 0))), kDecWarps * 32, smem, stream, &p, inl, rest...);
 }
 
 // launch(size, block) with the parameter block that the plan fits in: none (it is in device memory), small or mid
 template <class F>
 static cudaError_t with_plan_bytes(const HostPlan& hp, F launch)
 {
-    if (!hp.bytes) return launch(std::integral_constant<int, 0>{}, PlanBytes<0>{});
-    auto carry = [&](auto size) {
-        PlanBytes<decltype(size)::value> b;
-        std::memcpy(b.bytes, hp.bytes, hp.size);
-        return launch(size, b);
-    };
+    static const PlanBytes<0> none = {};
+    if (!hp.bytes) return launch(std::integral_constant<int, 0>{}, &none);
+    auto carry = [&](auto size) { return launch(size, reinterpret_cast<const PlanBytes<decltype(size)::value>*>(hp.bytes)); };
     if (hp.size <= (size_t)kSmallPlanBytes) return carry(std::integral_constant<int, kSmallPlanBytes>{});
     return hp.size <= (size_t)kMidPlanBytes ? carry(std::integral_constant<int, kMidPlanBytes>{}) : cudaErrorInvalidValue;
 }
@@ -939,7 +946,7 @@ static cudaError_t with_plan_bytes(const HostPlan& hp, F launch)
 template <int D>
 static cudaError_t launch_decode_t(const AttnParams& p, const HostPlan& hp, int n_items, cudaStream_t stream)
 {
-    return with_plan_bytes(hp, [&](auto size, const auto& inl) {
+    return with_plan_bytes(hp, [&](auto size, const auto* inl) {
         return launch_decode_grid<decode_splitk_kernel<D, kDecWarps, dec_stages<D>(), decltype(size)::value>>(
             n_items * p.Hkv, decode_smem_bytes<D>(), stream, p, inl);
     });
@@ -950,7 +957,7 @@ cudaError_t launch_decode_fp8(const AttnParams& p, const HostPlan& hp, int n_ite
     if (n_items <= 0) return cudaSuccess;
     const size_t ring = (size_t)kDecWarps * kDecStagesFp8 * 2 * 16 * 128;
     const size_t merge = (size_t)kDecWarps * 8 * (128 + 4) * 4 + (size_t)kDecWarps * 8 * 4 * 2;
-    return with_plan_bytes(hp, [&](auto size, const auto& inl) {
+    return with_plan_bytes(hp, [&](auto size, const auto* inl) {
         return launch_decode_grid<decode_splitk_fp8_kernel<kDecWarps, kDecStagesFp8, decltype(size)::value>>(
             n_items * p.Hkv, std::max(ring, merge), stream, p, inl);
     });
@@ -969,9 +976,10 @@ static cudaError_t launch_decode_shared_t(const AttnParams& p, const HostPlan& h
     constexpr int STAGES = kDecStages * 128 / D;       // the same 96 KB for both head sizes
     const size_t ring = (size_t)kDecWarps * STAGES * 2 * 16 * D * 2;
     const size_t merge = (size_t)kDecWarps * COLS * (D + 4) * 4 + (size_t)kDecWarps * COLS * 4 * 2;
-    return with_plan_bytes(hp, [&](auto size, const auto& inl) {
+    const int n_shared_ctas = n_shared_items * p.Hkv;
+    return with_plan_bytes(hp, [&](auto size, const auto* inl) {
         return launch_decode_grid<decode_with_shared_kernel<D, kDecWarps, STAGES, NCG, decltype(size)::value>>(
-            (n_shared_items + n_items) * p.Hkv, std::max(ring, merge), stream, p, inl, n_shared_items * p.Hkv);
+            (n_shared_items + n_items) * p.Hkv, std::max(ring, merge), stream, p, inl, &n_shared_ctas);
     });
 }
 
@@ -986,22 +994,10 @@ cudaError_t launch_decode_with_shared(const AttnParams& p, const HostPlan& hp, i
 cudaError_t launch_combine(const AttnParams& p, const HostPlan& hp, int head_dim, int n_items, cudaStream_t stream)
 {
     if (n_items <= 0) return cudaSuccess;
-    dim3 grid(n_items, p.Hq);
-    // programmatic dependent launch: the grid may be scheduled while the decode kernel drains; every CTA
-    // executes griddepcontrol.wait before touching the partials
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(head_dim == 128 ? 32 : 16);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return with_plan_bytes(hp, [&](auto size, const auto& inl) {
+    return with_plan_bytes(hp, [&](auto size, const auto* inl) {
         constexpr int INL = decltype(size)::value;
-        return head_dim == 128 ? cudaLaunchKernelEx(&cfg, combine_kernel<128, INL>, p, inl) : cudaLaunchKernelEx(&cfg, combine_kernel<64, INL>, p, inl);
+        const void* kernel = head_dim == 128 ? (const void*)combine_kernel<128, INL> : (const void*)combine_kernel<64, INL>;
+        return launch_serialised(kernel, dim3((unsigned)n_items, (unsigned)p.Hq), head_dim / 4, 0, stream, &p, inl);
     });
 }
 
@@ -1040,10 +1036,14 @@ StaticSetup g_static_setup[kMaxDevices];
 std::mutex g_static_setup_mutex;     // two host threads may make a device's first call at the same time
 
 struct StaticPlan {                  // fixed capacity, lives on the caller's stack (about 124 KB)
-    cf::DecodeItem items[kStaticMaxItems];
-    cf::CombineItem comb[kStaticMaxSeqs];
+    union {
+        float pages[cf::kTargetSeqs];                // while the chunk length is chosen
+        cf::DecodeItem items[kStaticMaxItems];
+    };
+    cf::CombineItem comb[kStaticMaxSeqs];            // moved up behind the items for a launch that carries the plan
     int n_items = 0, n_comb = 0, n_slots = 0;
 };
+static_assert(sizeof(cf::DecodeItem) * kStaticMaxItems >= (size_t)cf::kMidPlanBytes, "a carried plan is read from the items' storage");
 static_assert(sizeof(cf::DecodeItem) * kStaticMaxItems + 256 + sizeof(cf::CombineItem) * kStaticMaxSeqs <= kStaticPlanBytes,
               "the plan region of the scratch array holds the largest plan");
 
@@ -1103,11 +1103,11 @@ extern "C" cf_status cf_decode_attention_static(const cf_cache_desc* desc, const
     }
     const int32_t W = desc->window_size;
     auto first_page_of = [&](int32_t lc) -> int64_t { return (W > 0 && lc > W) ? (lc - W) / B : 0; };
+    StaticPlan pl;
     const int64_t target = decode_target_pages(
         num_seqs, [&](int32_t s) -> int64_t { return (int64_t)context_len[s] - first_page_of(context_len[s]) * B; }, B,
-        Hq, desc->num_kv_heads, D, false, cfg);
-
-    StaticPlan pl;
+        Hq, desc->num_kv_heads, D, false, cfg, pl.pages);
+    std::atomic_signal_fence(std::memory_order_seq_cst);      // the items take over the storage
     for (int32_t s = 0; s < num_seqs; ++s) {
         const int32_t lc = context_len[s];
         const int64_t page0 = first_page_of(lc);
@@ -1152,13 +1152,12 @@ extern "C" cf_status cf_decode_attention_static(const cf_cache_desc* desc, const
     // runtime stages the bytes before returning and the arrays may go out of scope as soon as this function returns
     // (three sequences of some 4000 tokens, 8 over 2 heads: 14.4 us per call with the copies, 9.7 us without).
     HostPlan hp;
-    alignas(16) uint8_t inline_plan[kMidPlanBytes];
     const size_t comb_at = (items_bytes + 15) / 16 * 16;
     const bool carried = comb_at + comb_bytes <= (size_t)kMidPlanBytes;
     if (carried) {
-        std::memcpy(inline_plan, pl.items, items_bytes);
-        if (comb_bytes) std::memcpy(inline_plan + comb_at, pl.comb, comb_bytes);
-        hp.bytes = inline_plan;
+        uint8_t* const bytes = reinterpret_cast<uint8_t*>(pl.items);
+        if (comb_bytes) std::memmove(bytes + comb_at, pl.comb, comb_bytes);
+        hp.bytes = bytes;
         hp.size = comb_at + comb_bytes;
     } else {
         if (cudaMemcpyAsync(su.base, pl.items, items_bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CF_ERR_CUDA;

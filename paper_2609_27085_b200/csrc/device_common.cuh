@@ -30,7 +30,8 @@ __device__ __forceinline__ const T* plan_list(const uint8_t* plan, int32_t offse
 {
     return reinterpret_cast<const T*>(plan + offset);
 }
-// the plan of a host-side call whose lists the launches carry (bytes null: p.plan.base is set instead)
+// The plan of a host-side call whose lists the launches carry (bytes null: p.plan.base is set instead).  `bytes` lies in a
+// buffer of at least kSmallPlanBytes, for larger plans of kMidPlanBytes: the launches read their parameter from there.
 struct HostPlan {
     const uint8_t* bytes = nullptr;
     size_t size = 0;

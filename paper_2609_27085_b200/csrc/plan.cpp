@@ -147,10 +147,11 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         return shared_pages.empty() ? first_page_of(context_len[s]) : (int64_t)shared_pages[(size_t)s];
     };
     auto decode_target = [&]() {
+        float pages[kTargetSeqs];
         return decode_target_pages(
             num_seqs,
             [&](int32_t s) -> int64_t { return query_len[s] == 1 ? (int64_t)context_len[s] - own_first_page(s) * B : -1; },
-            B, d->num_q_heads, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, cfg, extra_pages);
+            B, d->num_q_heads, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, cfg, pages, extra_pages);
     };
     int64_t target = decode_target();
 

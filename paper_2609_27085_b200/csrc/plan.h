@@ -140,12 +140,12 @@ cf_status validate_lengths(const cf_cache_desc* d, const int32_t* context_len, c
 // 64 of 4000 tokens, which four waves fitted, 167 -> 168 us; the 90 shapes 1.06 in the mean.
 constexpr int64_t kStaticPartBytes = (16ll << 20) - (128ll << 10);      // partials of the allocation-free entry point
 constexpr int32_t kStaticMaxItems = 3584;                              // and its chunks
+constexpr int32_t kTargetSeqs = 2048;               // larger batches: whole sequences are chunks enough
+// `pages`: scratch of kTargetSeqs floats
 template <class LcOf>
 inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int32_t Hq, int32_t Hkv, int32_t D, bool fp8,
-                                   const PlanConfig& cfg, int64_t extra_pages = 0)
+                                   const PlanConfig& cfg, float* pages, int64_t extra_pages = 0)
 {
-    constexpr int32_t kMax = 2048;                      // larger batches: whole sequences are chunks enough
-    float pages[kMax];
     int32_t n = 0;
     int64_t total = extra_pages, longest = 1;           // extra: pages streamed by shared-prefix items
     for (int32_t s = 0; s < num_seqs; ++s) {
@@ -154,7 +154,7 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
         const int64_t pg = (lc + B - 1) / B;
         total += pg;
         longest = pg > longest ? pg : longest;
-        if (n < kMax) pages[n] = (float)pg;
+        if (n < kTargetSeqs) pages[n] = (float)pg;
         ++n;
     }
     const int64_t quantum = cfg.decode_page_quantum > 1 ? cfg.decode_page_quantum : 1;
@@ -165,7 +165,7 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
     auto round_up = [&](int64_t c) { return (c + quantum - 1) / quantum * quantum; };
     const int64_t full = round_up((total * Hkv + 2 * sms * waves - 1) / (2 * sms * waves));      // fills `waves` waves of two CTAs per SM
     const int64_t slot_bytes = (int64_t)Hq * (D + 2) * 4, budget = std::min(cfg.part_bytes, kStaticPartBytes);
-    if (n > kMax || extra_pages > 0) {
+    if (n > kTargetSeqs || extra_pages > 0) {
         int64_t c = round_up((total * Hkv + slots * waves - 1) / (slots * waves));
         c = extra_pages > 0 ? (c > 32 ? c : c > lo ? 32 : lo) : (c > lo ? c : lo);
         if (cfg.part_bytes != INT64_MAX) {

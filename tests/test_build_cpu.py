@@ -22,3 +22,19 @@ def test_a_failed_build_leaves_no_temporaries(tmp_path):
                        capture_output=True, text=True, timeout=300)
     assert r.returncode != 0
     assert set(os.listdir(tmp_path / PKG)) <= before
+
+
+def test_the_allocation_free_call_keeps_to_its_stack(tmp_path):
+    """cf_decode_attention_static promises about 124 KB of stack: its own frame, and no other of its file worth mentioning (a plan
+    that the launches carry is not copied on the way).  Frame sizes as the host compiler reports them."""
+    src = os.path.join(ROOT, PKG, "csrc", "decode_splitk.cu")
+    nvcc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "bin", "nvcc")
+    subprocess.run([nvcc if os.path.exists(nvcc) else "nvcc", "-gencode", "arch=compute_100a,code=compute_100a", "-Xcicc", "-O0", "-O3", "-std=c++17",
+                    "-Xcompiler", "-fPIC,-fstack-usage", "--expt-relaxed-constexpr", "-c", src, "-o", str(tmp_path / "d.o")],
+                   check=True, capture_output=True, timeout=600)
+    frames = {}
+    for line in (tmp_path / "d.su").read_text().splitlines():
+        name, size, _ = line.split("\t")
+        frames[name] = int(size)
+    sizes = sorted(frames.values())                                   # the entry point's frame is the largest by far
+    assert 112 * 1024 < sizes[-1] <= 126 * 1024 and sizes[-2] <= 4096, sizes[-3:]
