@@ -173,10 +173,12 @@ bool arity(Py_ssize_t n, Py_ssize_t want)
     return false;
 }
 
-bool same(int32_t a, int32_t b)      // one length per sequence in every array
+// context_len says how many sequences there are; the other arrays have a value for each of them (or more: a caller may hand
+// over the front of padded arrays)
+bool enough(int32_t seqs, int32_t n)
 {
-    if (a == b) return true;
-    PyErr_SetString(PyExc_ValueError, "length arrays of different sizes");
+    if (n >= seqs) return true;
+    PyErr_SetString(PyExc_ValueError, "a length array is shorter than context_len");
     return false;
 }
 
@@ -196,7 +198,7 @@ PyObject* py_kv_append(PyObject*, PyObject* const* a, Py_ssize_t n)
     Held hd, hc, hq;
     if (!arity(n, 11) || !handle(a[0], &ctx) || !hd.desc(a[1], &d) || !address(a[2], &k) || !address(a[3], &v) || !address(a[4], &kn) ||
         !address(a[5], &vn) || !address(a[6], &bt) || !int32(a[7], &mb) || !hc.lengths(a[8], &lc, &S) || !hq.lengths(a[9], &lq, &S2) ||
-        !same(S, S2) || !stream_of(a[10], &s))
+        !enough(S, S2) || !stream_of(a[10], &s))
         return nullptr;
     return status([&] { return lib.kv_append(ctx, d, k, v, kn, vn, bt, mb, lc, lq, S, s); });
 }
@@ -206,7 +208,7 @@ PyObject* py_mixed_attention(PyObject*, PyObject* const* a, Py_ssize_t n)
     cf_ctx* ctx; const cf_cache_desc* d; void *out, *s; const void *q, *k, *v; float* lse; const int32_t *bt, *lc, *lq; int32_t mb, S, S2;
     Held hd, hc, hq;
     if (!arity(n, 12) || !handle(a[0], &ctx) || !hd.desc(a[1], &d) || !address(a[2], &q) || !address(a[3], &k) || !address(a[4], &v) ||
-        !address(a[5], &bt) || !int32(a[6], &mb) || !hc.lengths(a[7], &lc, &S) || !hq.lengths(a[8], &lq, &S2) || !same(S, S2) ||
+        !address(a[5], &bt) || !int32(a[6], &mb) || !hc.lengths(a[7], &lc, &S) || !hq.lengths(a[8], &lq, &S2) || !enough(S, S2) ||
         !address(a[9], &out) || !address(a[10], &lse) || !stream_of(a[11], &s))
         return nullptr;
     return status([&] { return lib.mixed_attention(ctx, d, q, k, v, bt, mb, lc, lq, S, out, lse, s); });
@@ -218,8 +220,8 @@ PyObject* py_mixed_attention_shared(PyObject*, PyObject* const* a, Py_ssize_t n)
     int32_t mb, S, S2, S3, S4;
     Held hd, hc, hq, hg, hl;
     if (!arity(n, 14) || !handle(a[0], &ctx) || !hd.desc(a[1], &d) || !address(a[2], &q) || !address(a[3], &k) || !address(a[4], &v) ||
-        !address(a[5], &bt) || !int32(a[6], &mb) || !hc.lengths(a[7], &lc, &S) || !hq.lengths(a[8], &lq, &S2) || !same(S, S2) ||
-        !hg.lengths(a[9], &sg, &S3) || !same(S, S3) || !hl.lengths(a[10], &sl, &S4) || !same(S, S4) || !address(a[11], &out) ||
+        !address(a[5], &bt) || !int32(a[6], &mb) || !hc.lengths(a[7], &lc, &S) || !hq.lengths(a[8], &lq, &S2) || !enough(S, S2) ||
+        !hg.lengths(a[9], &sg, &S3) || !enough(S, S3) || !hl.lengths(a[10], &sl, &S4) || !enough(S, S4) || !address(a[11], &out) ||
         !address(a[12], &lse) || !stream_of(a[13], &s))
         return nullptr;
     return status([&] { return lib.mixed_attention_shared(ctx, d, q, k, v, bt, mb, lc, lq, sg, sl, S, out, lse, s); });
@@ -249,7 +251,7 @@ PyObject* py_mixed_step_host(PyObject*, PyObject* const* a, Py_ssize_t n)
     Held hd, hc, hq;
     if (!arity(n, 13) || !handle(a[0], &ctx) || !hd.desc(a[1], &d) || !address(a[2], &q) || !address(a[3], &kn) || !address(a[4], &vn) ||
         !address(a[5], &k) || !address(a[6], &v) || !address(a[7], &bt) || !int32(a[8], &mb) || !hc.lengths(a[9], &lc, &S) ||
-        !hq.lengths(a[10], &lq, &S2) || !same(S, S2) || !address(a[11], &out) || !stream_of(a[12], &s))
+        !hq.lengths(a[10], &lq, &S2) || !enough(S, S2) || !address(a[11], &out) || !stream_of(a[12], &s))
         return nullptr;
     return status([&] { return lib.mixed_step_host(ctx, d, q, kn, vn, k, v, bt, mb, lc, lq, S, out, s); });
 }

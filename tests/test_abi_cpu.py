@@ -311,3 +311,18 @@ def test_decode_estimates_follow_the_present_kernels(Hq, Hkv, D, fp8, n, L, meas
                      v_scale=16 if fp8 else None)
     us, _, _ = cf.cf_estimate_us(d, [L] * n, [1] * n, 4096)
     assert abs(us / measured - 1.0) < 0.25, us
+
+
+def test_padded_length_arrays_are_accepted_and_short_ones_refused():
+    """The number of sequences is context_len's; the other arrays may be longer (the call itself is refused here for its null
+    context) but not shorter."""
+    d = cf.make_desc(32, 8, 128, 16, 64)
+    calls = [lambda lq: cf.cf_kv_append(None, d, 0, 0, 0, 0, 0, 4, [5, 7], lq, check=False),
+             lambda lq: cf.cf_mixed_attention(None, d, 0, 0, 0, 0, 4, [5, 7], lq, 0, check=False),
+             lambda lq: cf.cf_mixed_attention_shared(None, d, 0, 0, 0, 0, 4, [5, 7], lq, lq, lq, 0, check=False),
+             lambda lq: cf.cf_mixed_step_host(None, d, 0, 0, 0, 0, 0, 0, 4, [5, 7], lq, 0, check=False)]
+    for call in calls:
+        for lq in ([1, 1], [1, 1, 0, 0], np.array([1, 1, 9], np.int32), np.array([1, 1, 9], np.int64)):
+            assert call(lq) == cf.CF_ERR_INVALID_ARG
+        with pytest.raises(ValueError):
+            call([1])
