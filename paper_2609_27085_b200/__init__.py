@@ -16,13 +16,14 @@ from __future__ import annotations
 import ctypes
 import importlib.util
 import os
+import sysconfig
 from typing import Optional, Tuple
 
 import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libcrossflow_attn.so")
-MARSHAL_PATH = os.path.join(_HERE, "_marshal.so")
+MARSHAL_PATH = os.path.join(_HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))      # of this interpreter's ABI
 
 CF_OK = 0
 CF_ERR_INVALID_ARG = 1
@@ -87,7 +88,7 @@ def load_library() -> ctypes.CDLL:
         return _lib
     for path in (LIB_PATH, MARSHAL_PATH):
         if not os.path.exists(path):
-            raise ImportError(f"{path} is missing: build it with `python -m paper_2609_27085_b200.build`")
+            raise ImportError(f"{path} is missing: build it with `python -m paper_2609_27085_b200.build` (this interpreter)")
     lib = ctypes.CDLL(LIB_PATH)
     vp, i32, i32p, fp = ctypes.c_void_p, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_float)
     dp = ctypes.POINTER(CacheDesc)

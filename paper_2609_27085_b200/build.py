@@ -1,5 +1,5 @@
-"""Builds libcrossflow_attn.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _marshal.so (the CPython
-extension that marshals the arguments of the hot entry points) with g++.
+"""Builds libcrossflow_attn.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _marshal.<abi>.so (the CPython
+extension that marshals the arguments of the hot entry points) with g++ and the running interpreter's headers.
 
     python -m paper_2609_27085_b200.build [--force] [--verbose]
 
@@ -17,7 +17,9 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcrossflow_attn.so")
-MARSHAL = os.path.join(HERE, "_marshal.so")      # CPython extension: argument marshalling of the hot entry points
+# CPython extension: argument marshalling of the hot entry points.  The name carries the interpreter's ABI tag, so that another
+# interpreter misses the file instead of loading it; building it takes that interpreter's headers.
+MARSHAL = os.path.join(HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["api.cu", "plan.cpp", "kv_append.cu", "decode_splitk.cu", "prefill_tc.cu", "prefill_tc2.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]

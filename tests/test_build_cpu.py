@@ -3,6 +3,12 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
+
+import pytest
+
+import paper_2609_27085_b200 as cf
+from paper_2609_27085_b200 import build as cf_build
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 PKG = "paper_2609_27085_b200"
@@ -38,3 +44,14 @@ def test_the_allocation_free_call_keeps_to_its_stack(tmp_path):
         frames[name] = int(size)
     sizes = sorted(frames.values())                                   # the entry point's frame is the largest by far
     assert 112 * 1024 < sizes[-1] <= 126 * 1024 and sizes[-2] <= 4096, sizes[-3:]
+
+
+def test_the_marshalling_extension_is_the_interpreters_own(monkeypatch):
+    """Its name carries the ABI tag; an interpreter that it was not built for finds no file and says so."""
+    assert cf_build.MARSHAL == cf.MARSHAL_PATH and cf.MARSHAL_PATH.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    cf_build.build()
+    assert os.path.exists(cf.MARSHAL_PATH)
+    monkeypatch.setattr(cf, "_lib", None)
+    monkeypatch.setattr(cf, "MARSHAL_PATH", cf.MARSHAL_PATH.replace("cpython-", "cpython-9"))
+    with pytest.raises(ImportError, match="is missing"):
+        cf.load_library()
