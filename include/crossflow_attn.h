@@ -324,9 +324,10 @@ cf_status cf_estimate_us(const cf_cache_desc* desc, const int32_t* context_len, 
  *   decode_items  : int32 [cap, 6] = {seq, q_row, kv_begin, kv_end, partial_slot (-1 = writes out directly), chunk_index}
  *   combine_items : int32 [cap, 3] = {q_row, first_partial_slot, num_chunks}
  *   prefill_items : int32 [cap, 8] = {seq, q_row_of_tile, first_row_in_chunk, num_rows, query_head, kv_head,
- *                   first_kv_tile, end_kv_tile}, one entry per (q tile, query head, KV range) in launch
- *                   order; KV tiles are 128 tokens, end_kv_tile is clamped to the tile's own extent; an item
- *                   that is not KV-split has one entry covering all of its tiles
+ *                   first_kv_tile, end_kv_tile}, one entry per (run of rows, query head, KV range) in launch
+ *                   order: the tiles of the work items that carry consecutive rows of one 128-row block over the same
+ *                   range are one run.  KV tiles are 128 tokens, end_kv_tile is clamped to the rows' own extent; rows
+ *                   that are not KV-split have one entry covering all of their tiles
  *   counts        : int32 [6]      = {n_decode_items, n_combine_items, n_prefill_entries, n_partial_slots,
  *                                     n_prefill_work_items (KV ranges of split items counted; an item occupies one
  *                                     SM, or a pair of SMs where pairs are used and then carries four heads),

@@ -1432,33 +1432,10 @@ cf_status cf_plan_inspect(const cf_cache_desc* desc, const int32_t* context_len,
             int32_t* o = combine_items + 3 * i;
             o[0] = pl.combine[i].q_row; o[1] = pl.combine[i].part_first; o[2] = pl.combine[i].n_chunks;
         }
-    size_t n_pre = 0;
-    auto entry = [&](const PrefillTcItem& it, int32_t q_row, int32_t row0, int32_t n_rows, int32_t head) {
-        if (prefill_items && n_pre < (size_t)cap) {
-            const int32_t tiles = (it.prefix + row0 + n_rows + 127) / 128;      // KV tiles these rows can see
-            int32_t* o = prefill_items + 8 * n_pre;
-            o[0] = it.seq; o[1] = q_row; o[2] = row0; o[3] = n_rows; o[4] = head; o[5] = it.kvh;
-            o[6] = it.j_begin < tiles ? it.j_begin : tiles;
-            o[7] = it.j_end < tiles ? it.j_end : tiles;
-        }
-        ++n_pre;
-    };
-    const int32_t G = desc->num_q_heads / desc->num_kv_heads;
-    for (const PrefillTcItem& it : pl.prefill_tc) {
-        if (!pl.pair && G >= 2) {
-            // the items of a 128-row block and KV head carry all heads of the group and share their KV range: the
-            // block's entries are listed with its first item
-            if (it.row0[0] % 128 != 0) continue;
-            const int32_t rest = query_len[it.seq] - it.row0[0], n_rows = rest < 128 ? rest : 128;
-            for (int32_t h = 0; h < G; ++h) entry(it, it.q_row0[0], it.row0[0], n_rows, it.kvh * G + h);
-            continue;
-        }
-        for (int t = 0; t < 2; ++t) {
-            if (it.n_rows[t] <= 0) continue;
-            entry(it, it.q_row0[t], it.row0[t], it.n_rows[t], it.head[t]);
-            if (pl.pair) entry(it, it.q_row0[t], it.row0[t], it.n_rows[t], it.head[t] + 2);      // the second CTA of the pair: head + 2
-        }
-    }
+    static_assert(sizeof(PrefillEntry) == 8 * sizeof(int32_t), "copied out as rows of eight");
+    const std::vector<PrefillEntry> entries = list_prefill(desc, pl);
+    const size_t n_pre = entries.size();
+    if (prefill_items && n_pre) std::memcpy(prefill_items, entries.data(), sizeof(PrefillEntry) * std::min(n_pre, (size_t)cap));
     if (counts) {
         counts[0] = (int32_t)pl.decode.size();
         counts[1] = (int32_t)pl.combine.size();

@@ -1,9 +1,11 @@
 #include "plan.h"
 
 #include <algorithm>
+#include <array>
 #include <climits>
 #include <cmath>
 #include <functional>
+#include <map>
 #include <queue>
 #include <utility>
 #include <cstdint>
@@ -568,6 +570,48 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         }
     }
     return CF_OK;
+}
+
+std::vector<PrefillEntry> list_prefill(const cf_cache_desc* d, const Plan& plan)
+{
+    const int32_t G = d->num_q_heads / d->num_kv_heads;
+    const bool packed = !plan.pair && G >= 2;
+    struct Run { PrefillEntry e; int32_t prefix; };
+    std::vector<Run> runs;
+    std::map<std::array<int32_t, 6>, size_t> open;         // (sequence, KV head, head, block, KV range) -> its last run
+    for (const PrefillTcItem& it : plan.prefill_tc)
+        for (int t = 0; t < 2; ++t) {
+            if (it.n_rows[t] <= 0) continue;
+            const Run tile{{it.seq, it.q_row0[t], it.row0[t], it.n_rows[t], it.head[t], it.kvh, it.j_begin, it.j_end}, it.prefix};
+            if (packed) {
+                const auto key = std::array<int32_t, 6>{it.seq, it.kvh, it.head[t], it.row0[t] / 128, it.j_begin, it.j_end};
+                const auto at = open.find(key);
+                if (at != open.end()) {
+                    PrefillEntry& e = runs[at->second].e;
+                    if (e.row0 + e.n_rows == tile.e.row0 && e.q_row + e.n_rows == tile.e.q_row) {
+                        e.n_rows += tile.e.n_rows;
+                        continue;
+                    }
+                }
+                open[key] = runs.size();
+            }
+            runs.push_back(tile);
+            if (plan.pair) {                               // the second CTA of the pair: head + 2
+                runs.push_back(tile);
+                runs.back().e.head += 2;
+            }
+        }
+    std::vector<PrefillEntry> out;
+    for (const Run& r : runs)
+        for (int32_t h = 0; h < (packed ? G : 1); ++h) {
+            PrefillEntry e = r.e;
+            e.head += h;
+            const int32_t tiles = (r.prefix + e.row0 + e.n_rows + 127) / 128;      // KV tiles these rows can see
+            e.j_begin = std::min(e.j_begin, tiles);
+            e.j_end = std::min(e.j_end, tiles);
+            out.push_back(e);
+        }
+    return out;
 }
 
 void join_plans(const cf_cache_desc* d, const std::vector<const Plan*>& parts, const std::vector<int32_t>& seqs,

@@ -260,6 +260,14 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
                      int32_t num_seqs, int32_t max_blocks_per_seq, const PlanConfig& cfg, Plan* plan,
                      const int32_t* share_group = nullptr, const int32_t* shared_len = nullptr);
 
+// The prefill items of a plan for inspection, in launch order: one entry per (rows of a 128-row block, query head, KV range).
+// Tiles of packed items that carry consecutive rows of one block over the same KV range are listed as one run of rows; what
+// does not fit together - a missing tile, another row, another range - shows as runs of their own.
+struct PrefillEntry {
+    int32_t seq, q_row, row0, n_rows, head, kvh, j_begin, j_end;
+};
+std::vector<PrefillEntry> list_prefill(const cf_cache_desc* d, const Plan& plan);
+
 // The plans of consecutive parts of one batch (part i: sequences from seqs[i] on, packed rows from rows[i] on) as one plan of
 // the batch: the same items, chunks and KV ranges, so every row has the bits that its part gives it, queued as build_plan
 // queues them.

@@ -3,6 +3,7 @@ arguments on the host before touching a device, and its planner covers every tok
 import ctypes
 import os
 import re
+import subprocess
 
 import numpy as np
 import pytest
@@ -326,3 +327,59 @@ def test_padded_length_arrays_are_accepted_and_short_ones_refused():
             assert call(lq) == cf.CF_ERR_INVALID_ARG
         with pytest.raises(ValueError):
             call([1])
+
+
+LISTING = r"""
+#include <cstdio>
+#include <cstring>
+#include "plan.h"
+using namespace cf;
+static bool same(const std::vector<PrefillEntry>& a, const std::vector<PrefillEntry>& b)
+{
+    return a.size() == b.size() && (a.empty() || !std::memcmp(a.data(), b.data(), a.size() * sizeof a[0]));
+}
+int main()
+{
+    long changed = 0, unseen = 0;
+    const int geo[][3] = {{32, 8, 128}, {64, 8, 128}, {16, 8, 64}, {4, 4, 128}};
+    for (auto& g : geo)
+        for (int split : {1, 0, 3})
+            for (int window : {0, 300}) {
+                cf_cache_desc d = {};
+                d.num_q_heads = g[0]; d.num_kv_heads = g[1]; d.head_dim = g[2]; d.block_size = 16; d.num_blocks = 1 << 20; d.window_size = window;
+                const int lc[] = {3100 + 700, 129, 40 + 33, 900}, lq[] = {700, 129, 33, 1};
+                PlanConfig cfg;
+                cfg.prefill_force_split = split;
+                Plan plan;
+                if (build_plan(&d, lc, lq, 4, 1 << 16, cfg, &plan) != CF_OK) return 2;
+                const auto good = list_prefill(&d, plan);
+                for (size_t i = 0; i < plan.prefill_tc.size(); ++i)
+                    for (int what = 0; what < 7; ++what) {
+                        Plan bad = plan;
+                        PrefillTcItem& it = bad.prefill_tc[i];
+                        const int t = it.n_rows[1] > 0 ? 1 : 0;
+                        if (what == 0) bad.prefill_tc.erase(bad.prefill_tc.begin() + (long)i);
+                        if (what == 1) it.n_rows[t] -= 1;
+                        if (what == 2) { it.row0[t] += 1; it.q_row0[t] += 1; }
+                        if (what == 3) it.q_row0[t] += 1;
+                        if (what == 4) it.kvh = (it.kvh + 1) % d.num_kv_heads;
+                        if (what == 5) it.j_begin += 1;
+                        if (what == 6) it.j_end = it.j_begin;
+                        ++changed;
+                        unseen += same(good, list_prefill(&d, bad));
+                    }
+            }
+    std::printf("%ld %ld\n", changed, unseen);
+}
+"""
+
+
+def test_the_listing_of_prefill_items_shows_every_single_item(tmp_path):
+    """cf_plan_inspect's prefill entries are made from all work items: a plan with one item left out, or with one tile's rows,
+    output row, KV head or KV range changed, is listed differently (so the coverage checks above see it)."""
+    csrc = os.path.join(ROOT, "paper_2609_27085_b200", "csrc")
+    (tmp_path / "listing.cpp").write_text(LISTING)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-I", csrc, str(tmp_path / "listing.cpp"), os.path.join(csrc, "plan.cpp"), "-o",
+                    str(tmp_path / "listing")], check=True, timeout=300)
+    changed, unseen = map(int, subprocess.run([str(tmp_path / "listing")], check=True, capture_output=True, text=True, timeout=300).stdout.split())
+    assert changed > 3000 and unseen == 0
