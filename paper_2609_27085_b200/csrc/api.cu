@@ -58,7 +58,9 @@ struct QMapEntry {
     uint64_t stamp = 0;
     CUtensorMap map;
 };
-static constexpr int kPoolMaps = 32, kQMaps = 8;
+// q maps: a host-staged step has one base address per prefill part and staging set (with 8 entries the nine of three parts over three
+// sets were encoded anew in every step)
+static constexpr int kPoolMaps = 32, kQMaps = 8 + kHostStages * kHostParts;
 
 struct PlanSlot {
     uint8_t* host = nullptr;   // pinned
