@@ -91,7 +91,7 @@ def test_host_steps_in_parts(prefix, qlen, window):
 
 def test_host_steps_without_a_flush_in_between():
     """A step whose kernels outweigh its copies goes in parts when it comes first after a flush and in one piece when it
-    follows another: both against the oracle, three in flight."""
+    follows another: both against the oracle, three in flight, the same bits."""
     sc = small(74, 32, 8, 128, [40000, 3000], [[600, 1]], NB=3072)
     b = sc.batches[0]
     g = GpuScenario(sc)
@@ -109,7 +109,7 @@ def test_host_steps_without_a_flush_in_between():
     assert cf.cf_get_async_status(g.ctx) == cf.CF_OK
     for oh in outs:
         compare(oh.numpy().view(np.uint16), None, ref_o, None, rows=rows)
-    assert torch.equal(outs[1], outs[2])
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[1], outs[2])
     g.close()
 
 

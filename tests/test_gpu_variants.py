@@ -285,28 +285,25 @@ def test_two_share_groups_and_a_short_prefix():
 
 
 def test_shared_prefix_with_many_chunks_and_the_separate_combine_kernel():
-    """A 40K-token shared prefix (many shared chunks per member) with short and long suffixes, merged by the fused
-    merge and by the separate combine kernel: identical bits."""
+    """A 40K-token shared prefix (many shared chunks per member) with short and long suffixes.  Shared batches are merged by the
+    combine kernel; without the description the same batch is merged inside the decode kernel: both against the oracle."""
     geom = syn.Geometry(32, 8, 128, 16, 8192)
     sc, sg, sl = syn.shared_prefix_scenario("long-shared", geom, 75, 40000 // 16 * 16, [0, 15, 3000, 9000, 17, 600], [1] * 6, [0] * 6)
     b = sc.batches[0]
-    outs = []
-    for debug in (None, {cf.CF_DEBUG_SEPARATE_COMBINE: 1}):
-        g = GpuScenario(sc, debug=debug)
-        g.append(b)
-        bt = torch.from_numpy(b.block_table).cuda()
-        q = to_dev_bf16(b.q)
+    g = GpuScenario(sc)
+    g.append(b)
+    bt = torch.from_numpy(b.block_table).cuda()
+    q = to_dev_bf16(b.q)
+    k_ref, v_ref = g.pools_host()
+    ref_o, ref_lse = oracle.mixed_attention(b.q, k_ref, v_ref, b.block_table, b.context_len, b.query_len)
+    for share, launches in (((sg, sl), 2), ((np.full(6, -1, np.int32), np.zeros(6, np.int32)), 1)):
         out = torch.full_like(q, float("nan"))
         lse = torch.full((b.total_q, 32), float("nan"), dtype=torch.float32, device="cuda")
-        cf.cf_mixed_attention_shared(g.ctx, g.desc, q, g.k, g.v, bt, b.max_blocks, b.context_len, b.query_len, sg, sl, out, lse)
+        cf.cf_mixed_attention_shared(g.ctx, g.desc, q, g.k, g.v, bt, b.max_blocks, b.context_len, b.query_len, *share, out, lse)
         torch.cuda.synchronize()
-        assert cf.cf_get_last_plan_counts(g.ctx)[5] > 1
-        outs.append((to_host_bits(out), lse.cpu().numpy()))
-        k_ref, v_ref = g.pools_host()
-        g.close()
-    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
-    ref_o, ref_lse = oracle.mixed_attention(b.q, k_ref, v_ref, b.block_table, b.context_len, b.query_len)
-    compare(outs[0][0], outs[0][1], ref_o, ref_lse)
+        assert (cf.cf_get_last_plan_counts(g.ctx)[5] > 1) == (launches == 2) and cf.cf_get_last_launch_count(g.ctx) == launches
+        compare(to_host_bits(out), lse.cpu().numpy(), ref_o, ref_lse)
+    g.close()
 
 
 # ------------------------------------------------------------------ chunked prefill on pairs of SMs (opt-in kernel)
