@@ -44,11 +44,11 @@ WORKLOAD = ("configs[3] agentic long-context mixed batch: 16 decode seqs (ctx un
             "+ 1 prefill of 8192 new tokens over 24576 cached, 2048-token chunks; Hq 32, Hkv 8, D 128, block 16, bf16; "
             "one step = kv_append + mixed attention of one chunk iteration (t cycles 0..3)")
 # DRAM traffic per algorithmic byte of the split-K decode kernel, from an ncu capture on the reduced
-# decode case (dram bytes read + written: 560.9 MB for 555.2 MB algorithmic); traffic grows in
+# decode case (dram bytes read + written: 559.0 MB for 555.2 MB algorithmic); traffic grows in
 # proportion to the K/V bytes, so a full launch is scaled by its algorithmic bytes.
-DECODE_TRAFFIC_RATIO = 1.010
+DECODE_TRAFFIC_RATIO = 1.007
 # DRAM traffic per algorithmic byte of the tcgen05 prefill kernel, from an ncu capture of the headline's own prefill
-# launch in the serial sequence (first chunk iteration: 2048 new tokens over 24,576 cached; 162.5 MB moved for
+# launch in the serial sequence (first chunk iteration: 2048 new tokens over 24,576 cached; 162.1 MB moved for
 # 142.6 MB algorithmic: K/V once, q, out and the fp32 partial rows of the KV-split items).  A 4096-token chunk over
 # 8192 cached tokens measures 1.28.  Prefill is tensor-bound; the figure is scaled by the launch's algorithmic bytes
 # and is approximate for the later chunk iterations.
@@ -658,7 +658,7 @@ def small_case(name: str) -> syn.Scenario:
 def run_shared_prefix_case(args):
     """16 decode sequences (Hq 32, Hkv 8, D 128) that share an 8192-token prefix and have 200..900 tokens of their
     own: the same batch through cf_mixed_attention (every sequence streams the shared pages) and through
-    cf_mixed_attention_shared (the shared pages are streamed once per set of four sequences).  `--variant plain`
+    cf_mixed_attention_shared (the shared pages are streamed once for all sixteen).  `--variant plain`
     or `--variant shared` runs only that one (for a profiler capture)."""
     import torch
     import paper_2609_27085_b200 as cf

@@ -221,9 +221,8 @@ int32_t cf_spatial_share(const cf_cache_desc* desc, const int32_t* context_len, 
 
 /* Debug aid (synchronous): checks every block-table entry that cf_kv_append / cf_mixed_attention would
  * dereference for these lengths (entries [0, ceil(context_len/B)) of each row) against [0, num_blocks).
- * The kernels themselves trust the table - an entry outside the pool is an out-of-bounds access on the
- * device - so a serving engine runs this in its debug builds or after a scheduler change.  Reads the
- * table only.  Returns CF_OK, or CF_ERR_OUT_OF_RANGE with the number of bad entries in *num_bad. */
+ * The kernels check each entry as well and read page 0 in the place of one outside the pool; this call counts
+ * such entries ahead of time, for debug builds or after a scheduler change.  Reads the table only.  Returns CF_OK, or CF_ERR_OUT_OF_RANGE with the number of bad entries in *num_bad. */
 cf_status cf_validate_block_table(cf_ctx* ctx, const cf_cache_desc* desc, const int32_t* block_table,
                                   int32_t max_blocks_per_seq, const int32_t* context_len, const int32_t* query_len,
                                   int32_t num_seqs, void* cuda_stream, int32_t* num_bad);

@@ -215,7 +215,7 @@ static size_t layout_of(const Plan& pl, size_t n_stage_seqs, PlanRef* r)
 }
 static int32_t shared_units(const Plan& pl, const cf_cache_desc* d)
 {
-    const int32_t per_unit = std::max(1, 16 / (d->num_q_heads / d->num_kv_heads));       // members whose heads fill 16 columns
+    const int32_t per_unit = std::max(1, 16 / (d->num_q_heads / d->num_kv_heads));       // members whose heads fill the 16 columns of a warp
     int32_t n = 0;
     for (const SharedDecodeItem& it : pl.shared_decode) n += (it.n_members + per_unit - 1) / per_unit;
     return n;
@@ -962,8 +962,8 @@ namespace cf {
 // and each part is read back while the next one runs; decode, which has next to nothing to read back, comes last.
 // A part is a run of consecutive rows: whole sequences, or a chunk cut at a multiple of 128 rows (the rest of the
 // chunk sees the same cache: the whole step has been appended before).  Measured per step, in one piece -> in parts: chat mix
-// 480 -> 332 us, agentic mix 1164 -> 981 us, 512 rows beside 256 decodes on an fp8 cache 561 -> 421 us, 8192 rows beside 256
-// decodes 4.20 -> 3.93 ms.
+// 484 -> 331 us, agentic mix 1164 -> 975 us, 512 rows beside 256 decodes on an fp8 cache 561 -> 424 us, 8192 rows beside 256
+// decodes 4.20 -> 3.94 ms.
 struct HostPart {
     int32_t seq = 0, num_seqs = 0;               // sequences [seq, seq + num_seqs)
     int64_t row = 0, rows = 0;                   // packed rows
@@ -1134,8 +1134,8 @@ cf_status cf_mixed_step_host(cf_ctx* c, const cf_cache_desc* desc,
         }
         // A step that follows another without a flush in between has its read-back under the kernels of the next one anyway.
         // Where the kernels outweigh both directions of the link such steps are bound by them, and the parts' items run as one
-        // call, decode beside prefill (agentic, back to back: 994 -> 905 us per step); where the link weighs as much, parts
-        // still help.  The items are the parts' own, so a step's result does not depend on the steps before it.
+        // call, decode beside prefill (agentic, back to back, in parts 1006 us per step, as one call 914); where the link weighs as
+        // much, parts still help.  The items are the parts' own, so a step's result does not depend on the steps before it.
         if (!whole && kernel_bound && c->unflushed_steps > 0) {
             Unit u;
             if (join_units(c, desc, parts, units, context_len, query_len, num_seqs, max_blocks_per_seq, &u)) {

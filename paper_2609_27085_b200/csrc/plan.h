@@ -131,13 +131,13 @@ cf_status validate_lengths(const cf_cache_desc* d, const int32_t* context_len, c
 //     fit the budget: cfg.part_bytes, and the limits of the allocation-free entry point, which plans with this routine (no
 //     split needs none).
 //   decode_split: near-equal chunks of at most `target` pages, each a multiple of the page quantum.
-// The prediction, in microseconds, was fitted to 800 (batch, chunk length) pairs: 90 batches of 2 to 256 sequences on all
-// geometries, measured on a B200.  Streaming at full bandwidth (B) and one CTA's way through the longest chunk (g per page)
+// The prediction, in microseconds, was fitted to 800 (batch, chunk length) pairs: batches of 2 to 256 sequences of 100 to 20,000
+// tokens on all geometries, measured on a B200.  Streaming at full bandwidth (B) and one CTA's way through the longest chunk (g per page)
 // add up in the 1.7-norm, 2.5 for a split (partials, ticket, merge; fp8 cache: 3.2), 1.2 for every further eight chunks of a
 // sequence (the merge takes eight at a time), 2.2 (fp8: 3.5) for every further wave.  Against chunks of at least 32 pages
 // in four waves, decode kernel alone: 40 sequences of 400 tokens, 64 over 8 heads 18.2 -> 14.2 us; 100 of 600 tokens 54 -> 47 us,
 // with head_dim 64 31 -> 23 us; 16 of 600 tokens (head_dim 64) 9.3 -> 7.8 us; 64 of 1500 tokens on an fp8 cache 54 -> 47 us;
-// 64 of 4000 tokens, which four waves fitted, 167 -> 168 us; the 90 shapes 1.06 in the mean.
+// 64 of 4000 tokens, which four waves fitted, 167 -> 168 us; all of them 1.06 in the mean.
 constexpr int64_t kStaticPartBytes = (16ll << 20) - (128ll << 10);      // partials of the allocation-free entry point
 constexpr int32_t kStaticMaxItems = 3584;                              // and its chunks
 constexpr int32_t kTargetSeqs = 2048;               // larger batches: whole sequences are chunks enough

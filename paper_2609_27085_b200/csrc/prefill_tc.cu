@@ -22,8 +22,8 @@
 // Tensor memory (512 columns): S_0 | S_1 | O_0 | O_1, 128 fp32 columns each; P_t (bf16) overwrites
 // the first 64 columns of S_t and is consumed by the PV product straight from tensor memory.
 // Softmax: scores leave tensor memory once (tcgen05.ld), exp2 with the scale folded in, the
-// running maximum is only raised when it grows by more than 2^8 (then O_t is rescaled in tensor
-// memory), so almost every tile costs no correction pass.  The causal comparison j <= P + i is
+// reference maximum is only raised when a tile's scores outgrow it (by 2^15, or a row sum above that; then O_t is rescaled in
+// tensor memory), so almost every tile costs no correction pass.  The causal comparison j <= P + i is
 // evaluated only in warps whose rows can see a masked key of the tile; tiles above the diagonal
 // are never loaded.
 // Every wait is bounded: on expiry the CTA raises an abort flag, every role leaves its loop, the
@@ -627,7 +627,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             // Optimistic pass: exponentials against the current reference maximum, packed two per
             // FMA-pipe instruction.  Whether the reference has to be raised is read off the tile's row
-            // sum (a probability above 2^8 makes it exceed 2^15 long before anything can overflow); only
+            // sum of the first chunks and the largest score of the last (2^15 is far below what can overflow); only
             // then is the exact maximum taken, O_t rescaled in tensor memory and the pass repeated.
             float2 acc2[4];
             auto exp_pass = [&](auto EDGE, auto C0, auto C1, const float neg_m) {
