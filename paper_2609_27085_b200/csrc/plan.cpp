@@ -5,8 +5,8 @@
 #include <climits>
 #include <cmath>
 #include <functional>
-#include <map>
 #include <queue>
+#include <unordered_map>
 #include <utility>
 #include <cstdint>
 
@@ -578,13 +578,24 @@ std::vector<PrefillEntry> list_prefill(const cf_cache_desc* d, const Plan& plan)
     const bool packed = !plan.pair && G >= 2;
     struct Run { PrefillEntry e; int32_t prefix; };
     std::vector<Run> runs;
-    std::map<std::array<int32_t, 6>, size_t> open;         // (sequence, KV head, head, block, KV range) -> its last run
+    using Key = std::array<int32_t, 6>;                    // sequence, KV head, head, block, KV range
+    struct Hash {
+        size_t operator()(const Key& k) const
+        {
+            size_t h = 0;
+            for (int32_t v : k) h = h * 1000003u + (uint32_t)v;
+            return h;
+        }
+    };
+    std::unordered_map<Key, size_t, Hash> open;            // its last run
+    runs.reserve(2 * plan.prefill_tc.size());
+    open.reserve(plan.prefill_tc.size());
     for (const PrefillTcItem& it : plan.prefill_tc)
         for (int t = 0; t < 2; ++t) {
             if (it.n_rows[t] <= 0) continue;
             const Run tile{{it.seq, it.q_row0[t], it.row0[t], it.n_rows[t], it.head[t], it.kvh, it.j_begin, it.j_end}, it.prefix};
             if (packed) {
-                const auto key = std::array<int32_t, 6>{it.seq, it.kvh, it.head[t], it.row0[t] / 128, it.j_begin, it.j_end};
+                const auto key = Key{it.seq, it.kvh, it.head[t], it.row0[t] / 128, it.j_begin, it.j_end};
                 const auto at = open.find(key);
                 if (at != open.end()) {
                     PrefillEntry& e = runs[at->second].e;
@@ -602,6 +613,7 @@ std::vector<PrefillEntry> list_prefill(const cf_cache_desc* d, const Plan& plan)
             }
         }
     std::vector<PrefillEntry> out;
+    out.reserve(runs.size() * (size_t)(packed ? G : 1));
     for (const Run& r : runs)
         for (int32_t h = 0; h < (packed ? G : 1); ++h) {
             PrefillEntry e = r.e;

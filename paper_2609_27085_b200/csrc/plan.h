@@ -178,18 +178,22 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
         }
         return c;
     }
-    // all chunks, and those of sequences with more than one: upper bounds (near-equal chunks are rounded up later, and the
-    // slack covers the reciprocal's rounding)
-    auto chunks = [&](int64_t c, int64_t* split = nullptr) -> int64_t {
+    // chunks of all sequences, and of those that have more than one: upper bounds (near-equal chunks are rounded up later, and
+    // the slack covers the reciprocal's rounding)
+    auto chunks = [&](int64_t c) -> int64_t {
         const float inv = 1.000001f / (float)c, up = (float)(c - 1);
-        int64_t sum = 0, parts = 0;
+        int32_t sum = 0;
+        for (int32_t i = 0; i < n; ++i) sum += (int32_t)((pages[i] + up) * inv + 1e-4f);
+        return sum > n ? sum : n;
+    };
+    auto parts = [&](int64_t c) -> int64_t {
+        const float inv = 1.000001f / (float)c, up = (float)(c - 1);
+        int32_t sum = 0;
         for (int32_t i = 0; i < n; ++i) {
             const int32_t k = (int32_t)((pages[i] + up) * inv + 1e-4f);
-            sum += k;
-            parts += k > 1 ? k : 0;
+            sum += k > 1 ? k : 0;
         }
-        if (split) *split = parts;
-        return sum > n ? sum : n;
+        return sum;
     };
     const double page_bytes = 2.0 * B * D * (fp8 ? 1.0 : 2.0), g = fp8 ? 0.15 : D == 64 ? 0.077 : 0.113;
     const double rate = (fp8 ? 6.3e6 : 7.6e6) * (double)sms / 148.0;
@@ -205,10 +209,9 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
     auto consider = [&](int64_t c) {
         c = round_up(c < lo ? lo : c);
         if (c > hi && c < longest) c = hi / quantum * quantum;
-        int64_t split = 0;
-        const int64_t all = chunks(c, &split);
+        const int64_t all = chunks(c);
         if (all > kStaticMaxItems && all > n) return;
-        if (split * slot_bytes + 256 > budget) return;
+        if (all * slot_bytes + 256 > budget && parts(c) * slot_bytes + 256 > budget) return;
         const int64_t ctas = all * Hkv, len = c < longest ? c : longest, of_longest = (longest + c - 1) / c;
         // further waves: a whole one for any remainder when the chunks are alike, the remainder's part of one when most
         // are shorter than the longest (they leave their slots early)
