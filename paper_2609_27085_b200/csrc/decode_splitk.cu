@@ -130,13 +130,129 @@ __device__ __forceinline__ void page_softmax(float (&s)[N], float (&m_run)[2], f
         }
 }
 
+// Copies of one (page, head) of K and of V into a ring slot (cp.async, 16 bytes per lane and instruction), laid out by
+// tile_off<16>.  Step s of the copy moves the rows [ROWS s, ROWS s + ROWS): a lane's row and chunk are constants, and since its
+// row inside a step takes the low bits of the row index, the swizzle of step s differs from that of step 0 by an XOR with a
+// constant.  A whole page of contiguous tokens - all but the edges, in the recommended layout - is 2 x STEPS copies with constant
+// offsets from a few lane registers.  Before, every copy computed its own 64-bit address and mask.
+template <int D, bool FP8>
+struct PageCopy {
+    static constexpr int ELEM = FP8 ? 1 : 2, CPR = D * ELEM / 16;       // 16-byte chunks of a token's row
+    static constexpr int ROWS = 32 / CPR, STEPS = 16 / ROWS, PATTERNS = 8 / ROWS;
+    static constexpr int PAGE_BYTES = 16 * D * ELEM;                    // one (page, head) of K or of V
+    uint32_t dst[PATTERNS];
+    int lane;
+    uint64_t policy;
+    __device__ __forceinline__ explicit PageCopy(int lane_) : lane(lane_), policy(l2_policy_evict_first())
+    {
+#pragma unroll
+        for (int i = 0; i < PATTERNS; ++i) dst[i] = tile_off<16>(i * ROWS + lane / CPR, lane % CPR) - i * ROWS * 128;
+    }
+    // k, v: the page's first token; tokens outside [lo, end) - slack slots, tokens left of a sliding window - are zero-filled
+    __device__ __forceinline__ void operator()(uint32_t slot, const uint8_t* k, const uint8_t* v, int64_t k_stride, int64_t v_stride, int tok0, int lo, int end) const
+    {
+        if (k_stride == D && v_stride == D && tok0 + 16 <= end && tok0 >= lo) {
+            const uint8_t *const ks = k + lane * 16, *const vs = v + lane * 16;
+#pragma unroll
+            for (int s = 0; s < STEPS; ++s) {
+                cp_async16_hint(slot + dst[s % PATTERNS] + s * ROWS * 128, ks + s * 512, 16, policy);
+                cp_async16_hint(slot + dst[s % PATTERNS] + PAGE_BYTES + s * ROWS * 128, vs + s * 512, 16, policy);
+            }
+        } else {
+            const int t0 = lane / CPR, ch = lane % CPR;
+#pragma unroll
+            for (int s = 0; s < STEPS; ++s) {
+                const int t = s * ROWS + t0;
+                const bool in = tok0 + t < end && tok0 + t >= lo;
+                const int tt = in ? t : 0;
+                const uint32_t to = slot + dst[s % PATTERNS] + s * ROWS * 128;
+                cp_async16_hint(to, k + (tt * k_stride * ELEM + ch * 16), in ? 16 : 0, policy);
+                cp_async16_hint(to + PAGE_BYTES, v + (tt * v_stride * ELEM + ch * 16), in ? 16 : 0, policy);
+            }
+        }
+    }
+};
+
+// A warp's ring of NSTAGE pages (K, V) and the fetching into it: one cp.async group per page, NSTAGE - 1 pages ahead.
+template <int D, bool FP8, int NWARPS, int NSTAGE>
+struct PageRing {
+    using Copy = PageCopy<D, FP8>;
+    static constexpr int HALF = Copy::PAGE_BYTES, STAGE_BYTES = 2 * HALF, WARP_BYTES = NSTAGE * STAGE_BYTES;
+    const AttnParams& p;
+    const DecodeItem& it;
+    const Copy copy;
+    const int32_t* const bt;                    // block ids of this warp's pages, NWARPS apart
+    const uint8_t *const k, *const v;
+    const uint32_t base;
+    const int n, tok, lane;                     // pages of this warp; first token of the first one
+    int cache_base = 0;
+    int32_t ids;
+    __device__ __forceinline__ PageRing(const AttnParams& p_, const DecodeItem& it_, int kvh, uint32_t base_, int n_, int warp, int lane_)
+        : p(p_), it(it_), copy(lane_),
+          bt(p_.block_table + (int64_t)it_.seq * p_.max_blocks + (it_.kv_begin >> 4) + warp),
+          k(reinterpret_cast<const uint8_t*>(p_.k_cache) + (int64_t)kvh * p_.ks_head * Copy::ELEM),
+          v(reinterpret_cast<const uint8_t*>(p_.v_cache) + (int64_t)kvh * p_.vs_head * Copy::ELEM),
+          base(base_), n(n_), tok(it_.kv_begin + warp * 16), lane(lane_)
+    {
+        ids = lane < n ? checked(__ldg(bt + lane * NWARPS)) : 0;
+    }
+    // A block id outside the pool is never dereferenced: page 0 is read in its place and the error word is set
+    // (the result of that sequence is then meaningless, but nothing faults).
+    __device__ __forceinline__ int32_t checked(int32_t id) const
+    {
+        if ((uint32_t)id < (uint32_t)p.num_blocks) return id;
+        if (p.err) atomicOr(p.err, kErrBlockId);
+        return 0;
+    }
+    __device__ __forceinline__ void fetch(int i)
+    {
+        if (i < n) {
+            if (i - cache_base == 32) {         // refill the per-lane block-id cache
+                cache_base = i;
+                ids = i + lane < n ? checked(__ldg(bt + (i + lane) * NWARPS)) : 0;
+            }
+            const int32_t page = __shfl_sync(0xffffffffu, ids, i - cache_base);
+            const uint32_t slot = base + (i % NSTAGE) * STAGE_BYTES;
+            copy(slot, k + (int64_t)page * p.ks_block * Copy::ELEM, v + (int64_t)page * p.vs_block * Copy::ELEM, p.ks_token, p.vs_token,
+                 tok + i * NWARPS * 16, it.kv_lo, it.kv_end);
+        }
+        cp_async_commit();
+    }
+    __device__ __forceinline__ void start()
+    {
+#pragma unroll
+        for (int s = 0; s < NSTAGE - 1; ++s) fetch(s);
+    }
+    // page i in place: K at the returned address, V behind it; a later page is on its way
+    __device__ __forceinline__ uint32_t page(int i)
+    {
+        cp_async_wait<NSTAGE - 2>();
+        __syncwarp();
+        fetch(i + NSTAGE - 1);
+        return base + (i % NSTAGE) * STAGE_BYTES;
+    }
+};
+
+// A lane's fragment addresses inside a (page, head): K rows for ldmatrix, V rows for ldmatrix.trans, by k-step or output tile mod 4
+// (the others are 2 KB further on), as constants in the same way.
+template <int D>
+struct PageLanes {
+    static constexpr int N = D / 16 < 4 ? D / 16 : 4;
+    uint32_t k[N], v[N];
+    __device__ __forceinline__ explicit PageLanes(int lane)
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            k[i] = tile_off<16>((lane & 7) + ((lane >> 3) & 1) * 8, 2 * i + (lane >> 4));
+            v[i] = tile_off<16>((lane & 7) + (lane >> 4) * 8, 2 * i + ((lane >> 3) & 1));
+        }
+    }
+};
+
 template <int D, int NWARPS, int NSTAGE>
 __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* plan, const int cta)
 {
-    constexpr int CPR = D / 8;                  // 16-byte chunks per token row
-    constexpr int PAGE_BYTES = 16 * D * 2;      // one (page, head) of K or of V
-    constexpr int STAGE_BYTES = 2 * PAGE_BYTES;
-    constexpr int WARP_BYTES = NSTAGE * STAGE_BYTES;
+    using Ring = PageRing<D, false, NWARPS, NSTAGE>;
     constexpr int KSTEPS = D / 16;
     constexpr int DP = D + 4;                   // padded row of the merge buffer (bank-conflict free)
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -160,46 +276,10 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
         }
     }
 
-    const int first_page = it.kv_begin >> 4;
     const int n_pages = (it.kv_end - it.kv_begin + 15) >> 4;
     const int my_n = n_pages > warp ? (n_pages - warp + NWARPS - 1) / NWARPS : 0;
-    const int32_t* bt = p.block_table + (int64_t)it.seq * p.max_blocks + first_page + warp;
-    const uint32_t wbase = smem_u32(smem) + warp * WARP_BYTES;
-    const __nv_bfloat16* kbase = p.k_cache + (int64_t)kvh * p.ks_head;
-    const __nv_bfloat16* vbase = p.v_cache + (int64_t)kvh * p.vs_head;
-
-    // A block id outside the pool is never dereferenced: page 0 is read in its place and the error word is set
-    // (the result of that sequence is then meaningless, but nothing faults).
-    auto checked = [&](int32_t id) -> int32_t {
-        if ((uint32_t)id < (uint32_t)p.num_blocks) return id;
-        if (p.err) atomicOr(p.err, kErrBlockId);
-        return 0;
-    };
-    int cache_base = 0;
-    int32_t pid_cache = (lane < my_n) ? checked(__ldg(bt + lane * NWARPS)) : 0;
-    const uint64_t stream_once = l2_policy_evict_first();
-
-    auto issue = [&](int i) {
-        if (i - cache_base == 32) {             // refill the per-lane page-id cache
-            cache_base = i;
-            pid_cache = (i + lane < my_n) ? checked(__ldg(bt + (i + lane) * NWARPS)) : 0;
-        }
-        const int32_t pid = __shfl_sync(0xffffffffu, pid_cache, i - cache_base);
-        const int tok0 = it.kv_begin + (i * NWARPS + warp) * 16;
-        const uint32_t sbase = wbase + (i % NSTAGE) * STAGE_BYTES;
-        const __nv_bfloat16* kp = kbase + (int64_t)pid * p.ks_block;
-        const __nv_bfloat16* vp = vbase + (int64_t)pid * p.vs_block;
-#pragma unroll
-        for (int r = 0; r < (16 * CPR) / 32; ++r) {
-            const int id = r * 32 + lane;
-            const int t = id / CPR, c = id % CPR;
-            // slack slots of the last page and tokens left of a sliding window are zero-filled
-            const bool ok = tok0 + t < it.kv_end && tok0 + t >= it.kv_lo;
-            const int tt = ok ? t : 0;
-            cp_async16_hint(sbase + tile_off<16>(t, c), kp + tt * p.ks_token + c * 8, ok ? 16 : 0, stream_once);
-            cp_async16_hint(sbase + PAGE_BYTES + tile_off<16>(t, c), vp + tt * p.vs_token + c * 8, ok ? 16 : 0, stream_once);
-        }
-    };
+    Ring ring(p, it, kvh, smem_u32(smem) + warp * Ring::WARP_BYTES, my_n, warp, lane);
+    const PageLanes<D> at(lane);
 
     float o[KSTEPS][4];
 #pragma unroll
@@ -207,30 +287,18 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
     float m_run[2] = {-INFINITY, -INFINITY};
     float l_run[2] = {0.f, 0.f};
 
-#pragma unroll
-    for (int s = 0; s < NSTAGE - 1; ++s) {
-        if (s < my_n) issue(s);
-        cp_async_commit();
-    }
-
+    ring.start();
     for (int i = 0; i < my_n; ++i) {
-        cp_async_wait<NSTAGE - 2>();
-        __syncwarp();
-        if (i + NSTAGE - 1 < my_n) issue(i + NSTAGE - 1);
-        cp_async_commit();
-
-        const uint32_t sK = wbase + (i % NSTAGE) * STAGE_BYTES;
-        const uint32_t sV = sK + PAGE_BYTES;
+        const uint32_t sK = ring.page(i), sV = sK + Ring::HALF;
         const int tok0 = it.kv_begin + (i * NWARPS + warp) * 16;
 
         // S^T = K Q^T ; two accumulators break the dependent MMA chain
         float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
         {
-            const int t = (lane & 7) + ((lane >> 3) & 1) * 8;
 #pragma unroll
             for (int ks = 0; ks < KSTEPS; ++ks) {
                 uint32_t a[4];
-                ldmatrix_x4(a, sK + tile_off<16>(t, 2 * ks + (lane >> 4)));
+                ldmatrix_x4(a, sK + at.k[ks & 3] + (ks >> 2) * 2048);
                 if (ks & 1) mma_bf16_16816(s1, a, qf[ks][0], qf[ks][1]);
                 else        mma_bf16_16816(s0, a, qf[ks][0], qf[ks][1]);
             }
@@ -251,11 +319,10 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
         const uint32_t pb0 = movmatrix_trans(pack_bf16(s[0], s[1]));
         const uint32_t pb1 = movmatrix_trans(pack_bf16(s[2], s[3]));
         {
-            const int t = (lane & 7) + (lane >> 4) * 8;
 #pragma unroll
             for (int mt = 0; mt < KSTEPS; ++mt) {
                 uint32_t a[4];
-                ldmatrix_x4_trans(a, sV + tile_off<16>(t, 2 * mt + ((lane >> 3) & 1)));
+                ldmatrix_x4_trans(a, sV + at.v[mt & 3] + (mt >> 2) * 2048);
                 mma_bf16_16816(o[mt], a, pb0, pb1);
             }
         }
@@ -355,11 +422,10 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
 //   O^T = V^T P^T: output row i of MMA mt is head-dim element d = 16 (i % 8) + 2 mt + (i / 8), so thread (g, c) owns
 //     d in [16 g, 16 g + 16) and reads one 16-byte chunk per token for all 8 MMAs; byte pairs of two tokens are
 //     brought together with one byte-permute.
-__device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t two_codes)
+// four codes -> two pairs (the halves of the word are named, so that no instruction is needed to move the upper one down)
+__device__ __forceinline__ void e4m3x4_to_f16x4(uint32_t codes, uint32_t& lo, uint32_t& hi)
 {
-    uint32_t d;
-    asm("{\n.reg .b16 lo;\ncvt.u16.u32 lo, %1;\ncvt.rn.f16x2.e4m3x2 %0, lo;\n}" : "=r"(d) : "r"(two_codes));
-    return d;
+    asm("{\n.reg .b16 l, h;\nmov.b32 {l, h}, %2;\ncvt.rn.f16x2.e4m3x2 %0, l;\ncvt.rn.f16x2.e4m3x2 %1, h;\n}" : "=r"(lo), "=r"(hi) : "r"(codes));
 }
 __device__ __forceinline__ void mma_f16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
@@ -383,9 +449,7 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const
 {
     const uint8_t* const plan = INL > 0 ? inl.bytes : p.plan.base;
     constexpr int D = 128;
-    constexpr int PAGE_BYTES = 16 * D;          // one (page, head) of K or of V: 16 tokens x 128 one-byte codes
-    constexpr int STAGE_BYTES = 2 * PAGE_BYTES;
-    constexpr int WARP_BYTES = NSTAGE * STAGE_BYTES;
+    using Ring = PageRing<D, true, NWARPS, NSTAGE>;
     constexpr int KSTEPS = D / 16;
     constexpr int DP = D + 4;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -412,45 +476,9 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const
         }
     }
 
-    const int first_page = it.kv_begin >> 4;
     const int n_pages = (it.kv_end - it.kv_begin + 15) >> 4;
     const int my_n = n_pages > warp ? (n_pages - warp + NWARPS - 1) / NWARPS : 0;
-    const int32_t* bt = p.block_table + (int64_t)it.seq * p.max_blocks + first_page + warp;
-    const uint32_t wbase = smem_u32(smem) + warp * WARP_BYTES;
-    const uint8_t* kbase = reinterpret_cast<const uint8_t*>(p.k_cache) + (int64_t)kvh * p.ks_head;
-    const uint8_t* vbase = reinterpret_cast<const uint8_t*>(p.v_cache) + (int64_t)kvh * p.vs_head;
-
-    auto checked = [&](int32_t id) -> int32_t {
-        if ((uint32_t)id < (uint32_t)p.num_blocks) return id;
-        if (p.err) atomicOr(p.err, kErrBlockId);
-        return 0;
-    };
-    int cache_base = 0;
-    int32_t pid_cache = (lane < my_n) ? checked(__ldg(bt + lane * NWARPS)) : 0;
-    const uint64_t stream_once = l2_policy_evict_first();
-
-    // a page in shared memory: [16 tokens][128 bytes], the eight 16-byte chunks of a row XOR-swizzled by the row index
-    auto issue = [&](int i) {
-        if (i - cache_base == 32) {
-            cache_base = i;
-            pid_cache = (i + lane < my_n) ? checked(__ldg(bt + (i + lane) * NWARPS)) : 0;
-        }
-        const int32_t pid = __shfl_sync(0xffffffffu, pid_cache, i - cache_base);
-        const int tok0 = it.kv_begin + (i * NWARPS + warp) * 16;
-        const uint32_t sbase = wbase + (i % NSTAGE) * STAGE_BYTES;
-        const uint8_t* kp = kbase + (int64_t)pid * p.ks_block;
-        const uint8_t* vp = vbase + (int64_t)pid * p.vs_block;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int id = r * 32 + lane;
-            const int t = id >> 3, ch = id & 7;
-            const bool ok = tok0 + t < it.kv_end && tok0 + t >= it.kv_lo;     // slack slots and tokens left of a window: zero-filled
-            const int tt = ok ? t : 0;
-            const uint32_t off = (uint32_t)(t * 128 + ((ch ^ (t & 7)) << 4));
-            cp_async16_hint(sbase + off, kp + tt * p.ks_token + ch * 16, ok ? 16 : 0, stream_once);
-            cp_async16_hint(sbase + PAGE_BYTES + off, vp + tt * p.vs_token + ch * 16, ok ? 16 : 0, stream_once);
-        }
-    };
+    Ring ring(p, it, kvh, smem_u32(smem) + warp * Ring::WARP_BYTES, my_n, warp, lane);
 
     float o[KSTEPS][4];
 #pragma unroll
@@ -458,20 +486,9 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const
     float m_run[2] = {-INFINITY, -INFINITY};
     float l_run[2] = {0.f, 0.f};
 
-#pragma unroll
-    for (int s = 0; s < NSTAGE - 1; ++s) {
-        if (s < my_n) issue(s);
-        cp_async_commit();
-    }
-
+    ring.start();
     for (int i = 0; i < my_n; ++i) {
-        cp_async_wait<NSTAGE - 2>();
-        __syncwarp();
-        if (i + NSTAGE - 1 < my_n) issue(i + NSTAGE - 1);
-        cp_async_commit();
-
-        const uint32_t sK = wbase + (i % NSTAGE) * STAGE_BYTES;
-        const uint32_t sV = sK + PAGE_BYTES;
+        const uint32_t sK = ring.page(i), sV = sK + Ring::HALF;
         const int tok0 = it.kv_begin + (i * NWARPS + warp) * 16;
 
         // S^T = K Q^T
@@ -485,14 +502,13 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const
                 const uint32_t addr = sK + row * 128 + (((2 * m + (c >> 1)) ^ (row & 7)) << 4) + 8 * (c & 1);
                 asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(lo[rh]), "=r"(hi[rh]) : "r"(addr));
             }
-            {
-                const uint32_t a[4] = {e4m3x2_to_f16x2(lo[0]), e4m3x2_to_f16x2(lo[1]), e4m3x2_to_f16x2(lo[0] >> 16), e4m3x2_to_f16x2(lo[1] >> 16)};
-                mma_f16_16816(s0, a, qf[2 * m][0], qf[2 * m][1]);
-            }
-            {
-                const uint32_t a[4] = {e4m3x2_to_f16x2(hi[0]), e4m3x2_to_f16x2(hi[1]), e4m3x2_to_f16x2(hi[0] >> 16), e4m3x2_to_f16x2(hi[1] >> 16)};
-                mma_f16_16816(s1, a, qf[2 * m + 1][0], qf[2 * m + 1][1]);
-            }
+            uint32_t a[4];
+            e4m3x4_to_f16x4(lo[0], a[0], a[2]);
+            e4m3x4_to_f16x4(lo[1], a[1], a[3]);
+            mma_f16_16816(s0, a, qf[2 * m][0], qf[2 * m][1]);
+            e4m3x4_to_f16x4(hi[0], a[0], a[2]);
+            e4m3x4_to_f16x4(hi[1], a[1], a[3]);
+            mma_f16_16816(s1, a, qf[2 * m + 1][0], qf[2 * m + 1][1]);
         }
         float s[4];
         const int tA = tok0 + g;
@@ -522,7 +538,9 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const
             const int w = mt >> 1;
             const uint32_t sel = (mt & 1) ? 0x7362u : 0x5140u;
             const uint32_t pa = __byte_perm(vw[0][w], vw[1][w], sel), pc = __byte_perm(vw[2][w], vw[3][w], sel);
-            const uint32_t a[4] = {e4m3x2_to_f16x2(pa), e4m3x2_to_f16x2(pa >> 16), e4m3x2_to_f16x2(pc), e4m3x2_to_f16x2(pc >> 16)};
+            uint32_t a[4];
+            e4m3x4_to_f16x4(pa, a[0], a[1]);
+            e4m3x4_to_f16x4(pc, a[2], a[3]);
             mma_f16_16816(o[mt], a, pb0, pb1);
         }
     }
@@ -875,22 +893,15 @@ __global__ void __launch_bounds__(D / 4) combine_kernel(const AttnParams p, cons
 
 // ---------------------------------------------------------------------------------------------
 static constexpr int kDecWarps = 4;
+// Pages in a warp's ring: 96 KB per CTA and two CTAs on an SM; with head_dim 64 or an fp8 cache, whose pages are half the size, 64 KB and
+// three CTAs.
 static constexpr int kDecStages = 3;
-#ifndef CF_FP8_STAGES
-#define CF_FP8_STAGES 4
-#endif
-static constexpr int kDecStagesFp8 = CF_FP8_STAGES;   // pages of an fp8 cache are half the size: the ring can be deeper in the same shared memory
+template <int D, bool FP8> constexpr int dec_stages() { return D == 64 || FP8 ? 4 : kDecStages; }
 
-#ifndef CF_D64_STAGES
-#define CF_D64_STAGES 4
-#endif
-// head_dim 64: a (page, head) is 2 KB, so four stages per warp fit in 64 KB per CTA and three CTAs on an SM (+3.5 %)
-template <int D> constexpr int dec_stages() { return D == 64 ? CF_D64_STAGES : kDecStages; }
-
-template <int D>
+template <int D, bool FP8>
 static size_t decode_smem_bytes()
 {
-    const size_t ring = (size_t)kDecWarps * dec_stages<D>() * 2 * 16 * D * 2;
+    const size_t ring = (size_t)kDecWarps * PageRing<D, FP8, kDecWarps, dec_stages<D, FP8>()>::WARP_BYTES;
     const size_t merge = (size_t)kDecWarps * 8 * (D + 4) * 4 + (size_t)kDecWarps * 8 * 4 * 2;
     return ring > merge ? ring : merge;
 }
@@ -947,19 +958,17 @@ template <int D>
 static cudaError_t launch_decode_t(const AttnParams& p, const HostPlan& hp, int n_items, cudaStream_t stream)
 {
     return with_plan_bytes(hp, [&](auto size, const auto* inl) {
-        return launch_decode_grid<decode_splitk_kernel<D, kDecWarps, dec_stages<D>(), decltype(size)::value>>(
-            n_items * p.Hkv, decode_smem_bytes<D>(), stream, p, inl);
+        return launch_decode_grid<decode_splitk_kernel<D, kDecWarps, dec_stages<D, false>(), decltype(size)::value>>(
+            n_items * p.Hkv, decode_smem_bytes<D, false>(), stream, p, inl);
     });
 }
 
 cudaError_t launch_decode_fp8(const AttnParams& p, const HostPlan& hp, int n_items, cudaStream_t stream)
 {
     if (n_items <= 0) return cudaSuccess;
-    const size_t ring = (size_t)kDecWarps * kDecStagesFp8 * 2 * 16 * 128;
-    const size_t merge = (size_t)kDecWarps * 8 * (128 + 4) * 4 + (size_t)kDecWarps * 8 * 4 * 2;
     return with_plan_bytes(hp, [&](auto size, const auto* inl) {
-        return launch_decode_grid<decode_splitk_fp8_kernel<kDecWarps, kDecStagesFp8, decltype(size)::value>>(
-            n_items * p.Hkv, std::max(ring, merge), stream, p, inl);
+        return launch_decode_grid<decode_splitk_fp8_kernel<kDecWarps, dec_stages<128, true>(), decltype(size)::value>>(
+            n_items * p.Hkv, decode_smem_bytes<128, true>(), stream, p, inl);
     });
 }
 

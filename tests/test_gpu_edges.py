@@ -127,6 +127,18 @@ def test_decode_chunk_lengths(Hq, Hkv, D, fp8, lens):
     run_and_check(small(79, Hq, Hkv, D, [l - 1 for l in lens], [[1] * len(lens)], NB=4096), fp8=scales)
 
 
+@pytest.mark.parametrize("Hq,Hkv,D,fp8,layout", [(16, 2, 64, False, "HND"), (8, 2, 128, False, "HND"), (16, 2, 128, True, "HND"),
+                                                 (16, 2, 64, False, "NHD"), (8, 2, 128, False, "NHD")])
+@pytest.mark.parametrize("window", [0, 83])
+def test_decode_rings_of_every_depth(Hq, Hkv, D, fp8, layout, window):
+    """A decode warp's ring holds three or four pages; whole pages of contiguous tokens are copied
+    with constant offsets, the others token by token: every number of pages per warp around the ring's depth, past the 32 block
+    ids that a warp keeps, whole and cut last pages, a window's edge inside a page, both pool layouts."""
+    lens = [max(1, 16 * pages + extra) for pages in (0, 1, 2, 3, 4, 7, 8, 12, 13, 16, 19, 20, 24, 127, 130, 261) for extra in (0, 1, 15)]
+    scales = (np.full(Hkv, 0.02, np.float32), np.full(Hkv, 0.015, np.float32)) if fp8 else None
+    run_and_check(small(83, Hq, Hkv, D, [l - 1 for l in lens], [[1] * len(lens)], NB=4096), fp8=scales, layout=layout, window=window)
+
+
 @pytest.mark.parametrize("Hq,Hkv,D,members", [(2, 2, 128, 40), (8, 2, 128, 4), (8, 2, 128, 5), (8, 2, 128, 9), (8, 2, 128, 17),
                                               (16, 2, 64, 2), (16, 2, 64, 3), (16, 2, 64, 9), (4, 2, 128, 22), (4, 2, 64, 33)])
 @pytest.mark.parametrize("pages", [16, 33, 129])
