@@ -134,8 +134,11 @@ __device__ __forceinline__ void page_softmax(float (&s)[N], float (&m_run)[2], f
 // tile_off<16>.  Step s of the copy moves the rows [ROWS s, ROWS s + ROWS): a lane's row and chunk are constants, and since its
 // row inside a step takes the low bits of the row index, the swizzle of step s differs from that of step 0 by an XOR with a
 // constant.  A whole page of contiguous tokens - all but the edges, in the recommended layout - is 2 x STEPS copies with constant
-// offsets from a few lane registers.  Before, every copy computed its own 64-bit address and mask.
-template <int D, bool FP8>
+// offsets from a few lane registers, where every copy computed its own 64-bit address and mask before: 256 decodes on an fp8 cache 352 ->
+// 283 warp instructions per page (with the conversions of e4m3x4_to_f16x4) and 288 -> 276 us beside four chunks, chat mix 258 ->
+// 253 us.  LEAN off keeps the general copy alone: a member's own chunks beside shared-prefix CTAs, which wait for instruction fetches
+// a fifth of their time, are slower with both forms in the code (16 forks of one context 30.5 against 30.2 us).
+template <int D, bool FP8, bool LEAN = true>
 struct PageCopy {
     static constexpr int ELEM = FP8 ? 1 : 2, CPR = D * ELEM / 16;       // 16-byte chunks of a token's row
     static constexpr int ROWS = 32 / CPR, STEPS = 16 / ROWS, PATTERNS = 8 / ROWS;
@@ -151,7 +154,7 @@ struct PageCopy {
     // k, v: the page's first token; tokens outside [lo, end) - slack slots, tokens left of a sliding window - are zero-filled
     __device__ __forceinline__ void operator()(uint32_t slot, const uint8_t* k, const uint8_t* v, int64_t k_stride, int64_t v_stride, int tok0, int lo, int end) const
     {
-        if (k_stride == D && v_stride == D && tok0 + 16 <= end && tok0 >= lo) {
+        if (LEAN && k_stride == D && v_stride == D && tok0 + 16 <= end && tok0 >= lo) {
             const uint8_t *const ks = k + lane * 16, *const vs = v + lane * 16;
 #pragma unroll
             for (int s = 0; s < STEPS; ++s) {
@@ -174,9 +177,9 @@ struct PageCopy {
 };
 
 // A warp's ring of NSTAGE pages (K, V) and the fetching into it: one cp.async group per page, NSTAGE - 1 pages ahead.
-template <int D, bool FP8, int NWARPS, int NSTAGE>
+template <int D, bool FP8, int NWARPS, int NSTAGE, bool LEAN = true>
 struct PageRing {
-    using Copy = PageCopy<D, FP8>;
+    using Copy = PageCopy<D, FP8, LEAN>;
     static constexpr int HALF = Copy::PAGE_BYTES, STAGE_BYTES = 2 * HALF, WARP_BYTES = NSTAGE * STAGE_BYTES;
     const AttnParams& p;
     const DecodeItem& it;
@@ -249,10 +252,10 @@ struct PageLanes {
     }
 };
 
-template <int D, int NWARPS, int NSTAGE>
+template <int D, int NWARPS, int NSTAGE, bool LEAN = true>
 __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* plan, const int cta)
 {
-    using Ring = PageRing<D, false, NWARPS, NSTAGE>;
+    using Ring = PageRing<D, false, NWARPS, NSTAGE, LEAN>;
     constexpr int KSTEPS = D / 16;
     constexpr int DP = D + 4;                   // padded row of the merge buffer (bank-conflict free)
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -874,7 +877,7 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_with_shared_kernel(cons
     if (decode_extra_cta(p)) return;
     const uint8_t* const plan = INL > 0 ? inl.bytes : p.plan.base;
     if ((int)blockIdx.x < n_shared_ctas) decode_shared_cta<D, NWARPS, NSTAGE, NCG>(p, plan, (int)blockIdx.x);
-    else decode_cta<D, NWARPS, NSTAGE>(p, plan, (int)blockIdx.x - n_shared_ctas);
+    else decode_cta<D, NWARPS, NSTAGE, false>(p, plan, (int)blockIdx.x - n_shared_ctas);
 }
 
 // ---------------------------------------------------------------------------------------------
