@@ -300,6 +300,28 @@ def test_decode_plans_fit_the_allocation_free_entry_point(Hq, Hkv, D):
                 assert counts[0] <= 3584 and parts * Hq * (D + 2) * 4 + 256 <= (16 << 20) - (128 << 10), (S, L)
 
 
+@pytest.mark.parametrize("Hq,Hkv,D,n,L", [(8, 2, 128, 48, 4100), (32, 8, 128, 48, 4100), (64, 8, 64, 64, 3000), (32, 8, 128, 3, 900), (8, 2, 64, 1, 40)])
+def test_decode_chunks_beside_prefill(Hq, Hkv, D, n, L):
+    """Beside prefill the decode chunks are twice as long as alone where they are longer than 32 pages, and the same up to that;
+    either way they cover every sequence once and in order."""
+    d = cf.make_desc(Hq, Hkv, D, 16, 65536)
+    lens = [L + 37 * i for i in range(n)]
+
+    def chunks(lc, lq):
+        dec = np.asarray(cf.cf_plan_inspect(d, lc, lq, 4096, 148)[1])
+        of = [dec[dec[:, 0] == s] for s in range(n)]
+        for s in range(n):
+            c = of[s][np.argsort(of[s][:, 2])]
+            assert c[0, 2] == 0 and c[-1, 3] == lens[s] and np.array_equal(c[1:, 2], c[:-1, 3])
+        return (dec[:, 3] - dec[:, 2]).max() / 16
+    alone, beside = chunks(lens, [1] * n), chunks(lens + [3000], [1] * n + [500])
+    longest = np.ceil(max(lens) / 16)
+    if alone <= 32 or alone >= longest:
+        assert beside <= max(alone, 2 * 32)
+    else:
+        assert min(1.5 * alone, longest / 2) <= beside <= 2 * alone + 8
+
+
 @pytest.mark.parametrize("Hq,Hkv,D,fp8,n,L,measured", [
     (64, 8, 128, False, 5, 600, 13.2), (32, 8, 128, False, 16, 400, 11.3), (32, 8, 128, False, 40, 800, 30.7),
     (32, 8, 128, False, 64, 2000, 84.1), (32, 8, 128, False, 16, 20000, 199.9), (8, 2, 128, False, 64, 2000, 28.9),
