@@ -136,9 +136,8 @@ __device__ __forceinline__ void page_softmax(float (&s)[N], float (&m_run)[2], f
 // constant.  A whole page of contiguous tokens - all but the edges, in the recommended layout - is 2 x STEPS copies with constant
 // offsets from a few lane registers, where every copy computed its own 64-bit address and mask before: 256 decodes on an fp8 cache 352 ->
 // 283 warp instructions per page (with the conversions of e4m3x4_to_f16x4) and 288 -> 276 us beside four chunks, chat mix 258 ->
-// 253 us.  LEAN off keeps the general copy alone: a member's own chunks beside shared-prefix CTAs, which wait for instruction fetches
-// a fifth of their time, are slower with both forms in the code (16 forks of one context 30.5 against 30.2 us).
-template <int D, bool FP8, bool LEAN = true>
+// 253 us.
+template <int D, bool FP8>
 struct PageCopy {
     static constexpr int ELEM = FP8 ? 1 : 2, CPR = D * ELEM / 16;       // 16-byte chunks of a token's row
     static constexpr int ROWS = 32 / CPR, STEPS = 16 / ROWS, PATTERNS = 8 / ROWS;
@@ -154,7 +153,7 @@ struct PageCopy {
     // k, v: the page's first token; tokens outside [lo, end) - slack slots, tokens left of a sliding window - are zero-filled
     __device__ __forceinline__ void operator()(uint32_t slot, const uint8_t* k, const uint8_t* v, int64_t k_stride, int64_t v_stride, int tok0, int lo, int end) const
     {
-        if (LEAN && k_stride == D && v_stride == D && tok0 + 16 <= end && tok0 >= lo) {
+        if (k_stride == D && v_stride == D && tok0 + 16 <= end && tok0 >= lo) {
             const uint8_t *const ks = k + lane * 16, *const vs = v + lane * 16;
 #pragma unroll
             for (int s = 0; s < STEPS; ++s) {
@@ -177,9 +176,9 @@ struct PageCopy {
 };
 
 // A warp's ring of NSTAGE pages (K, V) and the fetching into it: one cp.async group per page, NSTAGE - 1 pages ahead.
-template <int D, bool FP8, int NWARPS, int NSTAGE, bool LEAN = true>
+template <int D, bool FP8, int NWARPS, int NSTAGE>
 struct PageRing {
-    using Copy = PageCopy<D, FP8, LEAN>;
+    using Copy = PageCopy<D, FP8>;
     static constexpr int HALF = Copy::PAGE_BYTES, STAGE_BYTES = 2 * HALF, WARP_BYTES = NSTAGE * STAGE_BYTES;
     const AttnParams& p;
     const DecodeItem& it;
@@ -252,10 +251,16 @@ struct PageLanes {
     }
 };
 
+// LEAN off, for a member's own chunks beside shared-prefix CTAs: the loop computes every address where it is used.  That
+// kernel waits for instruction fetches a fifth of its time and is slower with PageRing in its code (30 forks of one 7808-token
+// context, 64 over 8 heads of 64, 58.5 -> 64 us).
 template <int D, int NWARPS, int NSTAGE, bool LEAN = true>
 __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* plan, const int cta)
 {
-    using Ring = PageRing<D, false, NWARPS, NSTAGE, LEAN>;
+    constexpr int CPR = D / 8;                  // 16-byte chunks per token row
+    constexpr int PAGE_BYTES = 16 * D * 2;      // one (page, head) of K or of V
+    constexpr int STAGE_BYTES = 2 * PAGE_BYTES;
+    constexpr int WARP_BYTES = NSTAGE * STAGE_BYTES;
     constexpr int KSTEPS = D / 16;
     constexpr int DP = D + 4;                   // padded row of the merge buffer (bank-conflict free)
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -279,10 +284,10 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
         }
     }
 
+    const int first_page = it.kv_begin >> 4;
     const int n_pages = (it.kv_end - it.kv_begin + 15) >> 4;
     const int my_n = n_pages > warp ? (n_pages - warp + NWARPS - 1) / NWARPS : 0;
-    Ring ring(p, it, kvh, smem_u32(smem) + warp * Ring::WARP_BYTES, my_n, warp, lane);
-    const PageLanes<D> at(lane);
+    const uint32_t wbase = smem_u32(smem) + warp * WARP_BYTES;
 
     float o[KSTEPS][4];
 #pragma unroll
@@ -290,21 +295,19 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
     float m_run[2] = {-INFINITY, -INFINITY};
     float l_run[2] = {0.f, 0.f};
 
-    ring.start();
-    for (int i = 0; i < my_n; ++i) {
-        const uint32_t sK = ring.page(i), sV = sK + Ring::HALF;
+    // page i, its K at sK and V behind it; k_at and v_at: a lane's fragment addresses inside K and V
+    auto use_page = [&](const int i, const uint32_t sK, auto k_at, auto v_at) {
+        const uint32_t sV = sK + PAGE_BYTES;
         const int tok0 = it.kv_begin + (i * NWARPS + warp) * 16;
 
         // S^T = K Q^T ; two accumulators break the dependent MMA chain
         float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
-        {
 #pragma unroll
-            for (int ks = 0; ks < KSTEPS; ++ks) {
-                uint32_t a[4];
-                ldmatrix_x4(a, sK + at.k[ks & 3] + (ks >> 2) * 2048);
-                if (ks & 1) mma_bf16_16816(s1, a, qf[ks][0], qf[ks][1]);
-                else        mma_bf16_16816(s0, a, qf[ks][0], qf[ks][1]);
-            }
+        for (int ks = 0; ks < KSTEPS; ++ks) {
+            uint32_t a[4];
+            ldmatrix_x4(a, sK + k_at(ks));
+            if (ks & 1) mma_bf16_16816(s1, a, qf[ks][0], qf[ks][1]);
+            else        mma_bf16_16816(s0, a, qf[ks][0], qf[ks][1]);
         }
         float s[4];
         const int tA = tok0 + (lane >> 2);
@@ -321,13 +324,67 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
         // P^T as B operand: transpose the two 8x8 (token x head) blocks
         const uint32_t pb0 = movmatrix_trans(pack_bf16(s[0], s[1]));
         const uint32_t pb1 = movmatrix_trans(pack_bf16(s[2], s[3]));
-        {
 #pragma unroll
-            for (int mt = 0; mt < KSTEPS; ++mt) {
-                uint32_t a[4];
-                ldmatrix_x4_trans(a, sV + at.v[mt & 3] + (mt >> 2) * 2048);
-                mma_bf16_16816(o[mt], a, pb0, pb1);
+        for (int mt = 0; mt < KSTEPS; ++mt) {
+            uint32_t a[4];
+            ldmatrix_x4_trans(a, sV + v_at(mt));
+            mma_bf16_16816(o[mt], a, pb0, pb1);
+        }
+    };
+    if constexpr (LEAN) {
+        using Ring = PageRing<D, false, NWARPS, NSTAGE>;
+        static_assert(Ring::WARP_BYTES == WARP_BYTES, "one layout");
+        Ring ring(p, it, kvh, wbase, my_n, warp, lane);
+        const PageLanes<D> at(lane);
+        ring.start();
+        for (int i = 0; i < my_n; ++i)
+            use_page(i, ring.page(i), [&](int ks) { return at.k[ks & 3] + (ks >> 2) * 2048; }, [&](int mt) { return at.v[mt & 3] + (mt >> 2) * 2048; });
+    } else {
+        const int32_t* bt = p.block_table + (int64_t)it.seq * p.max_blocks + first_page + warp;
+        const __nv_bfloat16* kbase = p.k_cache + (int64_t)kvh * p.ks_head;
+        const __nv_bfloat16* vbase = p.v_cache + (int64_t)kvh * p.vs_head;
+        // as in PageRing: never dereferenced outside the pool
+        auto checked = [&](int32_t id) -> int32_t {
+            if ((uint32_t)id < (uint32_t)p.num_blocks) return id;
+            if (p.err) atomicOr(p.err, kErrBlockId);
+            return 0;
+        };
+        int cache_base = 0;
+        int32_t pid_cache = (lane < my_n) ? checked(__ldg(bt + lane * NWARPS)) : 0;
+        const uint64_t stream_once = l2_policy_evict_first();
+        auto issue = [&](int i) {
+            if (i - cache_base == 32) {             // refill the per-lane page-id cache
+                cache_base = i;
+                pid_cache = (i + lane < my_n) ? checked(__ldg(bt + (i + lane) * NWARPS)) : 0;
             }
+            const int32_t pid = __shfl_sync(0xffffffffu, pid_cache, i - cache_base);
+            const int tok0 = it.kv_begin + (i * NWARPS + warp) * 16;
+            const uint32_t sbase = wbase + (i % NSTAGE) * STAGE_BYTES;
+            const __nv_bfloat16* kp = kbase + (int64_t)pid * p.ks_block;
+            const __nv_bfloat16* vp = vbase + (int64_t)pid * p.vs_block;
+#pragma unroll
+            for (int r = 0; r < (16 * CPR) / 32; ++r) {
+                const int id = r * 32 + lane;
+                const int t = id / CPR, c = id % CPR;
+                // slack slots of the last page and tokens left of a sliding window are zero-filled
+                const bool ok = tok0 + t < it.kv_end && tok0 + t >= it.kv_lo;
+                const int tt = ok ? t : 0;
+                cp_async16_hint(sbase + tile_off<16>(t, c), kp + tt * p.ks_token + c * 8, ok ? 16 : 0, stream_once);
+                cp_async16_hint(sbase + PAGE_BYTES + tile_off<16>(t, c), vp + tt * p.vs_token + c * 8, ok ? 16 : 0, stream_once);
+            }
+        };
+#pragma unroll
+        for (int s = 0; s < NSTAGE - 1; ++s) {
+            if (s < my_n) issue(s);
+            cp_async_commit();
+        }
+        for (int i = 0; i < my_n; ++i) {
+            cp_async_wait<NSTAGE - 2>();
+            __syncwarp();
+            if (i + NSTAGE - 1 < my_n) issue(i + NSTAGE - 1);
+            cp_async_commit();
+            use_page(i, wbase + (i % NSTAGE) * STAGE_BYTES, [&](int ks) { return tile_off<16>((lane & 7) + ((lane >> 3) & 1) * 8, 2 * ks + (lane >> 4)); },
+                     [&](int mt) { return tile_off<16>((lane & 7) + (lane >> 4) * 8, 2 * mt + ((lane >> 3) & 1)); });
         }
     }
     cp_async_wait<0>();
