@@ -197,8 +197,8 @@ cf_status cf_get_async_status(cf_ctx* ctx);
  * partition of the node between prefill and decode.  Both are launch sequences of cf_mixed_attention; a
  * batch that holds both kinds of work runs the spatial one unless it is switched off.  The same plan gives the
  * same bits in either sequence (planned calls); an unplanned call plans for the sequence it will run (the
- * spatial one balances the prefill items over its first grid's SMs and may cut other items into KV ranges), so
- * across sequences unplanned results agree to rounding.
+ * spatial one balances the prefill items over its first grid's SMs and may cut other items into KV ranges, and decode
+ * sequences into chunks for the SMs that are left), so across sequences unplanned results agree to rounding.
  *   cf_set_overlap(ctx, 0): serial sequence, decode -> (combine) -> prefill -> (prefill combine) on the
  *     caller's stream alone.
  *   cf_set_overlap(ctx, n), n > 0 (the initial state is n = 1): n persistent prefill CTAs, one per SM (n = 1:
@@ -229,7 +229,8 @@ cf_status cf_validate_block_table(cf_ctx* ctx, const cf_cache_desc* desc, const 
 
 /* TEST ONLY: planner and launch-sequence switches that the test-suite uses to force paths the cost model
  * would not pick on small inputs.  Not part of the supported surface; values <= 0 restore the default.
- *   CF_DEBUG_PREFILL_SPLIT          k >= 2: cut every prefill item into k KV ranges; 1: never split
+ *   CF_DEBUG_PREFILL_SPLIT          k >= 2: cut every prefill item into k KV ranges; 1: never split, one plan for
+ *                                   both launch sequences
  *   CF_DEBUG_SEPARATE_COMBINE       1: merge split-K decode partials in the separate combine kernel
  *   CF_DEBUG_DECODE_WAVES           target number of decode CTA waves
  *   CF_DEBUG_DECODE_MIN_CHUNK_PAGES shortest decode chunk, in pages

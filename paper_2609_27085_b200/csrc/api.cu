@@ -1135,7 +1135,8 @@ cf_status cf_mixed_step_host(cf_ctx* c, const cf_cache_desc* desc,
         // A step that follows another without a flush in between has its read-back under the kernels of the next one anyway.
         // Where the kernels outweigh both directions of the link such steps are bound by them, and the parts' items run as one
         // call, decode beside prefill (agentic, back to back, in parts 1006 us per step, as one call 914); where the link weighs as
-        // much, parts still help.  The items are the parts' own, so a step's result does not depend on the steps before it.
+        // much, parts still help.  The items are the parts' own (decode in chunks for all SMs, as it runs alone in parts), so a step's
+        // result does not depend on the steps before it.
         if (!whole && kernel_bound && c->unflushed_steps > 0) {
             Unit u;
             if (join_units(c, desc, parts, units, context_len, query_len, num_seqs, max_blocks_per_seq, &u)) {

@@ -86,19 +86,11 @@ static bool head_by_head(const cf_cache_desc* d, int64_t longest)
     return d->num_q_heads / d->num_kv_heads >= 2 && longest * 2 * d->num_kv_heads * d->head_dim * 2 > kKvSetBytes;
 }
 
-cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const int32_t* query_len,
-                     int32_t num_seqs, int32_t max_blocks_per_seq, const PlanConfig& cfg, Plan* plan,
-                     const int32_t* share_group, const int32_t* shared_len)
+// Decode: near-equal KV chunks, of a length that suits `sms` SMs (those that the decode grid starts on).
+static void plan_decode(const cf_cache_desc* d, const int32_t* context_len, const int32_t* query_len, int32_t num_seqs,
+                        const PlanConfig& cfg, int32_t sms, const int32_t* share_group, const int32_t* shared_len, Plan* plan)
 {
-    *plan = Plan();
-    cf_status st = validate_lengths(d, context_len, query_len, num_seqs, max_blocks_per_seq, plan);
-    if (st != CF_OK) return st;
     const int32_t B = d->block_size;
-
-    // ---- decode: near-equal KV chunks, sized so that (chunks x kv heads) fills the machine a few times
-    for (int32_t s = 0; s < num_seqs; ++s)
-        if (query_len[s] == 1) ++plan->n_decode_seqs;
-        else if (query_len[s] > 1) ++plan->n_prefill_seqs;
     const int32_t quantum = std::max(1, cfg.decode_page_quantum);
     // With a sliding window a decode token at position Lc - 1 sees keys [Lc - W, Lc): the chunks cover the pages
     // from the one that holds the window's left edge onwards, and nothing left of it is ever touched.
@@ -148,19 +140,15 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
     auto own_first_page = [&](int32_t s) -> int64_t {
         return shared_pages.empty() ? first_page_of(context_len[s]) : (int64_t)shared_pages[(size_t)s];
     };
-    // Beside prefill a decode grid has about half of the SMs that the model fills with CTAs, so chunks there are twice as long: as many
-    // CTAs as fit at a time, and half as many starts, ends and partials.  (A rule on the batch and not on the launch sequence: both
-    // give the same bits.  Up to 32 pages, where latency decides, the model's length stays.)  One pass, the model's chunks ->
-    // twice as long: one rank of four of the chat mix 81 -> 75 us, 256 decodes on an fp8 cache beside four chunks 275.5 -> 272.4,
-    // chat mix 253 -> 252, agentic and sweep batches unchanged; 1.25 and 1.5 times 78 and 80.5 us for the rank of four, half
-    // as long 89.
+    // Shared prefixes have a rule of their own (below) that counts on every SM.
     auto decode_target = [&]() -> int64_t {
         float pages[kTargetSeqs];
-        const int64_t t = decode_target_pages(
+        PlanConfig on = cfg;
+        if (extra_pages == 0) on.num_sms = sms;
+        return decode_target_pages(
             num_seqs,
             [&](int32_t s) -> int64_t { return query_len[s] == 1 ? (int64_t)context_len[s] - own_first_page(s) * B : -1; },
-            B, d->num_q_heads, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, cfg, pages, extra_pages);
-        return plan->n_prefill_seqs > 0 && extra_pages == 0 && t > 32 ? 2 * t : t;
+            B, d->num_q_heads, d->num_kv_heads, d->head_dim, d->kv_dtype == CF_KV_FP8_E4M3, on, pages, extra_pages);
     };
     int64_t target = decode_target();
 
@@ -279,7 +267,21 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
     std::stable_sort(plan->decode.begin(), plan->decode.end(), [](const DecodeItem& a, const DecodeItem& b) {
         return (a.kv_end - a.kv_begin) > (b.kv_end - b.kv_begin);
     });
+}
 
+cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const int32_t* query_len,
+                     int32_t num_seqs, int32_t max_blocks_per_seq, const PlanConfig& cfg, Plan* plan,
+                     const int32_t* share_group, const int32_t* shared_len)
+{
+    *plan = Plan();
+    cf_status st = validate_lengths(d, context_len, query_len, num_seqs, max_blocks_per_seq, plan);
+    if (st != CF_OK) return st;
+
+    for (int32_t s = 0; s < num_seqs; ++s)
+        if (query_len[s] == 1) ++plan->n_decode_seqs;
+        else if (query_len[s] > 1) ++plan->n_prefill_seqs;
+    const int32_t B = d->block_size, G = d->num_q_heads / d->num_kv_heads, W = d->window_size;
+    const int64_t slot_bytes = (int64_t)d->num_q_heads * (d->head_dim + 2) * 4;
     // ---- prefill: q tiles of every chunk, the tile with the longest visible KV range first
     {
         // A block = 128 rows of a chunk (group size 1: two blocks of one head, one per q tile).  The work items of a
@@ -399,13 +401,13 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         // An item may be cut into k <= 8 KV ranges that write fp32 partials, merged by a combine pass; k
         // comes from the cost model's constants; a range never starts inside the diagonal band and has at
         // least 4 tiles.
-        const size_t M = (size_t)std::max(1, ((cfg.prefill_sms_mixed > 0 && !plan->decode.empty()) ? cfg.prefill_sms_mixed : cfg.num_sms) /
+        const size_t M = (size_t)std::max(1, ((cfg.prefill_sms_mixed > 0 && plan->n_decode_seqs > 0) ? cfg.prefill_sms_mixed : cfg.num_sms) /
                                                  (pair ? 2 : 1));      // slots that take an item: SMs, or pairs of SMs
         // Beside decode that lasts longer than the uncut items an incomplete last wave costs nothing - the call ends with
         // decode - while ranges would cost their partials and the combine pass (chat mix, 128 items on 88 SMs, one pass:
         // 40 of them cut in two 277 us, none 263 us).
         bool decode_outlasts = false;
-        if (cfg.prefill_sms_mixed > 0 && cfg.prefill_sms_mixed < cfg.num_sms && !plan->decode.empty() && !items.empty()) {
+        if (cfg.prefill_sms_mixed > 0 && cfg.prefill_sms_mixed < cfg.num_sms && plan->n_decode_seqs > 0 && !items.empty()) {
             double bytes = 0.0, tiles = 0.0;
             for (int32_t s = 0; s < num_seqs; ++s)
                 if (query_len[s] == 1)
@@ -492,7 +494,7 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         const size_t n_items = items.size();
         // The first prefill grid: as many SMs as the batch's share, or fewer that need no more rounds when the items are alike
         // (chat mix: two rounds of 64 instead of 88 and 40: 263 -> 256 us, decode has the SMs).
-        if (cfg.prefill_sms_mixed > 0 && !plan->decode.empty()) {
+        if (cfg.prefill_sms_mixed > 0 && plan->n_decode_seqs > 0) {
             plan->front_sms = cfg.prefill_sms_mixed;
             const size_t slots = M, rounds = n_items > 0 ? (n_items + slots - 1) / slots : 1;
             const bool whole = std::all_of(k_of.begin(), k_of.end(), [](int32_t k) { return k == 1; });
@@ -503,6 +505,22 @@ cf_status build_plan(const cf_cache_desc* d, const int32_t* context_len, const i
         }
         for (size_t i = 1; i < n_items; ++i)
             if (items[i].sub > 0) k_of[i] = k_of[i - 1];      // the items of a block and KV head are cut alike
+        // The decode grid of the spatial sequence starts on the SMs that the first prefill grid leaves, so its chunks are chosen for those,
+        // and in the serial sequence for all of them.  CTAs chosen to fill every SM once are up to a tenth too many beside even
+        // one small chunk, and the last of them wait for a whole one to end.  One pass on a B200, chunks for all SMs -> for those
+        // left: four of 16,000 tokens beside a 64-token chunk, 64 over 8 heads, fp8 cache 46.8 -> 37.9 us, heads of 64 32.4 -> 27.5; 32
+        // of 1K-8K beside 512 tokens, fp8 94 -> 87; one rank of four of the chat mix 72.3 -> 69.7; one of 32,000 (8 over 2
+        // heads) beside 64 18.9 -> 18.6; 190 batches 1.02 in the mean, the worst 10 of 17,000 beside 360 tokens with heads of 64 67.2 -> 72.9.
+        // A time-averaged count of SMs instead (more of them the shorter the prefill): 1.01.  A plan whose KV split is switched off
+        // does not depend on the launch sequence.
+        int32_t decode_sms = cfg.num_sms;
+        if (plan->front_sms > 0 && cfg.prefill_force_split != 1) {
+            int64_t slots = 0;
+            for (int32_t k : k_of) slots += k;
+            decode_sms -= (int32_t)std::min<int64_t>(plan->front_sms, slots * (pair ? 2 : 1));
+            decode_sms = std::max(decode_sms, cfg.num_sms / 8);
+        }
+        plan_decode(d, context_len, query_len, num_seqs, cfg, decode_sms, share_group, shared_len, plan);
         if (cfg.part_bytes != INT64_MAX) {                      // fewer ranges where the partial rows would outgrow the budget
             const int64_t left = cfg.part_bytes - (int64_t)plan->n_part_slots * slot_bytes;
             auto row_bytes = [&](int32_t most) {

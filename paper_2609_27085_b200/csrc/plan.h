@@ -93,7 +93,8 @@ struct PlanConfig {
     int32_t decode_page_quantum = 4;  // chunk lengths are multiples of this many pages (warps per CTA)
     int32_t prefill_sms_mixed = 0;    // > 0: SMs the prefill items are balanced over when the batch also holds decode
                                       // work (spatial launch sequence: the first prefill grid's share); 0: num_sms
-    int32_t prefill_force_split = 0;  // >= 2: split every tcgen05 item that many ways (tests); 0: cost model decides
+    int32_t prefill_force_split = 0;  // >= 2: split every tcgen05 item that many ways (tests); 1: none, and one plan for both launch
+                                      // sequences; 0: cost model decides
     int64_t part_bytes = INT64_MAX;   // bytes that the fp32 partials of split sequences and items may take (fixed workspace)
     bool prefill_pair = false;        // plan for the two-CTA kernel where the geometry allows it (head_dim 128, group
                                       // size a multiple of 4): an item carries four heads, the machine has num_sms / 2 slots
@@ -159,7 +160,7 @@ inline int64_t decode_target_pages(int32_t num_seqs, LcOf lc_of, int32_t B, int3
     }
     const int64_t quantum = cfg.decode_page_quantum > 1 ? cfg.decode_page_quantum : 1;
     const int64_t lo = ((cfg.decode_min_chunk_pages > 1 ? cfg.decode_min_chunk_pages : 1) + quantum - 1) / quantum * quantum;
-    const int64_t sms = cfg.num_sms > 1 ? cfg.num_sms : 1;      // of a mixed batch too: the sequences of launches agree bit for bit
+    const int64_t sms = cfg.num_sms > 1 ? cfg.num_sms : 1;      // those that the grid starts on
     const int64_t slots = sms * (D == 64 || fp8 ? 3 : 2);      // resident CTAs: 64 KB of shared memory each, or 96 KB
     const int32_t waves = cfg.decode_waves > 1 ? cfg.decode_waves : 1;
     auto round_up = [&](int64_t c) { return (c + quantum - 1) / quantum * quantum; };

@@ -300,26 +300,73 @@ def test_decode_plans_fit_the_allocation_free_entry_point(Hq, Hkv, D):
                 assert counts[0] <= 3584 and parts * Hq * (D + 2) * 4 + 256 <= (16 << 20) - (128 << 10), (S, L)
 
 
-@pytest.mark.parametrize("Hq,Hkv,D,n,L", [(8, 2, 128, 48, 4100), (32, 8, 128, 48, 4100), (64, 8, 64, 64, 3000), (32, 8, 128, 3, 900), (8, 2, 64, 1, 40)])
-def test_decode_chunks_beside_prefill(Hq, Hkv, D, n, L):
-    """Beside prefill the decode chunks are twice as long as alone where they are longer than 32 pages, and the same up to that;
-    either way they cover every sequence once and in order."""
-    d = cf.make_desc(Hq, Hkv, D, 16, 65536)
-    lens = [L + 37 * i for i in range(n)]
+def _decode_cuts(desc, lc, lq, **kw):
+    """((sequence, first token, end) of every decode chunk, prefill work items, those cut into KV ranges)"""
+    _, dec, *_, counts = cf.cf_plan_inspect(desc, lc, lq, 1 << 16, want_counts=True, **kw)
+    return [tuple(r) for r in dec[:, [0, 2, 3]].tolist()], int(counts[4]), int(counts[5])
 
-    def chunks(lc, lq):
-        dec = np.asarray(cf.cf_plan_inspect(d, lc, lq, 4096, 148)[1])
-        of = [dec[dec[:, 0] == s] for s in range(n)]
-        for s in range(n):
-            c = of[s][np.argsort(of[s][:, 2])]
-            assert c[0, 2] == 0 and c[-1, 3] == lens[s] and np.array_equal(c[1:, 2], c[:-1, 3])
-        return (dec[:, 3] - dec[:, 2]).max() / 16
-    alone, beside = chunks(lens, [1] * n), chunks(lens + [3000], [1] * n + [500])
-    longest = np.ceil(max(lens) / 16)
-    if alone <= 32 or alone >= longest:
-        assert beside <= max(alone, 2 * 32)
-    else:
-        assert min(1.5 * alone, longest / 2) <= beside <= 2 * alone + 8
+
+@pytest.mark.parametrize("new", [2, 64, 500])
+@pytest.mark.parametrize("Hq,Hkv,D,fp8,n,L", [
+    (8, 2, 128, False, 1, 32000), (8, 2, 128, False, 1, 131072), (32, 8, 128, False, 1, 131072), (8, 2, 128, False, 2, 32000),
+    (8, 2, 128, False, 16, 8192), (32, 8, 128, False, 16, 8000), (8, 2, 128, False, 48, 4100), (64, 8, 64, False, 64, 3000),
+    (64, 8, 128, True, 4, 16000), (64, 8, 128, True, 256, 1300), (32, 8, 128, False, 3, 900), (8, 2, 64, False, 1, 40),
+])
+def test_decode_chunks_suit_the_sms_that_prefill_leaves(Hq, Hkv, D, fp8, n, L, new):
+    """Beside prefill (spatial sequence) decode is cut as it would be alone on the SMs that the first prefill grid leaves at the start, in
+    the serial sequence as alone on all of them, and with the KV split switched off alike in both."""
+    d = cf.make_desc(Hq, Hkv, D, 16, 65536, kv_dtype=cf.CF_KV_FP8_E4M3 if fp8 else cf.CF_KV_BF16, k_scale=16 if fp8 else None,
+                     v_scale=16 if fp8 else None)
+    lens = [L + 37 * i for i in range(n)]
+    lc, lq = lens + [new + 6000], [1] * n + [new]
+    alone = _decode_cuts(d, lens, [1] * n)[0]
+    for s in range(n):
+        c = sorted(r[1:] for r in alone if r[0] == s)
+        assert c[0][0] == 0 and c[-1][1] == lens[s] and all(x[1] == y[0] for x, y in zip(c, c[1:]))
+    assert _decode_cuts(d, lc, lq)[0] == alone
+    assert _decode_cuts(d, lc, lq, prefill_sms_mixed=88, prefill_force_split=1)[0] == alone
+    beside, items, cut = _decode_cuts(d, lc, lq, prefill_sms_mixed=88)
+    # whole items that need several rounds on the 88 SMs, all of like length here, take as few SMs as need no more rounds
+    front = min(88, items) if cut or items <= 88 else -(-items // -(-items // 88))
+    assert beside == _decode_cuts(d, lens, [1] * n, num_sms=148 - front)[0]
+    assert len(beside) * Hkv >= min(0.9 * len(alone) * Hkv, 148 - front)     # no SM without a chunk that has one alone
+
+
+SHARED = r"""
+#include <cstring>
+#include "plan.h"
+using namespace cf;
+int main()
+{
+    cf_cache_desc d = {};
+    d.num_q_heads = 32; d.num_kv_heads = 8; d.head_dim = 128; d.block_size = 16; d.num_blocks = 1 << 20;
+    std::vector<int32_t> lc, lq, group, len;
+    for (int i = 0; i < 16; ++i) { lc.push_back(8300 + 130 * i); lq.push_back(1); group.push_back(0); len.push_back(8192); }
+    Plan p[3];
+    PlanConfig cfg;
+    if (build_plan(&d, lc.data(), lq.data(), 16, 1 << 16, cfg, &p[0], group.data(), len.data()) != CF_OK) return 2;
+    lc.push_back(1200); lq.push_back(600); group.push_back(-1); len.push_back(0);
+    for (int i = 1; i < 3; ++i) {
+        cfg.prefill_sms_mixed = i == 2 ? 88 : 0;
+        if (build_plan(&d, lc.data(), lq.data(), 17, 1 << 16, cfg, &p[i], group.data(), len.data()) != CF_OK) return 2;
+        if (p[i].prefill_tc.empty() || p[i].shared_decode.empty() || p[i].decode.size() != p[0].decode.size() ||
+            p[i].shared_decode.size() != p[0].shared_decode.size() ||
+            std::memcmp(p[i].decode.data(), p[0].decode.data(), p[0].decode.size() * sizeof p[0].decode[0]) ||
+            std::memcmp(p[i].shared_decode.data(), p[0].shared_decode.data(), p[0].shared_decode.size() * sizeof p[0].shared_decode[0]))
+            return 1;
+    }
+}
+"""
+
+
+def test_shared_prefix_chunks_do_not_depend_on_prefill_beside_them(tmp_path):
+    """The chunks of shared prefixes and of their members have rules of their own: the same alone, beside prefill in the serial sequence, and in
+    the spatial one."""
+    csrc = os.path.join(ROOT, "paper_2609_27085_b200", "csrc")
+    (tmp_path / "shared.cpp").write_text(SHARED)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-I", csrc, str(tmp_path / "shared.cpp"), os.path.join(csrc, "plan.cpp"), "-o",
+                    str(tmp_path / "shared")], check=True, timeout=300)
+    assert subprocess.run([str(tmp_path / "shared")], timeout=300).returncode == 0
 
 
 @pytest.mark.parametrize("Hq,Hkv,D,fp8,n,L,measured", [
