@@ -131,54 +131,51 @@ __device__ __forceinline__ void page_softmax(float (&s)[N], float (&m_run)[2], f
 }
 
 // Copies of one (page, head) of K and of V into a ring slot (cp.async, 16 bytes per lane and instruction), laid out by
-// tile_off<16>.  Step s of the copy moves the rows [ROWS s, ROWS s + ROWS): a lane's row and chunk are constants, and since its
-// row inside a step takes the low bits of the row index, the swizzle of step s differs from that of step 0 by an XOR with a
-// constant.  A whole page of contiguous tokens - all but the edges, in the recommended layout - is 2 x STEPS copies with constant
-// offsets from a few lane registers, where every copy computed its own 64-bit address and mask before: 256 decodes on an fp8 cache 352 ->
-// 283 warp instructions per page (with the conversions of e4m3x4_to_f16x4) and 288 -> 276 us beside four chunks, chat mix 258 ->
-// 253 us.
-template <int D, bool FP8>
+// tile_off<16>.  Step s of the copy moves the rows [ROWS s, ROWS s + ROWS), a lane always the same row of a step and the same chunk of it.
+// The swizzle depends on the row modulo 8, so the lane's place in the slot repeats every 8 / ROWS steps but for the step's own offset:
+// a few registers and constants.  In the pool it moves by the same stride with every step, a constant where a (page, head) holds its
+// tokens one behind the other (CONTIGUOUS); whether a row is one to copy is two compares with constants.  One form for whole pages and
+// for those that an edge cuts: with a form of its own for either, inlined at the four places that fetch, a CTA of a few pages waits for
+// instructions.  Decode kernel alone, every copy with its own address and mask -> two forms -> this one: 256 sequences behind a
+// 128-token window (32 over 8 heads) 32.6 -> 33.4 -> 32.1 us, 64 over 8 heads of 64 20.0 -> 20.5 -> 19.5, fp8 cache 28.2 -> 28.1
+// -> 27.2; in [blocks, tokens, heads, D] pools 34.1 -> 36.0 -> 33.6, 16 of 100-600 tokens 8.1 -> 9.2 -> 7.9; 64 of 1K-8K 176.7 ->
+// 175.3 -> 174.3, fp8 cache 103.4 -> 104.4 -> 103.2.  Without an instantiation of its own for CONTIGUOUS: fp8 cache, 64 of 200-1000 17.9 -> 18.4.
+template <int D, bool FP8, bool CONTIGUOUS>
 struct PageCopy {
     static constexpr int ELEM = FP8 ? 1 : 2, CPR = D * ELEM / 16;       // 16-byte chunks of a token's row
     static constexpr int ROWS = 32 / CPR, STEPS = 16 / ROWS, PATTERNS = 8 / ROWS;
     static constexpr int PAGE_BYTES = 16 * D * ELEM;                    // one (page, head) of K or of V
+    static_assert(CPR * ROWS == 32 && PATTERNS * ROWS == 8 && STEPS * ROWS == 16, "whole steps, and whole steps per period of the swizzle");
     uint32_t dst[PATTERNS];
-    int lane;
+    int row, chunk;                                                     // this lane's, of a step
     uint64_t policy;
-    __device__ __forceinline__ explicit PageCopy(int lane_) : lane(lane_), policy(l2_policy_evict_first())
+    __device__ __forceinline__ explicit PageCopy(int lane) : row(lane / CPR), chunk(lane % CPR), policy(l2_policy_evict_first())
     {
 #pragma unroll
-        for (int i = 0; i < PATTERNS; ++i) dst[i] = tile_off<16>(i * ROWS + lane / CPR, lane % CPR) - i * ROWS * 128;
+        for (int i = 0; i < PATTERNS; ++i) dst[i] = tile_off<16>(i * ROWS + row, chunk) - i * ROWS * 128;
     }
-    // k, v: the page's first token; tokens outside [lo, end) - slack slots, tokens left of a sliding window - are zero-filled
+    // this lane's 16 bytes of a page's first step, from the page's first token on
+    __device__ __forceinline__ int64_t source(int64_t stride) const { return CONTIGUOUS ? (row * CPR + chunk) * 16 : row * stride * ELEM + chunk * 16; }
+    // k, v: source() in the page; tokens outside [lo, end) - slack slots, tokens left of a sliding window - are zero-filled
+    // (a copy of no bytes reads nothing, and the address is inside the page all the same)
     __device__ __forceinline__ void operator()(uint32_t slot, const uint8_t* k, const uint8_t* v, int64_t k_stride, int64_t v_stride, int tok0, int lo, int end) const
     {
-        if (k_stride == D && v_stride == D && tok0 + 16 <= end && tok0 >= lo) {
-            const uint8_t *const ks = k + lane * 16, *const vs = v + lane * 16;
+        const int64_t k_step = ROWS * ELEM * (CONTIGUOUS ? D : k_stride), v_step = ROWS * ELEM * (CONTIGUOUS ? D : v_stride);
+        const int first = lo - tok0 - row, last = end - tok0 - row;
 #pragma unroll
-            for (int s = 0; s < STEPS; ++s) {
-                cp_async16_hint(slot + dst[s % PATTERNS] + s * ROWS * 128, ks + s * 512, 16, policy);
-                cp_async16_hint(slot + dst[s % PATTERNS] + PAGE_BYTES + s * ROWS * 128, vs + s * 512, 16, policy);
-            }
-        } else {
-            const int t0 = lane / CPR, ch = lane % CPR;
-#pragma unroll
-            for (int s = 0; s < STEPS; ++s) {
-                const int t = s * ROWS + t0;
-                const bool in = tok0 + t < end && tok0 + t >= lo;
-                const int tt = in ? t : 0;
-                const uint32_t to = slot + dst[s % PATTERNS] + s * ROWS * 128;
-                cp_async16_hint(to, k + (tt * k_stride * ELEM + ch * 16), in ? 16 : 0, policy);
-                cp_async16_hint(to + PAGE_BYTES, v + (tt * v_stride * ELEM + ch * 16), in ? 16 : 0, policy);
-            }
+        for (int s = 0; s < STEPS; ++s, k += k_step, v += v_step) {
+            const int bytes = s * ROWS >= first && s * ROWS < last ? 16 : 0;
+            const uint32_t to = slot + dst[s % PATTERNS] + s * ROWS * 128;
+            cp_async16_hint(to, k, bytes, policy);
+            cp_async16_hint(to + PAGE_BYTES, v, bytes, policy);
         }
     }
 };
 
 // A warp's ring of NSTAGE pages (K, V) and the fetching into it: one cp.async group per page, NSTAGE - 1 pages ahead.
-template <int D, bool FP8, int NWARPS, int NSTAGE>
+template <int D, bool FP8, int NWARPS, int NSTAGE, bool CONTIGUOUS>
 struct PageRing {
-    using Copy = PageCopy<D, FP8>;
+    using Copy = PageCopy<D, FP8, CONTIGUOUS>;
     static constexpr int HALF = Copy::PAGE_BYTES, STAGE_BYTES = 2 * HALF, WARP_BYTES = NSTAGE * STAGE_BYTES;
     const AttnParams& p;
     const DecodeItem& it;
@@ -192,8 +189,8 @@ struct PageRing {
     __device__ __forceinline__ PageRing(const AttnParams& p_, const DecodeItem& it_, int kvh, uint32_t base_, int n_, int warp, int lane_)
         : p(p_), it(it_), copy(lane_),
           bt(p_.block_table + (int64_t)it_.seq * p_.max_blocks + (it_.kv_begin >> 4) + warp),
-          k(reinterpret_cast<const uint8_t*>(p_.k_cache) + (int64_t)kvh * p_.ks_head * Copy::ELEM),
-          v(reinterpret_cast<const uint8_t*>(p_.v_cache) + (int64_t)kvh * p_.vs_head * Copy::ELEM),
+          k(reinterpret_cast<const uint8_t*>(p_.k_cache) + (int64_t)kvh * p_.ks_head * Copy::ELEM + copy.source(p_.ks_token)),
+          v(reinterpret_cast<const uint8_t*>(p_.v_cache) + (int64_t)kvh * p_.vs_head * Copy::ELEM + copy.source(p_.vs_token)),
           base(base_), n(n_), tok(it_.kv_begin + warp * 16), lane(lane_)
     {
         ids = lane < n ? checked(__ldg(bt + lane * NWARPS)) : 0;
@@ -254,7 +251,7 @@ struct PageLanes {
 // LEAN off, for a member's own chunks beside shared-prefix CTAs: the loop computes every address where it is used.  That
 // kernel waits for instruction fetches a fifth of its time and is slower with PageRing in its code (30 forks of one 7808-token
 // context, 64 over 8 heads of 64, 58.5 -> 64 us).
-template <int D, int NWARPS, int NSTAGE, bool LEAN = true>
+template <int D, int NWARPS, int NSTAGE, bool CONTIGUOUS, bool LEAN = true>
 __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* plan, const int cta)
 {
     constexpr int CPR = D / 8;                  // 16-byte chunks per token row
@@ -332,7 +329,7 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
         }
     };
     if constexpr (LEAN) {
-        using Ring = PageRing<D, false, NWARPS, NSTAGE>;
+        using Ring = PageRing<D, false, NWARPS, NSTAGE, CONTIGUOUS>;
         static_assert(Ring::WARP_BYTES == WARP_BYTES, "one layout");
         Ring ring(p, it, kvh, wbase, my_n, warp, lane);
         const PageLanes<D> at(lane);
@@ -504,12 +501,12 @@ __device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t v)
     return pack_f16(f.x, f.y);
 }
 
-template <int NWARPS, int NSTAGE, int INL>
+template <int NWARPS, int NSTAGE, bool CONTIGUOUS, int INL>
 __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_fp8_kernel(const AttnParams p, const __grid_constant__ PlanBytes<INL> inl)
 {
     const uint8_t* const plan = INL > 0 ? inl.bytes : p.plan.base;
     constexpr int D = 128;
-    using Ring = PageRing<D, true, NWARPS, NSTAGE>;
+    using Ring = PageRing<D, true, NWARPS, NSTAGE, CONTIGUOUS>;
     constexpr int KSTEPS = D / 16;
     constexpr int DP = D + 4;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -918,11 +915,11 @@ __device__ __forceinline__ void decode_shared_cta(const AttnParams& p, const uin
     else decode_shared_team<D, NWARPS, NSTAGE, NCG, 1>(p, it, members, kvh);
 }
 
-template <int D, int NWARPS, int NSTAGE, int INL>
+template <int D, int NWARPS, int NSTAGE, bool CONTIGUOUS, int INL>
 __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_kernel(const AttnParams p, const __grid_constant__ PlanBytes<INL> inl)
 {
     if (decode_extra_cta(p)) return;
-    decode_cta<D, NWARPS, NSTAGE>(p, INL > 0 ? inl.bytes : p.plan.base, (int)blockIdx.x);
+    decode_cta<D, NWARPS, NSTAGE, CONTIGUOUS>(p, INL > 0 ? inl.bytes : p.plan.base, (int)blockIdx.x);
 }
 
 // One grid for a batch with shared prefixes: the first n_shared_ctas CTAs serve the shared chunks (longer items
@@ -934,7 +931,7 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_with_shared_kernel(cons
     if (decode_extra_cta(p)) return;
     const uint8_t* const plan = INL > 0 ? inl.bytes : p.plan.base;
     if ((int)blockIdx.x < n_shared_ctas) decode_shared_cta<D, NWARPS, NSTAGE, NCG>(p, plan, (int)blockIdx.x);
-    else decode_cta<D, NWARPS, NSTAGE, false>(p, plan, (int)blockIdx.x - n_shared_ctas);
+    else decode_cta<D, NWARPS, NSTAGE, false, false>(p, plan, (int)blockIdx.x - n_shared_ctas);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -961,7 +958,7 @@ template <int D, bool FP8> constexpr int dec_stages() { return D == 64 || FP8 ? 
 template <int D, bool FP8>
 static size_t decode_smem_bytes()
 {
-    const size_t ring = (size_t)kDecWarps * PageRing<D, FP8, kDecWarps, dec_stages<D, FP8>()>::WARP_BYTES;
+    const size_t ring = (size_t)kDecWarps * PageRing<D, FP8, kDecWarps, dec_stages<D, FP8>(), true>::WARP_BYTES;
     const size_t merge = (size_t)kDecWarps * 8 * (D + 4) * 4 + (size_t)kDecWarps * 8 * 4 * 2;
     return ring > merge ? ring : merge;
 }
@@ -1014,11 +1011,20 @@ static cudaError_t with_plan_bytes(const HostPlan& hp, F launch)
     return hp.size <= (size_t)kMidPlanBytes ? carry(std::integral_constant<int, kMidPlanBytes>{}) : cudaErrorInvalidValue;
 }
 
+// launch(contiguous, size, block), contiguous: the tokens of a (page, head) lie one behind the other in both pools (PageCopy)
+template <int D, class F>
+static cudaError_t with_layout(const AttnParams& p, const HostPlan& hp, F launch)
+{
+    return with_plan_bytes(hp, [&](auto size, const auto* inl) {
+        return p.ks_token == D && p.vs_token == D ? launch(std::true_type{}, size, inl) : launch(std::false_type{}, size, inl);
+    });
+}
+
 template <int D>
 static cudaError_t launch_decode_t(const AttnParams& p, const HostPlan& hp, int n_items, cudaStream_t stream)
 {
-    return with_plan_bytes(hp, [&](auto size, const auto* inl) {
-        return launch_decode_grid<decode_splitk_kernel<D, kDecWarps, dec_stages<D, false>(), decltype(size)::value>>(
+    return with_layout<D>(p, hp, [&](auto contiguous, auto size, const auto* inl) {
+        return launch_decode_grid<decode_splitk_kernel<D, kDecWarps, dec_stages<D, false>(), decltype(contiguous)::value, decltype(size)::value>>(
             n_items * p.Hkv, decode_smem_bytes<D, false>(), stream, p, inl);
     });
 }
@@ -1026,8 +1032,8 @@ static cudaError_t launch_decode_t(const AttnParams& p, const HostPlan& hp, int 
 cudaError_t launch_decode_fp8(const AttnParams& p, const HostPlan& hp, int n_items, cudaStream_t stream)
 {
     if (n_items <= 0) return cudaSuccess;
-    return with_plan_bytes(hp, [&](auto size, const auto* inl) {
-        return launch_decode_grid<decode_splitk_fp8_kernel<kDecWarps, dec_stages<128, true>(), decltype(size)::value>>(
+    return with_layout<128>(p, hp, [&](auto contiguous, auto size, const auto* inl) {
+        return launch_decode_grid<decode_splitk_fp8_kernel<kDecWarps, dec_stages<128, true>(), decltype(contiguous)::value, decltype(size)::value>>(
             n_items * p.Hkv, decode_smem_bytes<128, true>(), stream, p, inl);
     });
 }

@@ -139,6 +139,42 @@ def test_decode_rings_of_every_depth(Hq, Hkv, D, fp8, layout, window):
     run_and_check(small(83, Hq, Hkv, D, [l - 1 for l in lens], [[1] * len(lens)], NB=4096), fp8=scales, layout=layout, window=window)
 
 
+@pytest.mark.parametrize("Hq,Hkv,D,fp8", [(16, 2, 64, False), (8, 2, 128, False), (16, 2, 128, True)])
+@pytest.mark.parametrize("window", [0, 83])
+def test_decode_from_pools_of_every_layout(Hq, Hkv, D, fp8, window):
+    """The decode kernels have an instantiation for pools whose (page, head) holds its tokens one behind the other, chosen when K and V
+    both do, and one for all others: K and V each as [blocks, heads, tokens, D], [blocks, tokens, heads, D] and with a padded row give
+    the same bits, decode and the pages of an fp8 cache that prefill reads (first and last pages cut, a window's edge inside a page)."""
+    lens = [1, 15, 16, 17, 63, 64, 65, 129, 700, 1100, 2500, 400]
+    scales = (np.full(Hkv, 0.02, np.float32), np.full(Hkv, 0.015, np.float32)) if fp8 else None
+    qlen = [1] * 11 + [130]
+    sc = small(89, Hq, Hkv, D, [l - q if q == 1 else l for l, q in zip(lens, qlen)], [qlen])
+    b = sc.batches[0]
+    g = GpuScenario(sc, window=window, fp8=scales)
+    g.append(b)
+    ref, ref_lse = g.attend(b)
+    bt, q = torch.from_numpy(b.block_table).cuda(), to_dev_bf16(b.q)
+    pad = 32
+
+    def laid_out(pool, how):
+        if how == "heads":
+            return pool, (Hkv * 16 * D, 16 * D, D)
+        rows = torch.zeros((pool.shape[0], 16, Hkv * D + (pad if how == "padded" else 0)), dtype=pool.dtype, device="cuda")
+        rows[:, :, :Hkv * D] = pool.permute(0, 2, 1, 3).reshape(pool.shape[0], 16, Hkv * D)
+        return rows, (16 * rows.shape[2], D, rows.shape[2])
+    scale = dict(kv_dtype=cf.CF_KV_FP8_E4M3, k_scale=g.k_scale_dev, v_scale=g.v_scale_dev) if fp8 else {}
+    for how_k, how_v in (("tokens", "tokens"), ("heads", "tokens"), ("tokens", "heads"), ("padded", "heads"), ("padded", "padded")):
+        (k, ks), (v, vs) = laid_out(g.k, how_k), laid_out(g.v, how_v)
+        d = cf.make_desc(Hq, Hkv, D, 16, sc.geom.num_blocks, k_strides=ks, v_strides=vs, window_size=window, **scale)
+        out, lse = torch.full_like(q, float("nan")), torch.full((b.total_q, Hq), float("nan"), dtype=torch.float32, device="cuda")
+        cf.cf_mixed_attention(g.ctx, d, q, k, v, bt, b.max_blocks, b.context_len, b.query_len, out, lse)
+        torch.cuda.synchronize()
+        assert cf.cf_get_async_status(g.ctx) == cf.CF_OK
+        assert np.array_equal(to_host_bits(out), ref) and np.array_equal(lse.cpu().numpy(), ref_lse), (how_k, how_v)
+    run_and_check(sc, window=window, fp8=scales)
+    g.close()
+
+
 @pytest.mark.parametrize("Hq,Hkv,D,members", [(2, 2, 128, 40), (8, 2, 128, 4), (8, 2, 128, 5), (8, 2, 128, 9), (8, 2, 128, 17),
                                               (16, 2, 64, 2), (16, 2, 64, 3), (16, 2, 64, 9), (4, 2, 128, 22), (4, 2, 64, 33)])
 @pytest.mark.parametrize("pages", [16, 33, 129])
