@@ -248,16 +248,11 @@ struct PageLanes {
     }
 };
 
-// LEAN off, for a member's own chunks beside shared-prefix CTAs: the loop computes every address where it is used.  That
-// kernel waits for instruction fetches a fifth of its time and is slower with PageRing in its code (30 forks of one 7808-token
-// context, 64 over 8 heads of 64, 58.5 -> 64 us).
-template <int D, int NWARPS, int NSTAGE, bool CONTIGUOUS, bool LEAN = true>
+// One (sequence, KV chunk, KV head): the whole of decode_splitk_kernel, and a member's own chunks beside shared-prefix CTAs.
+template <int D, int NWARPS, int NSTAGE, bool CONTIGUOUS>
 __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* plan, const int cta)
 {
-    constexpr int CPR = D / 8;                  // 16-byte chunks per token row
-    constexpr int PAGE_BYTES = 16 * D * 2;      // one (page, head) of K or of V
-    constexpr int STAGE_BYTES = 2 * PAGE_BYTES;
-    constexpr int WARP_BYTES = NSTAGE * STAGE_BYTES;
+    using Ring = PageRing<D, false, NWARPS, NSTAGE, CONTIGUOUS>;
     constexpr int KSTEPS = D / 16;
     constexpr int DP = D + 4;                   // padded row of the merge buffer (bank-conflict free)
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -281,10 +276,9 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
         }
     }
 
-    const int first_page = it.kv_begin >> 4;
     const int n_pages = (it.kv_end - it.kv_begin + 15) >> 4;
     const int my_n = n_pages > warp ? (n_pages - warp + NWARPS - 1) / NWARPS : 0;
-    const uint32_t wbase = smem_u32(smem) + warp * WARP_BYTES;
+    Ring ring(p, it, kvh, smem_u32(smem) + warp * Ring::WARP_BYTES, my_n, warp, lane);
 
     float o[KSTEPS][4];
 #pragma unroll
@@ -292,9 +286,10 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
     float m_run[2] = {-INFINITY, -INFINITY};
     float l_run[2] = {0.f, 0.f};
 
-    // page i, its K at sK and V behind it; k_at and v_at: a lane's fragment addresses inside K and V
-    auto use_page = [&](const int i, const uint32_t sK, auto k_at, auto v_at) {
-        const uint32_t sV = sK + PAGE_BYTES;
+    const PageLanes<D> at(lane);
+    ring.start();
+    for (int i = 0; i < my_n; ++i) {
+        const uint32_t sK = ring.page(i), sV = sK + Ring::HALF;
         const int tok0 = it.kv_begin + (i * NWARPS + warp) * 16;
 
         // S^T = K Q^T ; two accumulators break the dependent MMA chain
@@ -302,7 +297,7 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
 #pragma unroll
         for (int ks = 0; ks < KSTEPS; ++ks) {
             uint32_t a[4];
-            ldmatrix_x4(a, sK + k_at(ks));
+            ldmatrix_x4(a, sK + at.k[ks & 3] + (ks >> 2) * 2048);
             if (ks & 1) mma_bf16_16816(s1, a, qf[ks][0], qf[ks][1]);
             else        mma_bf16_16816(s0, a, qf[ks][0], qf[ks][1]);
         }
@@ -324,64 +319,8 @@ __device__ __forceinline__ void decode_cta(const AttnParams& p, const uint8_t* p
 #pragma unroll
         for (int mt = 0; mt < KSTEPS; ++mt) {
             uint32_t a[4];
-            ldmatrix_x4_trans(a, sV + v_at(mt));
+            ldmatrix_x4_trans(a, sV + at.v[mt & 3] + (mt >> 2) * 2048);
             mma_bf16_16816(o[mt], a, pb0, pb1);
-        }
-    };
-    if constexpr (LEAN) {
-        using Ring = PageRing<D, false, NWARPS, NSTAGE, CONTIGUOUS>;
-        static_assert(Ring::WARP_BYTES == WARP_BYTES, "one layout");
-        Ring ring(p, it, kvh, wbase, my_n, warp, lane);
-        const PageLanes<D> at(lane);
-        ring.start();
-        for (int i = 0; i < my_n; ++i)
-            use_page(i, ring.page(i), [&](int ks) { return at.k[ks & 3] + (ks >> 2) * 2048; }, [&](int mt) { return at.v[mt & 3] + (mt >> 2) * 2048; });
-    } else {
-        const int32_t* bt = p.block_table + (int64_t)it.seq * p.max_blocks + first_page + warp;
-        const __nv_bfloat16* kbase = p.k_cache + (int64_t)kvh * p.ks_head;
-        const __nv_bfloat16* vbase = p.v_cache + (int64_t)kvh * p.vs_head;
-        // as in PageRing: never dereferenced outside the pool
-        auto checked = [&](int32_t id) -> int32_t {
-            if ((uint32_t)id < (uint32_t)p.num_blocks) return id;
-            if (p.err) atomicOr(p.err, kErrBlockId);
-            return 0;
-        };
-        int cache_base = 0;
-        int32_t pid_cache = (lane < my_n) ? checked(__ldg(bt + lane * NWARPS)) : 0;
-        const uint64_t stream_once = l2_policy_evict_first();
-        auto issue = [&](int i) {
-            if (i - cache_base == 32) {             // refill the per-lane page-id cache
-                cache_base = i;
-                pid_cache = (i + lane < my_n) ? checked(__ldg(bt + (i + lane) * NWARPS)) : 0;
-            }
-            const int32_t pid = __shfl_sync(0xffffffffu, pid_cache, i - cache_base);
-            const int tok0 = it.kv_begin + (i * NWARPS + warp) * 16;
-            const uint32_t sbase = wbase + (i % NSTAGE) * STAGE_BYTES;
-            const __nv_bfloat16* kp = kbase + (int64_t)pid * p.ks_block;
-            const __nv_bfloat16* vp = vbase + (int64_t)pid * p.vs_block;
-#pragma unroll
-            for (int r = 0; r < (16 * CPR) / 32; ++r) {
-                const int id = r * 32 + lane;
-                const int t = id / CPR, c = id % CPR;
-                // slack slots of the last page and tokens left of a sliding window are zero-filled
-                const bool ok = tok0 + t < it.kv_end && tok0 + t >= it.kv_lo;
-                const int tt = ok ? t : 0;
-                cp_async16_hint(sbase + tile_off<16>(t, c), kp + tt * p.ks_token + c * 8, ok ? 16 : 0, stream_once);
-                cp_async16_hint(sbase + PAGE_BYTES + tile_off<16>(t, c), vp + tt * p.vs_token + c * 8, ok ? 16 : 0, stream_once);
-            }
-        };
-#pragma unroll
-        for (int s = 0; s < NSTAGE - 1; ++s) {
-            if (s < my_n) issue(s);
-            cp_async_commit();
-        }
-        for (int i = 0; i < my_n; ++i) {
-            cp_async_wait<NSTAGE - 2>();
-            __syncwarp();
-            if (i + NSTAGE - 1 < my_n) issue(i + NSTAGE - 1);
-            cp_async_commit();
-            use_page(i, wbase + (i % NSTAGE) * STAGE_BYTES, [&](int ks) { return tile_off<16>((lane & 7) + ((lane >> 3) & 1) * 8, 2 * ks + (lane >> 4)); },
-                     [&](int mt) { return tile_off<16>((lane & 7) + (lane >> 4) * 8, 2 * mt + ((lane >> 3) & 1)); });
         }
     }
     cp_async_wait<0>();
@@ -925,13 +864,13 @@ __global__ void __launch_bounds__(NWARPS * 32, 2) decode_splitk_kernel(const Att
 // One grid for a batch with shared prefixes: the first n_shared_ctas CTAs serve the shared chunks (longer items
 // first), the rest the sequences' own chunks.  Both kinds need half an SM's shared memory, so the larger register
 // footprint of the shared role costs no occupancy; batches without sharing launch decode_splitk_kernel.
-template <int D, int NWARPS, int NSTAGE, int NCG, int INL>
+template <int D, int NWARPS, int NSTAGE, int NCG, bool CONTIGUOUS, int INL>
 __global__ void __launch_bounds__(NWARPS * 32, 2) decode_with_shared_kernel(const AttnParams p, const __grid_constant__ PlanBytes<INL> inl, const int n_shared_ctas)
 {
     if (decode_extra_cta(p)) return;
     const uint8_t* const plan = INL > 0 ? inl.bytes : p.plan.base;
     if ((int)blockIdx.x < n_shared_ctas) decode_shared_cta<D, NWARPS, NSTAGE, NCG>(p, plan, (int)blockIdx.x);
-    else decode_cta<D, NWARPS, NSTAGE, false, false>(p, plan, (int)blockIdx.x - n_shared_ctas);
+    else decode_cta<D, NWARPS, NSTAGE, CONTIGUOUS>(p, plan, (int)blockIdx.x - n_shared_ctas);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1052,8 +991,8 @@ static cudaError_t launch_decode_shared_t(const AttnParams& p, const HostPlan& h
     const size_t ring = (size_t)kDecWarps * STAGES * 2 * 16 * D * 2;
     const size_t merge = (size_t)kDecWarps * COLS * (D + 4) * 4 + (size_t)kDecWarps * COLS * 4 * 2;
     const int n_shared_ctas = n_shared_items * p.Hkv;
-    return with_plan_bytes(hp, [&](auto size, const auto* inl) {
-        return launch_decode_grid<decode_with_shared_kernel<D, kDecWarps, STAGES, NCG, decltype(size)::value>>(
+    return with_layout<D>(p, hp, [&](auto contiguous, auto size, const auto* inl) {
+        return launch_decode_grid<decode_with_shared_kernel<D, kDecWarps, STAGES, NCG, decltype(contiguous)::value, decltype(size)::value>>(
             (n_shared_items + n_items) * p.Hkv, std::max(ring, merge), stream, p, inl, &n_shared_ctas);
     });
 }
