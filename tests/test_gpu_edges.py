@@ -129,14 +129,19 @@ def test_decode_chunk_lengths(Hq, Hkv, D, fp8, lens):
 
 @pytest.mark.parametrize("Hq,Hkv,D,fp8,layout", [(16, 2, 64, False, "HND"), (8, 2, 128, False, "HND"), (16, 2, 128, True, "HND"),
                                                  (16, 2, 64, False, "NHD"), (8, 2, 128, False, "NHD")])
-@pytest.mark.parametrize("window", [0, 83])
+@pytest.mark.parametrize("window", [0, 83, 2500])
 def test_decode_rings_of_every_depth(Hq, Hkv, D, fp8, layout, window):
-    """A decode warp's ring holds three or four pages; whole pages of contiguous tokens are copied
-    with constant offsets, the others token by token: every number of pages per warp around the ring's depth, past the 32 block
-    ids that a warp keeps, whole and cut last pages, a window's edge inside a page, both pool layouts."""
+    """A decode warp's ring holds three or four pages, and the warp keeps 32 block ids: every number of pages per warp around the
+    ring's depth, past 32 and 64 ids, whole and cut last pages, a window's edge inside a page, both pool layouts.  The shortest
+    chunk is set above every sequence's length, so that a warp has a quarter of its pages."""
     lens = [max(1, 16 * pages + extra) for pages in (0, 1, 2, 3, 4, 7, 8, 12, 13, 16, 19, 20, 24, 127, 130, 261) for extra in (0, 1, 15)]
+    d = cf.make_desc(Hq, Hkv, D, 16, 4096, window_size=window)
+    dec = cf.cf_plan_inspect(d, lens, [1] * len(lens), 512, decode_min_chunk_pages=272)[1]
+    pages = np.ceil((dec[:, 3] - dec[:, 2]) / 16).astype(int)
+    assert len(dec) == len(lens) and {1, 2, 3, 4, 5} <= set(pages.tolist()) and pages.max() == (262 if window == 0 else 7 if window == 83 else 158)
     scales = (np.full(Hkv, 0.02, np.float32), np.full(Hkv, 0.015, np.float32)) if fp8 else None
-    run_and_check(small(83, Hq, Hkv, D, [l - 1 for l in lens], [[1] * len(lens)], NB=4096), fp8=scales, layout=layout, window=window)
+    run_and_check(small(83, Hq, Hkv, D, [l - 1 for l in lens], [[1] * len(lens)], NB=4096), fp8=scales, layout=layout, window=window,
+                  debug={cf.CF_DEBUG_DECODE_MIN_CHUNK_PAGES: 272})
 
 
 @pytest.mark.parametrize("Hq,Hkv,D,fp8", [(16, 2, 64, False), (8, 2, 128, False), (16, 2, 128, True)])
